@@ -1,369 +1,244 @@
 // sg_score: window-query x key-cache scoring with a fused softmax and row-reduce (sm_100a).
 //
-// For one (layer, sequence, KV head) the R = G*W window queries are scored against all N keys:
-// a dense R x N x d contraction, so it runs on the 5th-generation tensor cores.  importance[t] =
-// sum_r softmax_row_r(s)[t] needs every row's normaliser before any probability can be summed
-// down a column, so the work is two passes over the keys:
+// For one (layer, sequence, KV head) -- a "part" -- the R = G*W window queries are scored against all N keys: a dense
+// R x N x d contraction, so it runs on the 5th-generation tensor cores.  importance[t] = sum_r softmax_row_r(s)[t] needs
+// every row's normaliser before any probability can be summed down a column, so the work is two passes over the keys,
+// each a kernel of its own:
 //
 //   pass 1 (row statistics)  D[row r][key t]  = Q_blk (A, 128 rows) x K_tile^T (B, 128 keys):
 //          each epilogue thread owns one query row (one TMEM lane) and keeps a running
-//          (max, sum-of-exp2) over the key columns -- no cross-thread reduction.
-//   pass 2 (column sums)     D[key t][row r]  = K_tile (A, 128 keys) x Q_blk^T (B, <=128 rows):
+//          (reference, sum of exp2) over the key columns -- no cross-thread reduction.
+//   pass 2 (column sums)     D[key t][row r]  = K_tile (A, 128 keys) x Q_blk^T (B, 128 rows):
 //          each epilogue thread owns one key (one TMEM lane) and adds exp2(s*c - lse_r) over the
 //          query-row columns; lse_r is a per-column constant read from shared memory.
 //
-// One persistent kernel runs both passes: one warp feeds Q and 128-key K tiles with TMA into 128-byte-swizzled
-// shared memory, one thread issues tcgen05.mma into four 128-column TMEM accumulator stages (one per epilogue
-// warpgroup), sixteen epilogue warps (four warpgroups, each owning every fourth block) drain them with tcgen05.ld.
-// The score matrix never leaves the SM.  Work items (a pass, a layer/KV head, a chunk of key tiles of one sequence)
-// are laid out so that pass 2 of a (layer, KV head) unit follows its pass 1 by a lag of a few units: close enough that
-// the unit's keys are still in L2 for the second read (K crosses HBM once), far enough that the statistics pass 2
-// needs are already published.  The epilogue warpgroups never meet at a CTA-wide barrier: each walks the items on its
-// own and only waits for accumulators; two helper warps do everything else at item boundaries -- they merge and
-// publish the row statistics of finished pass-1 items, bump a per-unit counter, wait (bounded) on that counter for
-// the CTA's next pass-2 item and merge the chunks' statistics into its rows' log-sum-exps, one item ahead of the
-// epilogue.  A pass-2 item only depends on items at smaller schedule positions and pass-1 items never wait, so the
-// schedule cannot deadlock for any grid size.
+// The score matrix never leaves the SM.  The key tiles of all parts of a launch, in order, are cut into one contiguous
+// range per CTA, so every CTA has the same work to within a tile; a CTA's piece of a part is a "segment".  Pass 1 leaves one
+// record per segment ((reference, sum) of every row), pass 2 merges a part's records into its rows' log-sum-exps.  The
+// kernel boundary is the only synchronisation between CTAs: measured against one persistent kernel that ran both passes
+// behind per-part counters in global memory, no CTA waits for another CTA's statistics in mid-kernel (a third of the time
+// of a one-layer call), and each kernel holds one hot loop.  The launches follow one another by programmatic dependent
+// launch: a kernel sets itself up and requests its first tiles while the one before it drains.
+//
+// Roles of a CTA (one per SM): twelve epilogue warps (three warpgroups, each taking every third block, a block being a
+// key tile x row block), one warp feeding Q and 128-key K tiles with TMA into 128-byte-swizzled shared memory, one issuing
+// tcgen05.mma into four 128-column TMEM stages, two helper warps (merging statistics and, for several row blocks per
+// tile, adding up the warpgroups' column sums) off the epilogue's path.
 //
 // Every wait is bounded: on expiry the CTA raises SG_ERR_TIMEOUT in the status word, stops issuing work, waits
 // (bounded) for its own TMA copies and MMAs, frees its TMEM and returns.
 #include <cuda.h>
 
-#include <vector>
-
 #include "common.cuh"
 #include "launch.h"
+#include "tcgen05.cuh"
 
 namespace sg {
 namespace {
 
-constexpr int kEpiGroups = 4;             // epilogue warpgroups (four warps each, one per TMEM lane quarter)
-constexpr int kEpiThreads = 128 * kEpiGroups;
-// Warp roles: warps 0-15 are the epilogue (four hardware-aligned warpgroups), warp 16 feeds TMA, warp 17 issues the MMAs and owns the TMEM allocation, warps 18 and 19 (the helpers)
-// merge row statistics off the epilogue's path.
-constexpr int kTmaWarp = kEpiThreads / 32;
-constexpr int kMmaWarp = kTmaWarp + 1;
-constexpr int kHelperWarp = kTmaWarp + 2;
-constexpr int kScoreThreads = kEpiThreads + 128;
+constexpr int kGroups = 3;                // epilogue warpgroups (four warps each, one per TMEM lane quarter)
+constexpr int kEpiWarps = 4 * kGroups;
+constexpr int kTmaWarp = kEpiWarps, kMmaWarp = kTmaWarp + 1, kHelperWarp = kMmaWarp + 1 /* two */;
+constexpr int kThreads = 32 * (kHelperWarp + 2);
 constexpr int kTileKeys = 128;
-constexpr int kAccStages = 4;             // 4 x 128 fp32 columns = the whole 512-column TMEM
-constexpr int kPartSlots = 8;             // pass 2, several row blocks per key tile: partial column sums of up to 8 tiles in flight
-constexpr uint32_t kTmemCols = 512;
+constexpr int kStages = 4;                // 4 x 128 fp32 columns = the whole 512-column TMEM
+constexpr int kColSlots = 4;              // pass 2, several row blocks per tile: partial column sums of four tiles in flight
 constexpr int kMaxKStages = 4;
 constexpr int kSmemLimit = 232448;        // 227 KB opt-in dynamic shared memory per CTA
 constexpr float kLog2e = 1.4426950408889634f;
 
-// Profiling build (-DSG_SCORE_PROFILE): selected threads add up the clocks they spend in each kind of wait and
-// write the sums behind the CTA's four clock words of the testing clock buffer (32 words per CTA).
-#ifdef SG_SCORE_PROFILE
-#define SG_PROF_DECL(...) long long __VA_ARGS__
-#define SG_PROF_BEGIN(t) const long long t = clock64()
-#define SG_PROF_ADD(acc, t) acc += clock64() - (t)
-#define SG_PROF_INC(acc) acc += 1
-#define SG_PROF_STORE(slot, v) do { if (p.clock_out) p.clock_out[32 * (size_t)blockIdx.x + (slot)] = (unsigned long long)(v); } while (0)
-constexpr int kClockWords = 32;
-#else
-#define SG_PROF_DECL(...)
-#define SG_PROF_BEGIN(t)
-#define SG_PROF_ADD(acc, t)
-#define SG_PROF_INC(acc)
-#define SG_PROF_STORE(slot, v)
-constexpr int kClockWords = 4;
-#endif
-
-// Debug build (-DSG_CHECKS): device-side checks of the shared-memory carve-up, of every TMA coordinate (16-byte
-// aligned innermost coordinate, tile inside the tensor or hanging over its end only where the fill value is
-// wanted) and of every TMEM address against the allocation.  A failed check never traps: it sets the
-// SG_ERR_INVALID bit of the status word and the access is still made only if it is known to be harmless (TMA
-// loads past the end are zero-filled by the hardware), so a debug run ends like any other and reports the bit.
+// Debug build (-DSG_CHECKS): device-side checks of the shared-memory carve-up and of every TMA coordinate (tile inside
+// the tensor or hanging over its end only where the fill value is wanted).  A failed check never traps: it sets the
+// SG_ERR_INVALID bit of the status word and the access is still made only if it is known to be harmless (TMA loads
+// past the end are zero-filled by the hardware), so a debug run ends like any other and reports the bit.
 #ifdef SG_CHECKS
 #define SG_CHECK(cond) do { if (!(cond)) raise(p.dev_status, SG_ERR_INVALID); } while (0)
 #else
 #define SG_CHECK(cond) do { } while (0)
 #endif
 
+// Profiling build (-DSG_SCORE_PROFILE): the MMA warp and one warp per warpgroup add up the clocks they spend waiting; the
+// sums go behind the CTA's four clock words of the testing clock buffer (32 words per CTA).
+#ifdef SG_SCORE_PROFILE
+constexpr int kClockWords = 32;
+#define SG_PROF_WAIT(acc, expr) do { const long long _t = clock64(); expr; acc += clock64() - _t; } while (0)
+#define SG_PROF_STORE(slot, v) do { if (p.clock_out && lane == 0) p.clock_out[32 * (size_t)blockIdx.x + (slot)] = (unsigned long long)(v); } while (0)
+#else
+constexpr int kClockWords = 4;
+#define SG_PROF_WAIT(acc, expr) do { expr; } while (0)
+#define SG_PROF_STORE(slot, v) do { (void)(v); } while (0)
+#endif
+
 struct ScoreParams {
   const int32_t* cu;
   float* importance;
-  int* p1_done;            // [U] per unit: two counts per published pass-1 item, one per helper warp (zeroed by the host call)
-  float2* part;            // [U][max_items][Ralloc] per-item row statistics (log2-domain max, sum of exp2)
+  float2* records;         // [parts of the group + CTAs][Ralloc] row statistics (log2-domain reference, sum of exp2) of a segment
   int32_t* dev_status;
   int64_t T;
-  int32_t B, Hkv, G, W, R, Rpad, Ralloc;
-  int32_t U;               // units = layers x KV heads
-  int32_t lag;             // pass 2 of unit u is scheduled `lag` units after its pass 1
-  int32_t compact;         // schedule layout: 0 = every slot 2*C positions, 1 = positions without an item removed
-  int32_t tiles_per_chunk, max_items, k_stages, q_bufs;
+  int32_t B, Hkv, G, W, R, Ralloc;
+  int32_t u0, units;       // the launch's (layer, KV head) units
+  int32_t k_stages, q_bufs;
+  int32_t more;            // another launch of the same call follows
   int32_t smem_bytes;      // dynamic shared memory of the launch (debug checks)
-  int32_t wgslots;         // statistics slots per item: 4 (one per epilogue warpgroup) or 1 (every row block has one owner)
-  int32_t withhold_unit;   // testing only: pass-1 items of this unit are never counted as done (-1 = none)
+  int32_t withhold_unit;   // testing only: the statistics of this unit's segments are never handed to the helpers (-1 = none)
   uint32_t wait_ns;        // limit of every bounded wait, nanoseconds
   unsigned long long* clock_out;   // testing only: per CTA {clock64 start, end, globaltimer start, end}, or null
   float scale_log2;
 };
 
-// ---------------------------------------------------------------- PTX wrappers
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+// ---------------------------------------------------------------- exponentials
+// The SFU gives 16 exp2 per clock and SM and is the first unit to fill up: a 128 x 128 block is 1024 clocks of it, while
+// the FMA pipe has 256 clocks of work (scale and sum, two at a time).  So a share of the exponentials is computed on the
+// FMA pipe with packed fp32 instructions.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
 }
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
 }
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
 }
-__device__ __forceinline__ uint64_t global_timer_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
 }
-// One try_wait: true when the phase has completed.
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
+__device__ __forceinline__ uint64_t pair_of(const uint32_t* v) { return pack2(__uint_as_float(v[0]), __uint_as_float(v[1])); }
+__device__ __forceinline__ uint64_t exp2_sfu2(uint64_t x) {
+  float x0, x1;
+  unpack2(x, x0, x1);
+  return pack2(exp2f(x0), exp2f(x1));
 }
-// Bounded wait: gives up after `limit_ns` (about one second in normal use), or once another thread has set
-// *abort_flag.  try_wait comes back after a short, hardware-chosen time whether or not the phase has completed, so a
-// thread that simply retries spins through a dozen instructions per attempt -- issue slots and, worse, entries of the
-// queue that the SFU instructions of the working warps go through (measured: one retry per 11 clocks and SM, 60 % of
-// all executed instructions, SFU pipe at 51 %).  A waiter therefore sleeps `sleep_ns` between attempts (chosen per
-// role: short on the MMA thread's critical path, long for the producer that runs ahead) and looks at the clock and the
-// abort flag only every 64th attempt.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, uint32_t limit_ns,
-                                          uint32_t sleep_ns) {
-  if (mbar_test(bar, parity)) return true;
-  uint64_t t0 = 0;
-  for (uint32_t it = 0;; ++it) {
-    if (sleep_ns) __nanosleep(sleep_ns);
-    if (mbar_test(bar, parity)) return true;
-    if ((it & 63u) == 63u) {
-      if (*abort_flag) return false;
-      const uint64_t now = global_timer_ns();
-      if (t0 == 0) t0 = now;
-      else if (now - t0 > (uint64_t)limit_ns) { *abort_flag = 1; return false; }
-    }
-  }
+// Two exp2 on the FMA pipe: x = n + f with n an integer and |f| <= 1/2, 2^f by a polynomial of degree 5 (minimax fit of
+// 2^f by iterated weighted least squares, constant term 1; relative error at most 1.6e-7 including the fp32 evaluation),
+// n added to the exponent field.  x is clamped to -127, where the sum of the exponent fields is 0, a subnormal that every
+// later operation flushes, and, where x may be large (pass 1, against a stale reference), to 127: a huge finite number,
+// which trips the range test of pass 1 as the SFU's inf does.
+template <bool kAbove>
+__device__ __forceinline__ uint64_t exp2_fma2(uint64_t x) {
+  float x0, x1;
+  unpack2(x, x0, x1);
+  x0 = fmaxf(x0, -127.f);
+  x1 = fmaxf(x1, -127.f);
+  if (kAbove) { x0 = fminf(x0, 127.f); x1 = fminf(x1, 127.f); }
+  x = pack2(x0, x1);
+  const uint64_t t = add2(x, pack2(12582912.f, 12582912.f));                 // 1.5 * 2^23: the low bits of t are round(x)
+  const uint64_t f = fma2(add2(t, pack2(-12582912.f, -12582912.f)), pack2(-1.f, -1.f), x);
+  uint64_t q = fma2(pack2(0.001326472731307149f, 0.001326472731307149f), f, pack2(0.009671512991189957f, 0.009671512991189957f));
+  q = fma2(q, f, pack2(0.05550733581185341f, 0.05550733581185341f));
+  q = fma2(q, f, pack2(0.24022242426872253f, 0.24022242426872253f));
+  q = fma2(q, f, pack2(0.6931470036506653f, 0.6931470036506653f));
+  q = fma2(q, f, pack2(1.f, 1.f));
+  float q0, q1, t0, t1;
+  unpack2(q, q0, q1);
+  unpack2(t, t0, t1);
+  return pack2(__int_as_float(__float_as_int(q0) + (__float_as_int(t0) << 23)), __int_as_float(__float_as_int(q1) + (__float_as_int(t1) << 23)));
 }
-__device__ __forceinline__ void fence_barrier_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2, int c3) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-      ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
-}
-__device__ __forceinline__ void tmem_alloc(uint32_t smem_dst, uint32_t cols) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(cols) : "memory");
-}
-__device__ __forceinline__ void tmem_relinquish() {
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
-}
-// D[tmem] = A[smem] * B[smem], bf16 x bf16 -> fp32, issued by one thread; the operands are shared-memory matrix
-// descriptors given as their low words (address field), the high word is the same for every operand.
-// All MMAs of one accumulator block in a single statement: NK k-steps of 16 elements, four per 128-byte
-// sub-tile (descriptor low word += 2 per step inside a sub-tile, += a_sub / b_sub to the next sub-tile).  The first
-// MMA overwrites the accumulator, the others add to it.  One statement keeps the issuing thread's instruction
-// stream to the bare minimum between two blocks: the tensor pipe drains its short queue within ~200 clocks of the
-// last issue, so every clock spent between blocks is an idle clock of the pipe.
-template <int NK>
-__device__ __forceinline__ void umma_block(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t a_sub, uint32_t b_sub,
-                                           uint32_t desc_hi, uint32_t idesc) {
-  static_assert(NK == 4 || NK == 8, "one or two 64-element sub-tiles along d");
-  if (NK == 8) {
-    asm volatile(
-        "{\n\t.reg .b64 da, db;\n\t.reg .b32 a, b;\n\t.reg .pred pf, pt;\n\t"
-        "setp.ne.u32 pf, %0, %0;\n\tsetp.eq.u32 pt, %0, %0;\n\t"
-        "mov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %6, pf;\n\t"
-        "add.u32 a, %1, 2;\n\tadd.u32 b, %2, 2;\n\tmov.b64 da, {a, %5};\n\tmov.b64 db, {b, %5};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %6, pt;\n\t"
-        "add.u32 a, %1, 4;\n\tadd.u32 b, %2, 4;\n\tmov.b64 da, {a, %5};\n\tmov.b64 db, {b, %5};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %6, pt;\n\t"
-        "add.u32 a, %1, 6;\n\tadd.u32 b, %2, 6;\n\tmov.b64 da, {a, %5};\n\tmov.b64 db, {b, %5};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %6, pt;\n\t"
-        "add.u32 a, %1, %3;\n\tadd.u32 b, %2, %4;\n\tmov.b64 da, {a, %5};\n\tmov.b64 db, {b, %5};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %6, pt;\n\t"
-        "add.u32 a, a, 2;\n\tadd.u32 b, b, 2;\n\tmov.b64 da, {a, %5};\n\tmov.b64 db, {b, %5};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %6, pt;\n\t"
-        "add.u32 a, a, 2;\n\tadd.u32 b, b, 2;\n\tmov.b64 da, {a, %5};\n\tmov.b64 db, {b, %5};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %6, pt;\n\t"
-        "add.u32 a, a, 2;\n\tadd.u32 b, b, 2;\n\tmov.b64 da, {a, %5};\n\tmov.b64 db, {b, %5};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %6, pt;\n\t}"
-        ::"r"(tmem_d), "r"(a_lo), "r"(b_lo), "r"(a_sub), "r"(b_sub), "r"(desc_hi), "r"(idesc) : "memory");
-  } else {
-    asm volatile(
-        "{\n\t.reg .b64 da, db;\n\t.reg .b32 a, b;\n\t.reg .pred pf, pt;\n\t"
-        "setp.ne.u32 pf, %0, %0;\n\tsetp.eq.u32 pt, %0, %0;\n\t"
-        "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, pf;\n\t"
-        "add.u32 a, %1, 2;\n\tadd.u32 b, %2, 2;\n\tmov.b64 da, {a, %3};\n\tmov.b64 db, {b, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, pt;\n\t"
-        "add.u32 a, %1, 4;\n\tadd.u32 b, %2, 4;\n\tmov.b64 da, {a, %3};\n\tmov.b64 db, {b, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, pt;\n\t"
-        "add.u32 a, %1, 6;\n\tadd.u32 b, %2, 6;\n\tmov.b64 da, {a, %3};\n\tmov.b64 db, {b, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, pt;\n\t}"
-        ::"r"(tmem_d), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc) : "memory");
-  }
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-// TMEM load of 32 consecutive fp32 columns of this thread's lane, issued without waiting: the registers hold
-// the data only after tmem_ld_wait().  A warp issues the load of its next 32 columns before it works on the
-// current ones, so the load's latency is covered by arithmetic.
-__device__ __forceinline__ void tmem_ld32_issue(uint32_t (&r)[32], uint32_t taddr) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr) : "memory");
-}
-// Waits for the thread's outstanding TMEM loads.  The empty statements that follow tie the 32 registers of the
-// load that has just completed to this point of the program: volatile statements keep their order, and every
-// later use of the registers depends on them, so the compiler cannot schedule arithmetic on the data ahead of the wait.
-__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[32]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+// Pairs of a 32-column chunk's sixteen whose exponentials run on the FMA pipe, spread evenly.
+constexpr int kFmaPairs1 = 4, kFmaPairs2 = 4;
+__device__ __forceinline__ constexpr bool on_fma(int pair, int share) { return ((pair + 1) * share) / 16 != (pair * share) / 16; }
+// Pass 1: adds exp2(score * scale - m) of a chunk's 32 columns to two pairs of accumulators (nm2 = {-m, -m}).
+__device__ __forceinline__ void chunk_rows(uint32_t (&cur)[32], uint64_t scale2, uint64_t nm2, uint64_t& s0, uint64_t& s1) {
 #pragma unroll
-  for (int i = 0; i < 32; i += 8)
-    asm volatile("" : "+r"(r[i]), "+r"(r[i + 1]), "+r"(r[i + 2]), "+r"(r[i + 3]), "+r"(r[i + 4]), "+r"(r[i + 5]),
-                      "+r"(r[i + 6]), "+r"(r[i + 7]) :: "memory");
-}
-
-// Shared-memory matrix descriptor of a K-major bf16 tile stored as rows of 128 bytes with the
-// 128-byte swizzle (what TMA writes with CU_TENSOR_MAP_SWIZZLE_128B).  High word: 8-row groups are 1024
-// bytes apart (stride byte offset, bits [32,46)), descriptor version 1 for sm_100 (bit 46), layout type
-// SWIZZLE_128B = 2 (bits [61,64)); the leading byte offset is unused for this layout.  Low word: the start
-// address in 16-byte units (bits [0,14)); advancing 16 elements along K inside the 128-byte span adds 2.
-constexpr uint32_t kSmemDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
-__device__ __forceinline__ uint32_t smem_desc_lo(uint32_t addr) { return (addr & 0x3FFFFu) >> 4; }
-// Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M x N tile.
-__device__ __forceinline__ uint32_t make_idesc(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-// Position in the persistent schedule -> work item.  The schedule is a sequence of slots; slot s holds the
-// pass-2 items of unit (s - lag) followed by the pass-1 items of unit s, a unit being one (layer, KV head)
-// with all its sequences (C items per pass).  CTA k walks positions k, k + grid, k + 2*grid, ...  A pass-2
-// item depends only on pass-1 items at smaller positions, and pass-1 items never wait, so the item at the
-// smallest unfinished position can always run: the schedule cannot deadlock whatever the grid size.
-// With few units (lag >= U) the schedule is simply all pass-1 items followed by all pass-2 items.
-struct SchedPos { int pass, unit, j; };    // pass 0 = no item at this position
-__host__ __device__ __forceinline__ long long schedule_length(int U, int C, int lag, bool compact) {
-  return (lag >= U || compact) ? (long long)U * 2 * C : (long long)(U + lag) * 2 * C;
-}
-// Three layouts.  lag >= U (few units): all pass-1 items, then all pass-2 items.  Padded: every slot has
-// 2*C positions, those of units that do not exist are empty (the first and the last `lag` slots are half
-// empty).  Compact: the same order with the empty positions removed.  Which of the last two finishes first
-// depends on how the items fall on the CTAs; the host simulates both and picks (see choose_layout).
-__host__ __device__ __forceinline__ SchedPos schedule_position(long long pos, int U, int C, int lag, bool compact) {
-  SchedPos sp;
-  if (lag >= U) {
-    const long long half = (long long)U * C;
-    const long long q = pos < half ? pos : pos - half;
-    sp.unit = (int)(q / C); sp.j = (int)(q - (long long)sp.unit * C); sp.pass = pos < half ? 1 : 2;
-    return sp;
+  for (int i = 0; i < 16; i += 2) {
+    const uint64_t x0 = fma2(pair_of(cur + 2 * i), scale2, nm2), x1 = fma2(pair_of(cur + 2 * i + 2), scale2, nm2);
+    s0 = add2(s0, on_fma(i, kFmaPairs1) ? exp2_fma2<true>(x0) : exp2_sfu2(x0));
+    s1 = add2(s1, on_fma(i + 1, kFmaPairs1) ? exp2_fma2<true>(x1) : exp2_sfu2(x1));
   }
-  if (compact) {
-    const long long head = (long long)lag * C, mid = (long long)(U - lag) * 2 * C;
-    if (pos < head) {
-      sp.unit = (int)(pos / C); sp.j = (int)(pos - (long long)sp.unit * C); sp.pass = 1;
-      return sp;
-    }
-    if (pos >= head + mid) {
-      const long long q = pos - head - mid;
-      const int k = (int)(q / C);
-      sp.unit = U - lag + k; sp.j = (int)(q - (long long)k * C); sp.pass = 2;
-      return sp;
-    }
-    pos += head;                                   // inside the middle part both layouts agree up to this shift
+}
+// Pass 2: adds exp2(score * scale + nl[column]) of a chunk's 32 columns (nl = negated log-sum-exps).
+__device__ __forceinline__ void chunk_cols(uint32_t (&cur)[32], uint64_t scale2, const float* nl, uint64_t& s0, uint64_t& s1) {
+#pragma unroll
+  for (int i = 0; i < 16; i += 2) {
+    const float4 l4 = *reinterpret_cast<const float4*>(nl + 2 * i);
+    const uint64_t x0 = fma2(pair_of(cur + 2 * i), scale2, pack2(l4.x, l4.y));
+    const uint64_t x1 = fma2(pair_of(cur + 2 * i + 2), scale2, pack2(l4.z, l4.w));
+    s0 = add2(s0, on_fma(i, kFmaPairs2) ? exp2_fma2<false>(x0) : exp2_sfu2(x0));
+    s1 = add2(s1, on_fma(i + 1, kFmaPairs2) ? exp2_fma2<false>(x1) : exp2_sfu2(x1));
   }
-  const int slot = (int)(pos / (2 * C));
-  const int r = (int)(pos - (long long)slot * (2 * C));
-  if (r < C) { sp.unit = slot - lag; sp.j = r; sp.pass = 2; } else { sp.unit = slot; sp.j = r - C; sp.pass = 1; }
-  if (sp.unit < 0 || sp.unit >= U) sp.pass = 0;
-  return sp;
 }
 
-struct ScoreItem {
-  int pass;          // 1 or 2; 0 = no item at this position
-  int unit, l, g, b;
-  int c0, N;         // first token and length of sequence b
-  int tile_beg, tile_end;
-  int item_in_unit;  // this item's index among the unit's C items (its partial-statistics slot)
-  int first_item_b;  // index of sequence b's first item in the unit
-  int nch_b;         // number of items (chunks) of sequence b
+// ---------------------------------------------------------------- schedule
+// CTAs that get tiles (the host sizes the grid by an upper bound of the tile count).
+__device__ __forceinline__ int busy_ctas(long long tt) { return tt < (long long)gridDim.x ? (int)tt : (int)gridDim.x; }
+// The CTA whose range holds tile `pos` of the launch's `tt`.
+__device__ __forceinline__ int cta_of(long long pos, long long tt, int busy) { return (int)(((pos + 1) * busy - 1) / tt); }
+// A CTA's segments: its range of the launch's key tiles [c * tt / busy, (c + 1) * tt / busy), cut at part boundaries.
+struct Segment {
+  int u, b;                // unit (counted over the whole call) and sequence
+  int c0, N;               // first token and length of sequence b
+  int tile_beg, tile_end;  // tiles of the part
+  int part;                // part within the launch
+};
+struct SegmentWalk {
+  int C, B, u0, pos, end;
+  const int *cu, *prefix;  // prefix[b] = tiles of the sequences before b (prefix[B] = C)
+  __device__ __forceinline__ SegmentWalk(int C_, int units, int B_, int u0_, const int* cu_, const int* prefix_)
+      : C(C_), B(B_), u0(u0_), cu(cu_), prefix(prefix_) {
+    const long long tt = (long long)units * C;
+    const int g = busy_ctas(tt);
+    pos = (int)blockIdx.x < g ? (int)(tt * blockIdx.x / g) : 0;
+    end = (int)blockIdx.x < g ? (int)(tt * (blockIdx.x + 1) / g) : 0;
+  }
+  __device__ __forceinline__ bool next(Segment& s) {
+    if (pos >= end) return false;
+    const int ul = pos / C, j = pos - ul * C;
+    int lo = 0, hi = B;
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (prefix[mid] <= j) lo = mid; else hi = mid;
+    }
+    s.u = u0 + ul;
+    s.b = lo;
+    s.c0 = cu[lo];
+    s.N = cu[lo + 1] - s.c0;
+    s.tile_beg = j - prefix[lo];
+    s.tile_end = min(prefix[lo + 1] - prefix[lo], s.tile_beg + (end - pos));
+    s.part = ul * B + lo;
+    pos += s.tile_end - s.tile_beg;
+    return true;
+  }
 };
 
-// s_cu[b] = cu_seqlens[b]; s_prefix[b] = number of items of the sequences before b (s_prefix[B] = C).
-__device__ __forceinline__ ScoreItem decode_position(const ScoreParams& p, long long pos, const int* s_cu, const int* s_prefix) {
-  ScoreItem it;
-  it.pass = 0;
-  const int C = s_prefix[p.B];
-  const SchedPos sp = schedule_position(pos, p.U, C, p.lag, p.compact != 0);
-  it.pass = sp.pass;
-  const int unit = sp.unit, j = sp.j;
-  if (it.pass == 0) return it;
-  it.unit = unit;
-  it.l = unit / p.Hkv;
-  it.g = unit - it.l * p.Hkv;
-  it.item_in_unit = j;
-  int lo = 0, hi = p.B;                                  // largest b with s_prefix[b] <= j
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (s_prefix[mid] <= j) lo = mid; else hi = mid;
+// Log-sum-exps of a part's rows from its segments' records: rows r0, r0 + step, ..., kFlight records in flight.  Negated, as
+// the epilogue of pass 2 adds them; rows outside the window get -inf: exp2(x - inf) = 0.
+template <int kFlight>
+__device__ __forceinline__ void merge_records(const ScoreParams& p, const Segment& sg, const int* prefix, int C, float* neg_lse, int r0, int step) {
+  const long long tt = (long long)p.units * C, first = (long long)(sg.u - p.u0) * C + prefix[sg.b];
+  const int busy = busy_ctas(tt), Weff = min(p.W, sg.N);
+  const int c_lo = cta_of(first, tt, busy), nrec = cta_of(first + (prefix[sg.b + 1] - prefix[sg.b]) - 1, tt, busy) - c_lo + 1;
+  for (int r = r0; r < p.Ralloc; r += step) {
+    const float2* rec = p.records + (size_t)(sg.part + c_lo) * p.Ralloc + r;
+    float M = -INFINITY, L = 0.f;
+    for (int i0 = 0; i0 < nrec; i0 += kFlight) {
+      float2 v[kFlight];
+#pragma unroll
+      for (int i = 0; i < kFlight; ++i) v[i] = i0 + i < nrec ? __ldcg(rec + (size_t)(i0 + i) * p.Ralloc) : make_float2(-INFINITY, 0.f);
+      float m = v[0].x;
+#pragma unroll
+      for (int i = 1; i < kFlight; ++i) m = fmaxf(m, v[i].x);
+      if (m != -INFINITY) {                            // else nothing of row r is visible in these segments
+        const float Mn = fmaxf(M, m);
+        float acc = L * exp2f(M - Mn);
+#pragma unroll
+        for (int i = 0; i < kFlight; ++i) acc += v[i].y * exp2f(v[i].x - Mn);    // a (-inf, 0) pair adds 0
+        M = Mn; L = acc;
+      }
+    }
+    neg_lse[r] = (r < p.R && r / p.G < Weff) ? -(M + log2f(L)) : -INFINITY;
   }
-  it.b = lo;
-  it.first_item_b = s_prefix[lo];
-  it.nch_b = s_prefix[lo + 1] - it.first_item_b;
-  it.c0 = s_cu[lo];
-  it.N = s_cu[lo + 1] - it.c0;
-  const int tiles_total = (it.N + kTileKeys - 1) / kTileKeys;
-  it.tile_beg = (j - it.first_item_b) * p.tiles_per_chunk;
-  it.tile_end = min(tiles_total, it.tile_beg + p.tiles_per_chunk);
-  return it;
 }
 
-__device__ __forceinline__ int ld_acquire_gpu(const int* ptr) {
-  int v;
-  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(ptr) : "memory");
-  return v;
-}
-// Rare path of pass 1: the sum of a 32-column chunk against the running reference m left the safe range (a value far
-// above m, or m still -inf at the start of a work item).  Takes the chunk's maximum, rescales the running sum and adds
-// the chunk against the new reference.  Kept out of line so that the hot loop holds nothing but its 32 x (fma, ex2, add).
-// (Everything is passed and returned by value: taking the address of the chunk's registers or of the running statistics
-// would move them to local memory in the hot loop as well.)
-__device__ __noinline__ float2 refresh_reference(float scale_log2, float m, float lsum, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, uint32_t c4, uint32_t c5, uint32_t c6, uint32_t c7, uint32_t c8, uint32_t c9, uint32_t c10, uint32_t c11, uint32_t c12, uint32_t c13, uint32_t c14, uint32_t c15, uint32_t c16, uint32_t c17, uint32_t c18, uint32_t c19, uint32_t c20, uint32_t c21, uint32_t c22, uint32_t c23, uint32_t c24, uint32_t c25, uint32_t c26, uint32_t c27, uint32_t c28, uint32_t c29, uint32_t c30, uint32_t c31) {
-  const uint32_t cur[32] = {c0, c1, c2, c3, c4, c5, c6, c7, c8, c9, c10, c11, c12, c13, c14, c15, c16, c17, c18, c19, c20, c21, c22, c23, c24, c25, c26, c27, c28, c29, c30, c31};
-  float mx = __uint_as_float(cur[0]);
-#pragma unroll
-  for (int c = 1; c < 32; ++c) mx = fmaxf(mx, __uint_as_float(cur[c]));
-  const float mn = fmaxf(m, mx * scale_log2);
-  float r0 = 0.f, r1 = 0.f;
-#pragma unroll
-  for (int c = 0; c < 32; c += 2) {
-    r0 += exp2f(fmaf(__uint_as_float(cur[c]), scale_log2, -mn));
-    r1 += exp2f(fmaf(__uint_as_float(cur[c + 1]), scale_log2, -mn));
-  }
-  return make_float2(mn, lsum * exp2f(m - mn) + (r0 + r1));
-}
-
-template <int D>
-__global__ void __launch_bounds__(kScoreThreads, 1)
+template <int D, int PASS>
+__global__ void __launch_bounds__(kThreads, 1)
 score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k, const ScoreParams p) {
   constexpr int kSub = D / 64;                        // 64-element (128-byte) sub-tiles along d
   constexpr int kKSubBytes = kTileKeys * 128;         // one sub-tile of a K stage
@@ -374,67 +249,72 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
   const int q_buf_bytes = kSub * q_sub_bytes;
   uint8_t* q_smem = smem;                                            // [q_bufs] Q operands
   uint8_t* k_smem = q_smem + p.q_bufs * q_buf_bytes;                  // [k_stages] K tiles
-  uint8_t* tail = k_smem + p.k_stages * kKStageBytes;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(tail);                 // 29 barriers (29 slots; the words behind them follow)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 29 * 8);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 29 * 8 + 4);
-  float* lse_buf = reinterpret_cast<float*>(tail + 240);              // [2][Ralloc] row log-sum-exps of two pass-2 items
-  float* sm_stat = lse_buf + 2 * p.Ralloc;                            // pass 1: [2 buffers]{m[wgslots][Ralloc], l[wgslots][Ralloc]}
-  float* sm_part = sm_stat + 4 * p.wgslots * p.Ralloc;                // pass 2, several blocks per tile: [slots][groups][128] partial column sums
-  const int part_slots = p.Rpad > 384 ? 4 : (p.Rpad > 128 ? 8 : 0);   // tiles in flight (see the pass-2 combine)
-  int* sm_cnt = reinterpret_cast<int*>(sm_part + part_slots * kEpiGroups * 128);   // [kPartSlots][4 lane quarters] partials written
-  int* s_cu = sm_cnt + kPartSlots * 4 + 8;                            // [B+1] (eight spare words before it)                                            // [B+1]
-  int* s_prefix = s_cu + p.B + 1;                                     // [B+1]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(k_smem + p.k_stages * kKStageBytes);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 38);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  float* table = reinterpret_cast<float*>(bars + 40);
+  // pass 1: [2 buffers][kGroups]{m[Ralloc], l[Ralloc]} running statistics of a segment
+  // pass 2: [2 buffers][Ralloc] negated log-sum-exps, [kColSlots][kGroups][128] partial column sums
+  float* const stat = table;
+  float* const neg_lse = table;
+  float* const cols = table + 2 * p.Ralloc;
+  int* s_cu = reinterpret_cast<int*>(table + (PASS == 1 ? 4 * kGroups * p.Ralloc : 2 * p.Ralloc + kColSlots * kGroups * 128));
+  int* s_prefix = s_cu + p.B + 1;
 
-  auto bar_qfull = [&](int s) { return smem_u32(&bars[s]); };
-  auto bar_qempty = [&](int s) { return smem_u32(&bars[2 + s]); };
-  auto bar_kfull = [&](int s) { return smem_u32(&bars[4 + s]); };
-  auto bar_kempty = [&](int s) { return smem_u32(&bars[8 + s]); };
-  auto bar_afull = [&](int s) { return smem_u32(&bars[12 + s]); };
-  auto bar_aempty = [&](int s) { return smem_u32(&bars[16 + s]); };
-  auto bar_lse_ready = [&](int s) { return smem_u32(&bars[20 + s]); };   // helper -> epilogue: lse_buf[s] holds the item's rows
-  auto bar_lse_free = [&](int s) { return smem_u32(&bars[22 + s]); };    // epilogue (16 warps) -> helper: lse_buf[s] may be rewritten
-  const uint32_t bar_drain = smem_u32(&bars[24]);
-  auto bar_stat_full = [&](int s) { return smem_u32(&bars[25 + s]); };   // epilogue (16 warps) -> helpers: the item's statistics are complete
-  auto bar_stat_free = [&](int s) { return smem_u32(&bars[27 + s]); };   // helpers -> epilogue: the statistics buffer was published                        // MMA thread: every MMA it issued has completed
+  const uint32_t bar0 = smem_u32(bars);
+  auto bar_qfull = [&](uint32_t s) { return bar0 + 8u * s; };
+  auto bar_qempty = [&](uint32_t s) { return bar0 + 8u * (2 + s); };
+  auto bar_kfull = [&](uint32_t s) { return bar0 + 8u * (4 + s); };
+  auto bar_kempty = [&](uint32_t s) { return bar0 + 8u * (8 + s); };
+  auto bar_afull = [&](uint32_t s) { return bar0 + 8u * (12 + s); };
+  auto bar_aempty = [&](uint32_t s) { return bar0 + 8u * (16 + s); };
+  // pass 1: statistics complete (epilogue -> helpers) / published; pass 2: log-sum-exps there (helper -> epilogue) / used
+  auto bar_tab_full = [&](uint32_t s) { return bar0 + 8u * (20 + s); };
+  auto bar_tab_free = [&](uint32_t s) { return bar0 + 8u * (22 + s); };
+  auto bar_cols_full = [&](uint32_t s) { return bar0 + 8u * (24 + s); };   // epilogue -> helper: partial column sums of a tile complete
+  auto bar_cols_free = [&](uint32_t s) { return bar0 + 8u * (28 + s); };
+  const uint32_t bar_drain = bar0 + 8u * 32u;
+  const uint32_t bar_first = bar0 + 8u * 33u;          // pass 2: the epilogue warps' own merge of the first segment's log-sum-exps
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  unsigned long long clk0 = 0, gt0 = 0;
+  if (p.clock_out && tid == 0) { clk0 = (unsigned long long)clock64(); gt0 = global_timer_ns(); }
+  const int nblk = p.Ralloc >> 7;                      // row blocks
+  if (warp == kTmaWarp && lane == 0) { tma_prefetch_map(&tmap_q); tma_prefetch_map(&tmap_k); }
   if (tid == 0) {
     SG_CHECK(reinterpret_cast<uint8_t*>(s_prefix + p.B + 1) <= smem_dyn + p.smem_bytes);     // carve-up fits the launch's shared memory
     SG_CHECK((smem_u32(q_smem) & 1023u) == 0 && (smem_u32(k_smem) & 1023u) == 0);            // swizzled operands on 1024-byte boundaries
-    SG_CHECK((smem_u32(bars) & 7u) == 0 && (smem_u32(lse_buf) & 15u) == 0);
-  }
-
-  if (tid == 0) {
     for (int s = 0; s < 2; ++s) {
       mbar_init(bar_qfull(s), 1); mbar_init(bar_qempty(s), 1);
+      mbar_init(bar_tab_full(s), PASS == 1 ? kEpiWarps : 1); mbar_init(bar_tab_free(s), PASS == 1 ? 2 : kEpiWarps);
     }
     for (int s = 0; s < kMaxKStages; ++s) { mbar_init(bar_kfull(s), 1); mbar_init(bar_kempty(s), 1); }
-    for (int s = 0; s < kAccStages; ++s) { mbar_init(bar_afull(s), 1); mbar_init(bar_aempty(s), 4); }
-    for (int s = 0; s < 2; ++s) { mbar_init(bar_lse_ready(s), 2); mbar_init(bar_lse_free(s), kEpiThreads / 32); }
+    for (int s = 0; s < kStages; ++s) { mbar_init(bar_afull(s), 1); mbar_init(bar_aempty(s), 4); }
+    for (int s = 0; s < kColSlots; ++s) { mbar_init(bar_cols_full(s), 4 * min(nblk, kGroups)); mbar_init(bar_cols_free(s), 1); }
     mbar_init(bar_drain, 1);
-    for (int s = 0; s < 2; ++s) { mbar_init(bar_stat_full(s), kEpiThreads / 32); mbar_init(bar_stat_free(s), 2); }
+    mbar_init(bar_first, kEpiWarps);
     *abort_flag = 0;
-    for (int i = 0; i < kPartSlots * 4; ++i) sm_cnt[i] = 0;
     fence_barrier_init();
     fence_proxy_async();
   }
   if (warp == kMmaWarp) {
-    tmem_alloc(smem_u32(tmem_slot), kTmemCols);
+    tmem_alloc(smem_u32(tmem_slot), 512);
     tmem_relinquish();
   }
   if (warp == 0) {
-    // sequence offsets and the per-sequence item prefix, once per CTA
+    // sequence offsets and the per-sequence tile prefix, once per CTA (one sequence: {0, T}, no load)
     int acc = 0;
     for (int b0 = 0; b0 <= p.B; b0 += 32) {
       const int b = b0 + lane;
-      int nch = 0;
-      if (b <= p.B) s_cu[b] = p.cu[b];
-      if (b < p.B) {
-        const int tiles = (p.cu[b + 1] - p.cu[b] + kTileKeys - 1) / kTileKeys;
-        nch = (tiles + p.tiles_per_chunk - 1) / p.tiles_per_chunk;
+      int nt = 0;
+      if (p.B == 1) {
+        if (b <= 1) s_cu[b] = b * (int)p.T;
+        if (b == 0) nt = ((int)p.T + kTileKeys - 1) / kTileKeys;
+      } else {
+        if (b <= p.B) s_cu[b] = p.cu[b];
+        if (b < p.B) nt = (p.cu[b + 1] - p.cu[b] + kTileKeys - 1) / kTileKeys;
       }
-      int inc = nch;
+      int inc = nt;
 #pragma unroll
       for (int off = 1; off < 32; off <<= 1) {
         const int v = __shfl_up_sync(0xffffffffu, inc, off);
@@ -452,7 +332,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
     for (int qb = 0; qb < p.q_bufs; ++qb)
       for (int dc = 0; dc < kSub; ++dc) {
         uint32_t* z = reinterpret_cast<uint32_t*>(q_smem + qb * q_buf_bytes + dc * q_sub_bytes + p.R * 128);
-        for (int i = tid; i < words; i += kScoreThreads) z[i] = 0u;
+        for (int i = tid; i < words; i += kThreads) z[i] = 0u;
       }
     fence_proxy_async();
   }
@@ -461,592 +341,369 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   const int C = s_prefix[p.B];
-  const long long npos = schedule_length(p.U, C, p.lag, p.compact != 0);
   volatile int never = 0;
-
-  unsigned long long clk0 = 0, gt0 = 0;
-  if (p.clock_out && tid == 0) { clk0 = (unsigned long long)clock64(); gt0 = global_timer_ns(); }
+  // Another launch of this call follows: let it be set up on every SM that this one leaves (it waits for this whole grid
+  // before it reads or overwrites anything that a launch wrote).
+  if (p.more) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  SegmentWalk walk(C, p.units, p.B, p.u0, s_cu, s_prefix);
+  Segment sg;
+  // A warp's wait: every lane sees the phase complete, or none goes on.
+  auto wait = [&](uint32_t bar, uint32_t parity) {
+    if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, abort_flag, p.wait_ns)) != 0;
+  };
+  long long w0 = 0, w1 = 0;                            // waiting clocks (profiling build)
 
   if (warp == kTmaWarp) {
     // ------------------------------------------------------------ TMA producer (one thread)
     if (lane == 0) {
-      int stage = 0, n_item = 0;
-      uint32_t phase = 0;
-      long long n_loads = 0;                          // K tiles requested so far
+      int nq = 0, nk = 0;                              // Q operands and K tiles requested so far
       bool ok = true;
-      SG_PROF_DECL(w_kempty = 0, w_qempty = 0);
-      for (long long pos = blockIdx.x; pos < npos && ok; pos += gridDim.x) {
-        const ScoreItem it = decode_position(p, pos, s_cu, s_prefix);
-        if (it.pass == 0) continue;
-        const int qb = n_item % p.q_bufs;
-        const uint32_t qph = (uint32_t)((n_item / p.q_bufs) & 1);
-        SG_PROF_BEGIN(tq);
-        ok = mbar_wait(bar_qempty(qb), qph ^ 1u, abort_flag, p.wait_ns, 200u);
-        SG_PROF_ADD(w_qempty, tq);
+      while (ok && walk.next(sg)) {
+        const int l = sg.u / p.Hkv, g = sg.u - l * p.Hkv, qs = nq % p.q_bufs;
+        ok = mbar_wait(bar_qempty(qs), (uint32_t)(((nq / p.q_bufs) & 1) ^ 1), abort_flag, p.wait_ns, 100u);
         if (!ok) break;
-        ++n_item;
-        SG_CHECK(qb >= 0 && qb < p.q_bufs && (it.g + 1) * p.G <= p.Hkv * p.G && it.b < p.B && p.G * p.W <= p.Ralloc);
-        mbar_arrive_expect_tx(bar_qfull(qb), (uint32_t)(kSub * p.G * p.W * 128));
+        ++nq;
+        mbar_arrive_expect_tx(bar_qfull(qs), (uint32_t)(kSub * p.G * p.W * 128));
 #pragma unroll
         for (int dc = 0; dc < kSub; ++dc)
-          tma_load_4d(smem_u32(q_smem + qb * q_buf_bytes + dc * q_sub_bytes), &tmap_q, bar_qfull(qb), dc * 64, it.g * p.G, 0,
-                      it.l * p.B + it.b);
-        for (int tile = it.tile_beg; tile < it.tile_end && ok; ++tile) {
-          SG_PROF_BEGIN(tk);
-          ok = mbar_wait(bar_kempty(stage), phase ^ 1u, abort_flag, p.wait_ns, 200u);
-          SG_PROF_ADD(w_kempty, tk);
+          tma_load_4d(smem_u32(q_smem + qs * q_buf_bytes + dc * q_sub_bytes), &tmap_q, bar_qfull(qs), dc * 64, g * p.G, 0, l * p.B + sg.b);
+        for (int tile = sg.tile_beg; tile < sg.tile_end; ++tile) {
+          const int ks = nk % p.k_stages;
+          ok = mbar_wait(bar_kempty(ks), (uint32_t)(((nk / p.k_stages) & 1) ^ 1), abort_flag, p.wait_ns, 100u);
           if (!ok) break;
-          SG_CHECK(stage >= 0 && stage < p.k_stages && it.c0 + tile * kTileKeys < p.T && it.g < p.Hkv && it.l * p.Hkv < p.U);
-          mbar_arrive_expect_tx(bar_kfull(stage), (uint32_t)kKStageBytes);
+          ++nk;
+          SG_CHECK(sg.c0 + tile * kTileKeys < p.T && g < p.Hkv && sg.b < p.B);
+          mbar_arrive_expect_tx(bar_kfull(ks), (uint32_t)kKStageBytes);
 #pragma unroll
           for (int dc = 0; dc < kSub; ++dc)
-            tma_load_4d(smem_u32(k_smem + stage * kKStageBytes + dc * kKSubBytes), &tmap_k, bar_kfull(stage), dc * 64, it.g,
-                        it.c0 + tile * kTileKeys, it.l);
-          ++n_loads;
-          if (++stage == p.k_stages) { stage = 0; phase ^= 1u; }
+            tma_load_4d(smem_u32(k_smem + ks * kKStageBytes + dc * kKSubBytes), &tmap_k, bar_kfull(ks), dc * 64, g, sg.c0 + tile * kTileKeys, l);
         }
       }
-      SG_PROF_STORE(4, w_kempty); SG_PROF_STORE(5, w_qempty);
-      if (ok) {
-        // Wait until the MMAs have released every K stage and Q buffer: no barrier arrival and no copy of this
-        // CTA is pending when it exits.
-        for (int i = 0; i < p.k_stages; ++i) {
-          if (!mbar_wait(bar_kempty(stage), phase ^ 1u, abort_flag, p.wait_ns, 200u)) break;
-          if (++stage == p.k_stages) { stage = 0; phase ^= 1u; }
-        }
-        for (int i = 0; i < p.q_bufs; ++i) {
-          const int n = n_item + i;
-          if (!mbar_wait(bar_qempty(n % p.q_bufs), (uint32_t)(((n / p.q_bufs) & 1) ^ 1), abort_flag, p.wait_ns, 200u)) break;
-        }
-      } else {
-        // Aborted: nobody may consume what was requested, so wait (bounded, ignoring the abort flag) for the copies
-        // themselves -- the `full` barrier of every K stage and Q buffer that still has a request outstanding --
-        // before this CTA's shared memory is given up.
-        const int back = (int)(n_loads < p.k_stages ? n_loads : p.k_stages);
-        for (int i = 1; i <= back; ++i) {
-          const long long n = n_loads - i;             // the i-th last request: stage n % k_stages, use n / k_stages
-          if (!mbar_wait(bar_kfull((int)(n % p.k_stages)), (uint32_t)((n / p.k_stages) & 1), &never, p.wait_ns, 200u)) break;
-        }
-        const int qback = n_item < p.q_bufs ? n_item : p.q_bufs;
-        for (int i = 1; i <= qback; ++i) {
-          const int n = n_item - i;
-          if (!mbar_wait(bar_qfull(n % p.q_bufs), (uint32_t)((n / p.q_bufs) & 1), &never, p.wait_ns, 200u)) break;
-        }
+      // No copy and no barrier arrival of this CTA may be pending when it exits: wait until the MMAs have released every
+      // buffer, or, on an aborted run (nobody consumes what was requested), for the copies themselves.
+      for (int i = 0; i < p.k_stages && ok; ++i)
+        ok = mbar_wait(bar_kempty((nk + i) % p.k_stages), (uint32_t)((((nk + i) / p.k_stages) & 1) ^ 1), abort_flag, p.wait_ns, 100u);
+      for (int i = 0; i < p.q_bufs && ok; ++i)
+        ok = mbar_wait(bar_qempty((nq + i) % p.q_bufs), (uint32_t)((((nq + i) / p.q_bufs) & 1) ^ 1), abort_flag, p.wait_ns, 100u);
+      if (!ok) {
+        for (int n = max(0, nk - p.k_stages); n < nk; ++n)
+          mbar_wait(bar_kfull(n % p.k_stages), (uint32_t)((n / p.k_stages) & 1), &never, p.wait_ns, 100u);
+        for (int n = max(0, nq - p.q_bufs); n < nq; ++n)
+          mbar_wait(bar_qfull(n % p.q_bufs), (uint32_t)((n / p.q_bufs) & 1), &never, p.wait_ns, 100u);
       }
     }
   } else if (warp == kMmaWarp) {
-    // ------------------------------------------------------------ MMA issuer (one thread)
-    // Accumulator stage w feeds epilogue warpgroup w; block n of the CTA's running count goes to stage n mod 4.
-    // Each stage is consumed by one warpgroup only, so no waiter ever falls more than one mbarrier phase behind.
-    if (lane == 0) {
-      int ks = 0, n_item = 0;
-      uint32_t kph = 0, phbits = 0, tile_count = 0;   // phbits: one phase bit per accumulator stage
-      bool ok = true;
-      SG_PROF_DECL(w_qfull = 0, w_kfull = 0, w_aempty = 0);
-      const uint32_t k_lo0 = smem_desc_lo(smem_u32(k_smem));
-      const uint32_t k_stage_lo = (uint32_t)kKStageBytes >> 4;
-      const uint32_t bar_afull0 = bar_afull(0), bar_aempty0 = bar_aempty(0);
-      for (long long pos = blockIdx.x; pos < npos && ok; pos += gridDim.x) {
-        const ScoreItem it = decode_position(p, pos, s_cu, s_prefix);
-        if (it.pass == 0) continue;
-        const int qb = n_item % p.q_bufs;
-        const uint32_t qph = (uint32_t)((n_item / p.q_bufs) & 1);
-        ++n_item;
-        SG_PROF_BEGIN(tq);
-        ok = mbar_wait(bar_qfull(qb), qph, abort_flag, p.wait_ns, 0u);
-        SG_PROF_ADD(w_qfull, tq);
+    // ------------------------------------------------------------ MMA issuer (converged warp, one elected lane issues)
+    // The tensor pipe holds about two MMAs (~200 clocks) behind the last one issued, and a single warp retires an
+    // instruction every 5-10 clocks: whatever stands between the last MMA of a block and the first of the next is time in
+    // which the pipe runs dry.  Hence a converged warp (waits and address arithmetic stay warp-uniform), per-segment
+    // constants, and every wait beyond its first attempt out of line: 730 clocks per block, 900 to 1400 with one thread
+    // and inline waits (micro-benchmark with streamed key tiles).
+    const bool leader = elect_one();
+    uint32_t ks = 0, kph = 0, n = 0;
+    int nq = 0;
+    bool ok = true;
+    const uint32_t k_lo0 = smem_desc_lo(smem_u32(k_smem)), k_stages = (uint32_t)p.k_stages, q_sub_lo = (uint32_t)q_sub_bytes >> 4;
+    constexpr uint32_t k_stage_lo = (uint32_t)kKStageBytes >> 4, k_sub_lo = (uint32_t)kKSubBytes >> 4, q_blk_lo = (128u * 128u) >> 4;
+    const uint32_t idesc = make_idesc(128, 128);
+    while (ok && walk.next(sg)) {
+      const int qs = nq % p.q_bufs;
+      SG_PROF_WAIT(w0, ok = wait(bar_qfull(qs), (uint32_t)((nq / p.q_bufs) & 1)));
+      if (!ok) break;
+      ++nq;
+      const uint32_t q_lo0 = smem_desc_lo(smem_u32(q_smem + qs * q_buf_bytes));
+      for (int tile = sg.tile_beg; tile < sg.tile_end && ok; ++tile) {
+        SG_PROF_WAIT(w0, ok = wait(bar_kfull(ks), kph));
         if (!ok) break;
-        tc_fence_after();
-        // per-item constants of the issue loop
-        const bool pass1 = it.pass == 1;
-        const int nblk = pass1 ? (p.R + 127) / 128 : (p.Rpad + 127) / 128;
-        const uint32_t q_lo0 = smem_desc_lo(smem_u32(q_smem + qb * q_buf_bytes));
-        const uint32_t q_blk_lo = (128u * 128u) >> 4;                      // next row block of the Q operand
-        const uint32_t a_sub = (uint32_t)(pass1 ? q_sub_bytes : kKSubBytes) >> 4;
-        const uint32_t b_sub = (uint32_t)(pass1 ? kKSubBytes : q_sub_bytes) >> 4;
-        const uint32_t idesc_full = make_idesc(128, 128);
-        const uint32_t idesc_last = pass1 ? idesc_full : make_idesc(128, p.Rpad - (nblk - 1) * 128);
-        for (int tile = it.tile_beg; tile < it.tile_end && ok; ++tile) {
-          SG_PROF_BEGIN(tk);
-          if (!mbar_test(bar_kfull(ks), kph)) ok = mbar_wait(bar_kfull(ks), kph, abort_flag, p.wait_ns, 0u);
-          SG_PROF_ADD(w_kfull, tk);
+        const uint32_t k_lo = k_lo0 + ks * k_stage_lo;
+        uint32_t q_lo = q_lo0;
+        for (int blk = 0; blk < nblk; ++blk, q_lo += q_blk_lo, ++n) {
+          const uint32_t st = n & (kStages - 1);
+          SG_PROF_WAIT(w1, ok = wait(bar_aempty(st), ((n / kStages) & 1u) ^ 1u));
           if (!ok) break;
           tc_fence_after();
-          const uint32_t k_lo = k_lo0 + (uint32_t)ks * k_stage_lo;
-          uint32_t q_lo = q_lo0;
-          for (int blk = 0; blk < nblk; ++blk, q_lo += q_blk_lo) {
-            const uint32_t as = (tile_count++) % kEpiGroups;               // blocks go to the warpgroups in rotation
-            const uint32_t par = ((phbits >> as) & 1u) ^ 1u;
-            SG_PROF_BEGIN(ta);
-            ok = mbar_wait(bar_aempty0 + as * 8u, par, abort_flag, p.wait_ns, 0u);
-            SG_PROF_ADD(w_aempty, ta);
-            if (!ok) break;
-            tc_fence_after();
-            umma_block<4 * kSub>(tmem_base + as * 128u, pass1 ? q_lo : k_lo, pass1 ? k_lo : q_lo, a_sub, b_sub, kSmemDescHi,
-                                 blk == nblk - 1 ? idesc_last : idesc_full);
-            umma_commit(bar_afull0 + as * 8u);
-            phbits ^= 1u << as;
+          if (leader) {
+            if (PASS == 1) umma_block<4 * kSub>(tmem_base + st * 128u, q_lo, k_lo, q_sub_lo, k_sub_lo, idesc);
+            else umma_block<4 * kSub>(tmem_base + st * 128u, k_lo, q_lo, k_sub_lo, q_sub_lo, idesc);
+            umma_commit(bar_afull(st));
+            if (blk == nblk - 1) umma_commit(bar_kempty(ks));
           }
-          if (ok) umma_commit(bar_kempty(ks));
-          if (++ks == p.k_stages) { ks = 0; kph ^= 1u; }
+          __syncwarp();
         }
-        if (ok) umma_commit(bar_qempty(qb));
+        if (++ks == k_stages) { ks = 0; kph ^= 1u; }
       }
-      // Every MMA this thread issued has completed before the CTA frees its tensor memory, also on an aborted run
-      // (the commit arrives when all earlier MMAs are done; the wait ignores the abort flag and is bounded).
-      SG_PROF_STORE(6, w_qfull); SG_PROF_STORE(7, w_kfull); SG_PROF_STORE(8, w_aempty);
+      if (ok && leader) umma_commit(bar_qempty(qs));
+      __syncwarp();
+    }
+    // Every MMA this warp issued has completed before the CTA frees its tensor memory, also on an aborted run
+    // (the commit arrives when all earlier MMAs are done; the wait ignores the abort flag and is bounded).
+    if (leader) {
       umma_commit(bar_drain);
       mbar_wait(bar_drain, 0u, &never, p.wait_ns, 0u);
     }
-  } else if (warp < kTmaWarp) {
+    __syncwarp();
+    SG_PROF_STORE(4, w0); SG_PROF_STORE(5, w1);
+  } else if (warp < kEpiWarps) {
     // ------------------------------------------------------------ epilogue warps
-    // Four warpgroups of four warps; each owns one accumulator stage and every fourth block (a key tile, or one
-    // row block of a key tile) of the CTA's running block count.  A thread sees all 128 accumulator columns of
-    // its TMEM lane.  The warpgroups never meet at a CTA-wide barrier: each walks the CTA's items on its own,
-    // publishes its own pass-1 statistics and waits only for accumulators and (pass 2) for the helper warp's
-    // log-sum-exps, so the others keep the SFU busy while one of them is between items.
-    const int wg = warp >> 2;
-    const int wg_tid = tid & 127;
-    (void)wg_tid;                                      // only the profiling build reads it
-    const int lane_grp = warp & 3;                     // TMEM lane quarter this warp may access
-    const int row_in_tile = lane_grp * 32 + lane;
-    const uint32_t t_lane = tmem_base + ((uint32_t)(lane_grp * 32) << 16);
-    const int as = wg;                                 // this warpgroup's accumulator stage
-    const uint32_t t_acc = t_lane + (uint32_t)(as * 128);
-    const int wgslot = p.wgslots == 4 ? wg : 0;
-    uint32_t aph = 0, tile_count = 0;
-    int n_p2 = 0;                                      // pass-2 items seen so far (selects the lse buffer)
-    int n_p1 = 0;                                      // pass-1 items seen so far (selects the statistics buffer)
+    // Block n of the CTA's running count is in stage n mod 4 and belongs to warpgroup n mod 3; one stage more than there are
+    // warpgroups, so the MMAs of a warpgroup's next block need not wait for its current one.
+    const int wg = warp >> 2, quarter = warp & 3;
+    const int row_in_tile = quarter * 32 + lane;       // this thread's TMEM lane: its row of the block (pass 1), its key (pass 2)
+    const uint32_t t_lane = tmem_base + ((uint32_t)(quarter * 32) << 16);
+    const uint64_t scale2 = pack2(p.scale_log2, p.scale_log2);
+    uint32_t n0 = 0;                                   // blocks of the CTA before this segment
+    int tiles0 = 0;                                    // tiles of the CTA before this segment
     bool ok = true;
-    SG_PROF_DECL(w_afull = 0, w_lse = 0, w_pub = 0, n_blocks = 0, w_sfree = 0);
-    // Releases the accumulator: called right after the block's last TMEM load has completed, before the
-    // arithmetic on those columns, so the MMAs of this warpgroup's next block overlap it.
-    auto release_acc = [&]() {
+    auto release = [&](uint32_t st) {
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar_aempty(as));
-      aph ^= 1u;
+      if (lane == 0) mbar_arrive(bar_aempty(st));
     };
-    for (long long pos = blockIdx.x; pos < npos; pos += gridDim.x) {   // no early exit: every thread meets its warpgroup's barriers
-      const ScoreItem it = decode_position(p, pos, s_cu, s_prefix);
-      if (it.pass == 0) continue;
-      const int N = it.N;
-      const int Weff = min(p.W, N);
-      const int first_win = N - Weff;                  // position of window row 0; keys <= it are visible to all rows
-
-      if (it.pass == 1) {
-        const int nblk = (p.R + 127) / 128;
-        const bool blockwise = nblk > 1;
-        const uint32_t n_item0 = tile_count;           // running block count at the start of the item
-        // Running statistics live in one of two shared-memory buffers (alternating pass-1 items, because the
-        // warpgroups drift apart by up to an item).  The buffer's previous item must have been merged and published
-        // by the helper warps (practically always true already; the wait is bounded).
-        const int sbuf = n_p1 & 1, suse = n_p1 >> 1;
-        ++n_p1;
-        SG_PROF_BEGIN(tsf);
-        if (ok && suse > 0) ok = mbar_wait(bar_stat_free(sbuf), (uint32_t)((suse - 1) & 1), abort_flag, p.wait_ns, 32u);
-        SG_PROF_ADD(w_sfree, tsf);
-        float* sm_m = sm_stat + (size_t)(sbuf * 2 * p.wgslots + wgslot) * p.Ralloc;   // this warpgroup's slot: max ...
-        float* sm_l = sm_m + p.wgslots * p.Ralloc;                                     // ... and sum of exp2
-        // Slot (wgslot, blk*128 + row_in_tile) is only ever touched by this thread during the item, so the running
-        // statistics need no barrier: with one slot per warpgroup every block's rows are initialised, with a shared
-        // slot (the number of row blocks is a multiple of four, so a row block always meets the same warpgroup)
-        // only the owned ones.
-        for (int blk = 0; blk < nblk; ++blk)
-          if (p.wgslots == 4 || ((n_item0 + (uint32_t)blk) % kEpiGroups) == (uint32_t)wg) {
-            sm_m[blk * 128 + row_in_tile] = -INFINITY;
-            sm_l[blk * 128 + row_in_tile] = 0.f;
-          }
-        // The item's tiles in two loops.  First the tiles that every window row sees completely, when all rows of this
-        // warp lie inside the window: the loop holds the hot body and nothing else -- with the masked variant compiled
-        // into the same loop the kernel, which runs at its 96-register limit, was 7-10 % slower as a whole.  Then the
-        // rest (the causal diagonal, or everything when some row of the warp is outside the window) in the general loop.
-        bool rows_ok = true;
-        for (int blk = 0; blk < nblk; ++blk) {
-          const int r = blk * 128 + row_in_tile;
-          rows_ok = rows_ok && r < p.R && (r / p.G) < Weff;
-        }
-        rows_ok = __all_sync(0xffffffffu, rows_ok);
-        const int vis_end = (first_win + 1) / kTileKeys;                    // tiles [0, vis_end) are visible to every window row
-        const int hot_end = rows_ok ? min(it.tile_end, max(it.tile_beg, vis_end)) : it.tile_beg;
-        for (int tile = it.tile_beg; tile < hot_end; ++tile) {
-          if (!blockwise && ((tile_count++) % kEpiGroups) != (uint32_t)wg) continue;   // (the wait below looks at `ok`)
-          for (int blk = 0; blk < nblk; ++blk) {
-            if (blockwise && (((tile_count++) % kEpiGroups) != (uint32_t)wg || !ok)) continue;
-            SG_PROF_BEGIN(ta);
-            if (ok) ok = mbar_wait(bar_afull(as), aph, abort_flag, p.wait_ns, 0u);
-            SG_PROF_ADD(w_afull, ta);
-            SG_PROF_INC(n_blocks);
-            if (!ok) continue;
-            tc_fence_after();
-            const int r = blk * 128 + row_in_tile;
-            float m = sm_m[r], lsum = sm_l[r];
-            uint32_t cur[32];
-            // The running reference m need not be the row maximum: fp32 keeps its relative precision for any exponent, so
-            // the sum of exp2(x - m) is as accurate with a stale (lower) m as with the true maximum, as long as nothing
-            // overflows.  A chunk is summed against the current m (no maximum over its 32 values); only if the sum leaves
-            // the safe range -- a value more than ~60 binary orders above m, or m still -inf at the start of an item --
-            // is the reference refreshed, out of line.  The loop body is 32 x (fma, ex2, add) and nothing else.
-#pragma unroll 2   // measured: 1, 2 and 4 give 685 / 667 / 680 us on the long-context shape
-            for (int j = 0; j < 4; ++j) {
-              SG_CHECK(as * 128 + j * 32 + 32 <= (int)kTmemCols);
-              tmem_ld32_issue(cur, t_acc + (uint32_t)(j * 32));
-              tmem_ld_wait(cur);
-              if (j == 3) release_acc();
-              float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+    for (int sidx = 0; ok && walk.next(sg); ++sidx) {
+      const int Weff = min(p.W, sg.N), first_win = sg.N - Weff;      // position of window row 0; keys <= it are visible to all rows
+      const int vis_end = (first_win + 1) / kTileKeys;               // tiles [0, vis_end) are visible to every window row
+      const uint32_t buf = (uint32_t)sidx & 1u, use = (uint32_t)sidx >> 1;
+      const uint32_t n_end = n0 + (uint32_t)((sg.tile_end - sg.tile_beg) * nblk);
+      uint32_t n = n0 + (kGroups + (uint32_t)wg - n0 % kGroups) % kGroups;     // this warpgroup's first block of the segment
+      int tile = sg.tile_beg, blk = (int)(n - n0);
+      while (blk >= nblk) { blk -= nblk; ++tile; }
+      if (PASS == 1) {
+        // The buffer's previous segment has been merged and published by the helpers (practically always true already).
+        // Slot (wg, row) is only ever touched by this thread during the segment, so the statistics need no barrier.
+        if (use > 0) ok = wait(bar_tab_free(buf), (use - 1u) & 1u);
+        if (!ok) break;
+        float* const sm_m = stat + (size_t)(buf * kGroups + wg) * 2 * p.Ralloc + row_in_tile;
+        float* const sm_l = sm_m + p.Ralloc;
+        for (int i = 0; i < nblk; ++i) { sm_m[i * 128] = -INFINITY; sm_l[i * 128] = 0.f; }
+        const bool all_rows = Weff == p.W;
+        for (; n < n_end; n += kGroups) {
+          const uint32_t st = n & (kStages - 1), t_acc = t_lane + st * 128u;
+          SG_PROF_WAIT(w0, ok = wait(bar_afull(st), (n / kStages) & 1u));
+          if (!ok) break;
+          tc_fence_after();
+          float m = sm_m[blk * 128], l = sm_l[blk * 128];
+          // The running reference m need not be the row maximum: fp32 keeps its relative precision for any exponent, so
+          // the sum of exp2(x - m) is as accurate with a stale (lower) m as with the true maximum, as long as nothing
+          // overflows.  A segment starts from the maximum of the block's first 32 columns; a block whose sum leaves the safe
+          // range (a value far above m) and a block with hidden scores are done carefully: true maximum first.
+          bool careful = tile >= vis_end || !all_rows;
+          if (!careful) {
+            uint32_t a[32], b[32];
+            tmem_ld32_issue(a, t_acc);
+            tmem_ld_wait(a);
+            tmem_ld32_issue(b, t_acc + 32u);
+            if (m == -INFINITY) {                      // (a row block's rows start together)
+              float x = fmaxf(__uint_as_float(a[0]), __uint_as_float(a[1]));
 #pragma unroll
-              for (int c = 0; c < 32; c += 4) {
-                s0 += exp2f(fmaf(__uint_as_float(cur[c]), p.scale_log2, -m));
-                s1 += exp2f(fmaf(__uint_as_float(cur[c + 1]), p.scale_log2, -m));
-                s2 += exp2f(fmaf(__uint_as_float(cur[c + 2]), p.scale_log2, -m));
-                s3 += exp2f(fmaf(__uint_as_float(cur[c + 3]), p.scale_log2, -m));
-              }
-              const float s = (s0 + s1) + (s2 + s3);
-              if (s < 0x1p60f) lsum += s;
-              else { const float2 ml = refresh_reference(p.scale_log2, m, lsum, cur[0], cur[1], cur[2], cur[3], cur[4], cur[5], cur[6], cur[7], cur[8], cur[9], cur[10], cur[11], cur[12], cur[13], cur[14], cur[15], cur[16], cur[17], cur[18], cur[19], cur[20], cur[21], cur[22], cur[23], cur[24], cur[25], cur[26], cur[27], cur[28], cur[29], cur[30], cur[31]); m = ml.x; lsum = ml.y; }
+              for (int c = 2; c < 32; c += 2) x = max3(x, __uint_as_float(a[c]), __uint_as_float(a[c + 1]));
+              m = x * p.scale_log2;
             }
-            sm_m[r] = m;
-            sm_l[r] = lsum;
+            const uint64_t nm2 = pack2(-m, -m);
+            uint64_t s0 = 0ull, s1 = 0ull;
+            chunk_rows(a, scale2, nm2, s0, s1);
+            tmem_ld_wait(b);
+            tmem_ld32_issue(a, t_acc + 64u);
+            chunk_rows(b, scale2, nm2, s0, s1);
+            tmem_ld_wait(a);
+            tmem_ld32_issue(b, t_acc + 96u);
+            chunk_rows(a, scale2, nm2, s0, s1);
+            tmem_ld_wait(b);
+            chunk_rows(b, scale2, nm2, s0, s1);
+            float lo, hi;
+            unpack2(add2(s0, s1), lo, hi);
+            const float s = lo + hi;
+            careful = !__all_sync(0xffffffffu, s < 0x1p60f);
+            if (!careful) l += s;
           }
-        }
-        for (int tile = hot_end; tile < it.tile_end; ++tile) {
-          if (!blockwise && (((tile_count++) % kEpiGroups) != (uint32_t)wg || !ok)) continue;
-          const int t0 = tile * kTileKeys;
-          const bool all_visible = t0 + kTileKeys - 1 <= first_win;
-          for (int blk = 0; blk < nblk; ++blk) {
-            if (blockwise && (((tile_count++) % kEpiGroups) != (uint32_t)wg || !ok)) continue;
-            SG_PROF_BEGIN(ta);
-            if (ok) ok = mbar_wait(bar_afull(as), aph, abort_flag, p.wait_ns, 0u);
-            SG_PROF_ADD(w_afull, ta);
-            SG_PROF_INC(n_blocks);
-            if (!ok) continue;
-            tc_fence_after();
+          if (careful) {
             const int r = blk * 128 + row_in_tile;
-            const bool row_ok = r < p.R && (r / p.G) < Weff;
-            const int cmax = row_ok ? (first_win + r / p.G - t0) : -1;    // last visible column of this tile
-            float m = sm_m[r], lsum = sm_l[r];
+            const int cmax = r < p.R && r / p.G < Weff ? first_win + r / p.G - tile * kTileKeys : -1;    // last visible column of this tile
+            float mx = -INFINITY;
             uint32_t cur[32];
-            // Chunk by chunk: where every row of the warp sees all 32 keys of the chunk (all but the last chunk or two
-            // of a tile on the causal diagonal, and every chunk of a fully visible tile) the hot body, else per-column
-            // masks with the true maximum.  (all_visible enters only to spare the vote on fully visible tiles.)
 #pragma unroll 1
             for (int j = 0; j < 4; ++j) {
-              const int col0 = j * 32;
-              SG_CHECK(as * 128 + col0 + 32 <= (int)kTmemCols);
-              tmem_ld32_issue(cur, t_acc + (uint32_t)col0);
-              tmem_ld_wait(cur);
-              if (j == 3) release_acc();
-              if (!__all_sync(0xffffffffu, row_ok && (all_visible || col0 + 31 <= cmax))) {
-                // Some (row, key) pairs of the chunk are hidden: a thread that sees nothing of it is done; the others
-                // replace their hidden scores by -inf, which the body below ignores (exp2 of it is 0, no maximum takes it).
-                if (col0 > cmax) continue;
-#pragma unroll
-                for (int c = 0; c < 32; ++c) cur[c] = (col0 + c <= cmax) ? cur[c] : 0xff800000u;
-              }
-              float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-#pragma unroll
-              for (int c = 0; c < 32; c += 4) {
-                s0 += exp2f(fmaf(__uint_as_float(cur[c]), p.scale_log2, -m));
-                s1 += exp2f(fmaf(__uint_as_float(cur[c + 1]), p.scale_log2, -m));
-                s2 += exp2f(fmaf(__uint_as_float(cur[c + 2]), p.scale_log2, -m));
-                s3 += exp2f(fmaf(__uint_as_float(cur[c + 3]), p.scale_log2, -m));
-              }
-              const float s = (s0 + s1) + (s2 + s3);
-              if (s < 0x1p60f) lsum += s;      // false also for the NaN that a hidden score gives while m is still -inf
-              else { const float2 ml = refresh_reference(p.scale_log2, m, lsum, cur[0], cur[1], cur[2], cur[3], cur[4], cur[5], cur[6], cur[7], cur[8], cur[9], cur[10], cur[11], cur[12], cur[13], cur[14], cur[15], cur[16], cur[17], cur[18], cur[19], cur[20], cur[21], cur[22], cur[23], cur[24], cur[25], cur[26], cur[27], cur[28], cur[29], cur[30], cur[31]); m = ml.x; lsum = ml.y; }
-            }
-            sm_m[r] = m;
-            sm_l[r] = lsum;
-          }
-        }
-        // End of the item for this warp: its rows' statistics are complete in shared memory.  The helper warps merge
-        // the warpgroups' slots, publish the item and count it as done for its unit, off this warp's path.
-        SG_PROF_BEGIN(tp);
-        __syncwarp();
-        if (lane == 0 && ok) mbar_arrive(bar_stat_full(sbuf));
-        SG_PROF_ADD(w_pub, tp);
-      } else {
-        const int nblk = (p.Rpad + 127) / 128;
-        const bool blockwise = nblk > 1;
-        // The helper warp has merged the unit's pass-1 statistics into this item's row log-sum-exps (it waited for
-        // the unit's counter); two buffers, so it works on the next pass-2 item while this one runs.  Every warp
-        // waits here, also one that gets no block of the item: passing this point proves that the buffer's previous
-        // use was released by all sixteen warps, which keeps the arrivals below in step with the barrier's phases.
-        const int lbuf = n_p2 & 1;
-        const uint32_t lph = (uint32_t)((n_p2 >> 1) & 1);
-        ++n_p2;
-        SG_PROF_BEGIN(tl);
-        if (ok) ok = mbar_wait(bar_lse_ready(lbuf), lph, abort_flag, p.wait_ns, 32u);
-        SG_PROF_ADD(w_lse, tl);
-        const float* lse2 = lse_buf + lbuf * p.Ralloc;   // [Ralloc] row log-sum-exps (log2 domain) of (unit, b)
-        // End of a tile for this warp: its partial (or whole) column sum goes out.
-        auto finish_tile = [&](const int tile, const int t, const float a0, const float a1, const float a2, const float a3, const uint32_t n0,
-                               const bool mine) {
-          float total = (a0 + a1) + (a2 + a3);
-          if (blockwise) {
-            // The tile's row blocks were dealt to different warpgroups.  Each warpgroup that had one leaves its partial
-            // column sums in shared memory; per lane quarter, the warp that writes the last partial adds them up in a
-            // fixed order (bitwise reproducible) and stores the importance -- no block-wide barrier per tile.  A slot
-            // is reused S tiles later: block m is issued only after blocks m-4 .. m-7 were released, and the
-            // warpgroups that released them had finished everything up to block m-8; with (S-1)*nblk >= 7 all
-            // partials of the slot's previous tile are summed before the slot is written again.
-            if (!mine) return;
-            const int nwg = nblk < kEpiGroups ? nblk : kEpiGroups;      // warpgroups that drain blocks of this tile
-            const int slot = tile & (nblk >= 4 ? 3 : 7);
-            float* part = sm_part + slot * (kEpiGroups * 128);
-            part[wg * 128 + row_in_tile] = total;
-            __threadfence_block();
-            __syncwarp();
-            int old = 0;
-            if (lane == 0) old = atomicAdd(&sm_cnt[slot * 4 + lane_grp], 1);
-            old = __shfl_sync(0xffffffffu, old, 0);
-            if (old != nwg - 1) return;
-            __threadfence_block();
-            total = 0.f;
-            for (int i = 0; i < nwg; ++i) total += part[((n0 + i) % kEpiGroups) * 128 + row_in_tile];
-            __syncwarp();
-            if (lane == 0) sm_cnt[slot * 4 + lane_grp] = 0;
-          }
-          SG_CHECK(!(ok && t < N) || (it.c0 + t < p.T && it.l * p.Hkv + it.g < p.U));
-          if (ok && t < N) p.importance[((size_t)it.l * p.Hkv + it.g) * p.T + it.c0 + t] = total;
-        };
-        // Two loops, as in pass 1: the tiles every window row sees completely, when every row block is full (hot body
-        // only), then the rest in the general loop.
-        const int vis_end = (first_win + 1) / kTileKeys;
-        const int hot_end = (p.Rpad & 127) == 0 ? min(it.tile_end, max(it.tile_beg, vis_end)) : it.tile_beg;
-        for (int tile = it.tile_beg; tile < hot_end; ++tile) {
-          if (!blockwise && ((tile_count++) % kEpiGroups) != (uint32_t)wg) continue;   // (the wait below looks at `ok`)
-          const int t = tile * kTileKeys + row_in_tile;  // this thread's key
-          float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-          const uint32_t n0 = tile_count;                // running block count at the start of this tile
-          bool mine = false;                             // this warpgroup drains at least one block of the tile
-          for (int blk = 0; blk < nblk; ++blk) {
-            if (blockwise && (((tile_count++) % kEpiGroups) != (uint32_t)wg || !ok)) continue;
-            mine = true;
-            SG_PROF_BEGIN(ta);
-            if (ok) ok = mbar_wait(bar_afull(as), aph, abort_flag, p.wait_ns, 0u);
-            SG_PROF_ADD(w_afull, ta);
-            SG_PROF_INC(n_blocks);
-            if (!ok) continue;
-            tc_fence_after();
-            uint32_t cur[32];
-            // nothing but 32 x (fma, ex2, add) and the rows' log-sum-exps from shared memory
-#pragma unroll 2
-            for (int j = 0; j < 4; ++j) {
-              SG_CHECK(as * 128 + j * 32 + 32 <= (int)kTmemCols && blk * 128 + j * 32 + 32 <= p.Ralloc);
               tmem_ld32_issue(cur, t_acc + (uint32_t)(j * 32));
               tmem_ld_wait(cur);
-              if (j == 3) release_acc();
-              const float* ls = lse2 + blk * 128 + j * 32;
 #pragma unroll
-              for (int c = 0; c < 32; c += 4) {
-                const float4 l4 = *reinterpret_cast<const float4*>(ls + c);
-                a0 += exp2f(fmaf(__uint_as_float(cur[c]), p.scale_log2, -l4.x));
-                a1 += exp2f(fmaf(__uint_as_float(cur[c + 1]), p.scale_log2, -l4.y));
-                a2 += exp2f(fmaf(__uint_as_float(cur[c + 2]), p.scale_log2, -l4.z));
-                a3 += exp2f(fmaf(__uint_as_float(cur[c + 3]), p.scale_log2, -l4.w));
+              for (int c = 0; c < 32; ++c)
+                if (j * 32 + c <= cmax) mx = fmaxf(mx, __uint_as_float(cur[c]));
+            }
+            const float mn = fmaxf(m, mx * p.scale_log2);
+            if (mn != -INFINITY) { l *= exp2f(m - mn); m = mn; }
+            const float ref = mn == -INFINITY ? 0.f : mn;
+#pragma unroll 1
+            for (int j = 0; j < 4; ++j) {
+              tmem_ld32_issue(cur, t_acc + (uint32_t)(j * 32));
+              tmem_ld_wait(cur);
+              float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+              for (int c = 0; c < 32; c += 2) {
+                s0 += j * 32 + c <= cmax ? exp2f(fmaf(__uint_as_float(cur[c]), p.scale_log2, -ref)) : 0.f;
+                s1 += j * 32 + c + 1 <= cmax ? exp2f(fmaf(__uint_as_float(cur[c + 1]), p.scale_log2, -ref)) : 0.f;
               }
+              l += s0 + s1;
             }
           }
-          finish_tile(tile, t, a0, a1, a2, a3, n0, mine);
+          release(st);
+          sm_m[blk * 128] = m;
+          sm_l[blk * 128] = l;
+          blk += kGroups;
+          while (blk >= nblk) { blk -= nblk; ++tile; }
         }
-        for (int tile = hot_end; tile < it.tile_end; ++tile) {
-          if (!blockwise && (((tile_count++) % kEpiGroups) != (uint32_t)wg || !ok)) continue;
-          const int t = tile * kTileKeys + row_in_tile;  // this thread's key
-          const bool all_visible = tile * kTileKeys + kTileKeys - 1 <= first_win;
-          const int rmin = (t - first_win) * p.G;        // rows below rmin cannot see key t
-          float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-          const uint32_t n0 = tile_count;                // running block count at the start of this tile
-          bool mine = false;                             // this warpgroup drains at least one block of the tile
-          for (int blk = 0; blk < nblk; ++blk) {
-            if (blockwise && (((tile_count++) % kEpiGroups) != (uint32_t)wg || !ok)) continue;
-            mine = true;
-            SG_PROF_BEGIN(ta);
-            if (ok) ok = mbar_wait(bar_afull(as), aph, abort_flag, p.wait_ns, 0u);
-            SG_PROF_ADD(w_afull, ta);
-            SG_PROF_INC(n_blocks);
-            if (!ok) continue;
-            tc_fence_after();
-            const int ncols = min(128, p.Rpad - blk * 128);
-            const int nchk = (ncols + 31) >> 5;          // 32-column chunks of this block (warp-uniform)
+        // This warp's statistics of the segment are complete; the helpers merge the warpgroups' slots and publish them.
+        __syncwarp();
+        if (lane == 0 && ok && sg.u != p.withhold_unit) mbar_arrive(bar_tab_full(buf));
+      } else {
+        if (sidx == 0) {
+          // The first segment's log-sum-exps are what the whole CTA waits for: all epilogue threads merge its records.
+          asm volatile("griddepcontrol.wait;" ::: "memory");
+          merge_records<12>(p, sg, s_prefix, C, neg_lse, tid, 32 * kEpiWarps);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_first);
+          ok = wait(bar_first, 0u);
+        } else {
+          // A helper has merged the part's records one segment ahead.  Every warp waits here, also one that gets no block of
+          // the segment: that keeps the arrivals below in step with the barrier's phases.
+          SG_PROF_WAIT(w1, ok = wait(bar_tab_full(buf), buf == 0u ? (use - 1u) & 1u : use & 1u));
+        }
+        if (!ok) break;
+        const float* nl = neg_lse + buf * p.Ralloc;
+        const int G = p.G;
+        uint64_t s0 = 0ull, s1 = 0ull;
+        while (n < n_end) {
+          const uint32_t st = n & (kStages - 1), t_acc = t_lane + st * 128u;
+          SG_PROF_WAIT(w0, ok = wait(bar_afull(st), (n / kStages) & 1u));
+          if (!ok) break;
+          tc_fence_after();
+          const int t = tile * kTileKeys + row_in_tile;                    // this thread's key
+          const float* ls = nl + blk * 128;
+          if (tile < vis_end && (blk + 1) * 128 <= p.R) {
+            uint32_t a[32], b[32];
+            tmem_ld32_issue(a, t_acc);
+            tmem_ld_wait(a);
+            tmem_ld32_issue(b, t_acc + 32u);
+            chunk_cols(a, scale2, ls, s0, s1);
+            tmem_ld_wait(b);
+            tmem_ld32_issue(a, t_acc + 64u);
+            chunk_cols(b, scale2, ls + 32, s0, s1);
+            tmem_ld_wait(a);
+            tmem_ld32_issue(b, t_acc + 96u);
+            chunk_cols(a, scale2, ls + 64, s0, s1);
+            tmem_ld_wait(b);
+            release(st);
+            chunk_cols(b, scale2, ls + 96, s0, s1);
+          } else {
+            const int nchk = (min(128, p.R - blk * 128) + 31) >> 5;       // 32-row chunks (rows past R have log-sum-exp +inf)
+            const int rmin = (t - first_win) * G;                          // rows below rmin cannot see key t
             uint32_t cur[32];
-            // Chunk by chunk: where all 32 rows of the chunk exist and see every key of the warp (on the causal diagonal:
-            // all warps but the one that holds the window's own keys) the hot body, else per-column masks.
 #pragma unroll 1
             for (int j = 0; j < nchk; ++j) {
-              const int col0 = j * 32;
-              SG_CHECK(as * 128 + col0 + 32 <= (int)kTmemCols && blk * 128 + col0 + 32 <= p.Ralloc);
-              tmem_ld32_issue(cur, t_acc + (uint32_t)col0);
+              tmem_ld32_issue(cur, t_acc + (uint32_t)(j * 32));
               tmem_ld_wait(cur);
-              if (j == nchk - 1) release_acc();
-              const float* ls = lse2 + blk * 128 + col0;
-              if (!(col0 + 32 <= ncols && (all_visible || __all_sync(0xffffffffu, blk * 128 + col0 >= rmin)))) {
-                // rows that do not see this thread's key (those below c_lo of this chunk), or that do not exist (from c_hi
-                // on, in a partial last chunk): score -inf, probability 0
-                const int c_lo = rmin - blk * 128 - col0, c_hi = ncols - col0;
-                if (c_hi >= 32) {
+              if (j == nchk - 1) release(st);
+              const int c_lo = rmin - blk * 128 - j * 32;
 #pragma unroll
-                  for (int c = 0; c < 32; ++c) cur[c] = c >= c_lo ? cur[c] : 0xff800000u;
-                } else {
-#pragma unroll
-                  for (int c = 0; c < 32; ++c) cur[c] = (c >= c_lo && c < c_hi) ? cur[c] : 0xff800000u;
-                }
-              }
-#pragma unroll
-              for (int c = 0; c < 32; c += 4) {
-                const float4 l4 = *reinterpret_cast<const float4*>(ls + c);
-                a0 += exp2f(fmaf(__uint_as_float(cur[c]), p.scale_log2, -l4.x));
-                a1 += exp2f(fmaf(__uint_as_float(cur[c + 1]), p.scale_log2, -l4.y));
-                a2 += exp2f(fmaf(__uint_as_float(cur[c + 2]), p.scale_log2, -l4.z));
-                a3 += exp2f(fmaf(__uint_as_float(cur[c + 3]), p.scale_log2, -l4.w));
-              }
+              for (int c = 0; c < 32; ++c) cur[c] = c >= c_lo ? cur[c] : 0xff800000u;
+              chunk_cols(cur, scale2, ls + j * 32, s0, s1);
             }
           }
-          finish_tile(tile, t, a0, a1, a2, a3, n0, mine);
+          const int tile_now = tile;
+          n += kGroups;
+          blk += kGroups;
+          while (blk >= nblk) { blk -= nblk; ++tile; }
+          if (tile == tile_now && n < n_end) continue;                     // more of this tile's row blocks are this warpgroup's
+          float lo, hi;
+          unpack2(add2(s0, s1), lo, hi);
+          s0 = s1 = 0ull;
+          if (nblk == 1) {
+            if (t < sg.N) p.importance[(size_t)sg.u * p.T + sg.c0 + t] = lo + hi;
+          } else {
+            // The tile's row blocks went to different warpgroups: leave the partial column sums for the helper.
+            const uint32_t ts = (uint32_t)(tiles0 + tile_now - sg.tile_beg), cs = ts % kColSlots, cu = ts / kColSlots;
+            if (cu > 0) ok = wait(bar_cols_free(cs), (cu - 1u) & 1u);
+            if (!ok) break;
+            cols[(cs * kGroups + wg) * 128 + row_in_tile] = lo + hi;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_cols_full(cs));
+          }
         }
         __syncwarp();
-        if (lane == 0 && ok) mbar_arrive(bar_lse_free(lbuf));        // this warp no longer reads lse_buf[lbuf]
+        if (lane == 0 && ok) mbar_arrive(bar_tab_free(buf));
       }
+      n0 = n_end;
+      tiles0 += sg.tile_end - sg.tile_beg;
     }
-#ifdef SG_SCORE_PROFILE
-    if (wg_tid == 0) { SG_PROF_STORE(9 + wg * 4, w_afull); SG_PROF_STORE(10 + wg * 4, w_lse); SG_PROF_STORE(11 + wg * 4, w_pub + w_sfree); SG_PROF_STORE(12 + wg * 4, n_blocks); }
-#endif
-  } else if (warp >= kHelperWarp) {
-    // ------------------------------------------------------------ helper warps (two: each handles half of the rows)
-    // Everything at an item boundary that is not arithmetic on scores runs here, off the epilogue's path:
-    //   publish(k), k-th pass-1 item of this CTA: when all sixteen epilogue warps have left their statistics in shared
-    //     memory, merge the warpgroups' slots per row, store one (max, sum) pair per row for the item, count the item
-    //     as done for its unit (stores ordered before the count by a fence), and hand the buffer back;
-    //   lse(j), j-th pass-2 item: when all pass-1 items of the unit are counted (bounded wait), merge the chunks' pairs
-    //     of the item's sequence into the rows' log-sum-exps for the epilogue; this runs one pass-2 item ahead of it.
-    // The two sequences advance independently and neither ever blocks: a task is taken only when a test shows that it
-    // can run, so a publication this CTA owes can never be held up behind a count some other CTA still owes.
+    if (quarter == 0) { SG_PROF_STORE(8 + 2 * wg, w0); SG_PROF_STORE(9 + 2 * wg, w1); SG_PROF_STORE(20, n0); }
+  } else {
+    // ------------------------------------------------------------ helper warps
     const int hw = warp - kHelperWarp;
-    long long pos1 = blockIdx.x, pos2 = blockIdx.x;      // schedule cursors of the next pass-1 / pass-2 item
-    int k1 = 0, j2 = 0;
-    ScoreItem it1, it2;
-    it1.pass = it2.pass = 0;
-    auto next_item = [&](long long& pos, ScoreItem& it, int pass) {   // advance to the next item of `pass` (it.pass = 0: none left)
-      for (; pos < npos; pos += gridDim.x) {
-        it = decode_position(p, pos, s_cu, s_prefix);
-        if (it.pass == pass) { pos += gridDim.x; return; }
-      }
-      it.pass = 0;
-    };
-    next_item(pos1, it1, 1);
-    next_item(pos2, it2, 2);
-    uint64_t idle_since = 0;
-    uint32_t idle_iters = 0;
-    SG_PROF_DECL(h_free = 0, h_cnt = 0, h_merge = 0);
-    while (it1.pass != 0 || it2.pass != 0) {
-      bool progressed = false;
-      if (it1.pass != 0 && mbar_test(bar_stat_full(k1 & 1), (uint32_t)((k1 >> 1) & 1))) {
-        SG_PROF_BEGIN(th0);
-        const int sbuf = k1 & 1;
-        const float* bm = sm_stat + (size_t)(sbuf * 2 * p.wgslots) * p.Ralloc;
-        const float* bl = bm + p.wgslots * p.Ralloc;
-        const size_t slot = ((size_t)it1.unit * p.max_items + it1.item_in_unit) * p.Ralloc;
+    // Everything below touches what an earlier launch of this call wrote or reads: wait until that has completed.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    bool ok = true;
+    if (PASS == 1) {
+      // merge the warpgroups' statistics of a finished segment and publish its record (half of the rows each)
+      for (int sidx = 0; ok && walk.next(sg); ++sidx) {
+        const uint32_t buf = (uint32_t)sidx & 1u, use = (uint32_t)sidx >> 1;
+        ok = wait(bar_tab_full(buf), use & 1u);
+        if (!ok) break;
+        const float* sm = stat + (size_t)buf * kGroups * 2 * p.Ralloc;
+        float2* rec = p.records + (size_t)(sg.part + (int)blockIdx.x) * p.Ralloc;
         for (int r = hw * 32 + lane; r < p.Ralloc; r += 64) {
-          float M = bm[r];
-          for (int w = 1; w < p.wgslots; ++w) M = fmaxf(M, bm[w * p.Ralloc + r]);
+          float m[kGroups], M = -INFINITY, L = 0.f;
+#pragma unroll
+          for (int w = 0; w < kGroups; ++w) { m[w] = sm[w * 2 * p.Ralloc + r]; M = fmaxf(M, m[w]); }
           const float Mu = M == -INFINITY ? 0.f : M;
-          float L = 0.f;
-          for (int w = 0; w < p.wgslots; ++w) L += bl[w * p.Ralloc + r] * exp2f(bm[w * p.Ralloc + r] - Mu);
-          p.part[slot + r] = make_float2(M, L);
+#pragma unroll
+          for (int w = 0; w < kGroups; ++w) L += sm[(w * 2 + 1) * p.Ralloc + r] * exp2f(m[w] - Mu);
+          rec[r] = make_float2(M, L);
         }
-        // each helper warp counts its half of the rows itself (a unit is complete at 2*C counts): its stores are ordered
-        // before its count by the warp barrier plus one cumulative fence, and no hand-shake between the two warps is needed
         __syncwarp();
-        if (lane == 0) {
-          __threadfence();
-          if (!*abort_flag && it1.unit != p.withhold_unit) atomicAdd(p.p1_done + it1.unit, 1);
-          mbar_arrive(bar_stat_free(sbuf));
-        }
-        ++k1;
-        next_item(pos1, it1, 1);
-        progressed = true;
-        SG_PROF_ADD(h_free, th0);
+        if (lane == 0) mbar_arrive(bar_tab_free(buf));
       }
-      if (it2.pass != 0) {
-        const int lbuf = j2 & 1, use = j2 >> 1;
-        bool can = use == 0 || mbar_test(bar_lse_free(lbuf), (uint32_t)((use - 1) & 1));
-        if (can) {
-          int cnt = 0;
-          if (lane == 0) cnt = ld_acquire_gpu(p.p1_done + it2.unit);
-          cnt = __shfl_sync(0xffffffffu, cnt, 0);
-          can = cnt >= 2 * C;
-        }
-        if (can) {
-          SG_PROF_BEGIN(th2);
-          __syncwarp();
-          __threadfence();                             // the other lanes' loads follow lane 0's acquire
-          float* lse2 = lse_buf + lbuf * p.Ralloc;
-          const int Weff = min(p.W, it2.N);
-          const size_t part_base = ((size_t)it2.unit * p.max_items + it2.first_item_b) * p.Ralloc;
-          const int nparts = it2.nch_b;
-          // a lane merges two neighbouring rows at a time (one 16-byte load per chunk), eight loads in flight
-          for (int r = 2 * (hw * 32 + lane); r < p.Ralloc; r += 128) {
-            float M0 = -INFINITY, L0 = 0.f, M1 = -INFINITY, L1 = 0.f;
-            for (int c0 = 0; c0 < nparts; c0 += 8) {
-              float4 v[8];
+    } else if (hw == 0) {
+      // merge the records of every segment but the first, one segment ahead of the epilogue
+      for (int sidx = 0; ok && walk.next(sg); ++sidx) {
+        if (sidx == 0) continue;
+        const uint32_t buf = (uint32_t)sidx & 1u, use = (uint32_t)sidx >> 1;
+        if (use > 0) ok = wait(bar_tab_free(buf), (use - 1u) & 1u);
+        if (!ok) break;
+        merge_records<16>(p, sg, s_prefix, C, neg_lse + buf * p.Ralloc, lane, 32);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_tab_full(buf));
+      }
+    } else if (nblk > 1) {
+      // add up the warpgroups' column sums of a tile, in the order of its row blocks (bitwise reproducible)
+      uint32_t n = 0, ts = 0;
+      const int nwg = min(nblk, kGroups);
+      while (ok && walk.next(sg)) {
+        for (int tile = sg.tile_beg; tile < sg.tile_end; ++tile, ++ts, n += (uint32_t)nblk) {
+          const uint32_t cs = ts % kColSlots;
+          ok = wait(bar_cols_full(cs), (ts / kColSlots) & 1u);
+          if (!ok) break;
+          const float* c = cols + cs * kGroups * 128;
 #pragma unroll
-              for (int i = 0; i < 8; ++i)
-                v[i] = c0 + i < nparts ? __ldcg(reinterpret_cast<const float4*>(p.part + part_base + (size_t)(c0 + i) * p.Ralloc + r))
-                                       : make_float4(-INFINITY, 0.f, -INFINITY, 0.f);
-              float m0 = v[0].x, m1 = v[0].z;
-#pragma unroll
-              for (int i = 1; i < 8; ++i) { m0 = fmaxf(m0, v[i].x); m1 = fmaxf(m1, v[i].z); }
-              if (m0 != -INFINITY) {                   // else nothing of row r is visible in these chunks
-                const float Mn = fmaxf(M0, m0);
-                float acc = L0 * exp2f(M0 - Mn);
-#pragma unroll
-                for (int i = 0; i < 8; ++i) acc += v[i].y * exp2f(v[i].x - Mn);   // a (-inf, 0) pair adds 0
-                M0 = Mn; L0 = acc;
-              }
-              if (m1 != -INFINITY) {
-                const float Mn = fmaxf(M1, m1);
-                float acc = L1 * exp2f(M1 - Mn);
-#pragma unroll
-                for (int i = 0; i < 8; ++i) acc += v[i].w * exp2f(v[i].z - Mn);
-                M1 = Mn; L1 = acc;
-              }
-            }
-            // rows outside the window get +inf: exp2(x - inf) = 0
-            lse2[r] = (r < p.R && (r / p.G) < Weff) ? M0 + log2f(L0) : INFINITY;
-            lse2[r + 1] = (r + 1 < p.R && ((r + 1) / p.G) < Weff) ? M1 + log2f(L1) : INFINITY;
+          for (int q = 0; q < 4; ++q) {
+            const int t = tile * kTileKeys + q * 32 + lane;
+            float s = 0.f;
+            for (int w = 0; w < nwg; ++w) s += c[(n + w) % kGroups * 128 + q * 32 + lane];
+            if (t < sg.N) p.importance[(size_t)sg.u * p.T + sg.c0 + t] = s;
           }
           __syncwarp();
-          if (lane == 0) mbar_arrive(bar_lse_ready(lbuf));
-          ++j2;
-          next_item(pos2, it2, 2);
-          progressed = true;
-          SG_PROF_ADD(h_merge, th2);
+          if (lane == 0) mbar_arrive(bar_cols_free(cs));
         }
       }
-      if (progressed) { idle_since = 0; idle_iters = 0; continue; }
-      // nothing could run: sleep a little; every 64th idle round look at the abort flag and the clock (bounded wait)
-      __nanosleep(40);
-      if ((++idle_iters & 63u) == 0u) {
-        if (*abort_flag) break;
-        const uint64_t now = global_timer_ns();
-        if (idle_since == 0) idle_since = now;
-        else if (now - idle_since > 2ull * p.wait_ns) { *abort_flag = 1; break; }
-      }
     }
-#ifdef SG_SCORE_PROFILE
-    if (warp == kHelperWarp && lane == 0) { SG_PROF_STORE(25, h_free); SG_PROF_STORE(26, h_cnt); SG_PROF_STORE(27, h_merge); }
-#endif
   }
-
   // ---------------------------------------------------------------- teardown
-  // This CTA has no work left: a kernel queued behind this one with programmatic stream serialization (the selection)
-  // may have its CTAs placed from now on; it still waits for this whole grid's completion before it reads anything.
+  // This CTA has no work left: a kernel queued behind this one with programmatic stream serialization (the selection) may
+  // have its CTAs placed from now on; it still waits for this whole grid's completion before it reads anything.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   tc_fence_before();
   __syncthreads();
   if (warp == kMmaWarp) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, kTmemCols);
+    tmem_dealloc(tmem_base, 512);
   }
   if (tid == 0 && *abort_flag) raise(p.dev_status, SG_ERR_TIMEOUT);
   if (p.clock_out && tid == 0) {
@@ -1077,28 +734,24 @@ std::atomic<int> g_test_wait_limit_ms{0};
 std::atomic<unsigned long long*> g_test_clock_out{nullptr};
 
 struct ScorePlan {
-  int R, Rpad, Ralloc, k_stages, q_bufs, tiles_per_chunk, max_items, smem_bytes, U, lag, wgslots;
-  size_t counter_bytes, workspace_bytes;
+  int R, Ralloc, k_stages, q_bufs, smem_bytes, U, group, groups, grid;
+  size_t workspace_bytes;
   bool ok;
 };
 
-ScorePlan plan_score(const sg_shape* s) {
+// `limit`: the most workspace there is (0 = whatever the plan needs); fewer CTAs need fewer records.
+ScorePlan plan_score(const sg_shape* s, size_t limit = 0) {
   ScorePlan pl{};
   const int D = s->head_dim;
   const int G = s->num_q_heads / s->num_kv_heads;
   pl.R = G * s->window;
-  pl.Rpad = (pl.R + 15) & ~15;
   pl.Ralloc = (pl.R + 127) & ~127;
   const int q_bytes = pl.Ralloc * D * 2;
   const int k_stage = kTileKeys * D * 2;
-  const int part_slots = pl.Rpad > 384 ? 4 : (pl.Rpad > 128 ? 8 : 0);
-  // Row blocks are dealt to the four epilogue warpgroups in rotation.  When their number is a multiple of four a
-  // row block always meets the same warpgroup, so one statistics slot per item suffices; otherwise every
-  // warpgroup keeps (and publishes) its own.
-  pl.wgslots = ((pl.Ralloc / 128) % kEpiGroups == 0) ? 1 : kEpiGroups;
-  const int tail = (240 + (2 + 4 * pl.wgslots) * pl.Ralloc * 4 + part_slots * kEpiGroups * 128 * 4 + kPartSlots * 4 * 4 + 32 + 2 * (s->batch + 1) * 4 + 15) & ~15;
+  const int table1 = 4 * kGroups * pl.Ralloc * 4, table2 = 2 * pl.Ralloc * 4 + kColSlots * kGroups * 128 * 4;
+  const int tail = (40 * 8 + (table1 > table2 ? table1 : table2) + 2 * (s->batch + 1) * 4 + 15) & ~15;
   const int avail = kSmemLimit - 1024 - tail;
-  // Two Q buffers let the next item's queries load while the current item computes; fall back to one
+  // Two Q buffers let the next segment's queries load while the current one computes; fall back to one
   // when that would leave fewer than three K stages.
   pl.q_bufs = 2;
   pl.k_stages = (avail - 2 * q_bytes) / k_stage;
@@ -1108,60 +761,35 @@ ScorePlan plan_score(const sg_shape* s) {
   pl.smem_bytes = 1024 + pl.q_bufs * q_bytes + pl.k_stages * k_stage + tail;
   if (pl.smem_bytes < 120 * 1024) pl.smem_bytes = 120 * 1024;     // one CTA per SM: each CTA takes the whole TMEM
   pl.U = s->num_layers * s->num_kv_heads;
-  // Chunking of the key axis.  Above the roofline ridge (R = G*W flop per K byte vs ~218) the second read of K
-  // need not come from L2, so items are long (32 tiles) to amortise the per-item work; below it they are shorter
-  // (16 tiles; 8 measured 16 % slower on the 8B shape) so that a unit's keys are still L2-resident when its pass 2 starts.  Either is halved while that
-  // leaves fewer than ~6 items per SM and pass.
-  const int64_t tiles_per_unit = (int64_t)s->total_tokens / kTileKeys + s->batch;
-  int tpc = pl.R >= 256 ? 32 : 16;
-  while (tpc > 4 && (tiles_per_unit / tpc + s->batch) * pl.U < 6 * kNumSMs) tpc /= 2;
-  pl.tiles_per_chunk = tpc;
-  pl.max_items = (int)(tiles_per_unit / tpc + s->batch + 1);
-  // Pass 2 of a unit trails its pass 1 by `lag` units.  The lag must span several times more schedule positions
-  // than there are CTAs (each slot holds about 2*C positions): a pass-2 item needs every pass-1 item of its unit
-  // published, and the helper warps prepare it one item ahead, so with a lag of one wave pass-2 items wait for
-  // statistics (measured on the 8B shape: 12-19 % of the epilogue's time at 1.25 waves, < 5 % at 3.5).  Beyond
-  // that it is kept small so that the unit's keys are still in L2 for the second read; 3.5 waves is where the
-  // time stops falling (8B shape 268 -> 232 us, long-context shape 808 -> 740 us from 1.25 to 3.5 waves).
-  const int64_t c_est = (tiles_per_unit - s->batch) / tpc + 1;
-  int64_t lag = (14 * kNumSMs / 4 + 2 * c_est - 1) / (2 * c_est) + 1;
-  if (2 * lag > pl.U) lag = pl.U;     // few units: all pass-1 items first, then all pass-2 items
-  pl.lag = (int)lag;
-  pl.counter_bytes = ((size_t)pl.U * sizeof(int) + 255) & ~(size_t)255;
-  pl.workspace_bytes = pl.counter_bytes + (size_t)2 * pl.U * pl.max_items * pl.Ralloc * sizeof(float);
+  pl.groups = 1;
+  pl.group = pl.U;
+  const int64_t tiles = (int64_t)pl.group * ((int64_t)s->total_tokens / kTileKeys + s->batch);      // upper bound
+  pl.grid = (int)(tiles < kNumSMs ? tiles : kNumSMs);
+  // records: a CTA adds at most one segment to the parts of a group
+  const int64_t record = (int64_t)pl.Ralloc * sizeof(float2), parts = (int64_t)pl.U * s->batch;
+  if (limit > 0) {
+    const int64_t most = ((int64_t)limit / record - parts) / pl.groups;
+    if (most >= 1 && most < pl.grid) pl.grid = (int)most;
+  }
+  pl.workspace_bytes = (size_t)((parts + (int64_t)pl.groups * pl.grid) * record);
   return pl;
 }
 
-// Finish time of the static schedule under a simple model (an item costs its tiles, pass 2 a little more;
-// a pass-2 item starts when its CTA is free and every pass-1 item of its unit is done).  CTA k takes
-// positions k, k + grid, ...; with items of 4-32 tiles, where the empty positions fall decides whether some
-// CTA ends up one item behind, so the host plays both layouts through and keeps the faster.
-double simulate_schedule(int U, int C, int lag, bool compact, int grid, int tiles) {
-  std::vector<double> clock((size_t)grid, 0.0), done1((size_t)U, 0.0);
-  const long long npos = schedule_length(U, C, lag, compact);
-  double end = 0.0;
-  for (long long pos = 0; pos < npos; ++pos) {
-    const SchedPos sp = schedule_position(pos, U, C, lag, compact);
-    if (sp.pass == 0) continue;
-    double& c = clock[(size_t)(pos % grid)];
-    double start = c;
-    if (sp.pass == 2 && done1[(size_t)sp.unit] > start) start = done1[(size_t)sp.unit];
-    c = start + (sp.pass == 2 ? 1.1 : 1.0) * tiles + 1.0;
-    if (sp.pass == 1 && c > done1[(size_t)sp.unit]) done1[(size_t)sp.unit] = c;
-    if (c > end) end = c;
-  }
-  return end;
-}
-
-bool choose_compact_layout(const sg_shape* s, const ScorePlan& pl, int grid) {
-  if (pl.lag >= pl.U) return false;                               // two-phase schedule: nothing to choose
-  // items per unit and pass: exact for one sequence, an estimate for a ragged batch (lengths live on the device)
-  const long long tiles_per_unit = s->batch == 1 ? ((long long)s->total_tokens + kTileKeys - 1) / kTileKeys
-                                                 : (long long)s->total_tokens / kTileKeys + (s->batch + 1) / 2;
-  const int C = (int)((tiles_per_unit + pl.tiles_per_chunk - 1) / pl.tiles_per_chunk);
-  if (schedule_length(pl.U, C, pl.lag, false) > 40000) return false;   // long schedules: the ends do not matter
-  return simulate_schedule(pl.U, C, pl.lag, true, grid, pl.tiles_per_chunk) <
-         simulate_schedule(pl.U, C, pl.lag, false, grid, pl.tiles_per_chunk);
+template <int D, int PASS>
+sg_status launch_pass(const CUtensorMap& q, const CUtensorMap& k, const ScoreParams& p, const ScorePlan& pl, bool chained, cudaStream_t s) {
+  SG_ENSURE_SMEM((score_kernel<D, PASS>), pl.smem_bytes);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)pl.grid);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = (size_t)pl.smem_bytes;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = chained ? 1 : 0;                     // the call's first launch is fully ordered behind earlier work
+  SG_CUDA_TRY(cudaLaunchKernelEx(&cfg, score_kernel<D, PASS>, q, k, p));
+  return SG_OK;
 }
 
 }  // namespace
@@ -1187,23 +815,22 @@ extern "C" int32_t sg_testing_score_grid(const sg_shape* shape) {
   using namespace sg;
   if (check_shape(shape, true) != SG_OK) return 0;
   const ScorePlan pl = plan_score(shape);
-  if (!pl.ok) return 0;
-  const long long max_pos = (long long)(pl.U + pl.lag) * 2 * pl.max_items;
-  return (int32_t)(max_pos < kNumSMs ? max_pos : kNumSMs);
+  return pl.ok ? pl.grid : 0;
 }
 
-extern "C" sg_status sg_score(const sg_shape* shape, const void* q_win, const void* k_cache, float* importance,
-                              void* workspace, size_t workspace_bytes, int32_t* dev_status, void* stream) {
-  using namespace sg;
+namespace sg {
+namespace {
+
+sg_status run_score(const sg_shape* shape, const void* q_win, const void* k_cache, float* importance, void* workspace,
+                    size_t workspace_bytes, size_t limit, int32_t* dev_status, void* stream) {
   sg_status st = check_shape(shape, true);
   if (st != SG_OK) return st;
   if (shape->total_tokens == 0) return SG_OK;
   if (!q_win || !k_cache || !importance) return SG_ERR_INVALID;
   if (!aligned16(q_win) || !aligned16(k_cache) || !aligned16(importance) || !aligned16(workspace)) return SG_ERR_INVALID;
-  const ScorePlan pl = plan_score(shape);
+  const ScorePlan pl = plan_score(shape, limit);
   if (!pl.ok) return SG_ERR_UNSUPPORTED;
-  const size_t need = score_workspace_bytes(shape);
-  if (!workspace || workspace_bytes < need) return SG_ERR_WORKSPACE;
+  if (!workspace || workspace_bytes < pl.workspace_bytes) return SG_ERR_WORKSPACE;
   EncodeTiledFn encode = encode_tiled_fn();
   if (!encode) return cuda_fail((int)cudaErrorUnknown);
 
@@ -1242,8 +869,6 @@ extern "C" sg_status sg_score(const sg_shape* shape, const void* q_win, const vo
   ScoreParams p;
   p.cu = shape->cu_seqlens;
   p.importance = importance;
-  p.p1_done = static_cast<int*>(workspace);
-  p.part = reinterpret_cast<float2*>(static_cast<uint8_t*>(workspace) + pl.counter_bytes);
   p.dev_status = dev_status;
   p.T = shape->total_tokens;
   p.B = shape->batch;
@@ -1251,16 +876,10 @@ extern "C" sg_status sg_score(const sg_shape* shape, const void* q_win, const vo
   p.G = G;
   p.W = shape->window;
   p.R = pl.R;
-  p.Rpad = pl.Rpad;
   p.Ralloc = pl.Ralloc;
-  p.U = pl.U;
-  p.lag = pl.lag;
-  p.tiles_per_chunk = pl.tiles_per_chunk;
-  p.max_items = pl.max_items;
   p.k_stages = pl.k_stages;
   p.q_bufs = pl.q_bufs;
   p.smem_bytes = pl.smem_bytes;
-  p.wgslots = pl.wgslots;
   p.withhold_unit = g_test_withhold_unit.load(std::memory_order_relaxed);
   const int limit_ms = g_test_wait_limit_ms.load(std::memory_order_relaxed);
   p.wait_ns = limit_ms > 0 ? (uint32_t)limit_ms * 1000000u : 1000000000u;
@@ -1268,23 +887,27 @@ extern "C" sg_status sg_score(const sg_shape* shape, const void* q_win, const vo
   p.scale_log2 = kLog2e / sqrtf((float)D);
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // the per-unit completion counters must start at zero on every call (also on every graph replay)
-  SG_CUDA_TRY(cudaMemsetAsync(workspace, 0, pl.counter_bytes, s));
-  int dev = 0, sms = kNumSMs;
-  SG_CUDA_TRY(cudaGetDevice(&dev));
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = kNumSMs;
-  const long long max_pos = (long long)(pl.U + pl.lag) * 2 * pl.max_items;
-  const unsigned grid = (unsigned)(max_pos < sms ? max_pos : sms);     // persistent: one CTA per SM
-  p.compact = choose_compact_layout(shape, pl, (int)grid) ? 1 : 0;
-  if (D == 128) {
-    SG_ENSURE_SMEM((score_kernel<128>), pl.smem_bytes);
-    score_kernel<128><<<grid, kScoreThreads, pl.smem_bytes, s>>>(tmap_q, tmap_k, p);
-  } else {
-    SG_ENSURE_SMEM((score_kernel<64>), pl.smem_bytes);
-    score_kernel<64><<<grid, kScoreThreads, pl.smem_bytes, s>>>(tmap_q, tmap_k, p);
+  const size_t buffer = (size_t)(pl.group * shape->batch + pl.grid) * pl.Ralloc;      // a group's records
+  for (int u = 0, i = 0; u < pl.U; u += pl.group, ++i) {
+    p.u0 = u;
+    p.units = pl.U - u < pl.group ? pl.U - u : pl.group;
+    p.records = static_cast<float2*>(workspace) + i * buffer;
+    p.more = 1;
+    st = D == 128 ? launch_pass<128, 1>(tmap_q, tmap_k, p, pl, i > 0, s) : launch_pass<64, 1>(tmap_q, tmap_k, p, pl, i > 0, s);
+    if (st != SG_OK) return st;
+    p.more = u + pl.group < pl.U;
+    st = D == 128 ? launch_pass<128, 2>(tmap_q, tmap_k, p, pl, true, s) : launch_pass<64, 2>(tmap_q, tmap_k, p, pl, true, s);
+    if (st != SG_OK) return st;
   }
-  SG_CUDA_TRY(cudaGetLastError());
   return SG_OK;
+}
+
+}  // namespace
+}  // namespace sg
+
+extern "C" sg_status sg_score(const sg_shape* shape, const void* q_win, const void* k_cache, float* importance,
+                              void* workspace, size_t workspace_bytes, int32_t* dev_status, void* stream) {
+  return sg::run_score(shape, q_win, k_cache, importance, workspace, workspace_bytes, 0, dev_status, stream);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1293,9 +916,7 @@ extern "C" sg_status sg_score(const sg_shape* shape, const void* q_win, const vo
 // The row statistics that pass 1 hands to pass 2 normally live in a caller-provided workspace.
 // Here they live in a fixed array that is part of the library image, so the caller needs no
 // allocator at all.  The array is shared by every call on a device and keeps the previous call's
-// contents.  The per-unit completion counters at its start must be zero when the kernel begins: the
-// call clears them with a memset on `stream`, exactly as sg_score does for a caller's workspace.
-// Every other word is written by pass 1 before pass 2 reads it.
+// contents; every word of it is written by pass 1 before pass 2 reads it.
 namespace sg {
 namespace {
 static __device__ __align__(256) unsigned char g_score_static_scratch[SG_SCORE_STATIC_SCRATCH_BYTES];
@@ -1309,7 +930,7 @@ extern "C" sg_status sg_score_static(const sg_shape* shape, const void* q_win, c
   if (st != SG_OK) return st;
   if (shape->total_tokens == 0) return SG_OK;
   if (!plan_score(shape).ok) return SG_ERR_UNSUPPORTED;      // same answer as sg_score for shapes no kernel covers
-  if (score_workspace_bytes(shape) > (size_t)SG_SCORE_STATIC_SCRATCH_BYTES) return SG_ERR_WORKSPACE;
+  if (plan_score(shape, SG_SCORE_STATIC_SCRATCH_BYTES).workspace_bytes > (size_t)SG_SCORE_STATIC_SCRATCH_BYTES) return SG_ERR_WORKSPACE;
   // In host code the array's name is only a handle; the device address has to be asked for, once per
   // device, with that device current.
   static std::atomic<void*> scratch_of_device[64];
@@ -1320,5 +941,6 @@ extern "C" sg_status sg_score_static(const sg_shape* shape, const void* q_win, c
     SG_CUDA_TRY(cudaGetSymbolAddress(&scratch, g_score_static_scratch));
     if (dev >= 0 && dev < 64) scratch_of_device[dev].store(scratch, std::memory_order_release);
   }
-  return sg_score(shape, q_win, k_cache, importance, scratch, (size_t)SG_SCORE_STATIC_SCRATCH_BYTES, dev_status, stream);
+  return run_score(shape, q_win, k_cache, importance, scratch, (size_t)SG_SCORE_STATIC_SCRATCH_BYTES, (size_t)SG_SCORE_STATIC_SCRATCH_BYTES,
+                   dev_status, stream);
 }
