@@ -1,9 +1,12 @@
 // sg_pack_kv: index-driven gather of selected K/V rows into a contiguous buffer.
 //
 // Pure byte movement, bound by HBM: every selected row (2*d bytes of K, 2*d bytes of V) is read
-// once and written once.  One group of d/8 threads moves one row with 16-byte vectors, so a
-// warp's accesses cover whole 128-byte lines on both sides; each group has kUnroll independent
-// rows (2*kUnroll loads) in flight before the first store.
+// once and written once.  A CTA takes 64 (d = 128) or 128 (d = 64) neighbouring entries of one (layer, KV head) of the
+// KV index.  First one thread per entry reads the index and works out where the row comes from and goes to; then
+// groups of d/8 threads move the rows with 16-byte vectors, so a warp's accesses cover whole 128-byte lines on both
+// sides, four rows (eight loads) per group in flight before the first store.  With every thread of a group working
+// out its own row (two 64-bit divisions, a search and four dependent loads per row), the address chain and not the bytes
+// set the pace of short and of counted calls.
 #include "common.cuh"
 
 namespace sg {
@@ -23,62 +26,65 @@ struct PackParams {
   uint16_t* packed_v;
   int32_t* dev_status;
   int64_t ls, ts, hs;
-  int64_t total_rows;      // L * K_tot * H_kv
-  int64_t rows_per_layer;  // K_tot * H_kv
   int32_t K_tot, B, Hkv;
+  int32_t chunks;          // CTAs per (layer, KV head)
 };
 
 // kCounted: rows beyond a head's count (PackParams::sel_count) are skipped; the plain instantiation carries none of it.
 template <int D, bool kCounted>
 __global__ void __launch_bounds__(kPackThreads) pack_kv_kernel(const PackParams p) {
   constexpr int kTPR = D / 8;                       // threads per row, 16 bytes each
-  constexpr int kRowsPerPass = kPackThreads / kTPR;
-  const int lane_in_row = threadIdx.x % kTPR;
-  const int group = threadIdx.x / kTPR;
-  const int64_t row0 = (int64_t)blockIdx.x * (kRowsPerPass * kUnroll) + group;
-
-  int4 kv[kUnroll][2];
-  bool ok[kUnroll], skip[kUnroll];
-#pragma unroll
-  for (int u = 0; u < kUnroll; ++u) {
-    const int64_t r = row0 + (int64_t)u * kRowsPerPass;
-    ok[u] = false;
-    skip[u] = false;
-    kv[u][0] = make_int4(0, 0, 0, 0);
-    kv[u][1] = make_int4(0, 0, 0, 0);
-    if (r < p.total_rows) {
-      const int64_t l = r / p.rows_per_layer;
-      const int64_t rr = r - l * p.rows_per_layer;
-      const int b = upper_segment(p.cu_k, p.B, rr, p.Hkv);
-      const int ck = p.cu_k[b];
-      const int kb = p.cu_k[b + 1] - ck;
-      const int rem = (int)(rr - (int64_t)ck * p.Hkv);
-      const int g = rem / kb;
-      const int j = rem - g * kb;
-      const int c0 = p.cu[b];
-      const int n = p.cu[b + 1] - c0;
-      if (kCounted && j >= p.sel_count[(l * p.B + b) * p.Hkv + g]) { skip[u] = true; continue; }   // not selected: slot left as it is
-      const int t = p.sel_idx[(l * p.Hkv + g) * (int64_t)p.K_tot + ck + j];
-      if (t >= 0 && t < n) {
-        ok[u] = true;
-        const int64_t src = l * p.ls + ((int64_t)c0 + t) * p.ts + (int64_t)g * p.hs + lane_in_row * 8;
-        kv[u][0] = __ldcs(reinterpret_cast<const int4*>(p.k_cache + src));
-        kv[u][1] = __ldcs(reinterpret_cast<const int4*>(p.v_cache + src));
-      } else if (lane_in_row == 0) {
-        raise(p.dev_status, SG_ERR_INDEX);
+  constexpr int kGroups = kPackThreads / kTPR, kRows = kGroups * kUnroll;
+  __shared__ int64_t s_src[kRows], s_dst[kRows];    // element offsets; source -1: zeros, destination -1: nothing to do
+  const int lg = blockIdx.x / p.chunks, e0 = (blockIdx.x - lg * p.chunks) * kRows;
+  const int l = lg / p.Hkv, g = lg - l * p.Hkv;
+  if (threadIdx.x < kRows) {
+    const int e = e0 + threadIdx.x, lane = threadIdx.x & 31;
+    int64_t src = -1, dst = -1;
+    // the sequence that holds the warp's first entry, then on from there
+    int b = 0;
+    if (p.B > 32) {
+      b = upper_segment(p.cu_k, p.B, e - lane);
+    } else if (p.B > 1) {
+      const int end = lane < p.B ? p.cu_k[lane + 1] : 0x7fffffff;
+      b = __popc(__ballot_sync(0xffffffffu, end <= e - lane));
+    }
+    if (e < p.K_tot) {
+      int ck = p.cu_k[b], ce = p.cu_k[b + 1];
+      while (e >= ce && b + 1 < p.B) { ++b; ck = ce; ce = p.cu_k[b + 1]; }
+      const int kb = ce - ck, j = e - ck;
+      if (!kCounted || j < p.sel_count[((int64_t)l * p.B + b) * p.Hkv + g]) {
+        dst = ((int64_t)l * p.K_tot * p.Hkv + (int64_t)ck * p.Hkv + (int64_t)g * kb + j) * D;
+        const int t = p.sel_idx[(int64_t)lg * p.K_tot + e];
+        const int c0 = p.cu[b];
+        if (t >= 0 && t < p.cu[b + 1] - c0) src = l * p.ls + ((int64_t)c0 + t) * p.ts + (int64_t)g * p.hs;
+        else raise(p.dev_status, SG_ERR_INDEX);
       }
     }
+    s_src[threadIdx.x] = src;
+    s_dst[threadIdx.x] = dst;
+  }
+  __syncthreads();
+  const int x = (threadIdx.x % kTPR) * 8, group = threadIdx.x / kTPR;
+  int4 kv[kUnroll][2];
+#pragma unroll
+  for (int u = 0; u < kUnroll; ++u) {
+    const int64_t src = s_src[group + u * kGroups];
+    kv[u][0] = make_int4(0, 0, 0, 0);
+    kv[u][1] = make_int4(0, 0, 0, 0);
+    if (src >= 0) {
+      kv[u][0] = __ldcs(reinterpret_cast<const int4*>(p.k_cache + src + x));
+      kv[u][1] = __ldcs(reinterpret_cast<const int4*>(p.v_cache + src + x));
+    }
   }
 #pragma unroll
   for (int u = 0; u < kUnroll; ++u) {
-    const int64_t r = row0 + (int64_t)u * kRowsPerPass;
-    if (r < p.total_rows && !(kCounted && skip[u])) {
-      const int64_t dst = r * D + lane_in_row * 8;
-      __stcs(reinterpret_cast<int4*>(p.packed_k + dst), kv[u][0]);
-      __stcs(reinterpret_cast<int4*>(p.packed_v + dst), kv[u][1]);
+    const int64_t dst = s_dst[group + u * kGroups];
+    if (dst >= 0) {
+      __stcs(reinterpret_cast<int4*>(p.packed_k + dst + x), kv[u][0]);
+      __stcs(reinterpret_cast<int4*>(p.packed_v + dst + x), kv[u][1]);
     }
   }
-  (void)ok;
 }
 
 }  // namespace
@@ -136,19 +142,15 @@ sg_status pack_kv_launch(const sg_shape* shape, const void* k_cache, const void*
   p.K_tot = total_sel;
   p.B = shape->batch;
   p.Hkv = shape->num_kv_heads;
-  p.rows_per_layer = (int64_t)total_sel * shape->num_kv_heads;
-  p.total_rows = p.rows_per_layer * shape->num_layers;
+  const int rows = kPackThreads / (shape->head_dim / 8) * kUnroll;
+  p.chunks = total_sel / rows + (total_sel % rows != 0);
+  const int64_t grid = (int64_t)p.chunks * shape->num_layers * shape->num_kv_heads;
+  if (grid > 0x7fffffffLL) return SG_ERR_UNSUPPORTED;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (shape->head_dim == 128) {
-    const int64_t rows_per_cta = (kPackThreads / 16) * kUnroll;
-    const int64_t grid = (p.total_rows + rows_per_cta - 1) / rows_per_cta;
-    if (grid > 0x7fffffffLL) return SG_ERR_UNSUPPORTED;
     if (sel_count) pack_kv_kernel<128, true><<<(unsigned)grid, kPackThreads, 0, s>>>(p);
     else pack_kv_kernel<128, false><<<(unsigned)grid, kPackThreads, 0, s>>>(p);
   } else {
-    const int64_t rows_per_cta = (kPackThreads / 8) * kUnroll;
-    const int64_t grid = (p.total_rows + rows_per_cta - 1) / rows_per_cta;
-    if (grid > 0x7fffffffLL) return SG_ERR_UNSUPPORTED;
     if (sel_count) pack_kv_kernel<64, true><<<(unsigned)grid, kPackThreads, 0, s>>>(p);
     else pack_kv_kernel<64, false><<<(unsigned)grid, kPackThreads, 0, s>>>(p);
   }
