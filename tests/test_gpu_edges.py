@@ -1,0 +1,78 @@
+"""GPU parity at the sizes where the kernels' own cuts fall: ends of tiles, chunks and register blocks, remainders, the
+smallest and the largest of each range.  Tolerances are those of the kernels' own test files (scores: 1e-4 relative, a
+bound on a few fp32 roundings of the exponent's argument; everything else exact)."""
+import numpy as np
+import pytest
+
+import oracle
+from helpers import cu_of, rand_bf16
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("lens,L,W,Hq,Hkv,d", [
+    ((1,), 1, 1, 1, 1, 64),                                # one key, one row
+    ((127,), 1, 32, 8, 2, 128), ((128,), 1, 32, 8, 2, 128), ((129,), 1, 32, 8, 2, 128),     # ends of a key tile
+    ((384, 1, 128, 5), 3, 32, 4, 1, 64),                   # tile multiples beside single keys; a CTA per tile
+    ((130,) * 40, 8, 16, 8, 2, 64),                        # 1280 tiles: every CTA's range crosses several sequences
+    ((2560,), 1, 48, 8, 2, 128),                           # R = 192: two row blocks, the second one partial
+    ((2560, 700), 1, 65, 20, 4, 64),                       # R = 325: three row blocks over three warpgroups
+    ((1300,), 2, 33, 16, 1, 64),                           # R = 528: five row blocks, a warpgroup takes two of a tile
+    ((19000,), 1, 8, 8, 8, 64),                            # 8 x 149 tiles: one more per KV head than there are SMs
+])
+def test_score_at_the_cuts(lens, L, W, Hq, Hkv, d):
+    import gpu_ops
+    rng = np.random.default_rng(11)
+    cu = cu_of(lens)
+    q, k = rand_bf16(rng, (L, len(lens), W, Hq, d)), rand_bf16(rng, (L, int(cu[-1]), Hkv, d))
+    want = oracle.score(q, k, cu).astype(np.float64)
+    got = gpu_ops.score(q, k, cu)
+    assert np.all(np.abs(got - want) <= 1e-4 * np.abs(want) + 1e-30)
+
+
+@pytest.mark.parametrize("ks,d,Hkv", [
+    ((1,), 128, 1), ((63,), 128, 3), ((64,), 128, 2), ((65,), 128, 2), ((127,), 64, 2), ((128,), 64, 2), ((129,), 64, 3),
+    ((0, 64, 0, 1, 200), 128, 2),                          # empty rows at and between the cuts of a CTA's entries
+    ((5,) * 32, 64, 2), ((3,) * 33, 128, 1), ((2,) * 70, 64, 2),         # 32 sequences and more: the two ways of the search
+])
+@pytest.mark.parametrize("counted", [False, True])
+def test_pack_at_the_cuts(ks, d, Hkv, counted):
+    import torch
+    import gpu_ops
+    import paper_2607_28150_b200.binding as sg
+    rng = np.random.default_rng(12)
+    L, lens = 2, tuple(k + 3 for k in ks)
+    cu, ck = cu_of(lens), cu_of(ks)
+    T, K = int(cu[-1]), int(ck[-1])
+    kc, vc = rand_bf16(rng, (L, T, Hkv, d)), rand_bf16(rng, (L, T, Hkv, d))
+    sel = np.zeros((L, Hkv, K), dtype=np.int32)
+    cnt = np.zeros((L, len(ks), Hkv), dtype=np.int32)
+    want_k, want_v = np.full((L, K * Hkv, d), 0x5555, np.uint16), np.full((L, K * Hkv, d), 0x5555, np.uint16)
+    for l in range(L):
+        for b, n in enumerate(lens):
+            for g in range(Hkv):
+                sel[l, g, ck[b]:ck[b + 1]] = np.sort(rng.choice(n, ks[b], replace=False))
+                cnt[l, b, g] = rng.integers(0, ks[b] + 1) if counted else ks[b]
+                for j in range(cnt[l, b, g]):
+                    r, t = ck[b] * Hkv + g * ks[b] + j, cu[b] + sel[l, g, ck[b] + j]
+                    want_k[l, r], want_v[l, r] = kc[l, t, g], vc[l, t, g]
+    if counted:
+        pk, pv = (gpu_ops.Guarded((L, K * Hkv, d), torch.int16, 0x5555) for _ in range(2))
+        st = gpu_ops.status_word()
+        sg.sg_pack_kv_counted(gpu_ops.shape_of(L, Hkv, Hkv, d, 1, cu), gpu_ops.dev(kc), gpu_ops.dev(vc), gpu_ops.dev(sel),
+                              gpu_ops.dev(ck), K, gpu_ops.dev(cnt), pk.view, pv.view, st)
+        got_k, got_v = pk.numpy(), pv.numpy()
+        assert gpu_ops.read_status(st) == 0
+    else:
+        got_k, got_v = gpu_ops.pack_kv(kc, vc, cu, sel, ck)
+    assert np.array_equal(got_k, want_k) and np.array_equal(got_v, want_v)
+
+
+@pytest.mark.parametrize("ks", [(31,), (32,), (33,), (1024, 1025, 0, 1), (8191,), (8192,), (8193,), (20000, 7)])
+def test_split_at_the_cuts(ks):
+    from test_gpu_split import make, run_gpu
+    idx, mask, cu, ck = make(13, tuple(k + 5 for k in ks), ks, 2, (0.1, 0.5, 0.4))
+    for reorder in (True, False):
+        want = oracle.split_index(idx, mask, cu, ck, reorder=reorder)
+        for a, b in zip(run_gpu(idx, mask, cu, ck, reorder), want):
+            assert np.array_equal(a, b)
