@@ -1,7 +1,8 @@
 // sg_select_threshold: threshold (alpha) selection under a cap.
 //
 // Per (layer, sequence, KV head): the tokens whose score exceeds the row maximum minus alpha, at most cap_b
-// of them (the largest, ties to the lower index), emitted in ascending order with their count.  A threshold
+// of them (the largest, ties to the lower index), emitted in ascending order with their count.  Rows that the
+// register-resident selection holds are done by one kernel (select_topk.cu, kThr).  For longer rows: a threshold
 // set is an upper set of the score order, so it is the exact top-cap_b set (sg_select_topk's exact selection,
 // run first with the cap as its budget) cut at the threshold: one CTA per row finds the row maximum among the
 // cap_b candidates, keeps the candidates above max - alpha with a stable block-wide compaction in place,
@@ -9,6 +10,7 @@
 // image of the scores, so subnormal scores are not flushed; a NaN is never selected (but may have taken one of
 // the cap_b candidate slots: NaN-free scores are part of the contract).
 #include "common.cuh"
+#include "launch.h"
 
 namespace sg {
 namespace {
@@ -118,6 +120,7 @@ extern "C" sg_status sg_select_threshold(const sg_shape* shape, const float* sco
   if (total_cap > 0 && (!sel_idx || !aligned16(sel_idx))) return SG_ERR_INVALID;
   const int64_t rows = (int64_t)shape->num_layers * shape->batch * shape->num_kv_heads;
   if (rows > 0x7fffffffLL) return SG_ERR_UNSUPPORTED;
+  if (select_threshold_fits(shape)) return select_threshold_launch(shape, scores, alpha, cu_cap, total_cap, sel_idx, sel_count, dev_status, stream);
   if (total_cap > 0) {
     st = sg_select_topk(shape, scores, cu_cap, total_cap, sel_idx, nullptr, 0, dev_status, stream);
     if (st != SG_OK) return st;

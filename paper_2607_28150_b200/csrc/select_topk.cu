@@ -35,6 +35,9 @@ struct SelParams {
   uint16_t* packed_k;
   uint16_t* packed_v;
   int64_t ls, ts, hs;
+  // threshold selection (select_topk_reg_kernel with kThr): keep only what exceeds the row maximum minus alpha
+  int32_t* sel_count;      // [L][B][Hkv]
+  float alpha;
 };
 
 // Takes the raw bit pattern: the row is read as uint32 so that no float instruction (and no
@@ -42,6 +45,9 @@ struct SelParams {
 __device__ __forceinline__ uint32_t order_key(uint32_t u) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
+
+__device__ __forceinline__ uint32_t key_to_bits(uint32_t k) { return (k & 0x80000000u) ? (k & 0x7fffffffu) : ~k; }
+constexpr uint32_t kKeyNegInf = 0x007fffffu, kKeyPosInf = 0xff800000u;
 
 // The selection kernels are launched with programmatic stream serialization: when the kernel before them in the
 // stream (normally the scoring kernel) lets its dependents go early, their CTAs are placed while it drains, and
@@ -198,6 +204,11 @@ __global__ void __launch_bounds__(kSelThreads, 1) select_topk_kernel(const SelPa
 // copies the row's kb selected K and V rows (16 bytes per thread, kPackUnroll rows in flight per thread group)
 // into the packed buffers.  Rows are independent, so while one CTA of an SM is in its latency-bound
 // selection another streams rows: the two phases overlap across CTAs without any inter-CTA wait.
+//
+// kThr is the threshold selection (sg_select_threshold): keys above row maximum - alpha, at most kb of them.  The threshold
+// is known from the row maximum alone, so the keys above it are counted first; only a row that has more than kb of them goes
+// through the narrowing (8B shape, 256 rows, cap 20 %: exact top-cap and a trimming kernel behind it took 13.7 + 7.6 us,
+// this 9.0 us when no row reaches its cap).  NaNs do not take part.
 constexpr int kPackUnroll = 4;
 constexpr int kFinishMax = 64;                         // interval populations up to this are finished by direct ranking
 constexpr int64_t kFuseMinRows = kNumSMs;               // fewer rows than SMs cannot fill the machine with their gathers
@@ -220,7 +231,7 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* w
   return before + inc - v;
 }
 
-template <int E, int T, int PD>
+template <int E, int T, int PD, bool kThr>
 __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
   pdl_wait();
   extern __shared__ __align__(16) uint32_t smem[];
@@ -239,7 +250,8 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
   const int N = p.cu[b + 1] - c0;
   const int ck = p.cu_k[b];
   const int kb = p.cu_k[b + 1] - ck;
-  if (kb <= 0) return;
+  auto write_count = [&](int n) { if (kThr && tid == 0) p.sel_count[((int64_t)l * p.B + b) * p.Hkv + g] = n; };
+  if (kb <= 0) { write_count(0); return; }
   int32_t* out = p.sel_idx + ((int64_t)l * p.Hkv + g) * p.K_tot + ck;
   // fused packing: thread group `grp` (D/8 threads, 16 bytes each) copies selected row j of this (layer, sequence, head)
   auto pack_rows = [&](auto pos_of) {
@@ -288,9 +300,11 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
     }
     for (int j = tid; j < kb; j += T) out[j] = -1;
     pack_rows([&](int) { return -1; });
+    write_count(0);
     return;
   }
-  if (kb >= N) {                                      // whole prompt (or an over-sized budget)
+  if (kThr && kb > N && tid == 0) raise(p.dev_status, SG_ERR_INVALID);
+  if (!kThr && kb >= N) {                             // whole prompt (or an over-sized budget)
     if (kb > N && tid == 0) {
       raise(p.dev_status, SG_ERR_INVALID);
       if (PD > 0) raise(p.dev_status, SG_ERR_INDEX);   // what the packing kernel reports for the -1 entries
@@ -303,7 +317,7 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
   for (int i = tid; i < kRegCopies * kRegBins; i += T) hist[i] = 0;
   const int first = tid * E;
   const int nvalid = min(max(N - first, 0), E);        // this thread's positions inside the row
-  const uint32_t vmask = nvalid >= 32 ? 0xffffffffu : ((1u << nvalid) - 1u);
+  uint32_t vmask = nvalid >= 32 ? 0xffffffffu : ((1u << nvalid) - 1u);
   uint32_t key[E];
   if ((reinterpret_cast<uintptr_t>(x) & 15u) == 0) {
     // 16-byte aligned row: every thread reads its own E consecutive values with 16-byte loads (the lines of a
@@ -347,6 +361,11 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
   // The digit of a pass is (key - lo) >> shift with shift chosen so that the interval spans at most 2048 bins:
   // unlike the fixed top bits of a float, it spreads whatever range the row really has over all bins, so the
   // threshold bin of the first pass keeps tens of keys, not a quarter of the row, and the later passes touch few.
+  if constexpr (kThr) {                                // the keys of -inf .. +inf: everything outside is a NaN
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+      if (key[e] < kKeyNegInf || key[e] > kKeyPosInf) vmask &= ~(1u << e);
+  }
   uint32_t kmin = 0xffffffffu, kmax = 0u;
 #pragma unroll
   for (int e = 0; e < E; ++e)
@@ -359,6 +378,24 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
   kmax = __reduce_max_sync(0xffffffffu, lane < T / 32 ? wsum[T / 32 + lane] : 0u);
   __syncthreads();                                     // wsum is reused by the scans below
   uint32_t lo = kmin, hi = kmax, need = (uint32_t)kb;
+  int above_thr = kb;                                  // kThr: number selected
+  if constexpr (kThr) {
+    float thr;                                         // IEEE subtraction without flush-to-zero, whatever the compile flags
+    asm("sub.rn.f32 %0, %1, %2;" : "=f"(thr) : "f"(__uint_as_float(key_to_bits(kmax))), "f"(p.alpha));
+    uint32_t thr_bits = __float_as_uint(thr);
+    if ((thr_bits & 0x7fffffffu) == 0u) thr_bits = 0u;  // -0 and +0 compare equal as floats: use +0's key
+    const uint32_t kthr = order_key(thr_bits);
+    uint32_t n = 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) n += ((vmask >> e) & 1u) && key[e] > kthr ? 1u : 0u;
+    n = __reduce_add_sync(0xffffffffu, n);
+    if (lane == 0) wsum[warp] = n;
+    __syncthreads();
+    above_thr = kmax == 0u ? 0 : (int)__reduce_add_sync(0xffffffffu, lane < T / 32 ? wsum[lane] : 0u);
+    __syncthreads();                                   // wsum is reused by the scans below
+    if (above_thr <= kb) { lo = hi = kmax == 0u ? 0xffffffffu : kthr; need = 0; }      // everything above, nothing equal
+    else above_thr = kb;
+  }
 #pragma unroll 1
   for (int pass = 0; lo != hi; ++pass) {
     const uint32_t width = hi - lo;
@@ -452,6 +489,10 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
     if constexpr (PD > 0) stage[slot] = (uint32_t)(first + e);
     ++slot;
   }
+  if constexpr (kThr) {
+    for (int j = above_thr + tid; j < kb; j += T) out[j] = -1;
+    write_count(above_thr);
+  }
   if constexpr (PD > 0) {
     __syncthreads();
     pack_rows([&](int j) { return (int)stage[j]; });
@@ -466,8 +507,10 @@ constexpr int select_reg_smem_bytes() { return (kRegCopies * kRegBins + 2 * (T /
 
 namespace sg {
 namespace {
-// Launches the selection; with `fuse` the register-resident kernels also pack (the caller has checked that the rows fit them).
-sg_status select_launch(const sg_shape* shape, SelParams& p, bool fuse, void* stream) {
+// Launches the selection.  kPack and kThreshold are done by the register-resident kernels only (the caller has checked that
+// the rows fit them).
+enum SelectKind { kSelect, kPack, kThreshold };
+sg_status select_launch(const sg_shape* shape, SelParams& p, SelectKind kind, void* stream) {
   const int64_t rows = (int64_t)shape->num_layers * shape->batch * shape->num_kv_heads;
   if (rows > 0x7fffffffLL) return SG_ERR_UNSUPPORTED;
   cudaLaunchAttribute attr;
@@ -478,24 +521,26 @@ sg_status select_launch(const sg_shape* shape, SelParams& p, bool fuse, void* st
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   cfg.gridDim = dim3((unsigned)rows);
-  const int pd = fuse ? shape->head_dim : 0;
-#define SG_LAUNCH_SELECT_REG_PD(E, T, PD)                                                       \
+  const int pd = kind == kPack ? shape->head_dim : 0;
+#define SG_LAUNCH_SELECT_REG_PD(E, T, PD, THR)                                                     \
   do {                                                                                          \
     p.capacity = (E) * (T);                                                                     \
-    SG_ENSURE_SMEM((select_topk_reg_kernel<E, T, PD>), (select_reg_smem_bytes<E, T>()));         \
+    SG_ENSURE_SMEM((select_topk_reg_kernel<E, T, PD, THR>), (select_reg_smem_bytes<E, T>()));         \
     cfg.blockDim = dim3(T);                                                                     \
     cfg.dynamicSmemBytes = select_reg_smem_bytes<E, T>();                                       \
-    SG_CUDA_TRY(cudaLaunchKernelEx(&cfg, select_topk_reg_kernel<E, T, PD>, p));                  \
+    SG_CUDA_TRY(cudaLaunchKernelEx(&cfg, select_topk_reg_kernel<E, T, PD, THR>, p));                  \
   } while (0)
-#define SG_LAUNCH_SELECT_REG(E, T)                        \
-  do {                                                    \
-    if (pd == 128) SG_LAUNCH_SELECT_REG_PD(E, T, 128);    \
-    else if (pd == 64) SG_LAUNCH_SELECT_REG_PD(E, T, 64); \
-    else SG_LAUNCH_SELECT_REG_PD(E, T, 0);                \
+#define SG_LAUNCH_SELECT_REG(E, T)                                              \
+  do {                                                                          \
+    if (kind == kThreshold) SG_LAUNCH_SELECT_REG_PD(E, T, 0, true);             \
+    else if (pd == 128) SG_LAUNCH_SELECT_REG_PD(E, T, 128, false);              \
+    else if (pd == 64) SG_LAUNCH_SELECT_REG_PD(E, T, 64, false);                \
+    else SG_LAUNCH_SELECT_REG_PD(E, T, 0, false);                               \
   } while (0)
-  if (rows < kNumSMs && !fuse && shape->max_seqlen <= 8192 && shape->max_seqlen > 4096) {
+  if (rows < kNumSMs && kind != kPack && shape->max_seqlen <= 8192 && shape->max_seqlen > 4096) {
     // fewer rows than SMs: one CTA per SM anyway, so twice the threads per row (half the keys each) shorten the chains
-    SG_LAUNCH_SELECT_REG_PD(8, 1024, 0);
+    if (kind == kThreshold) SG_LAUNCH_SELECT_REG_PD(8, 1024, 0, true);
+    else SG_LAUNCH_SELECT_REG_PD(8, 1024, 0, false);
   } else if (shape->max_seqlen <= 4096) {
     SG_LAUNCH_SELECT_REG(8, 512);
   } else if (shape->max_seqlen <= 8192) {
@@ -504,7 +549,7 @@ sg_status select_launch(const sg_shape* shape, SelParams& p, bool fuse, void* st
     SG_LAUNCH_SELECT_REG(16, 1024);
   } else if (shape->max_seqlen <= 32768) {
     SG_LAUNCH_SELECT_REG(32, 1024);
-  } else if (fuse) {
+  } else if (kind != kSelect) {
     return SG_ERR_UNSUPPORTED;
   } else if (shape->max_seqlen <= kSelKeyCap) {
     const int smem = kSelFixedSmem + shape->max_seqlen * 4;
@@ -525,6 +570,26 @@ sg_status select_launch(const sg_shape* shape, SelParams& p, bool fuse, void* st
   return SG_OK;
 }
 }  // namespace
+}  // namespace sg
+
+namespace sg {
+bool select_threshold_fits(const sg_shape* shape) { return shape->max_seqlen <= 32768; }
+sg_status select_threshold_launch(const sg_shape* shape, const float* scores, float alpha, const int32_t* cu_cap, int32_t total_cap,
+                                  int32_t* sel_idx, int32_t* sel_count, int32_t* dev_status, void* stream) {
+  SelParams p = {};
+  p.importance = scores;
+  p.cu = shape->cu_seqlens;
+  p.cu_k = cu_cap;
+  p.sel_idx = sel_idx;
+  p.dev_status = dev_status;
+  p.T = shape->total_tokens;
+  p.K_tot = total_cap;
+  p.B = shape->batch;
+  p.Hkv = shape->num_kv_heads;
+  p.sel_count = sel_count;
+  p.alpha = alpha;
+  return select_launch(shape, p, kThreshold, stream);
+}
 }  // namespace sg
 
 extern "C" sg_status sg_select_topk(const sg_shape* shape, const float* importance, const int32_t* cu_k,
@@ -549,7 +614,7 @@ extern "C" sg_status sg_select_topk(const sg_shape* shape, const float* importan
   p.K_tot = total_sel;
   p.B = shape->batch;
   p.Hkv = shape->num_kv_heads;
-  return select_launch(shape, p, false, stream);
+  return select_launch(shape, p, kSelect, stream);
 }
 
 extern "C" sg_status sg_select_pack_kv(const sg_shape* shape, const float* importance, const int32_t* cu_k,
@@ -590,5 +655,5 @@ extern "C" sg_status sg_select_pack_kv(const sg_shape* shape, const float* impor
   p.ls = shape->cache_layer_stride;
   p.ts = shape->cache_token_stride;
   p.hs = shape->cache_head_stride;
-  return select_launch(shape, p, true, stream);
+  return select_launch(shape, p, kPack, stream);
 }

@@ -76,3 +76,16 @@ def test_split_at_the_cuts(ks):
         want = oracle.split_index(idx, mask, cu, ck, reorder=reorder)
         for a, b in zip(run_gpu(idx, mask, cu, ck, reorder), want):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n", [1, 31, 4096, 4097, 8192, 8193, 16385, 32768, 32769])
+def test_threshold_at_the_cuts(n):
+    """Row lengths at the ends of every kernel variant; caps that bind, that are met exactly and that are the whole row."""
+    from test_gpu_threshold import run
+    rng = np.random.default_rng(14)
+    x = np.round(rng.standard_normal((2, 2, n)) * 8).astype(np.float32) / 4                # many ties
+    x[0, 0, n // 2] = -np.inf
+    above = int((x[1, 0] > x[1, 0].max() - 1.5).sum())
+    for cap in sorted({1, min(above, n), min(above + 1, n), max(1, above - 1), n}):
+        run(x, (n,), (cap,), 1.5)
+    run(np.full((1, 1, n), -np.inf, np.float32), (n,), (n,), 1.0)                           # nothing exceeds -inf
