@@ -2,13 +2,12 @@
 //
 // Every KV block of the call's layers whose flat id l*M + m is in the selected set is copied, all KV heads,
 // K and V, to the same token positions of the decode-side cache.  Pure byte movement, bound by HBM: a
-// selected row is read once and written once.  One CTA per (block, sequence, layer): it looks its block up
-// in the ascending selected list once (a uniform binary search, L2-resident) and leaves if the block is not
-// selected or holds no token of the sequence -- unselected blocks cost no cache traffic.  Otherwise one
-// group of d/8 threads moves one (token, head) row with 16-byte vectors, a warp covers whole 128-byte
-// lines, and each group has kUnroll independent rows (2*kUnroll loads) in flight before the first store.
-// The rows of a block form one contiguous run when the cache is dense.  Optionally the same CTA marks the
-// block's tokens as local (1) in the decode-side KV mask, the update the paper sends behind every pushed block.
+// selected row is read once and written once.  One CTA per selected block and sequence; a call whose list is longer than
+// the blocks of its layers (one layer out of a whole list) launches one CTA per block instead, which looks its block
+// up in the ascending list (a uniform binary search, L2-resident) and leaves if it is not there.  In a dense cache the
+// block's rows are one contiguous run, moved as such; else one group of d/8 threads moves one (token, head) row.  Either
+// way with 16-byte vectors, kUnroll of K and of V in flight per thread before the first store.  Optionally the same CTA
+// marks the block's tokens as local (1) in the decode-side KV mask, the update the paper sends behind every pushed block.
 #include "common.cuh"
 
 namespace sg {
@@ -27,27 +26,54 @@ struct PushParams {
   int8_t* kv_mask;         // [layers][T] decode-side KV mask to update (1 = local) for the pushed tokens, or null
   int64_t T;
   int64_t ls, ts, hs;
-  int32_t B, Hkv, M, layer, K_r;
+  int32_t B, Hkv, M, layer, layers, K_r;
 };
 
-template <int D>
+// kByList: blockIdx.x counts the list's entries, else the blocks of the call's layers.
+template <int D, bool kByList>
 __global__ void __launch_bounds__(kPushThreads) push_blocks_kernel(const PushParams p) {
   constexpr int kTPR = D / 8;                       // threads per row, 16 bytes each
   constexpr int kRowsPerPass = kPushThreads / kTPR;
-  const int m = blockIdx.x, b = blockIdx.y, l = blockIdx.z;
-  const int32_t id = (int32_t)(((int64_t)p.layer + l) * p.M + m);
-  int lo = 0, hi = p.K_r;                           // binary search in the ascending list, uniform over the CTA
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (p.selected[mid] < id) lo = mid + 1; else hi = mid;
+  const int b = blockIdx.y;
+  int l, m;
+  if constexpr (kByList) {
+    const int id = p.selected[blockIdx.x];
+    l = id / p.M - p.layer;
+    if (id < 0 || l < 0 || l >= p.layers) return;   // a block of another call's layers
+    m = id % p.M;
+  } else {
+    l = blockIdx.x / p.M;
+    m = blockIdx.x - l * p.M;
+    const int32_t id = (p.layer + l) * p.M + m;
+    int lo = 0, hi = p.K_r;                         // binary search in the ascending list, uniform over the CTA
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (p.selected[mid] < id) lo = mid + 1; else hi = mid;
+    }
+    if (lo >= p.K_r || p.selected[lo] != id) return;
   }
-  if (lo >= p.K_r || p.selected[lo] != id) return;
   const int64_t c0 = p.cu[b], N = p.cu[b + 1] - c0;
   // tokens t with floor(t * M / N) == m
   const int64_t t0 = ((int64_t)m * N + p.M - 1) / p.M, t1 = ((int64_t)(m + 1) * N + p.M - 1) / p.M;
   const int rows = (int)(t1 - t0) * p.Hkv;
   if (p.kv_mask)                                    // the pushed tokens are locally available from now on
     for (int t = threadIdx.x; t < (int)(t1 - t0); t += kPushThreads) p.kv_mask[(int64_t)l * p.T + c0 + t0 + t] = 1;
+  if (p.hs == D && p.ts == (int64_t)p.Hkv * D) {
+    const int64_t base = (int64_t)l * p.ls + (c0 + t0) * p.ts;
+    const int4 *sk = reinterpret_cast<const int4*>(p.src_k + base), *sv = reinterpret_cast<const int4*>(p.src_v + base);
+    int4 *dk = reinterpret_cast<int4*>(p.dst_k + base), *dv = reinterpret_cast<int4*>(p.dst_v + base);
+    const int64_t n = (int64_t)rows * kTPR;
+    for (int64_t i0 = threadIdx.x; i0 < n; i0 += kPushThreads * kUnroll) {
+      int4 kv[kUnroll][2];
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u)
+        if (i0 + u * kPushThreads < n) { kv[u][0] = __ldcs(sk + i0 + u * kPushThreads); kv[u][1] = __ldcs(sv + i0 + u * kPushThreads); }
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u)
+        if (i0 + u * kPushThreads < n) { __stcs(dk + i0 + u * kPushThreads, kv[u][0]); __stcs(dv + i0 + u * kPushThreads, kv[u][1]); }
+    }
+    return;
+  }
   const int lane_in_row = threadIdx.x % kTPR;
   const int group = threadIdx.x / kTPR;
   const int64_t base = (int64_t)l * p.ls + (c0 + t0) * p.ts + lane_in_row * 8;
@@ -106,12 +132,21 @@ extern "C" sg_status sg_push_blocks(const sg_shape* shape, int32_t num_blocks, i
   p.Hkv = shape->num_kv_heads;
   p.M = num_blocks;
   p.layer = layer;
+  p.layers = shape->num_layers;
   p.K_r = num_selected;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (shape->batch > 65535 || shape->num_layers > 65535) return SG_ERR_UNSUPPORTED;
-  const dim3 grid((unsigned)num_blocks, (unsigned)shape->batch, (unsigned)shape->num_layers);
-  if (shape->head_dim == 128) push_blocks_kernel<128><<<grid, kPushThreads, 0, s>>>(p);
-  else push_blocks_kernel<64><<<grid, kPushThreads, 0, s>>>(p);
+  const int64_t blocks = (int64_t)num_blocks * shape->num_layers;
+  // 8 layers, 1024 blocks each, 3277 of them listed: by list 35.3 us, by block 42.9
+  const bool by_list = num_selected <= blocks;
+  const dim3 grid((unsigned)(by_list ? num_selected : blocks), (unsigned)shape->batch);
+  if (shape->head_dim == 128) {
+    if (by_list) push_blocks_kernel<128, true><<<grid, kPushThreads, 0, s>>>(p);
+    else push_blocks_kernel<128, false><<<grid, kPushThreads, 0, s>>>(p);
+  } else {
+    if (by_list) push_blocks_kernel<64, true><<<grid, kPushThreads, 0, s>>>(p);
+    else push_blocks_kernel<64, false><<<grid, kPushThreads, 0, s>>>(p);
+  }
   SG_CUDA_TRY(cudaGetLastError());
   return SG_OK;
 }

@@ -89,3 +89,12 @@ def test_threshold_at_the_cuts(n):
     for cap in sorted({1, min(above, n), min(above + 1, n), max(1, above - 1), n}):
         run(x, (n,), (cap,), 1.5)
     run(np.full((1, 1, n), -np.inf, np.float32), (n,), (n,), 1.0)                           # nothing exceeds -inf
+
+
+@pytest.mark.parametrize("lens,Hkv,d,M,n_sel", [
+    ((640,), 3, 128, 64, 64), ((641, 1, 90), 2, 64, 64, 9), ((5,), 1, 64, 8, 1),      # a list no longer than the layer's blocks
+])
+@pytest.mark.parametrize("head_major", [False, True])
+def test_push_by_list(lens, Hkv, d, M, n_sel, head_major):
+    from test_gpu_push import run_case
+    run_case(15, lens, Hkv, d, M, 2, n_sel, head_major)
