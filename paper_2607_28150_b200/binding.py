@@ -1,9 +1,12 @@
-"""ctypes binding of libsmartgen.so: same names as the C ABI, argument marshalling only.
+"""Python binding of libsmartgen.so: same names as the C ABI, argument marshalling only.
 
 Every function takes torch CUDA tensors (PyTorch is used for device memory and streams, nothing
 else), checks dtypes/contiguity, passes raw pointers to the library and raises `SmartGenError` on a
 non-zero status.  All computation happens in the library's CUDA kernels; there is no fallback --
 importing this module without the built library raises.
+
+The calls of the hot path are marshalled by the extension module `_native` (csrc/native.cpp: a few dozen
+nanoseconds per tensor); the rest, which no timed loop contains, go through ctypes here.
 """
 from __future__ import annotations
 
@@ -30,6 +33,8 @@ if not os.path.exists(LIB_PATH):
     raise ImportError("libsmartgen.so is not built (%s): run `python __graft_entry__.py` or "
                       "`python -m paper_2607_28150_b200.build`; there is no CPU fallback" % LIB_PATH)
 _lib = ctypes.CDLL(LIB_PATH)
+
+from . import _native  # noqa: E402  (needs the library above)
 
 
 class SmartGenError(RuntimeError):
@@ -165,12 +170,6 @@ def _stream(stream) -> Optional[int]:
     return getattr(stream, "cuda_stream", stream) or None
 
 
-def _ws(workspace: Optional[torch.Tensor]):
-    if workspace is None:
-        return None, 0
-    return workspace.data_ptr(), workspace.numel() * workspace.element_size()
-
-
 def sg_strerror(status: int) -> str:
     return _lib.sg_strerror(status).decode()
 
@@ -191,11 +190,7 @@ def alloc_workspace(op: int, shape: Shape, total_sel: int = 0, total_loc: int = 
 
 def sg_score(shape: Shape, q_win: torch.Tensor, k_cache: torch.Tensor, importance: torch.Tensor,
              workspace: Optional[torch.Tensor] = None, dev_status: Optional[torch.Tensor] = None, stream=None) -> None:
-    _check(q_win, _BF16, "q_win"); _check(k_cache, _BF16, "k_cache"); _check(importance, torch.float32, "importance")
-    _check(dev_status, torch.int32, "dev_status", True)
-    w, wb = _ws(workspace)
-    rc = _lib.sg_score(ctypes.byref(shape), _ptr(q_win), k_cache.data_ptr(), _ptr(importance), w, wb,
-                       _ptr(dev_status), _stream(stream))
+    rc = _native.score(shape, q_win, k_cache, importance, workspace, dev_status, stream)
     if rc:
         raise SmartGenError(rc, "sg_score")
 
@@ -205,10 +200,7 @@ def sg_score_static(shape: Shape, q_win: torch.Tensor, k_cache: torch.Tensor, im
     """`sg_score` for callers that cannot allocate device memory: the scratch between the two scoring
     passes is a fixed array inside the library (SG_SCORE_STATIC_SCRATCH_BYTES), shared by all calls on a
     device, so calls must not overlap on the GPU.  Shapes that need more scratch raise SG_ERR_WORKSPACE."""
-    _check(q_win, _BF16, "q_win"); _check(k_cache, _BF16, "k_cache"); _check(importance, torch.float32, "importance")
-    _check(dev_status, torch.int32, "dev_status", True)
-    rc = _lib.sg_score_static(ctypes.byref(shape), _ptr(q_win), k_cache.data_ptr(), _ptr(importance),
-                              _ptr(dev_status), _stream(stream))
+    rc = _native.score_static(shape, q_win, k_cache, importance, dev_status, stream)
     if rc:
         raise SmartGenError(rc, "sg_score_static")
 
@@ -216,11 +208,7 @@ def sg_score_static(shape: Shape, q_win: torch.Tensor, k_cache: torch.Tensor, im
 def sg_select_topk(shape: Shape, importance: torch.Tensor, cu_k: torch.Tensor, total_sel: int,
                    sel_idx: torch.Tensor, workspace: Optional[torch.Tensor] = None,
                    dev_status: Optional[torch.Tensor] = None, stream=None) -> None:
-    _check(importance, torch.float32, "importance"); _check(cu_k, torch.int32, "cu_k")
-    _check(sel_idx, torch.int32, "sel_idx"); _check(dev_status, torch.int32, "dev_status", True)
-    w, wb = _ws(workspace)
-    rc = _lib.sg_select_topk(ctypes.byref(shape), _ptr(importance), cu_k.data_ptr(), total_sel, _ptr(sel_idx), w, wb,
-                             _ptr(dev_status), _stream(stream))
+    rc = _native.select_topk(shape, importance, cu_k, total_sel, sel_idx, workspace, dev_status, stream)
     if rc:
         raise SmartGenError(rc, "sg_select_topk")
 
@@ -228,11 +216,7 @@ def sg_select_topk(shape: Shape, importance: torch.Tensor, cu_k: torch.Tensor, t
 def sg_pack_kv(shape: Shape, k_cache: torch.Tensor, v_cache: torch.Tensor, sel_idx: torch.Tensor,
                cu_k: torch.Tensor, total_sel: int, packed_k: torch.Tensor, packed_v: torch.Tensor,
                dev_status: Optional[torch.Tensor] = None, stream=None) -> None:
-    _check(k_cache, _BF16, "k_cache"); _check(v_cache, _BF16, "v_cache"); _check(sel_idx, torch.int32, "sel_idx")
-    _check(cu_k, torch.int32, "cu_k"); _check(packed_k, _BF16, "packed_k"); _check(packed_v, _BF16, "packed_v")
-    _check(dev_status, torch.int32, "dev_status", True)
-    rc = _lib.sg_pack_kv(ctypes.byref(shape), k_cache.data_ptr(), v_cache.data_ptr(), _ptr(sel_idx), cu_k.data_ptr(),
-                         total_sel, _ptr(packed_k), _ptr(packed_v), _ptr(dev_status), _stream(stream))
+    rc = _native.pack_kv(shape, k_cache, v_cache, sel_idx, cu_k, total_sel, packed_k, packed_v, dev_status, stream)
     if rc:
         raise SmartGenError(rc, "sg_pack_kv")
 
@@ -244,16 +228,8 @@ def sg_sparse_decode_attn(shape: Shape, q: torch.Tensor, packed_k: Optional[torc
                           out: torch.Tensor, lse: Optional[torch.Tensor] = None, softmax_scale: float = 0.0,
                           workspace: Optional[torch.Tensor] = None, dev_status: Optional[torch.Tensor] = None,
                           stream=None) -> None:
-    _check(q, _BF16, "q"); _check(out, _BF16, "out"); _check(cu_k, torch.int32, "cu_k")
-    _check(cu_nloc, torch.int32, "cu_nloc"); _check(packed_k, _BF16, "packed_k", True)
-    _check(packed_v, _BF16, "packed_v", True); _check(local_k, _BF16, "local_k", True)
-    _check(local_v, _BF16, "local_v", True); _check(local_idx, torch.int32, "local_idx", True)
-    _check(lse, torch.float32, "lse", True); _check(dev_status, torch.int32, "dev_status", True)
-    w, wb = _ws(workspace)
-    rc = _lib.sg_sparse_decode_attn(ctypes.byref(shape), q.data_ptr(), _ptr(packed_k), _ptr(packed_v), cu_k.data_ptr(),
-                                    total_sel, _ptr(local_k), _ptr(local_v), _ptr(local_idx), cu_nloc.data_ptr(),
-                                    total_loc, softmax_scale, out.data_ptr(), _ptr(lse), w, wb, _ptr(dev_status),
-                                    _stream(stream))
+    rc = _native.sparse_decode_attn(shape, q, packed_k, packed_v, cu_k, total_sel, local_k, local_v, local_idx, cu_nloc, total_loc,
+                                    out, lse, softmax_scale, workspace, dev_status, stream)
     if rc:
         raise SmartGenError(rc, "sg_sparse_decode_attn")
 
@@ -264,13 +240,8 @@ def sg_split_index(shape: Shape, kv_index: torch.Tensor, cu_k: torch.Tensor, tot
                    dev_status: Optional[torch.Tensor] = None, stream=None) -> None:
     """Algorithm 1: split each KV index row into local (mask 1) and remote (mask 2) lists, optionally reordering
     the row so that remote entries come first."""
-    _check(kv_index, torch.int32, "kv_index"); _check(cu_k, torch.int32, "cu_k"); _check(kv_mask, torch.int8, "kv_mask")
-    _check(reordered, torch.int32, "reordered", True); _check(local_index, torch.int32, "local_index")
-    _check(remote_index, torch.int32, "remote_index"); _check(n_local, torch.int32, "n_local")
-    _check(n_remote, torch.int32, "n_remote"); _check(dev_status, torch.int32, "dev_status", True)
-    rc = _lib.sg_split_index(ctypes.byref(shape), _ptr(kv_index), cu_k.data_ptr(), total_sel, _ptr(kv_mask),
-                             1 if reorder else 0, _ptr(reordered), _ptr(local_index), _ptr(remote_index),
-                             n_local.data_ptr(), n_remote.data_ptr(), _ptr(dev_status), _stream(stream))
+    rc = _native.split_index(shape, kv_index, cu_k, total_sel, kv_mask, 1 if reorder else 0, reordered, local_index, remote_index,
+                             n_local, n_remote, dev_status, stream)
     if rc:
         raise SmartGenError(rc, "sg_split_index")
 
@@ -314,11 +285,7 @@ def sg_select_threshold(shape: Shape, scores: torch.Tensor, alpha: float, cu_cap
                         stream=None) -> None:
     """Threshold selection under a cap: per row the positions with score > row max - alpha (at most cap_b, the
     largest first, ties to the lower index), ascending then -1, plus the count per (layer, sequence, KV head)."""
-    _check(scores, torch.float32, "scores"); _check(cu_cap, torch.int32, "cu_cap")
-    _check(sel_idx, torch.int32, "sel_idx", total_cap == 0); _check(sel_count, torch.int32, "sel_count")
-    _check(dev_status, torch.int32, "dev_status", True)
-    rc = _lib.sg_select_threshold(ctypes.byref(shape), _ptr(scores), alpha, _ptr(cu_cap), total_cap, _ptr(sel_idx),
-                                  _ptr(sel_count), _ptr(dev_status), _stream(stream))
+    rc = _native.select_threshold(shape, scores, alpha, cu_cap, total_cap, sel_idx, sel_count, dev_status, stream)
     if rc:
         raise SmartGenError(rc, "sg_select_threshold")
 
@@ -327,12 +294,7 @@ def sg_select_pack_kv(shape: Shape, importance: torch.Tensor, cu_k: torch.Tensor
                       v_cache: torch.Tensor, sel_idx: torch.Tensor, packed_k: torch.Tensor, packed_v: torch.Tensor,
                       dev_status: Optional[torch.Tensor] = None, stream=None) -> None:
     """sg_select_topk then sg_pack_kv in one call (one fused kernel where that pays); same outputs as the two calls."""
-    _check(importance, torch.float32, "importance"); _check(cu_k, torch.int32, "cu_k")
-    _check(k_cache, _BF16, "k_cache"); _check(v_cache, _BF16, "v_cache"); _check(sel_idx, torch.int32, "sel_idx", total_sel == 0)
-    _check(packed_k, _BF16, "packed_k", total_sel == 0); _check(packed_v, _BF16, "packed_v", total_sel == 0)
-    _check(dev_status, torch.int32, "dev_status", True)
-    rc = _lib.sg_select_pack_kv(ctypes.byref(shape), _ptr(importance), _ptr(cu_k), total_sel, _ptr(k_cache), _ptr(v_cache),
-                                _ptr(sel_idx), _ptr(packed_k), _ptr(packed_v), _ptr(dev_status), _stream(stream))
+    rc = _native.select_pack_kv(shape, importance, cu_k, total_sel, k_cache, v_cache, sel_idx, packed_k, packed_v, dev_status, stream)
     if rc:
         raise SmartGenError(rc, "sg_select_pack_kv")
 
@@ -341,12 +303,7 @@ def sg_pack_kv_counted(shape: Shape, k_cache: torch.Tensor, v_cache: torch.Tenso
                        cu_cap: torch.Tensor, total_cap: int, sel_count: torch.Tensor, packed_k: torch.Tensor,
                        packed_v: torch.Tensor, dev_status: Optional[torch.Tensor] = None, stream=None) -> None:
     """sg_pack_kv for per-head counts: only the first sel_count[l][b][g] entries of each row of sel_idx are packed."""
-    _check(k_cache, _BF16, "k_cache"); _check(v_cache, _BF16, "v_cache"); _check(sel_idx, torch.int32, "sel_idx", total_cap == 0)
-    _check(cu_cap, torch.int32, "cu_cap"); _check(sel_count, torch.int32, "sel_count")
-    _check(packed_k, _BF16, "packed_k", total_cap == 0); _check(packed_v, _BF16, "packed_v", total_cap == 0)
-    _check(dev_status, torch.int32, "dev_status", True)
-    rc = _lib.sg_pack_kv_counted(ctypes.byref(shape), _ptr(k_cache), _ptr(v_cache), _ptr(sel_idx), _ptr(cu_cap), total_cap,
-                                 _ptr(sel_count), _ptr(packed_k), _ptr(packed_v), _ptr(dev_status), _stream(stream))
+    rc = _native.pack_kv_counted(shape, k_cache, v_cache, sel_idx, cu_cap, total_cap, sel_count, packed_k, packed_v, dev_status, stream)
     if rc:
         raise SmartGenError(rc, "sg_pack_kv_counted")
 
@@ -360,16 +317,8 @@ def sg_sparse_decode_attn_counted(shape: Shape, q: torch.Tensor, packed_k: Optio
                                   local_skip: Optional[torch.Tensor] = None) -> None:
     """sg_sparse_decode_attn for per-head counts: of the cap_b packed rows of (b, g) only the first packed_count[b][g]
     are attended, and the first local_skip[b][g] entries of its local-index row are left out."""
-    _check(q, _BF16, "q"); _check(out, _BF16, "out"); _check(cu_cap, torch.int32, "cu_cap"); _check(cu_nloc, torch.int32, "cu_nloc")
-    _check(packed_count, torch.int32, "packed_count", True); _check(local_skip, torch.int32, "local_skip", True)
-    _check(packed_k, _BF16, "packed_k", True); _check(packed_v, _BF16, "packed_v", True)
-    _check(local_k, _BF16, "local_k", True); _check(local_v, _BF16, "local_v", True)
-    _check(local_idx, torch.int32, "local_idx", True); _check(lse, torch.float32, "lse", True)
-    _check(dev_status, torch.int32, "dev_status", True)
-    rc = _lib.sg_sparse_decode_attn_counted(ctypes.byref(shape), _ptr(q), _ptr(packed_k), _ptr(packed_v), _ptr(cu_cap), total_cap,
-                                            _ptr(packed_count), _ptr(local_k), _ptr(local_v), _ptr(local_idx), _ptr(cu_nloc),
-                                            total_loc, _ptr(local_skip), softmax_scale, _ptr(out), _ptr(lse), _ptr(dev_status),
-                                            _stream(stream))
+    rc = _native.sparse_decode_attn_counted(shape, q, packed_k, packed_v, cu_cap, total_cap, packed_count, local_k, local_v, local_idx,
+                                            cu_nloc, total_loc, out, lse, softmax_scale, dev_status, stream, local_skip)
     if rc:
         raise SmartGenError(rc, "sg_sparse_decode_attn_counted")
 
@@ -381,15 +330,41 @@ def sg_push_blocks(shape: Shape, num_blocks: int, layer: int, selected: Optional
     `layer` .. `layer + shape.num_layers - 1` from the source cache to the same positions of the destination
     cache (the tensors start at `layer`); other rows are untouched.  With `kv_mask` (int8 [layers][T]) the pushed
     tokens are also marked local (1) in the decode-side KV mask."""
-    _check(selected, torch.int32, "selected", True)
-    for name, t in (("src_k", src_k), ("src_v", src_v), ("dst_k", dst_k), ("dst_v", dst_v)):
-        _check(t, _BF16, name)
-    _check(kv_mask, torch.int8, "kv_mask", True)
-    n = 0 if selected is None else selected.numel()
-    rc = _lib.sg_push_blocks(ctypes.byref(shape), num_blocks, layer, _ptr(selected), n, _ptr(src_k), _ptr(src_v),
-                             _ptr(dst_k), _ptr(dst_v), _ptr(kv_mask), _stream(stream))
+    rc = _native.push_blocks(shape, num_blocks, layer, selected, src_k, src_v, dst_k, dst_v, kv_mask, stream)
     if rc:
         raise SmartGenError(rc, "sg_push_blocks")
+
+
+def prefill(shape: Shape, q_win: torch.Tensor, k_cache: torch.Tensor, v_cache: torch.Tensor, importance: torch.Tensor,
+            workspace: Optional[torch.Tensor], cu_k: torch.Tensor, total_sel: int, sel_idx: torch.Tensor, packed_k: torch.Tensor,
+            packed_v: torch.Tensor, dev_status: Optional[torch.Tensor] = None, stream=None) -> None:
+    """sg_score, then sg_select_pack_kv, marshalled once."""
+    rc = _native.prefill(shape, q_win, k_cache, v_cache, importance, workspace, cu_k, total_sel, sel_idx, packed_k, packed_v, dev_status,
+                         stream)
+    if rc:
+        raise SmartGenError(rc & 255, ("sg_score", "sg_select_pack_kv")[rc >> 8])
+
+
+def prefill_layer(shape: Shape, layer: int, q_win: torch.Tensor, k_cache: torch.Tensor, v_cache: torch.Tensor, importance: torch.Tensor,
+                  workspace: Optional[torch.Tensor], cu_k: torch.Tensor, total_sel: int, sel_idx: torch.Tensor, packed_k: torch.Tensor,
+                  packed_v: torch.Tensor, dev_status: Optional[torch.Tensor] = None, stream=None) -> None:
+    """sg_score, sg_select_topk and sg_pack_kv of one layer, marshalled once.  The tensors hold all layers (each layer
+    contiguous); `shape` describes one."""
+    rc = _native.prefill_layer(shape, layer, q_win, k_cache, v_cache, importance, workspace, cu_k, total_sel, sel_idx, packed_k, packed_v,
+                               dev_status, stream)
+    if rc:
+        raise SmartGenError(rc & 255, ("sg_score", "sg_select_topk", "sg_pack_kv")[rc >> 8])
+
+
+def decode_layer(shape: Shape, layer: int, q: torch.Tensor, packed_k: torch.Tensor, packed_v: torch.Tensor, cu_k: torch.Tensor,
+                 total_sel: int, local_k: Optional[torch.Tensor], local_v: Optional[torch.Tensor], local_idx: Optional[torch.Tensor],
+                 cu_nloc: torch.Tensor, total_loc: int, out: torch.Tensor, lse: Optional[torch.Tensor] = None, softmax_scale: float = 0.0,
+                 workspace: Optional[torch.Tensor] = None, dev_status: Optional[torch.Tensor] = None, stream=None) -> None:
+    """sg_sparse_decode_attn on layer `layer` of packed tensors that hold all layers."""
+    rc = _native.decode_layer(shape, layer, q, packed_k, packed_v, cu_k, total_sel, local_k, local_v, local_idx, cu_nloc, total_loc, out, lse,
+                              softmax_scale, workspace, dev_status, stream)
+    if rc:
+        raise SmartGenError(rc, "sg_sparse_decode_attn")
 
 
 def sg_speculative_delivered(num_layers: int, num_blocks: int, k_r: int, ratio: float, iteration: int) -> int:

@@ -2,7 +2,8 @@
 
 Each csrc/*.cu is compiled to an object under build/ (in parallel, skipped when up to date) and
 the objects are linked into paper_2607_28150_b200/libsmartgen.so with the CUDA runtime linked
-statically, so the library loads on a machine without a GPU or a driver.
+statically, so the library loads on a machine without a GPU or a driver.  csrc/native.cpp, the marshalling
+between torch tensors and the library, becomes the extension module _native.so beside it.
 """
 from __future__ import annotations
 
@@ -12,6 +13,7 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -19,6 +21,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OBJDIR = os.path.join(ROOT, "build", "obj")
 LIB = os.path.join(HERE, "libsmartgen.so")
+NATIVE = os.path.join(HERE, "_native.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -54,6 +57,28 @@ def _compile(src: str, obj: str, verbose: bool) -> None:
         sys.stderr.write(res.stderr)
 
 
+def _build_native(force: bool) -> None:
+    src = os.path.join(CSRC, "native.cpp")
+    newest = max(os.path.getmtime(p) for p in (src, os.path.join(INCLUDE, "smartgen.h"), os.path.abspath(__file__)))
+    if not force and os.path.exists(NATIVE) and os.path.getmtime(NATIVE) >= newest:
+        return
+    import torch
+    inc = os.path.join(os.path.dirname(torch.__file__), "include")
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
+    tmp = NATIVE + ".tmp.%d" % os.getpid()
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch.compiled_with_cxx11_abi()), "-I", INCLUDE,
+           "-isystem", inc, "-isystem", os.path.join(inc, "torch", "csrc", "api", "include"),
+           "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(cuda, "include"), src, "-o", tmp,
+           "-L", HERE, "-l:libsmartgen.so", "-L", lib, "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda",
+           "-Wl,-rpath,$ORIGIN"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("building the marshalling module failed:\n%s\n%s" % (res.stdout, res.stderr))
+    os.replace(tmp, NATIVE)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     srcs = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
     if not srcs:
@@ -80,6 +105,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         if res.returncode != 0:
             raise RuntimeError("link failed:\n%s\n%s" % (res.stdout, res.stderr))
         os.replace(tmp, LIB)
+    _build_native(force)
     with open(_STAMP, "w") as f:
         f.write(" ".join(EXTRA_FLAGS))
     return LIB

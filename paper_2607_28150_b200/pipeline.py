@@ -74,8 +74,9 @@ class HotPath:
         return self.packed_k, self.packed_v
 
     def prefill(self, q_win, k_cache, v_cache, stream=None):
-        self.score(q_win, k_cache, stream)
-        return self.select_pack(k_cache, v_cache, stream)
+        sg.prefill(self.shape, q_win, k_cache, v_cache, self.importance, self.ws_score, self.cu_k, self.K_tot, self.sel_idx, self.packed_k,
+                   self.packed_v, self.status, stream)
+        return self.packed_k, self.packed_v
 
     def prefill_layer(self, layer: int, q_win: torch.Tensor, k_cache: torch.Tensor, v_cache: torch.Tensor,
                       stream=None, aux_stream=None):
@@ -84,18 +85,19 @@ class HotPath:
         `q_win`, `k_cache`, `v_cache` are the full [L][...] tensors.  With `aux_stream`, select and pack run
         there behind an event, so the next layer's scoring on `stream` does not wait for them; the caller joins
         with `join_aux` before reading the results on `stream`."""
+        if aux_stream is None:
+            sg.prefill_layer(self.shape1, layer, q_win, k_cache, v_cache, self.importance, self.ws_score, self.cu_k, self.K_tot,
+                             self.sel_idx, self.packed_k, self.packed_v, self.status, stream)
+            return
         main = stream if stream is not None else torch.cuda.current_stream(self.device)
         sg.sg_score(self.shape1, q_win[layer], k_cache[layer], self.importance[layer], self.ws_score, self.status, main)
-        side = main
-        if aux_stream is not None:
-            ev = torch.cuda.Event()
-            ev.record(main)
-            aux_stream.wait_event(ev)
-            side = aux_stream
+        ev = torch.cuda.Event()
+        ev.record(main)
+        aux_stream.wait_event(ev)
         sg.sg_select_topk(self.shape1, self.importance[layer], self.cu_k, self.K_tot, self.sel_idx[layer], None,
-                          self.status, side)
+                          self.status, aux_stream)
         sg.sg_pack_kv(self.shape1, k_cache[layer], v_cache[layer], self.sel_idx[layer], self.cu_k, self.K_tot,
-                      self.packed_k[layer], self.packed_v[layer], self.status, side)
+                      self.packed_k[layer], self.packed_v[layer], self.status, aux_stream)
 
     def join_aux(self, aux_stream, stream=None) -> None:
         """Make `stream` wait for everything queued on `aux_stream` so far."""
@@ -124,9 +126,8 @@ class HotPath:
                lse: Optional[torch.Tensor] = None, softmax_scale: float = 0.0, stream=None) -> torch.Tensor:
         """One layer of one decode step: packed rows of `layer` plus `local_idx`-addressed rows of local_k/v."""
         ws = self.decode_workspace(total_loc)
-        sg.sg_sparse_decode_attn(self.shape1, q, self.packed_k[layer], self.packed_v[layer], self.cu_k, self.K_tot,
-                                 local_k, local_v, local_idx, cu_nloc, total_loc, out, lse, softmax_scale, ws,
-                                 self.status, stream)
+        sg.decode_layer(self.shape1, layer, q, self.packed_k, self.packed_v, self.cu_k, self.K_tot, local_k, local_v, local_idx, cu_nloc,
+                        total_loc, out, lse, softmax_scale, ws, self.status, stream)
         return out
 
     def read_status(self) -> int:
