@@ -171,13 +171,15 @@ __device__ __forceinline__ void chunk_cols(uint32_t (&cur)[32], uint64_t scale2,
 __device__ __forceinline__ int busy_ctas(long long tt) { return tt < (long long)gridDim.x ? (int)tt : (int)gridDim.x; }
 // The CTA whose range holds tile `pos` of the launch's `tt`.
 __device__ __forceinline__ int cta_of(long long pos, long long tt, int busy) { return (int)(((pos + 1) * busy - 1) / tt); }
-// A CTA's segments: its range of the launch's key tiles [c * tt / busy, (c + 1) * tt / busy), cut at part boundaries.
+// A CTA's segments: its range of the launch's key tiles [c * tt / busy, (c + 1) * tt / busy), cut at part boundaries.  Pass 2
+// walks the range backwards, segments and tiles: what pass 1 read last is still in L2 (keys of %%).
 struct Segment {
   int u, b;                // unit (counted over the whole call) and sequence
   int c0, N;               // first token and length of sequence b
   int tile_beg, tile_end;  // tiles of the part
   int part;                // part within the launch
 };
+template <int PASS>
 struct SegmentWalk {
   int C, B, u0, pos, end;
   const int *cu, *prefix;  // prefix[b] = tiles of the sequences before b (prefix[B] = C)
@@ -190,7 +192,8 @@ struct SegmentWalk {
   }
   __device__ __forceinline__ bool next(Segment& s) {
     if (pos >= end) return false;
-    const int ul = pos / C, j = pos - ul * C;
+    const int at = PASS == 1 ? pos : end - 1;         // a tile of the segment
+    const int ul = at / C, j = at - ul * C;
     int lo = 0, hi = B;
     while (hi - lo > 1) {
       const int mid = (lo + hi) >> 1;
@@ -200,13 +203,17 @@ struct SegmentWalk {
     s.b = lo;
     s.c0 = cu[lo];
     s.N = cu[lo + 1] - s.c0;
-    s.tile_beg = j - prefix[lo];
-    s.tile_end = min(prefix[lo + 1] - prefix[lo], s.tile_beg + (end - pos));
+    const int tile = j - prefix[lo];
+    s.tile_beg = PASS == 1 ? tile : max(0, tile - (at - pos));
+    s.tile_end = PASS == 1 ? min(prefix[lo + 1] - prefix[lo], tile + (end - pos)) : tile + 1;
     s.part = ul * B + lo;
-    pos += s.tile_end - s.tile_beg;
+    if (PASS == 1) pos += s.tile_end - s.tile_beg; else end -= s.tile_end - s.tile_beg;
     return true;
   }
 };
+// The i-th tile of a segment in the order of the pass.
+template <int PASS>
+__device__ __forceinline__ int tile_at(const Segment& s, int i) { return PASS == 1 ? s.tile_beg + i : s.tile_end - 1 - i; }
 
 // Log-sum-exps of a part's rows from its segments' records: rows r0, r0 + step, ..., kFlight records in flight.  Negated, as
 // the epilogue of pass 2 adds them; rows outside the window get -inf: exp2(x - inf) = 0.
@@ -345,7 +352,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
   // Another launch of this call follows: let it be set up on every SM that this one leaves (it waits for this whole grid
   // before it reads or overwrites anything that a launch wrote).
   if (p.more) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  SegmentWalk walk(C, p.units, p.B, p.u0, s_cu, s_prefix);
+  SegmentWalk<PASS> walk(C, p.units, p.B, p.u0, s_cu, s_prefix);
   Segment sg;
   // A warp's wait: every lane sees the phase complete, or none goes on.
   auto wait = [&](uint32_t bar, uint32_t parity) {
@@ -368,8 +375,9 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
 #pragma unroll
         for (int dc = 0; dc < kSub; ++dc)
           tma_load_4d(smem_u32(q_smem + qs * q_buf_bytes + dc * q_sub_bytes), &tmap_q, bar_qfull(qs), dc * 64, g * p.G, 0, l * p.B + sg.b);
-        for (int tile = sg.tile_beg; tile < sg.tile_end; ++tile) {
-          const int ks = nk % p.k_stages;
+        const int tiles = sg.tile_end - sg.tile_beg;
+        for (int i = 0; i < tiles; ++i) {
+          const int tile = tile_at<PASS>(sg, i), ks = nk % p.k_stages;
           ok = mbar_wait(bar_kempty(ks), (uint32_t)(((nk / p.k_stages) & 1) ^ 1), abort_flag, p.wait_ns, 100u);
           if (!ok) break;
           ++nk;
@@ -466,8 +474,8 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
       const uint32_t buf = (uint32_t)sidx & 1u, use = (uint32_t)sidx >> 1;
       const uint32_t n_end = n0 + (uint32_t)((sg.tile_end - sg.tile_beg) * nblk);
       uint32_t n = n0 + (kGroups + (uint32_t)wg - n0 % kGroups) % kGroups;     // this warpgroup's first block of the segment
-      int tile = sg.tile_beg, blk = (int)(n - n0);
-      while (blk >= nblk) { blk -= nblk; ++tile; }
+      int ti = 0, blk = (int)(n - n0);                                // its tile, counted in the segment, and its row block
+      while (blk >= nblk) { blk -= nblk; ++ti; }
       if (PASS == 1) {
         // The buffer's previous segment has been merged and published by the helpers (practically always true already).
         // Slot (wg, row) is only ever touched by this thread during the segment, so the statistics need no barrier.
@@ -487,6 +495,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
           // the sum of exp2(x - m) is as accurate with a stale (lower) m as with the true maximum, as long as nothing
           // overflows.  A segment starts from the maximum of the block's first 32 columns; a block whose sum leaves the safe
           // range (a value far above m) and a block with hidden scores are done carefully: true maximum first.
+          const int tile = tile_at<PASS>(sg, ti);
           bool careful = tile >= vis_end || !all_rows;
           if (!careful) {
             uint32_t a[32], b[32];
@@ -549,7 +558,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
           sm_m[blk * 128] = m;
           sm_l[blk * 128] = l;
           blk += kGroups;
-          while (blk >= nblk) { blk -= nblk; ++tile; }
+          while (blk >= nblk) { blk -= nblk; ++ti; }
         }
         // This warp's statistics of the segment are complete; the helpers merge the warpgroups' slots and publish them.
         __syncwarp();
@@ -576,7 +585,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
           SG_PROF_WAIT(w0, ok = wait(bar_afull(st), (n / kStages) & 1u));
           if (!ok) break;
           tc_fence_after();
-          const int t = tile * kTileKeys + row_in_tile;                    // this thread's key
+          const int tile = tile_at<PASS>(sg, ti), t = tile * kTileKeys + row_in_tile;      // t: this thread's key
           const float* ls = nl + blk * 128;
           if (tile < vis_end && (blk + 1) * 128 <= p.R) {
             uint32_t a[32], b[32];
@@ -608,11 +617,11 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
               chunk_cols(cur, scale2, ls + j * 32, s0, s1);
             }
           }
-          const int tile_now = tile;
+          const int ti_now = ti;
           n += kGroups;
           blk += kGroups;
-          while (blk >= nblk) { blk -= nblk; ++tile; }
-          if (tile == tile_now && n < n_end) continue;                     // more of this tile's row blocks are this warpgroup's
+          while (blk >= nblk) { blk -= nblk; ++ti; }
+          if (ti == ti_now && n < n_end) continue;                     // more of this tile's row blocks are this warpgroup's
           float lo, hi;
           unpack2(add2(s0, s1), lo, hi);
           s0 = s1 = 0ull;
@@ -620,7 +629,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
             if (t < sg.N) p.importance[(size_t)sg.u * p.T + sg.c0 + t] = lo + hi;
           } else {
             // The tile's row blocks went to different warpgroups: leave the partial column sums for the helper.
-            const uint32_t ts = (uint32_t)(tiles0 + tile_now - sg.tile_beg), cs = ts % kColSlots, cu = ts / kColSlots;
+            const uint32_t ts = (uint32_t)(tiles0 + ti_now), cs = ts % kColSlots, cu = ts / kColSlots;
             if (cu > 0) ok = wait(bar_cols_free(cs), (cu - 1u) & 1u);
             if (!ok) break;
             cols[(cs * kGroups + wg) * 128 + row_in_tile] = lo + hi;
@@ -677,7 +686,9 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
       uint32_t n = 0, ts = 0;
       const int nwg = min(nblk, kGroups);
       while (ok && walk.next(sg)) {
-        for (int tile = sg.tile_beg; tile < sg.tile_end; ++tile, ++ts, n += (uint32_t)nblk) {
+        const int tiles = sg.tile_end - sg.tile_beg;
+        for (int i = 0; i < tiles; ++i, ++ts, n += (uint32_t)nblk) {
+          const int tile = tile_at<PASS>(sg, i);
           const uint32_t cs = ts % kColSlots;
           ok = wait(bar_cols_full(cs), (ts / kColSlots) & 1u);
           if (!ok) break;

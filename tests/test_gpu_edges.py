@@ -98,3 +98,29 @@ def test_threshold_at_the_cuts(n):
 def test_push_by_list(lens, Hkv, d, M, n_sel, head_major):
     from test_gpu_push import run_case
     run_case(15, lens, Hkv, d, M, 2, n_sel, head_major)
+
+
+@pytest.mark.parametrize("lens,L,W,Hq,Hkv,d", [
+    ((33000,), 1, 4, 8, 8, 128),                           # 67.6 MB of keys: groups of several KV heads of one layer
+    ((20000, 3, 14001), 2, 16, 16, 8, 128),                # ragged, 16 units, the last group smaller
+    ((130000,), 2, 8, 4, 4, 64),                           # long rows of 64-element heads
+])
+def test_score_keys_beyond_l2(lens, L, W, Hq, Hkv, d):
+    """Calls large enough to run both passes in turn, group by group, in one launch; the call is repeated on the same
+    workspace, whose words then hold the first call's records and counts."""
+    import torch
+    import gpu_ops
+    import paper_2607_28150_b200.binding as sg
+    rng = np.random.default_rng(16)
+    cu = cu_of(lens)
+    T = int(cu[-1])
+    q, k = rand_bf16(rng, (L, len(lens), W, Hq, d)), rand_bf16(rng, (L, T, Hkv, d))
+    want = oracle.score(q, k, cu).astype(np.float64)
+    shp = gpu_ops.shape_of(L, Hq, Hkv, d, W, cu)
+    ws, st = sg.alloc_workspace(sg.SG_OP_SCORE, shp), gpu_ops.status_word()
+    dq, dk = gpu_ops.dev(q), gpu_ops.dev(k)
+    for _ in range(2):
+        imp = gpu_ops.Guarded((L, Hkv, T), torch.float32, -7.0)
+        sg.sg_score(shp, dq, dk, imp.view, ws, st)
+        assert np.all(np.abs(imp.numpy() - want) <= 1e-4 * np.abs(want) + 1e-30)
+    assert gpu_ops.read_status(st) == 0
