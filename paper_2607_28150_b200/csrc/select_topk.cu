@@ -210,7 +210,12 @@ __global__ void __launch_bounds__(kSelThreads, 1) select_topk_kernel(const SelPa
 // through the narrowing (8B shape, 256 rows, cap 20 %: exact top-cap and a trimming kernel behind it took 13.7 + 7.6 us,
 // this 9.0 us when no row reaches its cap).  NaNs do not take part.
 constexpr int kPackUnroll = 4;
-constexpr int kFinishMax = 64;                         // interval populations up to this are finished by direct ranking
+// Interval populations up to kFinishMax are finished by direct ranking.  Rows of 8192 (one CTA each, 256 of them): 64 takes
+// 13.8 us (most rows need another histogram pass), 128 takes 10.1, 256 takes 12.8.  Up to kAtomicGather of them are gathered
+// with one shared atomic per thread that has any, more of them through a block-wide prefix sum: the atomics of 100 threads
+// took 9 k clocks in a row of 32768, the prefix sum costs rows of 8192 and less 0.1 us when there are few.
+constexpr int kFinishMax = 128;
+constexpr uint32_t kAtomicGather = 64;
 constexpr int64_t kFuseMinRows = kNumSMs;               // fewer rows than SMs cannot fill the machine with their gathers
 constexpr int kRegBins = 2048;
 constexpr int kRegCopies = 2;
@@ -237,8 +242,8 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
   extern __shared__ __align__(16) uint32_t smem[];
   uint32_t* hist = smem;                               // [kRegCopies][kRegBins]
   uint32_t* wsum = hist + kRegCopies * kRegBins;       // [2][T/32]
-  uint32_t* sh = wsum + 2 * (T / 32);                  // [0] chosen bin, [1] remaining need  (8 words)
-  uint32_t* stage = sh + 8;                            // [T][E + 4] keys, each thread's segment padded by 16 bytes
+  uint32_t* sh = wsum + 2 * (T / 32);                  // [0] chosen bin, [1] remaining need ... [6], [7] barrier
+  uint32_t* stage = sh + 8;                            // [T][E + 4] keys, or [T * E] values of the row; later lists
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int row = blockIdx.x;
@@ -314,17 +319,69 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
     return;
   }
   const uint32_t* x = reinterpret_cast<const uint32_t*>(p.importance) + ((int64_t)l * p.Hkv + g) * p.T + c0;
+  // Thread t owns E consecutive values of the row.  Up to 16 of them it reads itself, with 16-byte loads where the row is
+  // 16-byte aligned (the lines of a warp's first load serve its later ones from L1), else coalesced through a padded buffer.
+  // For E = 32 the row comes to shared memory with one bulk copy from the 16-byte boundary at or before it (`off` values
+  // early), the up to three values behind the last boundary with plain loads.  Thread t's values are then the positions
+  // from t*E - off; it reads them 16 bytes at a time, starting at another quad of its segment than its neighbours (no bank
+  // conflicts), so its registers hold the segment turned by `turn` quads, and bit masks over them are turned back before use.
+  // A row of 32768: 5.7 k clocks; by the threads themselves 10.7 k (the row is larger than the L1 that shared memory leaves:
+  // every line comes from L2 several times), coalesced through the padded buffer 8.5 k.  With 16 values or fewer the bulk
+  // copy loses: 3.8 against 2.9 k clocks for a row of 8192, 2.8 against 2.3 k for 1024.
+  constexpr bool kBulk = E > 16;
+  constexpr uint32_t kAll = E >= 32 ? 0xffffffffu : ((1u << (E & 31)) - 1u);
+  constexpr int kQuads = E / 4;
+  const int turn = kBulk ? (lane / (8 / (kQuads < 8 ? kQuads : 8))) % kQuads : 0;
+  auto turned = [&](uint32_t m, int by) -> uint32_t {  // rotate the E-bit mask left by `by` quads
+    if constexpr (!kBulk) return m;
+    const int sft = 4 * by;
+    return sft == 0 ? m : ((m << sft) | (m >> (E - sft))) & kAll;
+  };
+  int off = kBulk ? (int)((reinterpret_cast<uintptr_t>(x) & 15u) >> 2) : 0;
+  const bool bulk = kBulk && N + off <= E * T;         // else the values in front of the row would push its end out of the registers
+  if (!bulk) off = 0;
+  const int span = N + off, whole = bulk ? span & ~3 : 0;                // values from the boundary on; of the bulk copy
+  const uint32_t bar = smem_u32(sh + 6);               // 8 bytes, 8-byte aligned
+  if (bulk && tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(whole * 4) : "memory");
+    if (whole > 0)
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(stage)), "l"(x - off),
+                   "r"(whole * 4), "r"(bar) : "memory");
+  }
   for (int i = tid; i < kRegCopies * kRegBins; i += T) hist[i] = 0;
-  const int first = tid * E;
-  const int nvalid = min(max(N - first, 0), E);        // this thread's positions inside the row
+  const int first = tid * E - off;                     // position of the thread's first value (negative: before the row)
+  const int nvalid = min(max(N - first, 0), E);
   uint32_t vmask = nvalid >= 32 ? 0xffffffffu : ((1u << nvalid) - 1u);
+  if constexpr (kBulk) {
+    if (first < 0) vmask &= ~((1u << -first) - 1u);    // the boundary's values in front of the row
+    vmask = turned(vmask, (kQuads - turn) % kQuads);   // as the registers hold the segment
+  }
   uint32_t key[E];
-  if ((reinterpret_cast<uintptr_t>(x) & 15u) == 0) {
-    // 16-byte aligned row: every thread reads its own E consecutive values with 16-byte loads (the lines of a
-    // warp's first load serve its later ones from L1); no staging, no barrier
-    uint4 v[E / 4];
+  if constexpr (kBulk) {
+    for (int i = whole + tid; i < span; i += T) stage[i] = __ldg(x - off + i);
+    __syncthreads();                                   // barrier set up, histogram cleared, plainly loaded values there
+    uint32_t done = bulk ? 0u : 1u;
+    for (uint32_t tries = 0; tries < (1u << 22) && !done; ++tries)
+      asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(done) : "r"(bar) : "memory");
+    if (!__syncthreads_and((int)done)) {               // does not happen: the copy has a valid source and size
+      if (tid == 0) raise(p.dev_status, SG_ERR_TIMEOUT);
+      for (int j = tid; j < kb; j += T) out[j] = -1;
+      pack_rows([&](int) { return -1; });
+      write_count(0);
+      return;
+    }
 #pragma unroll
-    for (int q = 0; q < E / 4; ++q) {
+    for (int q = 0; q < kQuads; ++q) {
+      const uint4 v = *reinterpret_cast<const uint4*>(stage + tid * E + 4 * ((q + turn) % kQuads));
+      key[4 * q] = order_key(v.x); key[4 * q + 1] = order_key(v.y);
+      key[4 * q + 2] = order_key(v.z); key[4 * q + 3] = order_key(v.w);
+    }
+  } else if ((reinterpret_cast<uintptr_t>(x) & 15u) == 0) {
+    uint4 v[kQuads];
+#pragma unroll
+    for (int q = 0; q < kQuads; ++q) {
       const int i = first + 4 * q;
       if (i + 3 < N) {
         v[q] = __ldg(reinterpret_cast<const uint4*>(x + i));
@@ -336,7 +393,7 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
       }
     }
 #pragma unroll
-    for (int q = 0; q < E / 4; ++q) {
+    for (int q = 0; q < kQuads; ++q) {
       key[4 * q] = order_key(v[q].x); key[4 * q + 1] = order_key(v[q].y);
       key[4 * q + 2] = order_key(v[q].z); key[4 * q + 3] = order_key(v[q].w);
     }
@@ -439,23 +496,43 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
     need = sh[1];
     const uint32_t ncand = sh[2];
     if (lo != hi && ncand <= (uint32_t)kFinishMax) {
-      // Few keys left in the interval: instead of more block-wide passes, gather them and let one thread per key
-      // count the keys above it and equal to it; the key whose rank range covers `need` is the threshold.
+      // Few keys left in the interval: instead of more block-wide passes, gather them and count for each the keys above it
+      // and equal to it; the key whose rank range covers `need` is the threshold.
       uint32_t* list = stage;
       const uint32_t w = hi - lo;
+      uint32_t mine = 0;
 #pragma unroll
-      for (int e = 0; e < E; ++e)
-        if (((vmask >> e) & 1u) && key[e] - lo <= w) list[atomicAdd(&sh[3], 1u)] = key[e];
+      for (int e = 0; e < E; ++e) mine |= (key[e] - lo <= w ? 1u : 0u) << e;
+      mine &= vmask;
+      uint32_t at = 0;
+      if (ncand > kAtomicGather)
+        at = block_exclusive_scan<T>((uint32_t)__popc(mine), wsum, lane, warp);
+      else if (mine)
+        at = atomicAdd(&sh[3], (uint32_t)__popc(mine));
+      if (mine) {
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+          if ((mine >> e) & 1u) list[at++] = key[e];
+      }
       __syncthreads();
-      if (tid < (int)ncand) {
-        const uint32_t k = list[tid];
+      // four lanes per key, a quarter of the list each
+      for (int i0 = 0; i0 < (int)ncand; i0 += T / 4) {
+        const int i = i0 + (tid >> 2), part = tid & 3;
+        if (i0 + (warp << 3) >= (int)ncand) break;     // nothing for this warp
+        const uint32_t k = i < (int)ncand ? list[i] : 0u;
         uint32_t above = 0, same = 0;
-        for (uint32_t j = 0; j < ncand; ++j) {
-          const uint32_t o = list[j];
-          above += o > k ? 1u : 0u;
-          same += o == k ? 1u : 0u;
+        for (int j = 4 * part; j < (int)ncand; j += 16) {
+          const uint4 o = *reinterpret_cast<const uint4*>(list + j);     // values behind the list's end do not count
+          const int left = (int)ncand - j;
+          above += (o.x > k ? 1u : 0u) + (left > 1 && o.y > k ? 1u : 0u) + (left > 2 && o.z > k ? 1u : 0u) + (left > 3 && o.w > k ? 1u : 0u);
+          same += (o.x == k ? 1u : 0u) + (left > 1 && o.y == k ? 1u : 0u) + (left > 2 && o.z == k ? 1u : 0u) + (left > 3 && o.w == k ? 1u : 0u);
         }
-        if (above < need && need <= above + same) { sh[4] = k; sh[5] = need - above; }   // equal keys write equal values
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+          above += __shfl_xor_sync(0xffffffffu, above, o);
+          same += __shfl_xor_sync(0xffffffffu, same, o);
+        }
+        if (part == 0 && i < (int)ncand && above < need && need <= above + same) { sh[4] = k; sh[5] = need - above; }   // equal keys write equal values
       }
       __syncthreads();
       lo = hi = sh[4];
@@ -472,8 +549,8 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
     mgt |= (key[e] > tau ? 1u : 0u) << e;
     meq |= (key[e] == tau ? 1u : 0u) << e;
   }
-  mgt &= vmask;
-  meq &= vmask;
+  mgt = turned(mgt & vmask, turn);
+  meq = turned(meq & vmask, turn);
   const uint32_t cnt = (uint32_t)__popc(mgt) | ((uint32_t)__popc(meq) << 16);
   const uint32_t before = block_exclusive_scan<T>(cnt, wsum, lane, warp);
   const uint32_t gt_before = before & 0xffffu, eq_before = before >> 16;
@@ -500,7 +577,7 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
 }
 
 template <int E, int T>
-constexpr int select_reg_smem_bytes() { return (kRegCopies * kRegBins + 2 * (T / 32) + 8 + T * (E + 4)) * 4; }
+constexpr int select_reg_smem_bytes() { return (kRegCopies * kRegBins + 2 * (T / 32) + 8 + T * (E > 16 ? E : E + 4)) * 4; }
 
 }  // namespace
 }  // namespace sg

@@ -78,6 +78,20 @@ def test_split_at_the_cuts(ks):
             assert np.array_equal(a, b)
 
 
+@pytest.mark.parametrize("n", [5, 4093, 4096, 8189, 8190, 8192, 16383, 16384, 32765, 32768])
+def test_select_rows_off_the_16_byte_boundary(n):
+    """Rows that start 0 to 3 values behind a 16-byte boundary, up to the longest of every kernel variant; values from
+    all different to a handful, so that the last interval holds from one key to thousands."""
+    import gpu_ops
+    rng = np.random.default_rng(17)
+    for lead, steps in ((0, 1e9), (1, 2000.0), (2, 100.0), (3, 1.0)):
+        lens, ks = (lead, n, 2, n), (min(lead, 1), max(1, n // 10), 1, n - 1)
+        cu, ck = cu_of(lens), cu_of(ks)
+        x = (np.round(rng.standard_normal((1, 2, int(cu[-1]))) * steps) / steps).astype(np.float32)
+        want = oracle.select_topk(x, cu, ck)
+        assert np.array_equal(gpu_ops.select_topk(x, cu, ck), want)
+
+
 @pytest.mark.parametrize("n", [1, 31, 4096, 4097, 8192, 8193, 16385, 32768, 32769])
 def test_threshold_at_the_cuts(n):
     """Row lengths at the ends of every kernel variant; caps that bind, that are met exactly and that are the whole row."""
