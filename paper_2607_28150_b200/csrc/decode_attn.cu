@@ -1,14 +1,22 @@
 // sg_sparse_decode_attn: split-KV decode attention over a packed source plus an index-gathered source.
 //
-// Memory-bound: every attended token costs 2*d*2 bytes of K+V per KV head and only 4*G*d flops.
+// Every attended token costs 2*d*2 bytes of K+V per KV head and only 4*G*d flops: large batches are bound by HBM, small
+// ones by the chain of launch, first loads, a slice or two per warp, and merge.  In between a warp's instructions are what
+// takes the time: they issue one by one, four to five clocks each, with few warps per scheduler.
 // The token list of a (sequence, KV head) -- packed rows first, then local rows addressed through
 // local_idx -- is cut into slices of 16 tokens.  The slices are dealt out round robin over all warps of all
 // CTAs that share a (sequence, KV head), so every CTA gets the same mix of packed and gathered slices; a warp
-// streams its slices through a ring of three K/V slices of its own in shared memory (16-byte cp.async copies, XOR-swizzled rows so ldmatrix is
-// conflict-free; gathered rows are whole 2*d-byte lines, so sector efficiency stays 100 %).  The ring is
-// private to the warp, so the loop has no block-wide barrier: a warp waits only for its own copies.
-// S = Q K^T and O += P V run on bf16 tensor-core MMAs with the G query rows of the KV head padded to
-// 16; the online softmax (base 2) stays in registers.
+// streams its slices through a ring of its own in shared memory, half a slice (16 rows of K, or of V) per slot
+// (16-byte cp.async copies, XOR-swizzled rows so ldmatrix is conflict-free; gathered rows are whole 2*d-byte lines, so
+// sector efficiency stays 100 %).  The ring is private to the warp, so the loop has no block-wide barrier: a warp waits
+// only for its own copies.
+// S^T = K Q^T and O^T += V^T P^T run on bf16 tensor-core MMAs with the tokens (or the head dimension) on the 16-row side and
+// the G query rows of the KV head on the 8-column side: no row is padding at G = 8, half are at G = 4, and the accumulator
+// takes d/4 registers.  (With the queries on the 16-row side: twice the MMAs and accumulators, 420 instructions per slice
+// instead of 200, and so many registers and so deep a ring that an SM held one CTA of eight warps; it holds two now, and
+// consecutive calls overlap on it.  32 layers of 819 entries: 48.5 -> 39.7 us, 4 layers of 32 x 820 entries 78.7 -> 73.4,
+// one layer of 128 x 4096 entries 342 -> 305 us, 7.1 TB/s.)
+// The online softmax (base 2) stays in registers.
 // The split-KV partials (m, l, unnormalised O) never leave the chip: the warps of a CTA merge through
 // shared memory, and the CTAs of a (sequence, KV head) form a thread-block cluster (1, 2, 4 or 8 CTAs);
 // every CTA owns a slice of the G*d outputs and receives the other CTAs' partials of that slice in its own
@@ -27,7 +35,7 @@
 namespace sg {
 namespace {
 
-constexpr int kSlice = 16;         // tokens per warp step (one m16n8k16 k-extent of P V)
+constexpr int kSlice = 16;         // tokens per warp step (one m16n8k16 k-extent of V^T P^T)
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
@@ -47,13 +55,17 @@ struct DecParams {
   float* lse;
   int32_t* dev_status;
   int64_t ts, hs;
+  uint32_t ts_bytes;  // token stride in bytes, or 0 when it does not fit
   int32_t B, Hq, Hkv, G, K_tot, NL_tot;
   int32_t n_tokens;  // total tokens of the batch: with one sequence every prefix array is {0, total}, known on the host
   int32_t csize;     // CTAs per (sequence, KV head) = cluster size
   float scale_log2;
 };
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int src_bytes) {
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void* src, int src_bytes) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
@@ -114,23 +126,27 @@ __device__ __forceinline__ bool mbar_wait_cluster_bounded(uint64_t* bar) {
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// kHi: the KV head has more than 8 query rows, so MMA rows 8..15 carry data too.
-// kDecWarps warps per CTA, each with a private ring of kBuf slices: (8, 3) gives one CTA per SM, (4, 3) two.
-template <int D, bool kHi, int kDecWarps, int kBuf>
-__global__ void __launch_bounds__(kDecWarps * 32, kDecWarps == 4 ? 2 : 1) decode_partial_kernel(const DecParams p) {
+// Exchanges rows and columns of an 8 x 8 matrix of 16-bit values held as an MMA accumulator holds one (lane / 4 = row).
+__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t v) {
+  uint32_t r;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;\n" : "=r"(r) : "r"(v));
+  return r;
+}
+
+// kN: 8-row tiles of the KV head's query rows (1 for G <= 8, 2 up to 16).  kDecWarps warps per CTA, each with a private ring
+// of kSlots half slices: three leave room for two 8-warp CTAs per SM (d = 128), six for one.
+template <int D, int kN, int kDecWarps, int kSlots>
+__global__ void __launch_bounds__(kDecWarps * 32, (kN == 1 && kSlots * D <= 384 ? 16 : 8) / kDecWarps) decode_partial_kernel(const DecParams p) {
   constexpr int kDecThreads = kDecWarps * 32;
   constexpr int kRowBytes = D * 2;
   constexpr int kChunksPerRow = D / 8;                       // 16-byte chunks
-  constexpr int kSliceBytes = kSlice * kRowBytes;            // K (or V) rows of one slice
+  constexpr int kHalfBytes = kSlice * kRowBytes;             // K (or V) rows of one slice
   constexpr int kCopiesPerLane = kSlice * kChunksPerRow / 32;
   constexpr uint32_t kFull = 0xffffffffu;
-  extern __shared__ __align__(128) uint8_t smem_raw[];
-  // per warp: kBuf slices of K, then kBuf slices of V, rows XOR-swizzled; after all rings one validity
-  // word per (warp, buffer)
-  uint32_t* s_mask = reinterpret_cast<uint32_t*>(smem_raw + kDecWarps * kBuf * 2 * kSliceBytes);
+  extern __shared__ __align__(1024) uint8_t smem_raw[];       // per warp: kSlots half slices, rows XOR-swizzled
   // Receive area for the cluster merge, never aliased by the rings: the slice of the G*d outputs this CTA
   // owns, as every rank's partial: rx_o [8][per], rx_m [8][16], rx_l [8][16].
-  float* rx_m = reinterpret_cast<float*>(s_mask + kDecWarps * kBuf);
+  float* rx_m = reinterpret_cast<float*>(smem_raw + kDecWarps * kSlots * kHalfBytes);
   float* rx_l = rx_m + 8 * 16;
   float* rx_o = rx_l + 8 * 16;
   uint64_t* rx_bar = reinterpret_cast<uint64_t*>(rx_o + 16 * D);   // counts the bytes of the partials pushed into the three arrays
@@ -171,93 +187,91 @@ __global__ void __launch_bounds__(kDecWarps * 32, kDecWarps == 4 ? 2 : 1) decode
   const uint16_t* pv_base = p.packed_v + ((int64_t)ck0 * p.Hkv + (int64_t)g * kb) * D;
   const uint16_t* lk_base = p.local_k + (int64_t)c0 * p.ts + (int64_t)g * p.hs;
   const uint16_t* lv_base = p.local_v + (int64_t)c0 * p.ts + (int64_t)g * p.hs;
-  const uint32_t wk_u32 = smem_u32(smem_raw) + warp * (kBuf * 2 * kSliceBytes);   // this warp's K ring
-  const uint32_t wv_u32 = wk_u32 + kBuf * kSliceBytes;                            // and its V ring
+  const uint32_t ring = smem_u32(smem_raw) + warp * (kSlots * kHalfBytes);        // this warp's ring
 
   // The slices of the list [packed rows ++ local rows] of (b, g) are dealt out round robin over all warps of all CTAs of
   // the cluster (slice s goes to rank s % csize, warp (s / csize) % warps): every CTA gets the same mix of contiguous
   // packed slices and slower gathered ones, whatever the split of the list.
-  constexpr int pos_beg = 0;
   const int ntok = kbe + nl;
-  const int nslices = (ntok + kSlice - 1) / kSlice;
-  const int first_slice = warp * p.csize + c, slice_stride = kDecWarps * p.csize;
-  const int nmine = nslices > first_slice ? (nslices - first_slice + slice_stride - 1) / slice_stride : 0;
-  const int32_t* idx_base = p.local_idx + (int64_t)g * p.NL_tot + cl0 + lskip - kbe;   // indexed by list position
-  // Lane r (and r + 16) holds the local index of row r of the warp's j-th slice, read one slice ahead.
-  auto fetch_idx = [&](int j) -> int {
-    const int li = (first_slice + j * slice_stride) * kSlice + (lane & 15);
-    const int pos = pos_beg + li;
-    return (j < nmine && li < ntok && pos >= kbe) ? __ldg(idx_base + pos) : 0;
+  const int step = kDecWarps * p.csize * kSlice;               // list positions from a slice of this warp to its next
+  int li0 = (warp * p.csize + c) * kSlice;                     // first list position of the warp's slice
+  const int32_t* idx_base = p.local_idx + (int64_t)g * p.NL_tot + cl0 + lskip - kbe + (lane & 15);   // indexed by list position
+  // Lane r (and r + 16) holds the local index of row r of a slice, read ahead of its use.
+  auto fetch_idx = [&](int at) -> int {
+    const int li = at + (lane & 15);
+    return (li < ntok && li >= kbe) ? __ldg(idx_base + at) : 0;
   };
-  auto load_slice = [&](int j, int buf, int idx_reg) {
-    const int li0 = (first_slice + j * slice_stride) * kSlice;
-    if (li0 + kSlice <= ntok && pos_beg + li0 + kSlice <= kbe) {
+  // A warp is alone on its scheduler or shares it with a few others, and its instructions issue one by one: what a slice takes
+  // is its instruction count (2500 clocks for 600 of them).  So the copies' addresses are built from per-lane constants and
+  // immediate offsets, with one multiplication per gathered row; what does not occur in the bulk of a list (the slice where
+  // packed rows end, the last slice, bad indices, very large strides) goes through a loop.
+  constexpr int kRowsPerCopy = 32 / kChunksPerRow;
+  const int row0 = lane / kChunksPerRow, col0 = lane % kChunksPerRow;
+  const uint32_t dst0 = ring + row0 * kRowBytes + ((col0 ^ row0) << 4);
+  pk_base += lane * 8;
+  pv_base += lane * 8;
+  const uint8_t* const lk_lane = reinterpret_cast<const uint8_t*>(lk_base + col0 * 8);
+  const uint8_t* const lv_lane = reinterpret_cast<const uint8_t*>(lv_base + col0 * 8);
+  // Copies the K or V rows of the slice at list position `at` into a slot; returns the rows that hold a real token (bit r: row r).
+  auto load_half = [&](int at, bool is_v, int slot, int idx_reg) -> uint32_t {
+    const uint32_t dst = dst0 + slot * kHalfBytes;
+    auto dst_of = [&](int i) { return (dst ^ (((i * kRowsPerCopy) & 7) << 4)) + i * (kRowsPerCopy * kRowBytes); };
+    if (at + kSlice <= kbe) {
       // the whole slice lies in the packed buffer: 16 consecutive rows are one contiguous run of 16-byte pieces
-      if (lane == 0) s_mask[warp * kBuf + buf] = 0xffffu;
-      const uint16_t* srck = pk_base + (int64_t)(pos_beg + li0) * D + lane * 8;
-      const uint16_t* srcv = pv_base + (int64_t)(pos_beg + li0) * D + lane * 8;
+      const uint16_t* src = (is_v ? pv_base : pk_base) + (int64_t)at * D;
+#pragma unroll
+      for (int i = 0; i < kCopiesPerLane; ++i) cp_async16(dst_of(i), src + i * 256);
+      return 0xffffu;
+    }
+    const uint8_t* local = is_v ? lv_lane : lk_lane;
+    if (at >= kbe && at + kSlice <= ntok && p.ts_bytes && __all_sync(kFull, (uint32_t)idx_reg < (uint32_t)nseq)) {
 #pragma unroll
       for (int i = 0; i < kCopiesPerLane; ++i) {
-        const int qid = lane + i * 32;
-        const int row = qid / kChunksPerRow;
-        const int col = qid % kChunksPerRow;
-        const uint32_t off = buf * kSliceBytes + row * kRowBytes + ((col ^ (row & 7)) << 4);
-        cp_async16(wk_u32 + off, srck + i * 256, 16);
-        cp_async16(wv_u32 + off, srcv + i * 256, 16);
+        const uint32_t t = (uint32_t)__shfl_sync(kFull, idx_reg, row0 + i * kRowsPerCopy);
+        cp_async16(dst_of(i), local + (uint64_t)t * p.ts_bytes);
       }
-      return;
+      return 0xffffu;
     }
-    {
-      const int li = li0 + (lane & 15), pos = pos_beg + li;
-      const bool in_list = li < ntok;
-      const bool ok = in_list && (pos < kbe || (idx_reg >= 0 && idx_reg < nseq));
-      if (in_list && !ok && lane < 16) raise(p.dev_status, SG_ERR_INDEX);
-      const uint32_t mask = __ballot_sync(kFull, ok) & 0xffffu;
-      if (lane == 0) s_mask[warp * kBuf + buf] = mask;        // bit r: row r holds a real token
-    }
+    const int li = at + (lane & 15);
+    const bool ok = li < kbe || (li < ntok && (uint32_t)idx_reg < (uint32_t)nseq);
+    if (li < ntok && !ok && !is_v && lane < 16) raise(p.dev_status, SG_ERR_INDEX);
+    const uint32_t good = __ballot_sync(kFull, ok) & 0xffffu;
+    // lane r finds row r's source, its copiers ask it
+    const uint64_t mine = li < kbe ? (uint64_t)((is_v ? pv_base : pk_base) - lane * 8 + (int64_t)li * D) : (uint64_t)(local - col0 * 16 + (int64_t)idx_reg * p.ts * 2);
 #pragma unroll
     for (int i = 0; i < kCopiesPerLane; ++i) {
-      const int qid = lane + i * 32;
-      const int row = qid / kChunksPerRow;
-      const int col = qid % kChunksPerRow;
-      const int li = li0 + row;
-      const int pos = pos_beg + li;
-      const int t = __shfl_sync(kFull, idx_reg, row);
-      const uint16_t* srck = p.packed_k;
-      const uint16_t* srcv = p.packed_v;
-      int bytes = 0;
-      if (li < ntok) {
-        if (pos < kbe) {
-          srck = pk_base + (int64_t)pos * D + col * 8;
-          srcv = pv_base + (int64_t)pos * D + col * 8;
-          bytes = 16;
-        } else if (t >= 0 && t < nseq) {
-          srck = lk_base + (int64_t)t * p.ts + col * 8;
-          srcv = lv_base + (int64_t)t * p.ts + col * 8;
-          bytes = 16;
-        }
-      }
-      const uint32_t off = buf * kSliceBytes + row * kRowBytes + ((col ^ (row & 7)) << 4);
-      cp_async16(wk_u32 + off, srck, bytes);                  // bytes == 0 zero-fills the row
-      cp_async16(wv_u32 + off, srcv, bytes);
+      const int row = row0 + i * kRowsPerCopy;
+      const uint64_t src = __shfl_sync(kFull, mine, row) + col0 * 16;
+      cp_async16_zfill(dst_of(i), reinterpret_cast<const void*>(src), (good >> row) & 1u ? 16 : 0);   // rows without a token are zero
     }
+    return good;
   };
 
-  float o_acc[D / 8][4];
+  float o_acc[kN][D / 16][4], m_run[kN][2], l_run[kN][2];
 #pragma unroll
-  for (int i = 0; i < D / 8; ++i) { o_acc[i][0] = o_acc[i][1] = o_acc[i][2] = o_acc[i][3] = 0.f; }
-  float m_lo = -INFINITY, m_hi = -INFINITY, l_lo = 0.f, l_hi = 0.f;
+  for (int t = 0; t < kN; ++t) {
+#pragma unroll
+    for (int i = 0; i < D / 16; ++i) { o_acc[t][i][0] = o_acc[t][i][1] = o_acc[t][i][2] = o_acc[t][i][3] = 0.f; }
+    m_run[t][0] = m_run[t][1] = -INFINITY;
+    l_run[t][0] = l_run[t][1] = 0.f;
+  }
 
-  int idx_next;
+  // The halves K0 V0 K1 V1 ... go through the ring in order, half h into slot h mod kSlots; a slot is refilled, with half
+  // h + kSlots, as soon as its fragments are in registers.
+  static_assert(kSlots == 3 || kSlots == 6, "the order of the refills below");
+  constexpr int kAhead = kSlots == 3 ? 2 : 3;                 // slices that are asked for ahead of the current one
+  uint32_t mask[kAhead + 1] = {};                             // real rows of this slice and the next ones
+  int idx[kAhead];                                            // local indices of the next slices
   {
-    int idx_pro[kBuf - 1];
+    const int idx0 = fetch_idx(li0);
 #pragma unroll
-    for (int s = 0; s < kBuf - 1; ++s) idx_pro[s] = fetch_idx(s);
-    idx_next = fetch_idx(kBuf - 1);
-    static_assert(kBuf == 3, "the prologue below passes two index registers by selection");
+    for (int i = 0; i < kAhead; ++i) idx[i] = fetch_idx(li0 + (i + 1) * step);
 #pragma unroll 1
-    for (int s = 0; s < kBuf - 1; ++s) {                      // not unrolled: this code runs once per call, from a cold instruction cache
-      if (s < nmine) load_slice(s, s, s ? idx_pro[1] : idx_pro[0]);
+    for (int h = 0; h < kSlots; ++h) {                        // not unrolled: this code runs once per call, from a cold instruction cache
+      const int at = li0 + (h >> 1) * step;
+      const uint32_t got = at < ntok ? load_half(at, h & 1, h, h < 2 ? idx0 : h < 4 ? idx[0] : idx[1]) : 0u;
+#pragma unroll
+      for (int i = 0; i < kAhead; ++i) mask[i] = h == 2 * i ? got : mask[i];
       cp_async_commit();
     }
   }
@@ -267,165 +281,153 @@ __global__ void __launch_bounds__(kDecWarps * 32, kDecWarps == 4 ? 2 : 1) decode
   // written by a kernel that itself lets its dependents start early (such as the previous layer's call of this
   // kernel).  So nothing waits here: the dependency wait sits in front of the stores of out / lse, and consecutive
   // calls overlap everything but those stores.
-  // Q fragments (A operand, 16 x D, rows >= G are zero).
-  const int r_lo = lane >> 2, r_hi = r_lo + 8;
-  uint32_t qa[D / 16][4];
+  // Q fragments (B operand, D x 8 per tile; rows >= G are zero).
+  const int r8 = lane >> 2, c2 = 2 * (lane & 3);
+  uint32_t qf[kN][D / 16][2];
   {
     const uint16_t* qb = p.q + ((int64_t)b * p.Hq + (int64_t)g * p.G) * D;
 #pragma unroll
-    for (int kk = 0; kk < D / 16; ++kk) {
-      const int col = kk * 16 + 2 * (lane & 3);
-      qa[kk][0] = r_lo < p.G ? *reinterpret_cast<const uint32_t*>(qb + r_lo * D + col) : 0u;
-      qa[kk][2] = r_lo < p.G ? *reinterpret_cast<const uint32_t*>(qb + r_lo * D + col + 8) : 0u;
-      qa[kk][1] = (kHi && r_hi < p.G) ? *reinterpret_cast<const uint32_t*>(qb + r_hi * D + col) : 0u;
-      qa[kk][3] = (kHi && r_hi < p.G) ? *reinterpret_cast<const uint32_t*>(qb + r_hi * D + col + 8) : 0u;
+    for (int t = 0; t < kN; ++t) {
+      const int r = t * 8 + r8;
+#pragma unroll
+      for (int kk = 0; kk < D / 16; ++kk) {
+        qf[t][kk][0] = r < p.G ? *reinterpret_cast<const uint32_t*>(qb + r * D + kk * 16 + c2) : 0u;
+        qf[t][kk][1] = r < p.G ? *reinterpret_cast<const uint32_t*>(qb + r * D + kk * 16 + c2 + 8) : 0u;
+      }
     }
   }
 
   // The ring is private to the warp: no block-wide barrier inside the loop, the warps drift freely.
+  // K fragments (A operand): matrices of tokens 0-7 and 8-15 x two column pieces; V^T: two column pieces x tokens 0-7 and 8-15
+  const int mi = lane >> 3, r7 = lane & 7;
+  const uint32_t k_lane = ring + ((mi & 1) * 8 + r7) * kRowBytes + (((mi >> 1) ^ r7) << 4);
+  const uint32_t v_lane = ring + ((mi >> 1) * 8 + r7) * kRowBytes + (((mi & 1) ^ r7) << 4);
+  int slot = 0;                                               // of K of slice j; V is in the next one
 #pragma unroll 1
-  for (int j = 0; j < nmine; ++j) {
-    cp_async_wait<kBuf - 2>();
+  for (; li0 < ntok; li0 += step) {
+    const int vslot = slot == kSlots - 1 ? 0 : slot + 1;
+    cp_async_wait<kSlots - 1>();
+    __syncwarp();
+    uint32_t f[D / 16][4];                                    // all fragment loads of a half before its MMAs
+    {
+      const uint32_t at = k_lane + slot * kHalfBytes;
+#pragma unroll
+      for (int kk = 0; kk < D / 16; ++kk) ldmatrix_x4(f[kk], at ^ (kk << 5));
+    }
+    __syncwarp();
+    // S^T = K Q^T: 16 tokens x 8 query rows per tile, even and odd k-steps in chains of their own (a warp has only one or
+    // two slices at small batch: the length of the chain is what it waits for)
+    float s_acc[kN][4], s_odd[kN][4];
+#pragma unroll
+    for (int t = 0; t < kN; ++t) {
+      s_odd[t][0] = s_odd[t][1] = s_odd[t][2] = s_odd[t][3] = 0.f;
+      s_acc[t][0] = s_acc[t][1] = s_acc[t][2] = s_acc[t][3] = 0.f;
+#pragma unroll
+      for (int kk = 0; kk < D / 16; ++kk)
+        mma_bf16((kk & 1) ? s_odd[t] : s_acc[t], f[kk][0], f[kk][1], f[kk][2], f[kk][3], qf[t][kk][0], qf[t][kk][1]);
+    }
+    // The tensor cores are busy with S: refill K's slot, fetch the V fragments (into the registers of K's), refill V's slot.
+    if (kSlots == 3) {
+      if (li0 + step < ntok) load_half(li0 + step, true, slot, idx[0]);
+    } else {
+      if (li0 + 3 * step < ntok) mask[kAhead] = load_half(li0 + 3 * step, false, slot, idx[kAhead - 1]);
+    }
+    cp_async_commit();
+    const uint32_t rows = mask[0];
+    cp_async_wait<kSlots - 1>();
     __syncwarp();
     {
-      const int nj = j + kBuf - 1;
-      if (nj < nmine) load_slice(nj, nj % kBuf, idx_next);
-      cp_async_commit();
-      idx_next = fetch_idx(nj + 1);
+      const uint32_t at = v_lane + vslot * kHalfBytes;
+#pragma unroll
+      for (int dc = 0; dc < D / 16; ++dc) ldmatrix_x4_trans(f[dc], at ^ (dc << 5));
     }
-    const int buf = j % kBuf;
-    const uint32_t k_st = wk_u32 + buf * kSliceBytes;
-    const uint32_t v_st = wv_u32 + buf * kSliceBytes;
-    const uint32_t vmask = s_mask[warp * kBuf + buf];
-    constexpr int wrow = 0;
-
-    // S = Q K^T for 16 tokens (two n8 tiles)
-    // (even and odd k-steps accumulate separately: two dependent chains of half the length; a warp has only one or two
-    // slices at small batch, so the length of this chain is what it waits for)
-    float s_acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-    {
-      float s_odd[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-      const int mi = lane >> 3;
-      const int row = wrow + (mi >> 1) * 8 + (lane & 7);
-      // all fragment loads of the slice first, then the tensor-core chain: the statements are volatile and keep their
-      // order, so loading inside the chain would expose one shared-memory latency per k-step
-      uint32_t kf[D / 16][4];
-#pragma unroll
-      for (int kk = 0; kk < D / 16; ++kk) {
-        const int chunk = kk * 2 + (mi & 1);
-        ldmatrix_x4(kf[kk], k_st + row * kRowBytes + ((chunk ^ (row & 7)) << 4));
-      }
-#pragma unroll
-      for (int kk = 0; kk < D / 16; ++kk) {
-        mma_bf16((kk & 1) ? s_odd[0] : s_acc[0], qa[kk][0], qa[kk][1], qa[kk][2], qa[kk][3], kf[kk][0], kf[kk][1]);
-        mma_bf16((kk & 1) ? s_odd[1] : s_acc[1], qa[kk][0], qa[kk][1], qa[kk][2], qa[kk][3], kf[kk][2], kf[kk][3]);
-      }
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) s_acc[j][e] += s_odd[j][e];
-      }
+    __syncwarp();
+    if (kSlots == 3) {
+      if (li0 + 2 * step < ntok) mask[kAhead] = load_half(li0 + 2 * step, false, vslot, idx[kAhead - 1]);
+    } else {
+      if (li0 + 3 * step < ntok) load_half(li0 + 3 * step, true, vslot, idx[kAhead - 1]);
     }
-    // the V fragments are fetched now, ahead of the softmax arithmetic that P V has to wait for anyway
-    uint32_t vf[D / 16][4];
-    {
-      const int mi = lane >> 3;
-      const int row = wrow + (mi & 1) * 8 + (lane & 7);
+    cp_async_commit();
 #pragma unroll
-      for (int dc = 0; dc < D / 16; ++dc) {
-        const int chunk = dc * 2 + (mi >> 1);
-        ldmatrix_x4_trans(vf[dc], v_st + row * kRowBytes + ((chunk ^ (row & 7)) << 4));
-      }
-    }
-    // online softmax in base 2; mask padding and skipped indices
-    float mx_lo = -INFINITY, mx_hi = -INFINITY;
+    for (int i = 0; i < kAhead; ++i) mask[i] = mask[i + 1];
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
+    for (int i = 0; i + 1 < kAhead; ++i) idx[i] = idx[i + 1];
+    idx[kAhead - 1] = fetch_idx(li0 + (kAhead + 1) * step);
+    // online softmax in base 2; padding and skipped indices are masked.  The lane holds tokens r8 and r8 + 8 of query rows c2
+    // and c2 + 1 of a tile.
+    const bool ok0 = (rows >> r8) & 1u, ok1 = (rows >> (r8 + 8)) & 1u;
+    uint32_t pf[kN][2];
+    bool rescale = false;
+    float al[kN][2];
+#pragma unroll
+    for (int t = 0; t < kN; ++t) {
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
-        const bool valid = (vmask >> (j * 8 + 2 * (lane & 3) + e)) & 1u;
-        s_acc[j][e] = valid ? s_acc[j][e] * p.scale_log2 : -INFINITY;
-        mx_lo = fmaxf(mx_lo, s_acc[j][e]);
-        if (kHi) {
-          s_acc[j][2 + e] = valid ? s_acc[j][2 + e] * p.scale_log2 : -INFINITY;
-          mx_hi = fmaxf(mx_hi, s_acc[j][2 + e]);
+        const float a = ok0 ? s_acc[t][e] + s_odd[t][e] : -INFINITY, c = ok1 ? s_acc[t][2 + e] + s_odd[t][2 + e] : -INFINITY;
+        float mx = fmaxf(a, c);
+        mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, 4));
+        mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, 8));
+        mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, 16));
+        const float mn = fmaxf(m_run[t][e], mx * p.scale_log2), mu = mn == -INFINITY ? 0.f : mn;
+        al[t][e] = exp2f(m_run[t][e] - mu);
+        m_run[t][e] = mn;
+        const float p0 = exp2f(fmaf(a, p.scale_log2, -mu)), p1 = exp2f(fmaf(c, p.scale_log2, -mu));
+        // every lane keeps the part of the row sum that its own tokens make; the parts are added up once, after the last slice
+        l_run[t][e] = l_run[t][e] * al[t][e] + (p0 + p1);
+        s_acc[t][e] = p0;
+        s_acc[t][2 + e] = p1;
+        rescale = rescale || al[t][e] != 1.f;
+      }
+      pf[t][0] = movmatrix_trans(pack_bf16(s_acc[t][0], s_acc[t][1]));
+      pf[t][1] = movmatrix_trans(pack_bf16(s_acc[t][2], s_acc[t][3]));
+    }
+    if (__any_sync(kFull, rescale)) {
+#pragma unroll
+      for (int t = 0; t < kN; ++t) {
+#pragma unroll
+        for (int i = 0; i < D / 16; ++i) {
+          o_acc[t][i][0] *= al[t][0]; o_acc[t][i][1] *= al[t][1];
+          o_acc[t][i][2] *= al[t][0]; o_acc[t][i][3] *= al[t][1];
         }
       }
     }
-    mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 1));
-    mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 2));
-    const float mn_lo = fmaxf(m_lo, mx_lo);
-    const float mu_lo = mn_lo == -INFINITY ? 0.f : mn_lo;
-    const float al_lo = exp2f(m_lo - mu_lo);
-    m_lo = mn_lo;
-    float mu_hi = 0.f, al_hi = 1.f;
-    if (kHi) {
-      mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 1));
-      mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 2));
-      const float mn_hi = fmaxf(m_hi, mx_hi);
-      mu_hi = mn_hi == -INFINITY ? 0.f : mn_hi;
-      al_hi = exp2f(m_hi - mu_hi);
-      m_hi = mn_hi;
-    }
-    float sum_lo = 0.f, sum_hi = 0.f;
-    uint32_t pa[4];
+    // O^T += V^T P^T
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const float p0 = exp2f(s_acc[j][0] - mu_lo), p1 = exp2f(s_acc[j][1] - mu_lo);
-      sum_lo += p0 + p1;
-      pa[2 * j] = pack_bf16(p0, p1);
-      if (kHi) {
-        const float p2 = exp2f(s_acc[j][2] - mu_hi), p3 = exp2f(s_acc[j][3] - mu_hi);
-        sum_hi += p2 + p3;
-        pa[2 * j + 1] = pack_bf16(p2, p3);
-      } else {
-        pa[2 * j + 1] = 0u;
-      }
-    }
-    // the four lanes of a row keep their own part of the row sum (the rescale factor is the same for all four);
-    // the parts are added up once, after the last slice
-    l_lo = l_lo * al_lo + sum_lo;
-    if (kHi) l_hi = l_hi * al_hi + sum_hi;
-    const bool rescale = kHi ? (al_lo != 1.f || al_hi != 1.f) : (al_lo != 1.f);
-    if (__any_sync(0xffffffffu, rescale)) {
+    for (int t = 0; t < kN; ++t) {
 #pragma unroll
-      for (int i = 0; i < D / 8; ++i) {
-        o_acc[i][0] *= al_lo; o_acc[i][1] *= al_lo;
-        if (kHi) { o_acc[i][2] *= al_hi; o_acc[i][3] *= al_hi; }
-      }
+      for (int dc = 0; dc < D / 16; ++dc) mma_bf16(o_acc[t][dc], f[dc][0], f[dc][1], f[dc][2], f[dc][3], pf[t][0], pf[t][1]);
     }
-    // O += P V
-#pragma unroll
-    for (int dc = 0; dc < D / 16; ++dc) {
-      mma_bf16(o_acc[2 * dc], pa[0], pa[1], pa[2], pa[3], vf[dc][0], vf[dc][1]);
-      mma_bf16(o_acc[2 * dc + 1], pa[0], pa[1], pa[2], pa[3], vf[dc][2], vf[dc][3]);
-    }
+    slot = slot >= kSlots - 2 ? slot + 2 - kSlots : slot + 2;
   }
-  l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 1);
-  l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 2);
-  if (kHi) {
-    l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 1);
-    l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 2);
+#pragma unroll
+  for (int t = 0; t < kN; ++t) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      l_run[t][e] += __shfl_xor_sync(kFull, l_run[t][e], 4);
+      l_run[t][e] += __shfl_xor_sync(kFull, l_run[t][e], 8);
+      l_run[t][e] += __shfl_xor_sync(kFull, l_run[t][e], 16);
+    }
   }
   cp_async_wait<0>();
   __syncthreads();
 
   // merge the warps through shared memory (the rings are free now)
-  constexpr int kOStride = D + 8;                             // row stride of the partials: the rows of a store land in different banks
-  float* sm_o = reinterpret_cast<float*>(smem_raw);           // [kDecWarps][16][kOStride]
-  float* sm_m = sm_o + kDecWarps * 16 * kOStride;             // [kDecWarps][16]
+  constexpr int kOStride = D + 4;                             // row stride of the partials: the lanes of a store hit 32 different banks
+  float* sm_o = reinterpret_cast<float*>(smem_raw);           // [kDecWarps][8 kN][kOStride]
+  float* sm_m = sm_o + kDecWarps * 8 * kN * kOStride;         // [kDecWarps][16]
   float* sm_l = sm_m + kDecWarps * 16;
-  const bool w_lo = r_lo < p.G, w_hi = kHi && r_hi < p.G;      // rows >= G are padding and never read
-  if ((lane & 3) == 0) {
-    if (w_lo) { sm_m[warp * 16 + r_lo] = m_lo; sm_l[warp * 16 + r_lo] = l_lo; }
-    if (w_hi) { sm_m[warp * 16 + r_hi] = m_hi; sm_l[warp * 16 + r_hi] = l_hi; }
-  }
 #pragma unroll
-  for (int i = 0; i < D / 8; ++i) {
-    const int col = i * 8 + 2 * (lane & 3);
-    float* dst = sm_o + (warp * 16 + r_lo) * kOStride + col;
-    if (w_lo) *reinterpret_cast<float2*>(dst) = make_float2(o_acc[i][0], o_acc[i][1]);
-    if (w_hi) *reinterpret_cast<float2*>(dst + 8 * kOStride) = make_float2(o_acc[i][2], o_acc[i][3]);
+  for (int t = 0; t < kN; ++t) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int r = t * 8 + c2 + e;                           // rows >= G are padding and never read
+      if (r < p.G) {
+        if (r8 == 0) { sm_m[warp * 16 + r] = m_run[t][e]; sm_l[warp * 16 + r] = l_run[t][e]; }
+        float* dst = sm_o + (warp * 8 * kN + r) * kOStride + r8;
+#pragma unroll
+        for (int i = 0; i < D / 16; ++i) { dst[i * 16] = o_acc[t][i][e]; dst[i * 16 + 8] = o_acc[t][i][2 + e]; }
+      }
+    }
   }
   __syncthreads();
   // CTA-level partial of every output; with a cluster, each rank owns a slice of the G*d outputs and
@@ -447,7 +449,7 @@ __global__ void __launch_bounds__(kDecWarps * 32, kDecWarps == 4 ? 2 : 1) decode
 #pragma unroll
     for (int w = 0; w < kDecWarps; ++w) {
       const float f = exp2f(sm_m[w * 16 + r] - Mu);
-      const float2 o = *reinterpret_cast<const float2*>(sm_o + (w * 16 + r) * kOStride + col);
+      const float2 o = *reinterpret_cast<const float2*>(sm_o + (w * 8 * kN + r) * kOStride + col);
       L += sm_l[w * 16 + r] * f;
       O0 += o.x * f;
       O1 += o.y * f;
@@ -500,45 +502,44 @@ __global__ void __launch_bounds__(kDecWarps * 32, kDecWarps == 4 ? 2 : 1) decode
   }
 }
 
-template <int D, int kDecWarps, int kBuf>
-constexpr int decode_smem_bytes() {
-  return kDecWarps * kBuf * 2 * kSlice * D * 2 + kDecWarps * kBuf * 4 + (2 * 8 * 16 + 16 * D) * 4 + 16;   // rings, masks, receive area, its barrier
+// rings, and with a cluster the receive area and its barrier
+constexpr int decode_smem_bytes(int D, int warps, int slots, bool cluster) {
+  return warps * slots * kSlice * D * 2 + (cluster ? (2 * 8 * 16 + 16 * D) * 4 + 16 : 0);
 }
 
 }  // namespace
 
-// Launch shape, from what a sweep over batch sizes and list lengths measured.  CTAs beyond one wave
-// of resident CTAs never paid, so a (sequence, KV head) pair is split over a cluster only while all
-// clusters fit on the SMs at one CTA each.
-//  * pairs <= SMs: warps = 8, one CTA per SM; csize = the cluster size (a power of two <= 8, the
-//    portable limit) that gives each warp about one slice, capped by the SM count (12 warps per CTA
-//    measured slower than 8: the merge grows faster than the streaming shrinks);
-//  * more pairs: csize = 1 and warps = 4, two CTAs per SM, so that one CTA's prologue and merge overlap
-//    the other's streaming -- except long lists whose CTA count fills waves of one CTA per SM better.
-void decode_plan(const sg_shape* shape, int32_t total_sel, int32_t total_loc, int* csize, int* warps) {
+// Launch shape, from a sweep over 1 to 64 sequences of 8 KV heads and lists of 30 to 6400 entries, each timed as calls that
+// follow one another at once (a decode step replayed from a graph) and as a call behind an unrelated kernel.  A
+// (sequence, KV head) pair is split over a cluster of 1, 2, 4 or 8 CTAs; two 8-warp or four 4-warp CTAs fit on an SM.
+//  * pairs <= SMs: the clusters are spread one CTA per SM, which leaves room on every SM for the next call; the cluster size is
+//    the smallest power of two (<= 8, the portable limit) that gives each warp about one slice, or the largest that fits.
+//  * more pairs: one CTA each; eight warps once a list has 1024 entries (24 sequences of 1600: 30.2 us alone against 32.8 with
+//    four), else four, whose merge is half as wide (64 sequences of 200: 9.8 against 11.3 us).
+// Rings of three slots, two CTAs per SM and so two calls overlapped, are faster wherever rows are gathered (14 sequences of 1600
+// entries, half of them gathered, 12 layers: 186 us against 199 with six slots) and for short lists.  Long lists that are all
+// packed stream at HBM rate, and at most two calls are in flight: six slots then keep more bytes under way (14 x 1600: 176
+// against 182 us, 32 x 3200: 696 against 721; 14 x 800: 104 against 103).  With more than eight query rows per KV head the
+// registers allow one 8-warp CTA per SM anyway: six slots.
+void decode_plan(const sg_shape* shape, int32_t total_sel, int32_t total_loc, int* csize, int* warps, int* slots) {
   const int64_t pairs = (int64_t)shape->batch * shape->num_kv_heads;
   const int64_t avg_tokens = ((int64_t)total_sel + total_loc) / shape->batch;
-  int W = 4, cs = 1;
-  if (pairs <= kNumSMs) {
-    // largest cluster whose CTAs are all resident at once; clusters of eight one-CTA-per-SM CTAs must also leave half
-    // of the SMs to the next call, whose clusters cannot be placed otherwise while this call drains (2x slower)
+  int W = 8, cs = 1;
+  if (pairs > kNumSMs) {
+    W = avg_tokens >= 1024 ? 8 : 4;
+  } else if (avg_tokens > (pairs >= 64 ? 14 : 8) * kSlice) {   // else a slice or two per warp of one CTA already: no cluster to merge
     int fit = 1;
     while (fit < 8 && pairs * fit * 2 <= kNumSMs) fit *= 2;
-    const int fit8 = (fit == 8 && pairs * 16 > kNumSMs) ? 4 : fit;
+    // clusters of eight only while those of two calls fit side by side: one that cannot be placed waits for a whole call (2x)
+    if (fit == 8 && pairs * 16 > kNumSMs) fit = 4;
     // short lists: four warps per CTA already give every warp at most ~1.75 slices, and the merge is half as wide
     W = 4 * avg_tokens <= 7 * 4 * kSlice * fit ? 4 : 8;
-    if (W == 8) fit = fit8;
-    int work = 1;
-    while (work < 8 && (int64_t)work * W * kSlice < avg_tokens) work *= 2;
-    cs = fit < work ? fit : work;
-    // many short lists: one 8-warp CTA per list has a slice or two per warp already, and no cluster to merge
-    if (pairs >= 64 && avg_tokens <= 14 * kSlice) { W = 8; cs = 1; }
-  } else {
-    auto fill = [&](int64_t slots) { return (double)pairs / (double)(((pairs + slots - 1) / slots) * slots); };
-    W = (avg_tokens >= 1024 && fill(kNumSMs) > fill(2 * kNumSMs) + 0.05) ? 8 : 4;
+    while (cs < fit && (int64_t)cs * W * kSlice < avg_tokens) cs *= 2;
   }
   *csize = cs;
   *warps = W;
+  const bool streams = total_loc == 0 && avg_tokens >= 1024 && 2 * pairs > kNumSMs;
+  *slots = shape->num_q_heads / shape->num_kv_heads > 8 || streams ? 6 : 3;
 }
 
 size_t decode_workspace_bytes(const sg_shape*, int32_t, int32_t) { return 0; }   // partials stay on chip
@@ -620,6 +621,7 @@ sg_status decode_launch(const sg_shape* shape, const void* q, const void* packed
   p.lse = lse;
   p.dev_status = dev_status;
   p.ts = shape->cache_token_stride;
+  p.ts_bytes = p.ts > 0 && p.ts < (1 << 30) ? (uint32_t)p.ts * 2u : 0u;
   p.hs = shape->cache_head_stride;
   p.B = shape->batch;
   p.Hq = shape->num_q_heads;
@@ -628,8 +630,8 @@ sg_status decode_launch(const sg_shape* shape, const void* q, const void* packed
   p.K_tot = total_sel;
   p.NL_tot = total_loc;
   p.n_tokens = shape->total_tokens;
-  int warps = 4;
-  decode_plan(shape, total_sel, total_loc, &p.csize, &warps);
+  int warps = 4, slots = 3;
+  decode_plan(shape, total_sel, total_loc, &p.csize, &warps, &slots);
   p.scale_log2 = (softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)D)) * kLog2e;
   const int64_t grid_x = (int64_t)shape->batch * p.csize;
   if (grid_x > 0x7fffffffLL || shape->num_kv_heads > 65535) return SG_ERR_UNSUPPORTED;
@@ -648,20 +650,23 @@ sg_status decode_launch(const sg_shape* shape, const void* q, const void* packed
   cfg.blockDim = dim3((unsigned)warps * 32);
   // one launch: sequences with empty lists still get out = 0 and lse = -inf
   cfg.gridDim = dim3((unsigned)grid_x, (unsigned)shape->num_kv_heads);
-#define SG_LAUNCH_DECODE(DD, HI, WW, BB)                                                      \
-  do {                                                                                        \
-    SG_ENSURE_SMEM((decode_partial_kernel<DD, HI, WW, BB>), (decode_smem_bytes<DD, WW, BB>())); \
-    cfg.dynamicSmemBytes = decode_smem_bytes<DD, WW, BB>();                                   \
-    SG_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_partial_kernel<DD, HI, WW, BB>, p));          \
+  cfg.dynamicSmemBytes = (size_t)decode_smem_bytes(D, warps, slots, p.csize > 1);
+#define SG_LAUNCH_DECODE(DD, NN, WW, SS)                                                         \
+  do {                                                                                           \
+    SG_ENSURE_SMEM((decode_partial_kernel<DD, NN, WW, SS>), decode_smem_bytes(DD, WW, SS, true)); \
+    SG_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_partial_kernel<DD, NN, WW, SS>, p));             \
   } while (0)
-#define SG_LAUNCH_DECODE_W(DD, HI)                         \
-  do {                                                     \
-    if (warps == 8) SG_LAUNCH_DECODE(DD, HI, 8, 3);        \
-    else SG_LAUNCH_DECODE(DD, HI, 4, 3);                   \
+#define SG_LAUNCH_DECODE_D(DD)                                            \
+  do {                                                                    \
+    if (G > 8 && warps == 8) SG_LAUNCH_DECODE(DD, 2, 8, 6);               \
+    else if (G > 8) SG_LAUNCH_DECODE(DD, 2, 4, 6);                        \
+    else if (warps == 4) SG_LAUNCH_DECODE(DD, 1, 4, 3);                   \
+    else if (slots == 6) SG_LAUNCH_DECODE(DD, 1, 8, 6);                   \
+    else SG_LAUNCH_DECODE(DD, 1, 8, 3);                                   \
   } while (0)
-  if (D == 128) { if (G > 8) SG_LAUNCH_DECODE_W(128, true); else SG_LAUNCH_DECODE_W(128, false); }
-  else          { if (G > 8) SG_LAUNCH_DECODE_W(64, true);  else SG_LAUNCH_DECODE_W(64, false); }
-#undef SG_LAUNCH_DECODE_W
+  if (D == 128) SG_LAUNCH_DECODE_D(128);
+  else SG_LAUNCH_DECODE_D(64);
+#undef SG_LAUNCH_DECODE_D
 #undef SG_LAUNCH_DECODE
   return SG_OK;
 }

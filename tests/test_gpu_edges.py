@@ -138,3 +138,31 @@ def test_score_keys_beyond_l2(lens, L, W, Hq, Hkv, d):
         sg.sg_score(shp, dq, dk, imp.view, ws, st)
         assert np.all(np.abs(imp.numpy() - want) <= 1e-4 * np.abs(want) + 1e-30)
     assert gpu_ops.read_status(st) == 0
+
+
+# Lists that give the eight warps of a CTA none to several slices of 16, cut one entry to either side, the packed part ending
+# on, behind and before a slice boundary.
+RING_KS = (0, 1, 15, 16, 127, 129, 256, 383, 511, 640, 769, 1023)
+
+
+@pytest.mark.parametrize("ks,nls,Hq,Hkv,d", [
+    (RING_KS, tuple(reversed(RING_KS)), 32, 8, 128),              # one CTA per pair, rings of three
+    (RING_KS, tuple(reversed(RING_KS)), 64, 8, 64),               # G = 8
+    (RING_KS, tuple(reversed(RING_KS)), 72, 8, 128),              # G = 9: two tiles of query rows, rings of six
+    (RING_KS, tuple(reversed(RING_KS)), 128, 8, 64),              # G = 16
+    (tuple(4 * k for k in RING_KS), (0,) * 12, 32, 8, 128), # packed rows only, 1024 and more on average: rings of six
+    (tuple(4 * k for k in RING_KS), (0,) * 12, 16, 8, 64),
+    ((1500,) * 20, RING_KS[:10] * 2, 32, 8, 128),                 # the same, long ones: eight warps
+])
+def test_decode_rings(ks, nls, Hq, Hkv, d):
+    """Against the oracle on inputs where one dropped or misplaced row shows (tolerances: see test_gpu_decode_sentinel)."""
+    from test_gpu_decode_sentinel import build_sentinel, check
+    check(build_sentinel(3, tuple(a + b + 5 for a, b in zip(ks, nls)), ks, nls, Hq, Hkv, d))
+
+
+def test_decode_rings_of_short_lists():
+    """More pairs than SMs, four warps.  Values of N(0, 1): the sentinels of a three-entry list average to 20, where bf16
+    rounding alone (2^-9 relative, of the weights and of the output) is beyond the absolute tolerance."""
+    from test_gpu_decode import build, compare
+    nls = RING_KS[:10] * 2
+    compare(build(3, tuple(n + 8 for n in nls), (3,) * 20, nls, 32, 8, 128))
