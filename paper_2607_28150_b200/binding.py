@@ -348,12 +348,12 @@ def prefill(shape: Shape, q_win: torch.Tensor, k_cache: torch.Tensor, v_cache: t
 def prefill_layer(shape: Shape, layer: int, q_win: torch.Tensor, k_cache: torch.Tensor, v_cache: torch.Tensor, importance: torch.Tensor,
                   workspace: Optional[torch.Tensor], cu_k: torch.Tensor, total_sel: int, sel_idx: torch.Tensor, packed_k: torch.Tensor,
                   packed_v: torch.Tensor, dev_status: Optional[torch.Tensor] = None, stream=None) -> None:
-    """sg_score, sg_select_topk and sg_pack_kv of one layer, marshalled once.  The tensors hold all layers (each layer
+    """sg_score, then sg_select_pack_kv, of one layer, marshalled once.  The tensors hold all layers (each layer
     contiguous); `shape` describes one."""
     rc = _native.prefill_layer(shape, layer, q_win, k_cache, v_cache, importance, workspace, cu_k, total_sel, sel_idx, packed_k, packed_v,
                                dev_status, stream)
     if rc:
-        raise SmartGenError(rc & 255, ("sg_score", "sg_select_topk", "sg_pack_kv")[rc >> 8])
+        raise SmartGenError(rc & 255, ("sg_score", "sg_select_pack_kv")[rc >> 8])
 
 
 def decode_layer(shape: Shape, layer: int, q: torch.Tensor, packed_k: torch.Tensor, packed_v: torch.Tensor, cu_k: torch.Tensor,

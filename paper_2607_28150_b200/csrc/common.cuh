@@ -41,6 +41,28 @@ inline sg_status cuda_fail(int err) {
     }                                                                                                 \
   } while (0)
 
+// Programmatic dependent launch.  A kernel launched by launch_chained() may be placed, and set itself up, while the one before
+// it in the stream finishes: it reads and writes nothing of anybody else's before pdl_wait(), which returns once that kernel
+// has completed and its writes are visible.  (After pdl_wait() shared inputs are read with plain loads: the compiler may move
+// read-only-cache loads across it.)
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next kernel in the stream be placed before this one ends.
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename Params>
+inline sg_status launch_chained(void (*kernel)(const Params), dim3 grid, int threads, const Params& p, void* stream) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.stream = static_cast<cudaStream_t>(stream);
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  SG_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, p));
+  return SG_OK;
+}
+
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // Checks common to every call.  `need_window` also validates shape->window.

@@ -121,11 +121,6 @@ __device__ __forceinline__ bool mbar_wait_cluster_bounded(uint64_t* bar) {
   } while (clock64() - t0 < 1000000000LL);
   return false;
 }
-// Programmatic dependent launch: let the next kernel in the stream start its prologue now, and wait
-// for the previous kernel's memory before touching anything it may have written.
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // Exchanges rows and columns of an 8 x 8 matrix of 16-bit values held as an MMA accumulator holds one (lane / 4 = row).
 __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t v) {
   uint32_t r;

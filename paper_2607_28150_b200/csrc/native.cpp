@@ -315,10 +315,8 @@ SG_FN(prefill_layer) {
   return call(x, [&]() -> int {
     int rc = sg_score(s, q, k, (float*)imp, w, wb, (int32_t*)st, stream);
     if (rc) return rc;
-    rc = sg_select_topk(s, (float*)imp, (int32_t*)cu_k, total, (int32_t*)sel, nullptr, 0, (int32_t*)st, stream);
-    if (rc) return rc + 256;
-    rc = sg_pack_kv(s, k, v, (int32_t*)sel, (int32_t*)cu_k, total, pk, pv, (int32_t*)st, stream);
-    return rc ? rc + 512 : 0;
+    rc = sg_select_pack_kv(s, (float*)imp, (int32_t*)cu_k, total, k, v, (int32_t*)sel, pk, pv, (int32_t*)st, stream);
+    return rc ? rc + 256 : 0;
   });
 }
 

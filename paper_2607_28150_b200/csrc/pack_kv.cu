@@ -36,6 +36,7 @@ __global__ void __launch_bounds__(kPackThreads) pack_kv_kernel(const PackParams 
   constexpr int kTPR = D / 8;                       // threads per row, 16 bytes each
   constexpr int kGroups = kPackThreads / kTPR, kRows = kGroups * kUnroll;
   __shared__ int64_t s_src[kRows], s_dst[kRows];    // element offsets; source -1: zeros, destination -1: nothing to do
+  pdl_wait();
   const int lg = blockIdx.x / p.chunks, e0 = (blockIdx.x - lg * p.chunks) * kRows;
   const int l = lg / p.Hkv, g = lg - l * p.Hkv;
   if (threadIdx.x < kRows) {
@@ -146,16 +147,9 @@ sg_status pack_kv_launch(const sg_shape* shape, const void* k_cache, const void*
   p.chunks = total_sel / rows + (total_sel % rows != 0);
   const int64_t grid = (int64_t)p.chunks * shape->num_layers * shape->num_kv_heads;
   if (grid > 0x7fffffffLL) return SG_ERR_UNSUPPORTED;
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (shape->head_dim == 128) {
-    if (sel_count) pack_kv_kernel<128, true><<<(unsigned)grid, kPackThreads, 0, s>>>(p);
-    else pack_kv_kernel<128, false><<<(unsigned)grid, kPackThreads, 0, s>>>(p);
-  } else {
-    if (sel_count) pack_kv_kernel<64, true><<<(unsigned)grid, kPackThreads, 0, s>>>(p);
-    else pack_kv_kernel<64, false><<<(unsigned)grid, kPackThreads, 0, s>>>(p);
-  }
-  SG_CUDA_TRY(cudaGetLastError());
-  return SG_OK;
+  if (shape->head_dim == 128)
+    return launch_chained(sel_count ? pack_kv_kernel<128, true> : pack_kv_kernel<128, false>, dim3((unsigned)grid), kPackThreads, p, stream);
+  return launch_chained(sel_count ? pack_kv_kernel<64, true> : pack_kv_kernel<64, false>, dim3((unsigned)grid), kPackThreads, p, stream);
 }
 }  // namespace
 }  // namespace sg

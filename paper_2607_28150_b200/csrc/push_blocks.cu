@@ -36,6 +36,7 @@ __global__ void __launch_bounds__(kPushThreads) push_blocks_kernel(const PushPar
   constexpr int kRowsPerPass = kPushThreads / kTPR;
   const int b = blockIdx.y;
   int l, m;
+  pdl_wait();
   if constexpr (kByList) {
     const int id = p.selected[blockIdx.x];
     l = id / p.M - p.layer;
@@ -134,19 +135,12 @@ extern "C" sg_status sg_push_blocks(const sg_shape* shape, int32_t num_blocks, i
   p.layer = layer;
   p.layers = shape->num_layers;
   p.K_r = num_selected;
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (shape->batch > 65535 || shape->num_layers > 65535) return SG_ERR_UNSUPPORTED;
   const int64_t blocks = (int64_t)num_blocks * shape->num_layers;
   // 8 layers, 1024 blocks each, 3277 of them listed: by list 35.3 us, by block 42.9
   const bool by_list = num_selected <= blocks;
   const dim3 grid((unsigned)(by_list ? num_selected : blocks), (unsigned)shape->batch);
-  if (shape->head_dim == 128) {
-    if (by_list) push_blocks_kernel<128, true><<<grid, kPushThreads, 0, s>>>(p);
-    else push_blocks_kernel<128, false><<<grid, kPushThreads, 0, s>>>(p);
-  } else {
-    if (by_list) push_blocks_kernel<64, true><<<grid, kPushThreads, 0, s>>>(p);
-    else push_blocks_kernel<64, false><<<grid, kPushThreads, 0, s>>>(p);
-  }
-  SG_CUDA_TRY(cudaGetLastError());
-  return SG_OK;
+  if (shape->head_dim == 128)
+    return launch_chained(by_list ? push_blocks_kernel<128, true> : push_blocks_kernel<128, false>, grid, kPushThreads, p, stream);
+  return launch_chained(by_list ? push_blocks_kernel<64, true> : push_blocks_kernel<64, false>, grid, kPushThreads, p, stream);
 }

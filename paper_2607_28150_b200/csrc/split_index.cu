@@ -37,6 +37,7 @@ __global__ void __launch_bounds__(kSplitThreads) split_index_kernel(const SplitP
   __shared__ uint32_t tot[3];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x / p.Hkv, g = blockIdx.x - b * p.Hkv;
+  pdl_wait();
   const int c0 = p.cu[b], N = p.cu[b + 1] - c0;
   const int ck = p.cu_k[b], kb = p.cu_k[b + 1] - ck;
   const int64_t base = (int64_t)g * p.K_tot + ck;
@@ -48,12 +49,12 @@ __global__ void __launch_bounds__(kSplitThreads) split_index_kernel(const SplitP
 #pragma unroll
     for (int i = 0; i < kFlight; ++i) {
       const int j = j0 + 32 * i + lane;
-      t[i] = j < end ? __ldg(p.kv_index + base + j) : -1;
+      t[i] = j < end ? p.kv_index[base + j] : -1;
     }
 #pragma unroll
     for (int i = 0; i < kFlight; ++i) {
       const bool in = t[i] >= 0 && t[i] < N;
-      const int m = in ? __ldg(p.kv_mask + c0 + t[i]) : 0;
+      const int m = in ? p.kv_mask[c0 + t[i]] : 0;
       cls[i] = j0 + 32 * i + lane >= end ? 3 : (m == 2 ? 0 : (m == 1 ? 1 : 2));
       if (cls[i] != 3 && !in) raise(p.dev_status, SG_ERR_INDEX);
     }
@@ -139,7 +140,5 @@ extern "C" sg_status sg_split_index(const sg_shape* shape, const int32_t* kv_ind
   p.B = shape->batch;
   p.Hkv = shape->num_kv_heads;
   p.reorder = reorder ? 1 : 0;
-  split_index_kernel<<<(unsigned)rows, kSplitThreads, 0, static_cast<cudaStream_t>(stream)>>>(p);
-  SG_CUDA_TRY(cudaGetLastError());
-  return SG_OK;
+  return launch_chained(split_index_kernel, dim3((unsigned)rows), kSplitThreads, p, stream);
 }
