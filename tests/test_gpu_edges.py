@@ -18,6 +18,7 @@ pytestmark = pytest.mark.gpu
     ((2560,), 1, 48, 8, 2, 128),                           # R = 192: two row blocks, the second one partial
     ((2560, 700), 1, 65, 20, 4, 64),                       # R = 325: three row blocks over three warpgroups
     ((1300,), 2, 33, 16, 1, 64),                           # R = 528: five row blocks, a warpgroup takes two of a tile
+    ((700, 130, 900), 8, 38, 32, 8, 128),                  # R = 152, a few segments per CTA: records of several rows merged together
     ((19000,), 1, 8, 8, 8, 64),                            # 8 x 149 tiles: one more per KV head than there are SMs
 ])
 def test_score_at_the_cuts(lens, L, W, Hq, Hkv, d):
@@ -120,8 +121,8 @@ def test_push_by_list(lens, Hkv, d, M, n_sel, head_major):
     ((130000,), 2, 8, 4, 4, 64),                           # long rows of 64-element heads
 ])
 def test_score_keys_beyond_l2(lens, L, W, Hq, Hkv, d):
-    """Calls large enough to run both passes in turn, group by group, in one launch; the call is repeated on the same
-    workspace, whose words then hold the first call's records and counts."""
+    """Calls whose keys exceed L2 and whose CTAs' ranges cross many parts; the call is repeated on the same workspace,
+    whose words then hold the first call's records."""
     import torch
     import gpu_ops
     import paper_2607_28150_b200.binding as sg
