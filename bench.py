@@ -783,7 +783,7 @@ def run_ours(args):
                 "frac": a / peaks["hbm_gbs"], "peak_source": peaks["source"] + " (copy)", "ms_per_step": ms,
                 "launches_per_step": launches, "traffic": ncu.get(name)}
     roofs = {
-        "score": hbm("score", work["score"]["bytes"], st["score"], 1),
+        "score": hbm("score", work["score"]["bytes"], st["score"], 2),
         "select": hbm("select", work["select"]["bytes"], st["select"], 1),
         "pack": hbm("pack", work["pack"]["bytes"], st["pack"], 1),
         "select_pack": hbm("select_pack", work["select"]["bytes"] + work["pack"]["bytes"], st["select_pack"], 1),
@@ -865,7 +865,7 @@ def run_ours(args):
         "stage_ms": st,
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                 "ms_per_step": ms_e2e, "decode_tokens_per_s": e2e_dec_tok, "stage_ms": st_e, "steps": e2e_steps},
-        "gpu_launches": args.steps * (2 + ncalls_dec),
+        "gpu_launches": args.steps * (3 + ncalls_dec),      # scoring 2, selection and gather 1
         "roofline": dominant, "rooflines": roofs, "cpu_baseline": cpu, "clocks": clocks,
         "decode_sweep": sweep, "configs": configs, "next_rows": next_rows, "prefill_layerwise": layerwise, "prefill_full_first_two": first_two, "score_select_handover": handover,
         "e2e_pipelined": None if ms_pipe is None else {
