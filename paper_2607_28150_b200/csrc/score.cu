@@ -323,7 +323,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
     SG_CHECK((smem_u32(q_smem) & 1023u) == 0 && (smem_u32(k_smem) & 1023u) == 0);            // swizzled operands on 1024-byte boundaries
     for (int s = 0; s < 2; ++s) {
       mbar_init(bar_qfull(s), 1); mbar_init(bar_qempty(s), 1);
-      mbar_init(bar_tab_full(s), PASS == 1 ? kEpiWarps : 1); mbar_init(bar_tab_free(s), PASS == 1 ? 2 : kEpiWarps);
+      mbar_init(bar_tab_full(s), PASS == 1 ? kEpiWarps : nblk == 1 ? 2 : 1); mbar_init(bar_tab_free(s), PASS == 1 ? 2 : kEpiWarps);
     }
     for (int s = 0; s < kMaxKStages; ++s) { mbar_init(bar_kfull(s), 1); mbar_init(bar_kempty(s), 1); }
     for (int s = 0; s < kStages; ++s) { mbar_init(bar_afull(s), 1); mbar_init(bar_aempty(s), 4); }
@@ -702,14 +702,17 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_tab_free(buf));
       }
-    } else if (hw == 0) {
-      // merge the records of every segment but the first, one segment ahead of the epilogue
+    } else if (hw == 0 || nblk == 1) {
+      // Merge the records of every segment but the first, one segment ahead of the epilogue.  Both helpers, half of the rows
+      // each, when there are no column sums to add up; 24 records in flight: the CTAs at the part boundaries of a one-layer
+      // call have a segment or two of a tile each, and parts of twenty records (8192 keys:
+      // 28.8 -> 26.6 us for the whole call; one helper, 16 in flight, took eight L2 round trips per segment).
       for (int sidx = 0; ok && walk.next(sg); ++sidx) {
         if (sidx == 0) continue;
         const uint32_t buf = (uint32_t)sidx & 1u, use = (uint32_t)sidx >> 1;
         if (use > 0) ok = wait(bar_tab_free(buf), (use - 1u) & 1u);
         if (!ok) break;
-        merge_records<16, 4>(p, sg, s_prefix, C, neg_lse + buf * p.Ralloc, lane, 32);
+        merge_records<24, 4>(p, sg, s_prefix, C, neg_lse + buf * p.Ralloc, nblk == 1 ? hw * 32 + lane : lane, nblk == 1 ? 64 : 32);
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_tab_full(buf));
       }
