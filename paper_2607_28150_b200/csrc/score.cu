@@ -223,11 +223,11 @@ __device__ __forceinline__ void merge_records(const ScoreParams& p, const Segmen
   const long long tt = (long long)p.units * C, first = (long long)(sg.u - p.u0) * C + prefix[sg.b];
   const int busy = busy_ctas(tt), Weff = min(p.W, sg.N);
   const int c_lo = cta_of(first, tt, busy), nrec = cta_of(first + (prefix[sg.b + 1] - prefix[sg.b]) - 1, tt, busy) - c_lo + 1;
-  if (kRows > 1 && nrec <= kFlight / kRows) {
+  constexpr int kRecs = 4;
+  if (kRows > 1 && nrec <= kRecs) {
     // Short parts: a warp has many rows of one or two records each and a segment of the next part every few microseconds, so
     // several rows' records are in flight together (640 parts of 486 to 827 keys, 152 query rows, whole call: 136.9 us with
     // one row at a time, which made the helper the slowest warp; 116.5 with four; one layer of 8192 keys 30.8 -> 28.9).
-    constexpr int kRecs = kFlight / kRows;
     for (int rb = r0; rb < p.Ralloc; rb += kRows * step) {
       float2 v[kRows][kRecs];
 #pragma unroll
