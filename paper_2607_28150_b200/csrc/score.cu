@@ -339,7 +339,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
     tmem_relinquish();
   }
   if (warp == 0) {
-    if (PASS == 1 && p.B > 1) pdl_wait();              // (pass 2 follows pass 1, which has waited)
+    if (PASS == 1 && p.B > 1) pdl_wait();              // (pass 2 is let go by pass 1 only behind its wait, below)
     // sequence offsets and the per-sequence tile prefix, once per CTA (one sequence: {0, T}, no load)
     int acc = 0;
     for (int b0 = 0; b0 <= p.B; b0 += 32) {
@@ -380,8 +380,11 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
   const uint32_t tmem_base = *tmem_slot;
   const int C = s_prefix[p.B];
   volatile int never = 0;
-  // Another launch of this call follows: let it be set up on every SM that this one leaves (it waits for this whole grid
-  // before it reads or overwrites anything that a launch wrote).
+  // Pass 1 waits for whatever precedes the call (it may have written the queries, the keys, the sequence offsets) before it
+  // lets pass 2 be set up: pass 2 loads queries, keys and offsets without a wait of its own, so everything ahead of the call
+  // has to be complete and visible by then, also behind a kernel that starts its dependents early.  (Pass 2 does wait
+  // for all of pass 1 before it reads or overwrites anything that a launch wrote.)
+  if (PASS == 1) pdl_wait();
   if (p.more) pdl_launch_dependents();
   SegmentWalk<PASS> walk(C, p.units, p.B, p.u0, s_cu, s_prefix);
   Segment sg;
@@ -394,7 +397,6 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
 
   if (warp == kTmaWarp) {
     // ------------------------------------------------------------ TMA producer (one thread)
-    if (PASS == 1) pdl_wait();                         // whatever wrote the queries and keys
     if (lane == 0) {
       int nq = 0, nk = 0;                              // Q operands and K tiles requested so far
       bool ok = true;

@@ -1,0 +1,72 @@
+"""GPU: ordering of calls that are launched programmatically dependent on one another.
+
+`sg_sparse_decode_attn` lets the next kernel in the stream start while it runs and writes its output at its very end, so it
+serves as the producer that a following call must wait for: a long list (few sequences, a million index entries each, all
+within a few rows of the cache) keeps it running for several hundred microseconds on half of the SMs, and the
+following call's kernels are placed beside it at once.
+"""
+import numpy as np
+import pytest
+
+from helpers import cu_of, rand_bf16
+
+pytestmark = pytest.mark.gpu
+
+
+class SlowProducer:
+    """One attention call of `rows` sequences with `heads` heads: out bf16 [rows][heads][d], written after `entries` index
+    entries per list have been attended."""
+
+    def __init__(self, rows, heads, d, entries=1 << 20, tokens=64, seed=0):
+        import torch
+        import gpu_ops
+        rng = np.random.default_rng(seed)
+        cu = cu_of((tokens,) * rows)
+        self.shape = gpu_ops.shape_of(1, heads, heads, d, 1, cu)
+        self.q = gpu_ops.dev(rand_bf16(rng, (rows, heads, d)))
+        self.k = gpu_ops.dev(rand_bf16(rng, (rows * tokens, heads, d)))
+        self.v = gpu_ops.dev(rand_bf16(rng, (rows * tokens, heads, d)))
+        self.nloc = rows * entries
+        self.idx = torch.randint(0, tokens, (heads, self.nloc), dtype=torch.int32, device="cuda")
+        self.cu_nloc = torch.arange(rows + 1, dtype=torch.int32, device="cuda") * entries
+        self.cu_k = torch.zeros(rows + 1, dtype=torch.int32, device="cuda")
+        self.out = torch.zeros((rows, heads, d), dtype=torch.int16, device="cuda")
+
+    def __call__(self):
+        import paper_2607_28150_b200.binding as sg
+        sg.sg_sparse_decode_attn(self.shape, self.q, None, None, self.cu_k, 0, self.k, self.v, self.idx, self.cu_nloc, self.nloc, self.out)
+
+
+@pytest.mark.parametrize("late", ["keys", "queries"])
+def test_score_waits_for_a_producer_that_lets_it_start_early(late):
+    """One sequence and few key tiles leave SMs free for both scoring kernels while the producer of the keys, or of the
+    window queries, is still running: neither may read them before it has ended."""
+    import torch
+    import gpu_ops
+    import paper_2607_28150_b200.binding as sg
+    rng = np.random.default_rng(21)
+    heads, d, n = 2, 128, 4
+    W = n if late == "queries" else 2
+    make = SlowProducer(n, heads, d)
+    T = 300 if late == "queries" else n
+    k = gpu_ops.dev(rand_bf16(rng, (1, T, heads, d))) if late == "queries" else make.out.view(1, n, heads, d)
+    q = make.out.view(1, 1, W, heads, d) if late == "queries" else gpu_ops.dev(rand_bf16(rng, (1, 1, W, heads, d)))
+    shp = gpu_ops.shape_of(1, heads, heads, d, W, cu_of((T,)))
+    ws = sg.alloc_workspace(sg.SG_OP_SCORE, shp)
+
+    def score():
+        imp, st = torch.full((1, heads, T), -1.0, dtype=torch.float32, device="cuda"), gpu_ops.status_word()
+        sg.sg_score(shp, q, k, imp, ws, st)
+        return imp, st
+
+    early, _ = score()                                    # on the zeros that the producer will overwrite
+    torch.cuda.synchronize()
+    for _ in range(3):
+        make.out.zero_()
+        imp, st = torch.full((1, heads, T), -1.0, dtype=torch.float32, device="cuda"), gpu_ops.status_word()
+        torch.cuda.synchronize()
+        make()
+        sg.sg_score(shp, q, k, imp, ws, st)
+        assert gpu_ops.read_status(st) == 0
+        want, _ = score()                                 # again, when everything has been written
+        assert torch.equal(imp, want) and not torch.allclose(want, early, rtol=1e-3)
