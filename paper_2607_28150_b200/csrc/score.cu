@@ -388,10 +388,12 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
   if (p.more) pdl_launch_dependents();
   SegmentWalk<PASS> walk(C, p.units, p.B, p.u0, s_cu, s_prefix);
   Segment sg;
+  // In pass 2 loads and MMAs run ahead while the epilogue waits for pass 1: what their limits count starts behind pass 1.
+  constexpr bool kBehind = PASS == 1;
   // A warp's wait: every lane sees the phase complete, or none goes on.
   auto wait = [&](uint32_t bar, uint32_t parity) {
     if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return true;
-    return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, abort_flag, p.wait_ns)) != 0;
+    return __all_sync(0xffffffffu, mbar_wait_slow<kBehind>(bar, parity, abort_flag, p.wait_ns)) != 0;
   };
   long long w0 = 0, w1 = 0;                            // waiting clocks (profiling build)
 
@@ -402,7 +404,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
       bool ok = true;
       while (ok && walk.next(sg)) {
         const int l = sg.u / p.Hkv, g = sg.u - l * p.Hkv, qs = nq % p.q_bufs;
-        ok = mbar_wait(bar_qempty(qs), (uint32_t)(((nq / p.q_bufs) & 1) ^ 1), abort_flag, p.wait_ns, 100u);
+        ok = mbar_wait<kBehind>(bar_qempty(qs), (uint32_t)(((nq / p.q_bufs) & 1) ^ 1), abort_flag, p.wait_ns, 100u);
         if (!ok) break;
         ++nq;
         mbar_arrive_expect_tx(bar_qfull(qs), (uint32_t)(kSub * p.G * p.W * 128));
@@ -412,7 +414,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
         const int tiles = sg.tile_end - sg.tile_beg;
         for (int i = 0; i < tiles; ++i) {
           const int tile = tile_at<PASS>(sg, i), ks = nk % p.k_stages;
-          ok = mbar_wait(bar_kempty(ks), (uint32_t)(((nk / p.k_stages) & 1) ^ 1), abort_flag, p.wait_ns, 100u);
+          ok = mbar_wait<kBehind>(bar_kempty(ks), (uint32_t)(((nk / p.k_stages) & 1) ^ 1), abort_flag, p.wait_ns, 100u);
           if (!ok) break;
           ++nk;
           SG_CHECK(sg.c0 + tile * kTileKeys < p.T && g < p.Hkv && sg.b < p.B);
@@ -425,14 +427,14 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
       // No copy and no barrier arrival of this CTA may be pending when it exits: wait until the MMAs have released every
       // buffer, or, on an aborted run (nobody consumes what was requested), for the copies themselves.
       for (int i = 0; i < p.k_stages && ok; ++i)
-        ok = mbar_wait(bar_kempty((nk + i) % p.k_stages), (uint32_t)((((nk + i) / p.k_stages) & 1) ^ 1), abort_flag, p.wait_ns, 100u);
+        ok = mbar_wait<kBehind>(bar_kempty((nk + i) % p.k_stages), (uint32_t)((((nk + i) / p.k_stages) & 1) ^ 1), abort_flag, p.wait_ns, 100u);
       for (int i = 0; i < p.q_bufs && ok; ++i)
-        ok = mbar_wait(bar_qempty((nq + i) % p.q_bufs), (uint32_t)((((nq + i) / p.q_bufs) & 1) ^ 1), abort_flag, p.wait_ns, 100u);
+        ok = mbar_wait<kBehind>(bar_qempty((nq + i) % p.q_bufs), (uint32_t)((((nq + i) / p.q_bufs) & 1) ^ 1), abort_flag, p.wait_ns, 100u);
       if (!ok) {
         for (int n = max(0, nk - p.k_stages); n < nk; ++n)
-          mbar_wait(bar_kfull(n % p.k_stages), (uint32_t)((n / p.k_stages) & 1), &never, p.wait_ns, 100u);
+          mbar_wait<kBehind>(bar_kfull(n % p.k_stages), (uint32_t)((n / p.k_stages) & 1), &never, p.wait_ns, 100u);
         for (int n = max(0, nq - p.q_bufs); n < nq; ++n)
-          mbar_wait(bar_qfull(n % p.q_bufs), (uint32_t)((n / p.q_bufs) & 1), &never, p.wait_ns, 100u);
+          mbar_wait<kBehind>(bar_qfull(n % p.q_bufs), (uint32_t)((n / p.q_bufs) & 1), &never, p.wait_ns, 100u);
       }
     }
   } else if (warp == kMmaWarp) {
@@ -482,7 +484,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
     // (the commit arrives when all earlier MMAs are done; the wait ignores the abort flag and is bounded).
     if (leader) {
       umma_commit(bar_drain);
-      mbar_wait(bar_drain, 0u, &never, p.wait_ns, 0u);
+      mbar_wait<kBehind>(bar_drain, 0u, &never, p.wait_ns, 0u);
     }
     __syncwarp();
     SG_PROF_STORE(4, w0); SG_PROF_STORE(5, w1);

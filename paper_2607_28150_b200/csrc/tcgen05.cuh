@@ -39,9 +39,14 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
 // all executed instructions, SFU pipe at 51 %).  A waiter therefore sleeps `sleep_ns` between attempts (chosen per
 // role: short on the MMA thread's critical path, long for the producer that runs ahead) and looks at the clock and the
 // abort flag only every 64th attempt.
+// kBehind: the thread has executed pdl_wait().  Otherwise the work it waits for may itself be waiting for the kernel in
+// front of this one, whose time does not count: when the limit first runs out, the thread waits for that kernel and
+// starts its limit again.
+template <bool kBehind>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, uint32_t limit_ns,
                                           uint32_t sleep_ns) {
   if (mbar_test(bar, parity)) return true;
+  bool behind = kBehind;
   uint64_t t0 = 0;
   for (uint32_t it = 0;; ++it) {
     if (sleep_ns) __nanosleep(sleep_ns);
@@ -49,14 +54,21 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     if ((it & 63u) == 63u) {
       if (*abort_flag) return false;
       const uint64_t now = global_timer_ns();
-      if (t0 == 0) t0 = now;
-      else if (now - t0 > (uint64_t)limit_ns) { *abort_flag = 1; return false; }
+      if (t0 == 0) {
+        t0 = now;
+      } else if (now - t0 > (uint64_t)limit_ns) {
+        if (behind) { *abort_flag = 1; return false; }
+        pdl_wait();
+        behind = true;
+        t0 = global_timer_ns();
+      }
     }
   }
 }
 // The same wait for code that issues work on its critical path: everything but a first attempt stays out of line.
+template <bool kBehind>
 static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag, uint32_t limit_ns) {
-  return mbar_wait(bar, parity, abort_flag, limit_ns, 0u);
+  return mbar_wait<kBehind>(bar, parity, abort_flag, limit_ns, 0u);
 }
 __device__ __forceinline__ void fence_barrier_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }

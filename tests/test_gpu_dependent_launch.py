@@ -70,3 +70,35 @@ def test_score_waits_for_a_producer_that_lets_it_start_early(late):
         assert gpu_ops.read_status(st) == 0
         want, _ = score()                                 # again, when everything has been written
         assert torch.equal(imp, want) and not torch.allclose(want, early, rtol=1e-3)
+
+
+def test_pass_2_of_scoring_waits_as_long_as_pass_1_takes():
+    """More (layer, sequence, KV head) parts than the fixed scratch of sg_score_static holds at full width: pass 1 runs for
+    several milliseconds on a few CTAs while those of pass 2 are set up beside it.  Their bounded waits, shortened to one
+    millisecond, count from the end of pass 1."""
+    import torch
+    import gpu_ops
+    import paper_2607_28150_b200.binding as sg
+    B, n, heads, G, d, W = 252, 3000, 8, 8, 64, 64        # 2016 parts of 512 rows: records of 4 KB, 8 MB hold 32 more
+    cu = cu_of((n,) * B)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(3)
+    q = torch.randn((1, B, W, heads * G, d), generator=gen, device="cuda", dtype=torch.bfloat16)
+    k = torch.randn((1, B * n, heads, d), generator=gen, device="cuda", dtype=torch.bfloat16)
+    shp = gpu_ops.shape_of(1, heads * G, heads, d, W, cu)
+    imp = torch.full((1, heads, B * n), -1.0, dtype=torch.float32, device="cuda")
+    want, st, st2 = torch.empty_like(imp), gpu_ops.status_word(), gpu_ops.status_word()
+    sg.sg_score(shp, q, k, want, sg.alloc_workspace(sg.SG_OP_SCORE, shp), st2)
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    try:
+        sg.sg_testing_score_fault(-1, 1)
+        a.record()
+        sg.sg_score_static(shp, q, k, imp, st)
+        b.record()
+        torch.cuda.synchronize()
+    finally:
+        sg.sg_testing_score_fault(-1, 0)
+    assert a.elapsed_time(b) > 4.0                        # else the limit would not have been exceeded
+    assert gpu_ops.read_status(st) == 0 and gpu_ops.read_status(st2) == 0
+    # the same sums, cut at other places: a few roundings of fp32 partial sums
+    assert torch.all((imp - want).abs() <= 1e-5 * want.abs() + 1e-30)
