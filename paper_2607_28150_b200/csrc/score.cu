@@ -118,18 +118,35 @@ __device__ __forceinline__ uint64_t exp2_sfu2(uint64_t x) {
   unpack2(x, x0, x1);
   return pack2(exp2f(x0), exp2f(x1));
 }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+// Bounds that let a NaN through (fmaxf and fminf return the bound in its place).
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.ftz.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float min_nan(float a, float b) {
+  float r;
+  asm("min.ftz.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
 // Two exp2 on the FMA pipe: x = n + f with n an integer and |f| <= 1/2, 2^f by a polynomial of degree 5 (minimax fit of
-// 2^f by iterated weighted least squares, constant term 1; relative error at most 1.6e-7 including the fp32 evaluation),
-// n added to the exponent field.  x is clamped to -127, where the sum of the exponent fields is 0, a subnormal that every
-// later operation flushes, and, where x may be large (pass 1, against a stale reference), to 127: a huge finite number,
-// which trips the range test of pass 1 as the SFU's inf does.
+// 2^f by iterated weighted least squares, constant term 1; relative error at most 1.7e-7 including the fp32 evaluation),
+// times 2^n put together from its exponent field.  x is clamped to -127, where that field is 0 and so is the factor, and,
+// where x may be large (pass 1, against a stale reference), to 127: a huge finite number, which trips the range test of
+// pass 1 as the SFU's inf does.  A NaN passes the clamps and the polynomial and is a NaN behind the product, as the
+// SFU's is: a non-finite score shows in the sums whatever column it stands in.
 template <bool kAbove>
 __device__ __forceinline__ uint64_t exp2_fma2(uint64_t x) {
   float x0, x1;
   unpack2(x, x0, x1);
-  x0 = fmaxf(x0, -127.f);
-  x1 = fmaxf(x1, -127.f);
-  if (kAbove) { x0 = fminf(x0, 127.f); x1 = fminf(x1, 127.f); }
+  x0 = max_nan(x0, -127.f);
+  x1 = max_nan(x1, -127.f);
+  if (kAbove) { x0 = min_nan(x0, 127.f); x1 = min_nan(x1, 127.f); }
   x = pack2(x0, x1);
   const uint64_t t = add2(x, pack2(12582912.f, 12582912.f));                 // 1.5 * 2^23: the low bits of t are round(x)
   const uint64_t f = fma2(add2(t, pack2(-12582912.f, -12582912.f)), pack2(-1.f, -1.f), x);
@@ -138,10 +155,9 @@ __device__ __forceinline__ uint64_t exp2_fma2(uint64_t x) {
   q = fma2(q, f, pack2(0.24022242426872253f, 0.24022242426872253f));
   q = fma2(q, f, pack2(0.6931470036506653f, 0.6931470036506653f));
   q = fma2(q, f, pack2(1.f, 1.f));
-  float q0, q1, t0, t1;
-  unpack2(q, q0, q1);
+  float t0, t1;
   unpack2(t, t0, t1);
-  return pack2(__int_as_float(__float_as_int(q0) + (__float_as_int(t0) << 23)), __int_as_float(__float_as_int(q1) + (__float_as_int(t1) << 23)));
+  return mul2(q, pack2(__int_as_float((__float_as_int(t0) << 23) + 0x3f800000), __int_as_float((__float_as_int(t1) << 23) + 0x3f800000)));
 }
 // Pairs of a 32-column chunk's sixteen whose exponentials run on the FMA pipe, spread evenly.
 constexpr int kFmaPairs1 = 4, kFmaPairs2 = 4;
