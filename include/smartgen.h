@@ -165,13 +165,16 @@ sg_status sg_select_pack_kv(const sg_shape* shape, const float* importance, cons
  *
  * Stream ordering: the kernel is launched with programmatic dependent launch and lets the next kernel
  * in the stream start early.  out / lse are written only after all earlier work in the stream has completed.
- * Every INPUT -- q, the KV sources (packed_k/v, local_k/v), local_idx, the per-head count arrays and the
- * prefix arrays (cu_seqlens, cu_k, cu_nloc) -- is treated as a stable input of the decode step and may be
- * read while an immediately preceding kernel THAT ITSELF OPTED IN to programmatic dependent launch (such as
- * the previous layer's sg_sparse_decode_attn, or sg_score) is still running: inputs must not be outputs of
- * such a kernel.  Ordinary preceding kernels (the projection that produces q, a copy, anything launched the
- * usual way) are fully ordered before this call as usual.  Independent calls issued back to back therefore
- * overlap everything but their output stores.
+ * Every INPUT -- q, the KV sources (packed_k/v, local_k/v), local_idx and the prefix arrays (cu_seqlens, cu_k,
+ * cu_nloc) -- is treated as a stable input of the decode step and is read without waiting for a preceding kernel
+ * that lets its dependents start early (griddepcontrol.launch_dependents,
+ * cudaTriggerProgrammaticLaunchCompletion).  The rule: an input must not be an output of a kernel in the unbroken
+ * run of such kernels directly in front of this call in the stream.  Of this library the attention calls and
+ * sg_score / sg_score_static let their dependents start early; all others (selection, packing, splitting, pushing,
+ * profiling) do not, nor do ordinary kernels and copies: those have ended when this call's kernel
+ * begins, so their outputs -- the projection's q, packed rows, index lists -- may be its inputs directly.
+ * Independent calls issued back to back therefore overlap everything but their output stores.
+ * sg_sparse_decode_attn_counted makes no such exception: it reads nothing before all earlier work has completed.
  */
 sg_status sg_sparse_decode_attn(const sg_shape* shape, const void* q, const void* packed_k,
                                 const void* packed_v, const int32_t* cu_k, int32_t total_sel,

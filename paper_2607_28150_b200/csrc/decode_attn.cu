@@ -163,6 +163,10 @@ __global__ void __launch_bounds__(kDecWarps * 32, (kN == 1 && kSlots * D <= 384 
     }
     cluster_arrive_release();                                  // "this CTA runs, its barrier is set up": awaited before the first remote store
   }
+  // The counts, rows and index lists of a counted call come from the calls right in front of it (split, pack): it reads
+  // nothing before they are complete and visible.  (They have ended when its CTAs are placed, so the wait is short.)
+  // Everything it reads is read with plain loads: the compiler may move read-only-cache loads across the wait.
+  if (p.packed_count || p.local_skip) pdl_wait();
   const int b = blockIdx.x / p.csize;                          // grid.x = B * cluster size
   const int c = blockIdx.x - b * p.csize;                      // rank in the cluster
   // A single sequence (the latency-critical case) needs no prefix loads: a dependent round trip to L2 less before the
@@ -170,10 +174,10 @@ __global__ void __launch_bounds__(kDecWarps * 32, (kN == 1 && kSlots * D <= 384 
   const bool one = p.B == 1;
   const int ck0 = one ? 0 : p.cu_k[b];
   const int kb = one ? p.K_tot : p.cu_k[b + 1] - ck0;          // packed rows per KV head (the slot size in the buffer)
-  const int kbe = p.packed_count ? min(kb, max(0, __ldg(p.packed_count + (int64_t)b * p.Hkv + g))) : kb;   // ... of which in the list
+  const int kbe = p.packed_count ? min(kb, max(0, p.packed_count[(int64_t)b * p.Hkv + g])) : kb;   // ... of which in the list
   const int cl0 = one ? 0 : p.cu_nloc[b];
   const int nl_row = one ? p.NL_tot : p.cu_nloc[b + 1] - cl0;
-  const int lskip = p.local_skip ? min(nl_row, max(0, __ldg(p.local_skip + (int64_t)b * p.Hkv + g))) : 0;
+  const int lskip = p.local_skip ? min(nl_row, max(0, p.local_skip[(int64_t)b * p.Hkv + g])) : 0;
   const int nl = nl_row - lskip;
   const int c0 = one ? 0 : p.cu[b];
   const int nseq = one ? p.n_tokens : p.cu[b + 1] - c0;
@@ -194,7 +198,7 @@ __global__ void __launch_bounds__(kDecWarps * 32, (kN == 1 && kSlots * D <= 384 
   // Lane r (and r + 16) holds the local index of row r of a slice, read ahead of its use.
   auto fetch_idx = [&](int at) -> int {
     const int li = at + (lane & 15);
-    return (li < ntok && li >= kbe) ? __ldg(idx_base + at) : 0;
+    return (li < ntok && li >= kbe) ? idx_base[at] : 0;
   };
   // A warp is alone on its scheduler or shares it with a few others, and its instructions issue one by one: what a slice takes
   // is its instruction count (2500 clocks for 600 of them).  So the copies' addresses are built from per-lane constants and
@@ -272,8 +276,8 @@ __global__ void __launch_bounds__(kDecWarps * 32, (kN == 1 && kSlots * D <= 384 
   }
 
   // Everything in this kernel up to its output stores reads only inputs of the decode step -- the KV sources, the
-  // index lists, the prefix arrays and the query rows -- which the contract treats as stable: they must not be
-  // written by a kernel that itself lets its dependents start early (such as the previous layer's call of this
+  // index lists, the prefix arrays and the query rows -- which the contract of the plain call treats as stable: they must
+  // not be written by a kernel that itself lets its dependents start early (such as the previous layer's call of this
   // kernel).  So nothing waits here: the dependency wait sits in front of the stores of out / lse, and consecutive
   // calls overlap everything but those stores.
   // Q fragments (B operand, D x 8 per tile; rows >= G are zero).

@@ -102,3 +102,66 @@ def test_pass_2_of_scoring_waits_as_long_as_pass_1_takes():
     assert gpu_ops.read_status(st) == 0 and gpu_ops.read_status(st2) == 0
     # the same sums, cut at other places: a few roundings of fp32 partial sums
     assert torch.all((imp - want).abs() <= 1e-5 * want.abs() + 1e-30)
+
+
+@pytest.mark.parametrize("late", ["packed rows", "queries"])
+def test_counted_attention_waits_for_a_producer_that_lets_it_start_early(late):
+    import torch
+    import gpu_ops
+    import paper_2607_28150_b200.binding as sg
+    rng = np.random.default_rng(22)
+    heads, d, n = 2, 128, 4
+    make = SlowProducer(n, heads, d)                       # out [n][heads][d]: n packed rows of each of the heads, or n sequences' queries
+    B = n if late == "queries" else 1
+    rows = make.out if late == "packed rows" else gpu_ops.dev(rand_bf16(rng, (B * 3, heads, d)))
+    q = make.out if late == "queries" else gpu_ops.dev(rand_bf16(rng, (B, heads, d)))
+    per = 3 if late == "queries" else n                    # packed rows per list
+    packed = rows.view(B * per * heads, d)
+    cu_cap = torch.arange(B + 1, dtype=torch.int32, device="cuda") * per
+    shp = gpu_ops.shape_of(1, heads, heads, d, 1, cu_of((8,) * B))
+    count = torch.full((B, heads), per, dtype=torch.int32, device="cuda")
+    none = torch.zeros(B + 1, dtype=torch.int32, device="cuda")
+    out, want = (torch.zeros((B, heads, d), dtype=torch.int16, device="cuda") for _ in range(2))
+
+    def attend(o):
+        sg.sg_sparse_decode_attn_counted(shp, q, packed, packed, cu_cap, B * per, count, None, None, None, none, 0, o)
+
+    attend(out)
+    torch.cuda.synchronize()
+    early = out.clone()                                    # on the zeros that the producer will overwrite
+    for _ in range(3):
+        make.out.zero_()
+        torch.cuda.synchronize()
+        make()
+        attend(out)
+        torch.cuda.synchronize()
+        attend(want)                                       # again, when everything has been written
+        torch.cuda.synchronize()
+        assert torch.equal(out, want) and not torch.equal(want, early)
+
+
+def test_attention_directly_behind_packing_reads_the_packed_rows():
+    """The rows that sg_pack_kv has just written are inputs of the next call, whose kernel reads them without waiting."""
+    import torch
+    import gpu_ops
+    import paper_2607_28150_b200.binding as sg
+    rng = np.random.default_rng(23)
+    Hq, Hkv, d, N, K = 32, 8, 128, 4096, 800
+    cu, ck = gpu_ops.dev(cu_of((N,))), gpu_ops.dev(cu_of((K,)))
+    shp = gpu_ops.shape_of(1, Hq, Hkv, d, 1, cu_of((N,)))
+    caches = [tuple(gpu_ops.dev(rand_bf16(rng, (1, N, Hkv, d))) for _ in range(2)) for _ in range(2)]
+    sel = torch.stack([torch.randperm(N, device="cuda")[:K].sort().values for _ in range(Hkv)]).int()[None].contiguous()
+    q = gpu_ops.dev(rand_bf16(rng, (1, Hq, d)))
+    none = torch.zeros(2, dtype=torch.int32, device="cuda")
+    pk, pv = (torch.zeros((1, K * Hkv, d), dtype=torch.int16, device="cuda") for _ in range(2))
+    outs = torch.zeros((402, 1, Hq, d), dtype=torch.int16, device="cuda")
+    for i in range(402):
+        if i < 2:
+            torch.cuda.synchronize()
+        sg.sg_pack_kv(shp, *caches[i % 2], sel, ck, K, pk, pv)
+        if i < 2:
+            torch.cuda.synchronize()                       # the first two are the references
+        sg.sg_sparse_decode_attn(shp, q, pk[0], pv[0], ck, K, None, None, None, none, 0, outs[i])
+    torch.cuda.synchronize()
+    assert not torch.equal(outs[0], outs[1])
+    assert torch.equal(outs[2::2], outs[0].expand(200, 1, Hq, d)) and torch.equal(outs[3::2], outs[1].expand(200, 1, Hq, d))
