@@ -94,9 +94,9 @@ __global__ void __launch_bounds__(kSelThreads, 1) select_topk_kernel(const SelPa
   const uint32_t* x = reinterpret_cast<const uint32_t*>(p.importance) + ((int64_t)l * p.Hkv + g) * p.T + c0;
 
   if (kInSmem) {
-    for (int t = tid; t < N; t += kSelThreads) keys[t] = order_key(__ldg(x + t));
+    for (int t = tid; t < N; t += kSelThreads) keys[t] = order_key(x[t]);
   }
-  auto key_at = [&](int t) -> uint32_t { return kInSmem ? keys[t] : order_key(__ldg(x + t)); };
+  auto key_at = [&](int t) -> uint32_t { return kInSmem ? keys[t] : order_key(x[t]); };
 
   // ---- radix select: find the kb-th largest key ----
   uint32_t prefix = 0, decided = 0, need = (uint32_t)kb;
@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
   }
   uint32_t key[E];
   if constexpr (kBulk) {
-    for (int i = whole + tid; i < span; i += T) stage[i] = __ldg(x - off + i);
+    for (int i = whole + tid; i < span; i += T) stage[i] = x[i - off];
     __syncthreads();                                   // barrier set up, histogram cleared, plainly loaded values there
     uint32_t done = bulk ? 0u : 1u;
     for (uint32_t tries = 0; tries < (1u << 22) && !done; ++tries)
@@ -383,11 +383,11 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
     for (int q = 0; q < kQuads; ++q) {
       const int i = first + 4 * q;
       if (i + 3 < N) {
-        v[q] = __ldg(reinterpret_cast<const uint4*>(x + i));
+        v[q] = *reinterpret_cast<const uint4*>(x + i);
       } else {
-        v[q].x = i < N ? __ldg(x + i) : 0u;
-        v[q].y = i + 1 < N ? __ldg(x + i + 1) : 0u;
-        v[q].z = i + 2 < N ? __ldg(x + i + 2) : 0u;
+        v[q].x = i < N ? x[i] : 0u;
+        v[q].y = i + 1 < N ? x[i + 1] : 0u;
+        v[q].z = i + 2 < N ? x[i + 2] : 0u;
         v[q].w = 0u;
       }
     }
@@ -401,7 +401,7 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
     {
       uint32_t v[E];                                   // all E loads of the thread are issued before the first store
 #pragma unroll
-      for (int e = 0; e < E; ++e) { const int i = tid + e * T; v[e] = i < N ? __ldg(x + i) : 0u; }
+      for (int e = 0; e < E; ++e) { const int i = tid + e * T; v[e] = i < N ? x[i] : 0u; }
 #pragma unroll
       for (int e = 0; e < E; ++e) { const int i = tid + e * T; stage[i + 4 * (i / E)] = i < N ? order_key(v[e]) : 0u; }
     }
