@@ -117,7 +117,8 @@ sg_status sg_select_topk(const sg_shape* shape, const float* importance, const i
  * (Section 4.2); the prefill node selects the required entries locally before sending them.
  *     packed_k[l][cu_k[b]*H_kv + g*k_b + j][:] = k_cache[l][cu[b] + sel_idx[l][g][cu_k[b]+j]][g][:]
  * and the same for V.  An index outside [0, N_b) sets the SG_ERR_INDEX device bit and its row is
- * written as zeros.
+ * written as zeros.  A total_sel above cu_k[B] sets the SG_ERR_INVALID device bit; the entries behind
+ * cu_k[B] are skipped.
  *
  * packed_k/v  bf16 [L][K_tot*H_kv][d], fully overwritten.
  */

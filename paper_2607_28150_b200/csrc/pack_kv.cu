@@ -48,13 +48,15 @@ __global__ void __launch_bounds__(kPackThreads) pack_kv_kernel(const PackParams 
       b = upper_segment(p.cu_k, p.B, e - lane);
     } else if (p.B > 1) {
       const int end = lane < p.B ? p.cu_k[lane + 1] : 0x7fffffff;
-      b = __popc(__ballot_sync(0xffffffffu, end <= e - lane));
+      b = min(__popc(__ballot_sync(0xffffffffu, end <= e - lane)), p.B - 1);
     }
     if (e < p.K_tot) {
       int ck = p.cu_k[b], ce = p.cu_k[b + 1];
       while (e >= ce && b + 1 < p.B) { ++b; ck = ce; ce = p.cu_k[b + 1]; }
       const int kb = ce - ck, j = e - ck;
-      if (!kCounted || j < p.sel_count[((int64_t)l * p.B + b) * p.Hkv + g]) {
+      if (j >= kb) {
+        raise(p.dev_status, SG_ERR_INVALID);          // the host's total is larger than cu_k[B]: no row owns the entry
+      } else if (!kCounted || j < p.sel_count[((int64_t)l * p.B + b) * p.Hkv + g]) {
         dst = ((int64_t)l * p.K_tot * p.Hkv + (int64_t)ck * p.Hkv + (int64_t)g * kb + j) * D;
         const int t = p.sel_idx[(int64_t)lg * p.K_tot + e];
         const int c0 = p.cu[b];

@@ -200,3 +200,29 @@ def test_score_non_finite_input_marks_its_part(value, where, at):
     part[l, g, int(cu[b]):int(cu[b + 1])] = True
     assert bool(got[part].isnan().all())
     assert torch.equal(got[~part], clean[~part]) and bool(clean.isfinite().all())
+
+
+@pytest.mark.parametrize("B", [1, 2, 32, 33])
+@pytest.mark.parametrize("counted", [False, True])
+def test_pack_total_above_the_prefix_array(B, counted):
+    """A host total larger than cu_k[B] is flagged; the entries that belong to no row are skipped, the others packed."""
+    import torch
+    import gpu_ops
+    import paper_2607_28150_b200.binding as sg
+    rng = np.random.default_rng(15)
+    k, more, Hkv, d = 9, 200, 1, 128                       # one KV head: the rows of the surplus lie behind all others
+    cu, ck = cu_of((12,) * B), cu_of((k,) * B)
+    K = B * k
+    kc = rand_bf16(rng, (1, 12 * B, Hkv, d))
+    sel = np.tile(np.arange(k, dtype=np.int32), B + more)[None, None, :K + more].copy()
+    pk, pv = (gpu_ops.Guarded((1, (K + more) * Hkv, d), torch.int16, 0x5555) for _ in range(2))
+    shp, st = gpu_ops.shape_of(1, Hkv, Hkv, d, 1, cu), gpu_ops.status_word()
+    args = [shp, gpu_ops.dev(kc), gpu_ops.dev(kc), gpu_ops.dev(sel), gpu_ops.dev(ck), K + more]
+    if counted:
+        sg.sg_pack_kv_counted(*args, torch.full((1, B, Hkv), k, dtype=torch.int32, device="cuda"), pk.view, pv.view, st)
+    else:
+        sg.sg_pack_kv(*args, pk.view, pv.view, st)
+    assert gpu_ops.read_status(st) == 1 << sg.SG_ERR_INVALID
+    want = np.concatenate([kc[0, 12 * b:12 * b + k, 0] for b in range(B)])
+    for got in (pk.numpy(), pv.numpy()):
+        assert np.array_equal(got[0, :K], want) and np.all(got[0, K:] == 0x5555)
