@@ -9,6 +9,7 @@
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "smartgen.h"
@@ -138,7 +139,16 @@ PyObject* call(const Args& x, F f) {
   Py_END_ALLOW_THREADS
   return PyLong_FromLong(rc);
 }
-#define SG_FN(name) PyObject* name(PyObject*, PyObject* const* a, Py_ssize_t n)
+// A function of the module.  A tensor's accessors throw C++ exceptions (no storage, no CUDA device); they become Python
+// errors here and never leave a C function.
+#define SG_FN(name)                                                         \
+  PyObject* name##_args(PyObject* const* a, Py_ssize_t n);                  \
+  PyObject* name(PyObject*, PyObject* const* a, Py_ssize_t n) {             \
+    HANDLE_TH_ERRORS                                                        \
+    return name##_args(a, n);                                               \
+    END_HANDLE_TH_ERRORS                                                    \
+  }                                                                         \
+  PyObject* name##_args(PyObject* const* a, Py_ssize_t n)
 
 SG_FN(score) {
   Args x(a, n, 7);
