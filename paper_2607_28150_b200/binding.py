@@ -349,7 +349,7 @@ def prefill_layer(shape: Shape, layer: int, q_win: torch.Tensor, k_cache: torch.
                   workspace: Optional[torch.Tensor], cu_k: torch.Tensor, total_sel: int, sel_idx: torch.Tensor, packed_k: torch.Tensor,
                   packed_v: torch.Tensor, dev_status: Optional[torch.Tensor] = None, stream=None) -> None:
     """sg_score, then sg_select_pack_kv, of one layer, marshalled once.  The tensors hold all layers (each layer
-    contiguous); `shape` describes one."""
+    contiguous; a sequence of one tensor per layer is taken, too); `shape` describes one."""
     rc = _native.prefill_layer(shape, layer, q_win, k_cache, v_cache, importance, workspace, cu_k, total_sel, sel_idx, packed_k, packed_v,
                                dev_status, stream)
     if rc:

@@ -33,9 +33,13 @@ struct Args {
   PyObject* const* a;
   Py_ssize_t n, i = 0;
   bool ok = true;
+  PyObject* held[8];                                    // layers taken out of sequences, kept for the length of the call
+  int n_held = 0;
   Args(PyObject* const* a_, Py_ssize_t n_, Py_ssize_t want) : a(a_), n(n_) {
     if (n != want) { PyErr_Format(PyExc_TypeError, "expected %zd arguments, got %zd", want, n); ok = false; }
   }
+  Args(const Args&) = delete;
+  ~Args() { while (n_held > 0) Py_DECREF(held[--n_held]); }
   const sg_shape* shape() {
     if (!ok) return nullptr;
     Py_buffer view;
@@ -59,8 +63,9 @@ struct Args {
   }
   // Checked tensor; undefined when None is given and allowed.  An empty tensor's address is null.
   const at::Tensor* tensor(Kind kind, const char* name, bool allow_none = false, bool whole = true) {
-    if (!ok) return nullptr;
-    PyObject* o = a[i++];
+    return ok ? tensor_of(a[i++], kind, name, allow_none, whole) : nullptr;
+  }
+  const at::Tensor* tensor_of(PyObject* o, Kind kind, const char* name, bool allow_none, bool whole) {
     if (o == Py_None) {
       if (!allow_none) { PyErr_Format(PyExc_TypeError, "%s is required", name); ok = false; }
       return nullptr;
@@ -87,8 +92,17 @@ struct Args {
     const at::Tensor* t = tensor(kind, name, allow_none);
     return t == nullptr || t->numel() == 0 ? nullptr : t->data_ptr();
   }
-  // t[layer] of a tensor whose layers are contiguous each.
+  // t[layer] of a tensor whose layers are contiguous each, or of a sequence of tensors, one per layer.
   void* layer_ptr(Kind kind, const char* name, long long layer) {
+    if (ok && a[i] != Py_None && !THPVariable_Check(a[i])) {
+      PyObject* index = PyLong_FromLongLong(layer);
+      PyObject* item = index == nullptr ? nullptr : PyObject_GetItem(a[i++], index);
+      Py_XDECREF(index);
+      if (item == nullptr) { ok = false; return nullptr; }
+      held[n_held++] = item;
+      const at::Tensor* t = tensor_of(item, kind, name, false, true);
+      return t == nullptr || t->numel() == 0 ? nullptr : t->data_ptr();
+    }
     const at::Tensor* t = tensor(kind, name, false, false);
     if (t == nullptr) return nullptr;
     if (t->dim() < 1 || layer < -t->size(0) || layer >= t->size(0)) {

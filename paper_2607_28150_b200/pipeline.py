@@ -82,7 +82,7 @@ class HotPath:
                       stream=None, aux_stream=None):
         """score -> select -> pack of ONE layer, as a prefill engine calls them when that layer's KV is ready
         (the paper transfers layer by layer, overlapped with the prefill of the following layers).
-        `q_win`, `k_cache`, `v_cache` are the full [L][...] tensors.  With `aux_stream`, select and pack run
+        `q_win`, `k_cache`, `v_cache` are the full [L][...] tensors or sequences of one tensor per layer.  With `aux_stream`, select and pack run
         there behind an event, so the next layer's scoring on `stream` does not wait for them; the caller joins
         with `join_aux` before reading the results on `stream`."""
         if aux_stream is None:

@@ -88,3 +88,20 @@ def test_layer_by_layer_prefill_matches_the_oracle_chain(two_streams):
     pk_o, pv_o = oracle.pack_kv(data["k"], data["v"], cu, sel_o, ck)
     assert np.array_equal(hp.packed_k.cpu().numpy().view(np.uint16), pk_o)
     assert np.array_equal(hp.packed_v.cpu().numpy().view(np.uint16), pv_o)
+
+
+def test_layers_of_a_list_of_caches():
+    """A cache kept as one tensor per layer gives what the [L] tensor gives."""
+    import torch
+    from paper_2607_28150_b200.pipeline import HotPath
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(4)
+    L, Hq, Hkv, d, W, lens = 3, 8, 2, 128, 16, [600, 250]
+    q = torch.randn((L, 2, W, Hq, d), generator=gen, device="cuda", dtype=torch.bfloat16)
+    k, v = (torch.randn((L, sum(lens), Hkv, d), generator=gen, device="cuda", dtype=torch.bfloat16) for _ in range(2))
+    hps = [HotPath(L, Hq, Hkv, d, W, lens, [60, 24]) for _ in range(2)]
+    hps[0].prefill_layerwise(q, k, v)
+    hps[1].prefill_layerwise([x.clone() for x in q], [x.clone() for x in k], [x.clone() for x in v])
+    torch.cuda.synchronize()
+    for name in ("importance", "sel_idx", "packed_k", "packed_v"):
+        assert torch.equal(getattr(hps[0], name), getattr(hps[1], name)), name

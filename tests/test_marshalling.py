@@ -85,3 +85,16 @@ def test_exceptions_of_tensor_accessors_become_python_errors():
             "    for call in %r:\n        try:\n            eval(call)\n        except RuntimeError:\n            print('RuntimeError')\n" % (calls,))
     res = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True)
     assert res.returncode == 0 and res.stdout.split() == ["RuntimeError"] * len(calls), res.stderr[-2000:]
+
+
+@pytest.mark.parametrize("layer", [0, 1, -1])
+def test_a_layer_out_of_a_sequence_of_tensors(layer):
+    e, f, i = ([fake(t, 0), fake(t, 0)] for t in (torch.bfloat16, torch.float32, torch.int32))
+    with pytest.raises(sg.SmartGenError):
+        sg.prefill_layer(SHAPE, layer, e, tuple(e), {layer: e[0]}, f, None, i[0], 4, i, e, e, None, 0)
+    with pytest.raises(IndexError):
+        sg.prefill_layer(SHAPE, 2, e, e, e, f, None, i[0], 4, i, e, e, None, 0)
+    with pytest.raises(TypeError, match="CUDA tensor"):
+        sg.prefill_layer(SHAPE, layer, e, [1, 2], e, f, None, i[0], 4, i, e, e, None, 0)
+    with pytest.raises(TypeError):
+        sg.prefill_layer(SHAPE, layer, e, 17, e, f, None, i[0], 4, i, e, e, None, 0)
