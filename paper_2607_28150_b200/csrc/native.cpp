@@ -130,14 +130,29 @@ struct Args {
     *bytes = t.nbytes();
     return t.data_ptr();
   }
-  // None: the current device's current stream; a torch stream; or a raw handle.
+  // None: the current device's current stream; a torch stream; or a raw handle (an integer or a ctypes pointer, 0 or empty
+  // for the default stream).
   void* stream() {
     if (!ok) return nullptr;
     PyObject* o = a[i++];
     if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
-    PyObject* raw = PyLong_Check(o) ? Py_NewRef(o) : PyObject_GetAttrString(o, "cuda_stream");
-    if (raw == nullptr) { ok = false; return nullptr; }
-    void* p = PyLong_AsVoidPtr(raw);
+    PyObject* raw = Py_NewRef(o);
+    for (const char* name : {"cuda_stream", "value"}) {
+      if (PyLong_Check(raw) || raw == Py_None) break;
+      PyObject* inner = PyObject_GetAttrString(raw, name);
+      if (inner == nullptr) {
+        if (!PyErr_ExceptionMatches(PyExc_AttributeError)) { Py_DECREF(raw); ok = false; return nullptr; }
+        PyErr_Clear();
+        continue;
+      }
+      Py_DECREF(raw);
+      raw = inner;
+    }
+    void* p = nullptr;
+    if (raw != Py_None) {
+      if (PyLong_Check(raw)) p = PyLong_AsVoidPtr(raw);
+      else PyErr_SetString(PyExc_TypeError, "stream must be a stream or a stream handle");
+    }
     Py_DECREF(raw);
     if (p == nullptr && PyErr_Occurred()) ok = false;
     return p;

@@ -1,5 +1,6 @@
 """The argument checks of the hot calls, without a GPU: empty fake tensors claim to be on a CUDA device and reach every check;
 the library refuses their null addresses before it launches anything."""
+import ctypes
 import subprocess
 import sys
 
@@ -85,6 +86,13 @@ def test_exceptions_of_tensor_accessors_become_python_errors():
             "    for call in %r:\n        try:\n            eval(call)\n        except RuntimeError:\n            print('RuntimeError')\n" % (calls,))
     res = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True)
     assert res.returncode == 0 and res.stdout.split() == ["RuntimeError"] * len(calls), res.stderr[-2000:]
+
+
+@pytest.mark.parametrize("stream", [0, ctypes.c_void_p(0), ctypes.c_void_p(None), type("S", (), {"cuda_stream": 0})(), type("S", (), {"cuda_stream": None})()])
+def test_forms_of_a_stream_handle(stream):
+    e = fake(torch.bfloat16, 0)
+    with pytest.raises(sg.SmartGenError):                 # the arguments are taken; the library refuses the null addresses
+        sg.sg_score(SHAPE, e, e, fake(torch.float32, 0), None, None, stream)
 
 
 @pytest.mark.parametrize("layer", [0, 1, -1])
