@@ -34,7 +34,15 @@ if not os.path.exists(LIB_PATH):
                       "`python -m paper_2607_28150_b200.build`; there is no CPU fallback" % LIB_PATH)
 _lib = ctypes.CDLL(LIB_PATH)
 
-from . import _native  # noqa: E402  (needs the library above)
+from .build import native_stamp  # noqa: E402
+
+try:
+    from . import _native  # noqa: E402  (needs the library above)
+    if _native.BUILT_FOR != native_stamp():
+        raise ImportError(_native.BUILT_FOR)
+except ImportError as e:
+    raise ImportError("the marshalling module does not fit this torch or interpreter (%s; running: %s): run `python "
+                      "__graft_entry__.py` or `python -m paper_2607_28150_b200.build`" % (e, native_stamp())) from e
 
 
 class SmartGenError(RuntimeError):

@@ -3,7 +3,7 @@
 Each csrc/*.cu is compiled to an object under build/ (in parallel, skipped when up to date) and
 the objects are linked into paper_2607_28150_b200/libsmartgen.so with the CUDA runtime linked
 statically, so the library loads on a machine without a GPU or a driver.  csrc/native.cpp, the marshalling
-between torch tensors and the library, becomes the extension module _native.so beside it.
+between torch tensors and the library, becomes the extension module _native (with the interpreter's suffix) beside it.
 """
 from __future__ import annotations
 
@@ -21,7 +21,8 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OBJDIR = os.path.join(ROOT, "build", "obj")
 LIB = os.path.join(HERE, "libsmartgen.so")
-NATIVE = os.path.join(HERE, "_native.so")
+EXT_SUFFIX = sysconfig.get_config_var("EXT_SUFFIX")          # names the interpreter
+NATIVE = os.path.join(HERE, "_native" + EXT_SUFFIX)
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -57,18 +58,38 @@ def _compile(src: str, obj: str, verbose: bool) -> None:
         sys.stderr.write(res.stderr)
 
 
-def _build_native(force: bool) -> None:
+def native_stamp() -> str:
+    """What the extension module is compiled against: it reads tensors through inline code of torch's headers, so it fits
+    one version of torch and one interpreter.  The module carries the stamp (BUILT_FOR)."""
+    import torch
+    return "built for torch %s, CUDA %s, C++11 ABI %d, Python %s" % (torch.__version__, torch.version.cuda,
+                                                                    int(torch.compiled_with_cxx11_abi()), EXT_SUFFIX)
+
+
+def native_is_current() -> bool:
     src = os.path.join(CSRC, "native.cpp")
     newest = max(os.path.getmtime(p) for p in (src, os.path.join(INCLUDE, "smartgen.h"), os.path.abspath(__file__)))
-    if not force and os.path.exists(NATIVE) and os.path.getmtime(NATIVE) >= newest:
+    if not os.path.exists(NATIVE) or os.path.getmtime(NATIVE) < newest:
+        return False
+    with open(NATIVE, "rb") as f:
+        return native_stamp().encode() in f.read()
+
+
+def _build_native(force: bool) -> None:
+    plain = os.path.join(HERE, "_native.so")                 # a module without the interpreter's suffix would be imported by any
+    if os.path.exists(plain):
+        os.remove(plain)
+    if not force and native_is_current():
         return
+    src = os.path.join(CSRC, "native.cpp")
     import torch
     inc = os.path.join(os.path.dirname(torch.__file__), "include")
     lib = os.path.join(os.path.dirname(torch.__file__), "lib")
     cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
     tmp = NATIVE + ".tmp.%d" % os.getpid()
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch.compiled_with_cxx11_abi()), "-I", INCLUDE,
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch.compiled_with_cxx11_abi()),
+           "-DSG_BUILT_FOR=\"%s\"" % native_stamp(), "-I", INCLUDE,
            "-isystem", inc, "-isystem", os.path.join(inc, "torch", "csrc", "api", "include"),
            "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(cuda, "include"), src, "-o", tmp,
            "-L", HERE, "-l:libsmartgen.so", "-L", lib, "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda",

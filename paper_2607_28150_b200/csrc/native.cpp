@@ -368,4 +368,11 @@ PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, kMethods, 
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__native() { return PyModule_Create(&kModule); }
+#ifndef SG_BUILT_FOR
+#error "SG_BUILT_FOR: the torch and the interpreter that the module is compiled against (build.py)"
+#endif
+PyMODINIT_FUNC PyInit__native() {
+  PyObject* m = PyModule_Create(&kModule);
+  if (m != nullptr && PyModule_AddStringConstant(m, "BUILT_FOR", SG_BUILT_FOR) != 0) Py_CLEAR(m);
+  return m;
+}

@@ -106,3 +106,14 @@ def test_a_layer_out_of_a_sequence_of_tensors(layer):
         sg.prefill_layer(SHAPE, layer, e, [1, 2], e, f, None, i[0], 4, i, e, e, None, 0)
     with pytest.raises(TypeError):
         sg.prefill_layer(SHAPE, layer, e, 17, e, f, None, i[0], 4, i, e, e, None, 0)
+
+
+def test_module_built_against_another_torch_is_rebuilt_and_not_imported(monkeypatch):
+    from paper_2607_28150_b200 import build
+    assert sg._native.BUILT_FOR == build.native_stamp() and build.native_is_current()
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    assert not build.native_is_current()
+    code = ("import torch\ntorch.__version__ = '0.0.1'\ntry:\n    import paper_2607_28150_b200.binding\n"
+            "except ImportError as e:\n    print(e)\n")
+    res = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True)
+    assert "does not fit this torch" in res.stdout and "torch 0.0.1" in res.stdout, res.stderr[-2000:]
