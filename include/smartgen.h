@@ -315,7 +315,7 @@ sg_status sg_sparse_decode_attn_counted(const sg_shape* shape, const void* q, co
 /*
  * sg_score_static -- sg_score without a workspace argument, for callers that cannot allocate.
  *
- * The paper has no counterpart to this call: it computes exactly what sg_score computes.  It exists
+ * The paper has no counterpart to this call: it computes what sg_score computes.  It exists
  * for hosts of this library that may not call cudaMalloc (or any allocating routine) at the point
  * where they score -- code running under a fixed memory plan, inside a region where allocation is
  * forbidden, or in a process whose allocator belongs to another runtime.  The scratch that pass 1
@@ -323,8 +323,12 @@ sg_status sg_sparse_decode_attn_counted(const sg_shape* shape, const void* q, co
  * SG_SCORE_STATIC_SCRATCH_BYTES long; every GPU that loads the library holds that much memory until
  * the process exits.
  *
- *   - Shapes whose sg_workspace_bytes(SG_OP_SCORE, ...) exceeds SG_SCORE_STATIC_SCRATCH_BYTES are
- *     rejected with SG_ERR_WORKSPACE before anything is launched; use sg_score for those.
+ *   - The array holds 8 * R bytes, R = G*W rounded up to a multiple of 128, for every (layer, KV head,
+ *     sequence) and for every CTA of a launch.  Shapes whose sg_workspace_bytes(SG_OP_SCORE, ...) fits run
+ *     exactly as sg_score runs them.  Of larger ones, those that leave room for at least 32 CTAs run on as many CTAs
+ *     as there is room for: slower, and with the sums over keys cut at other places, so equal to sg_score's to
+ *     rounding and not bit by bit.  All others are rejected with SG_ERR_WORKSPACE before anything is launched; use
+ *     sg_score for those.
  *   - The call allocates nothing and frees nothing.  The first call on each device looks up the
  *     array's device address (one cudaGetSymbolAddress with that device current); make that first
  *     call before starting any stream capture on the device.

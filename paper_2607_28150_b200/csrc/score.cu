@@ -805,7 +805,9 @@ struct ScorePlan {
   bool ok;
 };
 
-// `limit`: the most workspace there is (0 = whatever the plan needs); fewer CTAs need fewer records.
+// `limit`: the most workspace there is (0 = whatever the plan needs).  Fewer CTAs need fewer records, but a call is not squeezed
+// onto fewer than kFewestCtas.
+constexpr int kFewestCtas = 32;
 ScorePlan plan_score(const sg_shape* s, size_t limit = 0) {
   ScorePlan pl{};
   const int D = s->head_dim;
@@ -835,7 +837,7 @@ ScorePlan plan_score(const sg_shape* s, size_t limit = 0) {
   const int64_t record = (int64_t)pl.Ralloc * sizeof(float2), parts = (int64_t)pl.U * s->batch;
   if (limit > 0) {
     const int64_t most = ((int64_t)limit / record - parts) / pl.groups;
-    if (most >= 1 && most < pl.grid) pl.grid = (int)most;
+    if (most >= kFewestCtas && most < pl.grid) pl.grid = (int)most;
   }
   pl.workspace_bytes = (size_t)((parts + (int64_t)pl.groups * pl.grid) * record);
   return pl;

@@ -67,3 +67,29 @@ def test_static_scratch_rejects_shapes_beyond_its_fixed_size():
     # a shape no scoring kernel covers is reported as such, as sg_score reports it (not as a size problem)
     odd = sg.Shape(1, 1, 64, 2, 128, 64, 16384, 16384, 0x1000, 16384 * 256, 256, 128)      # G*W = 2048 rows
     assert sg._lib.sg_score_static(ctypes.byref(odd), fake, fake, fake, None, None) == sg.SG_ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("B,runs", [(252, True), (253, False)])
+def test_static_scratch_runs_on_fewer_ctas_down_to_a_limit(B, runs):
+    """8 KV heads of 512 rows: 2048 records of 4 KB in all, one per part, what is left for the CTAs of a launch (32 and 24)."""
+    import torch
+    import gpu_ops
+    import oracle
+    import paper_2607_28150_b200.binding as sg
+    rng = np.random.default_rng(2)
+    G, Hkv, d, W = 8, 8, 64, 64
+    lens = tuple(int(x) for x in rng.integers(1, 260, B))
+    cu = cu_of(lens)
+    q_h, k_h = rand_bf16(rng, (1, B, W, G * Hkv, d)), rand_bf16(rng, (1, int(cu[-1]), Hkv, d))
+    shp, st = gpu_ops.shape_of(1, G * Hkv, Hkv, d, W, cu), gpu_ops.status_word()
+    assert sg.sg_workspace_bytes(sg.SG_OP_SCORE, shp) > sg.SG_SCORE_STATIC_SCRATCH_BYTES
+    got = torch.full((1, Hkv, int(cu[-1])), -2.0, dtype=torch.float32, device="cuda")
+    if not runs:
+        with pytest.raises(sg.SmartGenError) as e:
+            sg.sg_score_static(shp, gpu_ops.dev(q_h), gpu_ops.dev(k_h), got, st)
+        assert e.value.status == sg.SG_ERR_WORKSPACE
+        return
+    sg.sg_score_static(shp, gpu_ops.dev(q_h), gpu_ops.dev(k_h), got, st)
+    assert gpu_ops.read_status(st) == 0
+    want = oracle.score(q_h, k_h, cu).astype(np.float64)
+    assert np.all(np.abs(got.cpu().numpy().astype(np.float64) - want) <= RTOL * np.abs(want) + ATOL)
