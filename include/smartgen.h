@@ -175,7 +175,8 @@ sg_status sg_select_pack_kv(const sg_shape* shape, const float* importance, cons
  * profiling) do not, nor do ordinary kernels and copies: those have ended when this call's kernel
  * begins, so their outputs -- the projection's q, packed rows, index lists -- may be its inputs directly.
  * Independent calls issued back to back therefore overlap everything but their output stores.
- * sg_sparse_decode_attn_counted makes no such exception: it reads nothing before all earlier work has completed.
+ * sg_sparse_decode_attn_counted with local_skip makes no such exception: it reads nothing before all earlier work has
+ * completed.
  */
 sg_status sg_sparse_decode_attn(const sg_shape* shape, const void* q, const void* packed_k,
                                 const void* packed_v, const int32_t* cu_k, int32_t total_sel,

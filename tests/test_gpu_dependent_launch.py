@@ -105,7 +105,7 @@ def test_pass_2_of_scoring_waits_as_long_as_pass_1_takes():
 
 
 @pytest.mark.parametrize("late", ["packed rows", "queries"])
-def test_counted_attention_waits_for_a_producer_that_lets_it_start_early(late):
+def test_two_lane_attention_waits_for_a_producer_that_lets_it_start_early(late):
     import torch
     import gpu_ops
     import paper_2607_28150_b200.binding as sg
@@ -120,11 +120,11 @@ def test_counted_attention_waits_for_a_producer_that_lets_it_start_early(late):
     cu_cap = torch.arange(B + 1, dtype=torch.int32, device="cuda") * per
     shp = gpu_ops.shape_of(1, heads, heads, d, 1, cu_of((8,) * B))
     count = torch.full((B, heads), per, dtype=torch.int32, device="cuda")
-    none = torch.zeros(B + 1, dtype=torch.int32, device="cuda")
+    none, skip = torch.zeros(B + 1, dtype=torch.int32, device="cuda"), torch.zeros((B, heads), dtype=torch.int32, device="cuda")
     out, want = (torch.zeros((B, heads, d), dtype=torch.int16, device="cuda") for _ in range(2))
 
     def attend(o):
-        sg.sg_sparse_decode_attn_counted(shp, q, packed, packed, cu_cap, B * per, count, None, None, None, none, 0, o)
+        sg.sg_sparse_decode_attn_counted(shp, q, packed, packed, cu_cap, B * per, count, None, None, None, none, 0, o, local_skip=skip)
 
     attend(out)
     torch.cuda.synchronize()
