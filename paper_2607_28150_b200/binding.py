@@ -65,6 +65,8 @@ class Shape(ctypes.Structure):
 
 _vp, _i32, _sz, _f = ctypes.c_void_p, ctypes.c_int32, ctypes.c_size_t, ctypes.c_float
 _sp = ctypes.POINTER(Shape)
+# what is called through ctypes: queries, host arithmetic, the profile calls; and the scoring and attention entry points as a
+# C caller sees them
 _lib.sg_strerror.restype = ctypes.c_char_p
 _lib.sg_strerror.argtypes = [ctypes.c_int]
 _lib.sg_last_cuda_error.restype = ctypes.c_int
@@ -74,10 +76,6 @@ _lib.sg_score.restype = ctypes.c_int
 _lib.sg_score.argtypes = [_sp, _vp, _vp, _vp, _vp, _sz, _vp, _vp]
 _lib.sg_score_static.restype = ctypes.c_int
 _lib.sg_score_static.argtypes = [_sp, _vp, _vp, _vp, _vp, _vp]
-_lib.sg_select_topk.restype = ctypes.c_int
-_lib.sg_select_topk.argtypes = [_sp, _vp, _vp, _i32, _vp, _vp, _sz, _vp, _vp]
-_lib.sg_pack_kv.restype = ctypes.c_int
-_lib.sg_pack_kv.argtypes = [_sp, _vp, _vp, _vp, _vp, _i32, _vp, _vp, _vp, _vp]
 _lib.sg_profile_accumulate.restype = ctypes.c_int
 _lib.sg_profile_accumulate.argtypes = [_sp, _vp, _vp, _i32, _vp, _vp, _vp]
 _lib.sg_block_importance.restype = ctypes.c_int
@@ -88,18 +86,6 @@ _lib.sg_speculative_delivered.restype = ctypes.c_int64
 _lib.sg_speculative_delivered.argtypes = [_i32, _i32, ctypes.c_int64, ctypes.c_double, _i32]
 _lib.sg_proactive_mask.restype = ctypes.c_int
 _lib.sg_proactive_mask.argtypes = [_sp, _i32, _i32, _vp, _i32, _vp, _vp]
-_lib.sg_select_pack_kv.restype = ctypes.c_int
-_lib.sg_select_pack_kv.argtypes = [_sp, _vp, _vp, _i32, _vp, _vp, _vp, _vp, _vp, _vp, _vp]
-_lib.sg_pack_kv_counted.restype = ctypes.c_int
-_lib.sg_pack_kv_counted.argtypes = [_sp, _vp, _vp, _vp, _vp, _i32, _vp, _vp, _vp, _vp, _vp]
-_lib.sg_sparse_decode_attn_counted.restype = ctypes.c_int
-_lib.sg_sparse_decode_attn_counted.argtypes = [_sp, _vp, _vp, _vp, _vp, _i32, _vp, _vp, _vp, _vp, _vp, _i32, _vp, _f, _vp, _vp, _vp, _vp]
-_lib.sg_select_threshold.restype = ctypes.c_int
-_lib.sg_select_threshold.argtypes = [_sp, _vp, _f, _vp, _i32, _vp, _vp, _vp, _vp]
-_lib.sg_push_blocks.restype = ctypes.c_int
-_lib.sg_push_blocks.argtypes = [_sp, _i32, _i32, _vp, _i32, _vp, _vp, _vp, _vp, _vp, _vp]
-_lib.sg_split_index.restype = ctypes.c_int
-_lib.sg_split_index.argtypes = [_sp, _vp, _vp, _i32, _vp, _i32, _vp, _vp, _vp, _vp, _vp, _vp, _vp]
 _lib.sg_sparse_decode_attn.restype = ctypes.c_int
 _lib.sg_sparse_decode_attn.argtypes = [_sp, _vp, _vp, _vp, _vp, _i32, _vp, _vp, _vp, _vp, _i32, _f, _vp, _vp, _vp,
                                        _sz, _vp, _vp]
@@ -116,7 +102,7 @@ _lib.sg_testing_score_grid.argtypes = [_sp]
 
 
 def sg_testing_score_fault(withhold_unit: int = -1, wait_limit_ms: int = 0) -> None:
-    """Test hook: withhold the done-count of one scoring unit and/or shorten every bounded wait (0 / -1 = off)."""
+    """Test hook: withhold the row statistics of one scoring unit and/or shorten every bounded wait (0 / -1 = off)."""
     _lib.sg_testing_score_fault(withhold_unit, wait_limit_ms)
 
 
@@ -163,9 +149,6 @@ def _check(t: Optional[torch.Tensor], dtype, name: str, allow_none: bool = False
         raise TypeError("%s: expected dtype %s, got %s" % (name, dtypes, t.dtype))
     if not t.is_contiguous():
         raise ValueError("%s must be contiguous (strided caches go through the sg_shape strides)" % name)
-
-
-_BF16 = (torch.bfloat16, torch.int16, torch.uint16)
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:

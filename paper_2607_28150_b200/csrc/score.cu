@@ -73,13 +73,12 @@ constexpr int kClockWords = 4;
 struct ScoreParams {
   const int32_t* cu;
   float* importance;
-  float2* records;         // [parts of the group + CTAs][Ralloc] row statistics (log2-domain reference, sum of exp2) of a segment
+  float2* records;         // [parts + CTAs][Ralloc] row statistics (log2-domain reference, sum of exp2) of a segment
   int32_t* dev_status;
   int64_t T;
   int32_t B, Hkv, G, W, R, Ralloc;
-  int32_t u0, units;       // the launch's (layer, KV head) units
+  int32_t units;           // (layer, KV head) units of the call
   int32_t k_stages, q_bufs;
-  int32_t more;            // another launch of the same call follows
   int32_t smem_bytes;      // dynamic shared memory of the launch (debug checks)
   int32_t withhold_unit;   // testing only: the statistics of this unit's segments are never handed to the helpers (-1 = none)
   uint32_t wait_ns;        // limit of every bounded wait, nanoseconds
@@ -191,17 +190,16 @@ __device__ __forceinline__ int cta_of(long long pos, long long tt, int busy) { r
 // A CTA's segments: its range of the launch's key tiles [c * tt / busy, (c + 1) * tt / busy), cut at part boundaries.  Pass 2
 // walks the range backwards, segments and tiles: what pass 1 read last is still in L2.
 struct Segment {
-  int u, b;                // unit (counted over the whole call) and sequence
+  int u, b;                // unit and sequence
   int c0, N;               // first token and length of sequence b
   int tile_beg, tile_end;  // tiles of the part
-  int part;                // part within the launch
+  int part;
 };
 template <int PASS>
 struct SegmentWalk {
-  int C, B, u0, pos, end;
+  int C, B, pos, end;
   const int *cu, *prefix;  // prefix[b] = tiles of the sequences before b (prefix[B] = C)
-  __device__ __forceinline__ SegmentWalk(int C_, int units, int B_, int u0_, const int* cu_, const int* prefix_)
-      : C(C_), B(B_), u0(u0_), cu(cu_), prefix(prefix_) {
+  __device__ __forceinline__ SegmentWalk(int C_, int units, int B_, const int* cu_, const int* prefix_) : C(C_), B(B_), cu(cu_), prefix(prefix_) {
     const long long tt = (long long)units * C;
     const int g = busy_ctas(tt);
     pos = (int)blockIdx.x < g ? (int)(tt * blockIdx.x / g) : 0;
@@ -210,20 +208,20 @@ struct SegmentWalk {
   __device__ __forceinline__ bool next(Segment& s) {
     if (pos >= end) return false;
     const int at = PASS == 1 ? pos : end - 1;         // a tile of the segment
-    const int ul = at / C, j = at - ul * C;
+    const int u = at / C, j = at - u * C;
     int lo = 0, hi = B;
     while (hi - lo > 1) {
       const int mid = (lo + hi) >> 1;
       if (prefix[mid] <= j) lo = mid; else hi = mid;
     }
-    s.u = u0 + ul;
+    s.u = u;
     s.b = lo;
     s.c0 = cu[lo];
     s.N = cu[lo + 1] - s.c0;
     const int tile = j - prefix[lo];
     s.tile_beg = PASS == 1 ? tile : max(0, tile - (at - pos));
     s.tile_end = PASS == 1 ? min(prefix[lo + 1] - prefix[lo], tile + (end - pos)) : tile + 1;
-    s.part = ul * B + lo;
+    s.part = u * B + lo;
     if (PASS == 1) pos += s.tile_end - s.tile_beg; else end -= s.tile_end - s.tile_beg;
     return true;
   }
@@ -236,7 +234,7 @@ __device__ __forceinline__ int tile_at(const Segment& s, int i) { return PASS ==
 // the epilogue of pass 2 adds them; rows outside the window get -inf: exp2(x - inf) = 0.
 template <int kFlight, int kRows>
 __device__ __forceinline__ void merge_records(const ScoreParams& p, const Segment& sg, const int* prefix, int C, float* neg_lse, int r0, int step) {
-  const long long tt = (long long)p.units * C, first = (long long)(sg.u - p.u0) * C + prefix[sg.b];
+  const long long tt = (long long)p.units * C, first = (long long)sg.u * C + prefix[sg.b];
   const int busy = busy_ctas(tt), Weff = min(p.W, sg.N);
   const int c_lo = cta_of(first, tt, busy), nrec = cta_of(first + (prefix[sg.b + 1] - prefix[sg.b]) - 1, tt, busy) - c_lo + 1;
   constexpr int kRecs = 4;
@@ -400,9 +398,11 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
   // lets pass 2 be set up: pass 2 loads queries, keys and offsets without a wait of its own, so everything ahead of the call
   // has to be complete and visible by then, also behind a kernel that starts its dependents early.  (Pass 2 does wait
   // for all of pass 1 before it reads or overwrites anything that a launch wrote.)
-  if (PASS == 1) pdl_wait();
-  if (p.more) pdl_launch_dependents();
-  SegmentWalk<PASS> walk(C, p.units, p.B, p.u0, s_cu, s_prefix);
+  if (PASS == 1) {
+    pdl_wait();
+    pdl_launch_dependents();
+  }
+  SegmentWalk<PASS> walk(C, p.units, p.B, s_cu, s_prefix);
   Segment sg;
   // In pass 2 loads and MMAs run ahead while the epilogue waits for pass 1: what their limits count starts behind pass 1.
   constexpr bool kBehind = PASS == 1;
@@ -699,7 +699,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
   } else {
     // ------------------------------------------------------------ helper warps
     const int hw = warp - kHelperWarp;
-    // Everything below touches what an earlier launch of this call wrote or reads: wait until that has completed.
+    // Everything below touches what the launch before this one wrote or reads: wait until that has completed.
     pdl_wait();
     bool ok = true;
     if (PASS == 1) {
@@ -800,7 +800,7 @@ std::atomic<int> g_test_wait_limit_ms{0};
 std::atomic<unsigned long long*> g_test_clock_out{nullptr};
 
 struct ScorePlan {
-  int R, Ralloc, k_stages, q_bufs, smem_bytes, U, group, groups, grid;
+  int R, Ralloc, k_stages, q_bufs, smem_bytes, U, grid;
   size_t workspace_bytes;
   bool ok;
 };
@@ -829,17 +829,15 @@ ScorePlan plan_score(const sg_shape* s, size_t limit = 0) {
   pl.smem_bytes = 1024 + pl.q_bufs * q_bytes + pl.k_stages * k_stage + tail;
   if (pl.smem_bytes < 120 * 1024) pl.smem_bytes = 120 * 1024;     // one CTA per SM: each CTA takes the whole TMEM
   pl.U = s->num_layers * s->num_kv_heads;
-  pl.groups = 1;
-  pl.group = pl.U;
-  const int64_t tiles = (int64_t)pl.group * ((int64_t)s->total_tokens / kTileKeys + s->batch);      // upper bound
+  const int64_t tiles = (int64_t)pl.U * ((int64_t)s->total_tokens / kTileKeys + s->batch);      // upper bound
   pl.grid = (int)(tiles < kNumSMs ? tiles : kNumSMs);
-  // records: a CTA adds at most one segment to the parts of a group
+  // records: a CTA adds at most one segment to the parts
   const int64_t record = (int64_t)pl.Ralloc * sizeof(float2), parts = (int64_t)pl.U * s->batch;
   if (limit > 0) {
-    const int64_t most = ((int64_t)limit / record - parts) / pl.groups;
+    const int64_t most = (int64_t)limit / record - parts;
     if (most >= kFewestCtas && most < pl.grid) pl.grid = (int)most;
   }
-  pl.workspace_bytes = (size_t)((parts + (int64_t)pl.groups * pl.grid) * record);
+  pl.workspace_bytes = (size_t)((parts + pl.grid) * record);
   return pl;
 }
 
@@ -955,19 +953,11 @@ sg_status run_score(const sg_shape* shape, const void* q_win, const void* k_cach
   p.scale_log2 = kLog2e / sqrtf((float)D);
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const size_t buffer = (size_t)(pl.group * shape->batch + pl.grid) * pl.Ralloc;      // a group's records
-  for (int u = 0, i = 0; u < pl.U; u += pl.group, ++i) {
-    p.u0 = u;
-    p.units = pl.U - u < pl.group ? pl.U - u : pl.group;
-    p.records = static_cast<float2*>(workspace) + i * buffer;
-    p.more = 1;
-    st = D == 128 ? launch_pass<128, 1>(tmap_q, tmap_k, p, pl, s) : launch_pass<64, 1>(tmap_q, tmap_k, p, pl, s);
-    if (st != SG_OK) return st;
-    p.more = u + pl.group < pl.U;
-    st = D == 128 ? launch_pass<128, 2>(tmap_q, tmap_k, p, pl, s) : launch_pass<64, 2>(tmap_q, tmap_k, p, pl, s);
-    if (st != SG_OK) return st;
-  }
-  return SG_OK;
+  p.units = pl.U;
+  p.records = static_cast<float2*>(workspace);
+  st = D == 128 ? launch_pass<128, 1>(tmap_q, tmap_k, p, pl, s) : launch_pass<64, 1>(tmap_q, tmap_k, p, pl, s);
+  if (st != SG_OK) return st;
+  return D == 128 ? launch_pass<128, 2>(tmap_q, tmap_k, p, pl, s) : launch_pass<64, 2>(tmap_q, tmap_k, p, pl, s);
 }
 
 }  // namespace
