@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(kDecWarps * 32, (kN == 1 && kSlots * D <= 384 
     return (li < ntok && li >= kbe) ? idx_base[at] : 0;
   };
   // A warp is alone on its scheduler or shares it with a few others, and its instructions issue one by one: what a slice takes
-  // is its instruction count (2500 clocks for 600 of them).  So the copies' addresses are built from per-lane constants and
+  // is its instruction count (a first form with 600 of them took 2500 clocks, this one has about 200).  So the copies' addresses are built from per-lane constants and
   // immediate offsets, with one multiplication per gathered row; what does not occur in the bulk of a list (the slice where
   // packed rows end, the last slice, bad indices, very large strides) goes through a loop.
   constexpr int kRowsPerCopy = 32 / kChunksPerRow;
@@ -518,16 +518,26 @@ constexpr int decode_smem_bytes(int D, int warps, int slots, bool cluster) {
 //  * more pairs: one CTA each; eight warps once a list has 1024 entries (24 sequences of 1600: 30.2 us alone against 32.8 with
 //    four), else four, whose merge is half as wide (64 sequences of 200: 9.8 against 11.3 us).
 // Rings of three slots, two CTAs per SM and so two calls overlapped, are faster wherever rows are gathered (14 sequences of 1600
-// entries, half of them gathered, 12 layers: 186 us against 199 with six slots) and for short lists.  Long lists that are all
-// packed stream at HBM rate, and at most two calls are in flight: six slots then keep more bytes under way (14 x 1600: 176
-// against 182 us, 32 x 3200: 696 against 721; 14 x 800: 104 against 103).  With more than eight query rows per KV head the
-// registers allow one 8-warp CTA per SM anyway: six slots.
+// entries, half of them gathered, 12 layers: 186 us against 199 with six slots) and for short lists.  Lists that are all
+// packed stream at HBM rate once every warp has six slices or more; six slots then keep more bytes under way (a call behind an
+// unrelated kernel / calls in sequence, three slots -> six: 14 sequences of 820 entries 11.3 -> 10.5 / 7.2 -> 7.0 us, 8 of 1640
+// 12.6 -> 11.8 / 8.3 -> 8.1, 14 of 4096 38.4 -> 37.7 / 32.2 -> 32.1; with five slices per warp 10 of 600 8.35 -> 8.18 / 4.0 -> 4.4).
+// Clusters have to fill three quarters of the SMs for that (96 CTAs of 6 x 4096 entries: 20.1 -> 19.4 / 13.5 -> 14.1).
+// With more pairs than SMs six slots at d = 128 mean one CTA per SM, and up to one and a half CTAs per SM that is a second wave
+// nearly empty: there four warps and three slots, all CTAs resident at once (19 sequences of 1640 entries 29.8 -> 25.5 / 18.3 ->
+// 15.5 us, 24 of 4096 66.4 -> 62.6 / 54.5 -> 53.7; equal at 28 sequences; at d = 64 two six-slot CTAs fit and stay ahead: 19
+// of 1640 14.7 against 17.0).  With more than eight query rows per KV head the registers allow one 8-warp CTA per SM
+// anyway: six slots.
+// A two-lane call names one row of the KV index as its packed and as its indexed list, so avg_tokens is up to twice what it
+// attends.  Planned for the row's length, the chain of split, pack and attention is slower more often than faster
+// (19 sequences of 820 entries 30.2 -> 32.7 us, 1 of 820 11.8 -> 12.3, 64 of 820 87.9 -> 83.4): it stays.
 void decode_plan(const sg_shape* shape, int32_t total_sel, int32_t total_loc, int* csize, int* warps, int* slots) {
   const int64_t pairs = (int64_t)shape->batch * shape->num_kv_heads;
   const int64_t avg_tokens = ((int64_t)total_sel + total_loc) / shape->batch;
+  const bool packed_only = total_loc == 0;
   int W = 8, cs = 1;
   if (pairs > kNumSMs) {
-    W = avg_tokens >= 1024 ? 8 : 4;
+    W = avg_tokens < 1024 || (packed_only && shape->head_dim == 128 && 2 * pairs <= 3 * kNumSMs) ? 4 : 8;
   } else if (avg_tokens > (pairs >= 64 ? 14 : 8) * kSlice) {   // else a slice or two per warp of one CTA already: no cluster to merge
     int fit = 1;
     while (fit < 8 && pairs * fit * 2 <= kNumSMs) fit *= 2;
@@ -539,7 +549,7 @@ void decode_plan(const sg_shape* shape, int32_t total_sel, int32_t total_loc, in
   }
   *csize = cs;
   *warps = W;
-  const bool streams = total_loc == 0 && avg_tokens >= 1024 && 2 * pairs > kNumSMs;
+  const bool streams = packed_only && W == 8 && avg_tokens >= 6 * kSlice * W * cs && (cs == 1 ? 2 * pairs > kNumSMs : 4 * pairs * cs > 3 * kNumSMs);
   *slots = shape->num_q_heads / shape->num_kv_heads > 8 || streams ? 6 : 3;
 }
 

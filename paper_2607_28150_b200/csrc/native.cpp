@@ -339,7 +339,7 @@ SG_FN(prefill) {
     return rc ? rc + 256 : 0;
   });
 }
-// sg_score, sg_select_topk, sg_pack_kv of one layer of tensors that hold all of them (shape: one layer).
+// sg_score, then sg_select_pack_kv, of one layer of tensors that hold all of them (shape: one layer).
 SG_FN(prefill_layer) {
   Args x(a, n, 14);
   const sg_shape* s = x.shape();

@@ -116,13 +116,13 @@ def test_push_by_list(lens, Hkv, d, M, n_sel, head_major):
 
 
 @pytest.mark.parametrize("lens,L,W,Hq,Hkv,d", [
-    ((33000,), 1, 4, 8, 8, 128),                           # 67.6 MB of keys: groups of several KV heads of one layer
-    ((20000, 3, 14001), 2, 16, 16, 8, 128),                # ragged, 16 units, the last group smaller
-    ((130000,), 2, 8, 4, 4, 64),                           # long rows of 64-element heads
+    ((33000,), 1, 4, 8, 8, 128),                           # 67.6 MB of keys, one layer: every KV head is cut over many CTAs
+    ((20000, 3, 14001), 2, 16, 16, 8, 128),                # ragged, 139 MB of keys, a part of three keys between long ones
+    ((130000,), 2, 8, 4, 4, 64),                           # 133 MB of keys, long rows of 64-element heads
 ])
 def test_score_keys_beyond_l2(lens, L, W, Hq, Hkv, d):
-    """Calls whose keys exceed L2 and whose CTAs' ranges cross many parts; the call is repeated on the same workspace,
-    whose words then hold the first call's records."""
+    """Calls with half of L2 to more than all of it in keys; the call is repeated on the same workspace, whose words then
+    hold the first call's records."""
     import torch
     import gpu_ops
     import paper_2607_28150_b200.binding as sg
@@ -154,6 +154,10 @@ RING_KS = (0, 1, 15, 16, 127, 129, 256, 383, 511, 640, 769, 1023)
     (tuple(4 * k for k in RING_KS), (0,) * 12, 32, 8, 128), # packed rows only, 1024 and more on average: rings of six
     (tuple(4 * k for k in RING_KS), (0,) * 12, 16, 8, 64),
     ((1500,) * 20, RING_KS[:10] * 2, 32, 8, 128),                 # the same, long ones: eight warps
+    ((767,) * 10 + (770,), (0,) * 11, 32, 8, 128), ((769,) * 11, (0,) * 11, 32, 8, 128),   # packed only, to either side of six slices per warp
+    ((1535,) * 8, (0,) * 8, 32, 8, 128), ((1537,) * 8, (0,) * 8, 32, 8, 128),     # the same for clusters of two
+    ((1100,) * 19, (0,) * 19, 32, 8, 128), ((1023,) * 19, (0,) * 19, 32, 8, 128),  # packed only, up to one and a half CTAs per SM
+    ((1100,) * 28, (0,) * 28, 32, 8, 128), ((1100,) * 19, (0,) * 19, 32, 8, 64),   # ... and what keeps eight warps
 ])
 def test_decode_rings(ks, nls, Hq, Hkv, d):
     """Against the oracle on inputs where one dropped or misplaced row shows (tolerances: see test_gpu_decode_sentinel)."""

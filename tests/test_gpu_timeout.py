@@ -1,7 +1,7 @@
 """GPU: a bounded device-side wait of the scoring kernel is made to run out, on purpose and harmlessly.
 
-The test withholds the done-count of one (layer, KV head) unit through the library's testing hook and shortens every
-wait to 10 ms.  The pass-2 work items of that unit then wait for a count that never comes; the wait gives up, the CTA
+The test withholds the row statistics of one (layer, KV head) unit through the library's testing hook and shortens every
+wait to 10 ms.  The warps of pass 1 that publish them then wait for statistics that never come; the wait gives up, the CTA
 sets SG_ERR_TIMEOUT in the status word, waits (bounded) for its own copies and MMAs, frees its tensor memory and
 returns.  Nothing traps, nothing spins without a limit, and the context stays usable: an ordinary sg_score call right
 afterwards matches the oracle.
