@@ -5,17 +5,12 @@
 // the row by class -- remote first, then local, then padding -- with ballots and prefix counts: no atomics, so
 // the output order is a pure function of the input.  The partitioned row (when asked for) and the local and
 // remote index lists with their counts are written.  Integer work only, bound by latency (a row is a few KB): two
-// dependent loads per entry, index then mask.  So every thread has eight entries in flight, and a row of up to 8192
-// entries is looked up once and stays in registers between the counting and the placing; 256 threads that took one
-// entry at a time, twice, needed 10.9 us for 64 rows of up to 3277 entries, this 5.5 us.
+// dependent loads per entry, index then mask.  So every thread has several entries in flight, and a row that they cover is
+// looked up once and stays in registers between the counting and the placing.
 #include "common.cuh"
 
 namespace sg {
 namespace {
-
-constexpr int kSplitThreads = 1024;
-constexpr int kSplitWarps = kSplitThreads / 32;
-constexpr int kFlight = 8;                         // entries in flight per thread
 
 struct SplitParams {
   const int32_t* kv_index;
@@ -31,7 +26,10 @@ struct SplitParams {
   int32_t K_tot, B, Hkv, reorder;
 };
 
+// kFlight: entries in flight per thread.
+template <int kSplitThreads, int kFlight>
 __global__ void __launch_bounds__(kSplitThreads) split_index_kernel(const SplitParams p) {
+  constexpr int kSplitWarps = kSplitThreads / 32;
   __shared__ uint32_t w_cnt[3][kSplitWarps];     // per-warp counts of classes remote / local / padding
   __shared__ uint32_t w_base[3][kSplitWarps];
   __shared__ uint32_t tot[3];
@@ -70,14 +68,14 @@ __global__ void __launch_bounds__(kSplitThreads) split_index_kernel(const SplitP
   if (lane == 0) { w_cnt[0][warp] = cnt[0]; w_cnt[1][warp] = cnt[1]; w_cnt[2][warp] = cnt[2]; }
   __syncthreads();
   if (warp < 3) {
-    const uint32_t v = w_cnt[warp][lane];
+    const uint32_t v = lane < kSplitWarps ? w_cnt[warp][lane] : 0u;
     uint32_t inc = v;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
       const uint32_t u = __shfl_up_sync(0xffffffffu, inc, off);
       if (lane >= off) inc += u;
     }
-    w_base[warp][lane] = inc - v;
+    if (lane < kSplitWarps) w_base[warp][lane] = inc - v;
     if (lane == 31) tot[warp] = inc;
   }
   __syncthreads();
@@ -140,5 +138,19 @@ extern "C" sg_status sg_split_index(const sg_shape* shape, const int32_t* kv_ind
   p.B = shape->batch;
   p.Hkv = shape->num_kv_heads;
   p.reorder = reorder ? 1 : 0;
-  return launch_chained(split_index_kernel, dim3((unsigned)rows), kSplitThreads, p, stream);
+  // The CTA size is chosen for a row of the longest sequence, if the budgets are shares of the lengths (any row is split
+  // correctly): four entries per thread hold the row in registers, two for the shortest rows, eight up to 8192 entries; longer
+  // rows are looked up twice in flights of four.  More threads or entries than the row needs are idle steps in every ballot
+  // loop, and fewer CTAs are resident.  Microseconds (1024 threads with eight entries each for every row -> these rules; 256
+  // threads, one entry at a time): 320 rows of 128 entries 7.8 -> 2.2 (3.0), 320 of 820 12.4 -> 3.7 (5.6), 64 of 2000 5.2 -> 3.3
+  // (7.7), 64 of 3277 5.3 -> 4.1 (11.2), 64 of 6000 6.3 (20.7; four entries per thread 7.5), 64 of 16000 14.8 -> 14.3 (51.7).
+  const int64_t average = total_sel / shape->batch;
+  const int64_t scaled = shape->total_tokens > 0 ? (int64_t)total_sel * shape->max_seqlen / shape->total_tokens : 0;
+  const int64_t longest = scaled > average ? scaled : average;
+  const dim3 grid((unsigned)rows);
+  if (longest <= 256) return launch_chained(split_index_kernel<128, 2>, grid, 128, p, stream);
+  if (longest <= 1024) return launch_chained(split_index_kernel<256, 4>, grid, 256, p, stream);
+  if (longest <= 2048) return launch_chained(split_index_kernel<512, 4>, grid, 512, p, stream);
+  if (longest > 4096 && longest <= 8192) return launch_chained(split_index_kernel<1024, 8>, grid, 1024, p, stream);
+  return launch_chained(split_index_kernel<1024, 4>, grid, 1024, p, stream);
 }

@@ -79,6 +79,21 @@ def test_split_at_the_cuts(ks):
             assert np.array_equal(a, b)
 
 
+@pytest.mark.parametrize("lens,ks", [
+    ((300,), (256,)), ((300,), (257,)), ((1100,), (1024,)), ((1100,), (1025,)), ((2500,), (2048,)), ((2500,), (2049,)),   # ends of the CTA sizes
+    ((5000,), (4096,)), ((5000,), (4097,)),
+    ((1300, 40, 1), (1024, 0, 1)), ((3000,) + (100,) * 60, (2900,) + (0,) * 60),      # a row longer than the CTA was chosen for
+    ((700,) * 30, (90,) * 30),
+])
+def test_split_cta_sizes(lens, ks):
+    from test_gpu_split import make, run_gpu
+    idx, mask, cu, ck = make(17, lens, ks, 3, (0.1, 0.5, 0.4))
+    for reorder in (True, False):
+        want = oracle.split_index(idx, mask, cu, ck, reorder=reorder)
+        for a, b in zip(run_gpu(idx, mask, cu, ck, reorder), want):
+            assert np.array_equal(a, b)
+
+
 @pytest.mark.parametrize("n", [5, 4093, 4096, 8189, 8190, 8192, 16383, 16384, 32765, 32768])
 def test_select_rows_off_the_16_byte_boundary(n):
     """Rows that start 0 to 3 values behind a 16-byte boundary, up to the longest of every kernel variant; values from
