@@ -288,7 +288,21 @@ __device__ __forceinline__ void merge_records(const ScoreParams& p, const Segmen
   }
 }
 
-template <int D, int PASS>
+// Pass 2, several row blocks per tile: a helper warp merges a later segment's records one segment ahead, hidden behind the
+// segment before it if that is long enough.  Round trips to L2 per lane that takes, each about as long as a block of the epilogue:
+__host__ __device__ __forceinline__ int helper_trips(int Ralloc, int nrec) {
+  return nrec <= 4 ? Ralloc >> 7 : (Ralloc >> 5) * ((nrec + 23) / 24);
+}
+// A part over many CTAs behind a short segment is not hidden (two layers of one KV head, 1024 query rows, sequences of 30000, 10
+// and 200 keys: 74 records of 1024 rows merged by one warp while a CTA's epilogue stood, 158 us; 82 with this rule, 107
+// before the helpers merged at all): then the epilogue warps merge the records themselves.  `per` = key tiles per CTA.
+__device__ __forceinline__ bool epilogue_merges(const ScoreParams& p, int part_tiles, int per, int blocks_before) {
+  const int nrec = part_tiles / per + 1;
+  return helper_trips(p.Ralloc, nrec) > blocks_before + (p.Ralloc + 32 * kEpiWarps - 1) / (32 * kEpiWarps) * ((nrec + 11) / 12);
+}
+
+// kOwn (pass 2): the epilogue warps may merge later segments, too (plan_score says when).
+template <int D, int PASS, bool kOwn>
 __global__ void __launch_bounds__(kThreads, 1)
 score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k, const ScoreParams p) {
   constexpr int kSub = D / 64;                        // 64-element (128-byte) sub-tiles along d
@@ -303,6 +317,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
   uint64_t* bars = reinterpret_cast<uint64_t*>(k_smem + p.k_stages * kKStageBytes);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 38);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  int* const s_per = reinterpret_cast<int*>(bars + 39);              // key tiles per CTA (kOwn)
   float* table = reinterpret_cast<float*>(bars + 40);
   // pass 1: [2 buffers][kGroups]{m[Ralloc], l[Ralloc]} running statistics of a segment
   // pass 2: [2 buffers][Ralloc] negated log-sum-exps, [kColSlots][kGroups][128] partial column sums
@@ -325,7 +340,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
   auto bar_cols_full = [&](uint32_t s) { return bar0 + 8u * (24 + s); };   // epilogue -> helper: partial column sums of a tile complete
   auto bar_cols_free = [&](uint32_t s) { return bar0 + 8u * (28 + s); };
   const uint32_t bar_drain = bar0 + 8u * 32u;
-  const uint32_t bar_first = bar0 + 8u * 33u;          // pass 2: the epilogue warps' own merge of the first segment's log-sum-exps
+  const uint32_t bar_own = bar0 + 8u * 33u;            // pass 2: the epilogue warps' own merge of a segment's log-sum-exps
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   unsigned long long clk0 = 0, gt0 = 0;
@@ -343,7 +358,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
     for (int s = 0; s < kStages; ++s) { mbar_init(bar_afull(s), 1); mbar_init(bar_aempty(s), 4); }
     for (int s = 0; s < kColSlots; ++s) { mbar_init(bar_cols_full(s), 4 * min(nblk, kGroups)); mbar_init(bar_cols_free(s), 1); }
     mbar_init(bar_drain, 1);
-    mbar_init(bar_first, kEpiWarps);
+    mbar_init(bar_own, kEpiWarps);
     *abort_flag = 0;
     fence_barrier_init();
     fence_proxy_async();
@@ -376,6 +391,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
       acc += __shfl_sync(0xffffffffu, inc, 31);
     }
     if (lane == 0) s_prefix[0] = 0;
+    if (kOwn && lane == 0) *s_per = max(1, (int)((long long)p.units * acc / gridDim.x));
   }
   if (p.R < p.Ralloc) {
     // Rows R..Ralloc-1 of the Q operands are never written by TMA: zero them once so that padded MMA
@@ -514,6 +530,8 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
     const uint64_t scale2 = pack2(p.scale_log2, p.scale_log2);
     uint32_t n0 = 0;                                   // blocks of the CTA before this segment
     int tiles0 = 0;                                    // tiles of the CTA before this segment
+    int blocks_before = 0;                             // blocks of the segment before this one
+    uint32_t merges = 0;                               // pass 2: parities of the helper's merges (bit per buffer) and of these warps' (bit 2)
     bool ok = true;
     auto release = [&](uint32_t st) {
       tc_fence_before();
@@ -616,17 +634,23 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
         __syncwarp();
         if (lane == 0 && ok && sg.u != p.withhold_unit) mbar_arrive(bar_tab_full(buf));
       } else {
-        if (sidx == 0) {
-          // The first segment's log-sum-exps are what the whole CTA waits for: all epilogue threads merge its records.
-          pdl_wait();
-          merge_records<12, 1>(p, sg, s_prefix, C, neg_lse, tid, 32 * kEpiWarps);
+        if (sidx == 0 || (kOwn && epilogue_merges(p, s_prefix[sg.b + 1] - s_prefix[sg.b], *s_per, blocks_before))) {
+          // The first segment's log-sum-exps, and those of a part that the helper would be late with, are what the whole
+          // CTA waits for: all epilogue threads merge its records.
+          if (sidx == 0) pdl_wait();
+          else if (kOwn && use > 0) ok = wait(bar_tab_free(buf), (use - 1u) & 1u);
+          if (!ok) break;
+          merge_records<12, 1>(p, sg, s_prefix, C, kOwn ? neg_lse + buf * p.Ralloc : neg_lse, tid, 32 * kEpiWarps);
           __syncwarp();
-          if (lane == 0) mbar_arrive(bar_first);
-          ok = wait(bar_first, 0u);
+          if (lane == 0) mbar_arrive(bar_own);
+          ok = wait(bar_own, kOwn ? merges >> 2 : 0u);
+          merges ^= 4u;
         } else {
           // A helper has merged the part's records one segment ahead.  Every warp waits here, also one that gets no block of
           // the segment: that keeps the arrivals below in step with the barrier's phases.
-          SG_PROF_WAIT(w1, ok = wait(bar_tab_full(buf), buf == 0u ? (use - 1u) & 1u : use & 1u));
+          const uint32_t phase = kOwn ? (merges >> buf) & 1u : buf == 0u ? (use - 1u) & 1u : use & 1u;
+          SG_PROF_WAIT(w1, ok = wait(bar_tab_full(buf), phase));
+          merges ^= 1u << buf;
         }
         if (!ok) break;
         const float* nl = neg_lse + buf * p.Ralloc;
@@ -692,6 +716,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
         __syncwarp();
         if (lane == 0 && ok) mbar_arrive(bar_tab_free(buf));
       }
+      blocks_before = (int)(n_end - n0);
       n0 = n_end;
       tiles0 += sg.tile_end - sg.tile_beg;
     }
@@ -727,11 +752,15 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
       // each, when there are no column sums to add up; 24 records in flight: the CTAs at the part boundaries of a one-layer
       // call have a segment or two of a tile each, and parts of twenty records (8192 keys:
       // 28.8 -> 26.6 us for the whole call; one helper, 16 in flight, took eight L2 round trips per segment).
+      int blocks_before = 0;
       for (int sidx = 0; ok && walk.next(sg); ++sidx) {
+        const int blocks = (sg.tile_end - sg.tile_beg) * nblk, before = blocks_before;
+        blocks_before = blocks;
         if (sidx == 0) continue;
         const uint32_t buf = (uint32_t)sidx & 1u, use = (uint32_t)sidx >> 1;
-        if (use > 0) ok = wait(bar_tab_free(buf), (use - 1u) & 1u);
+        if (use > 0) ok = wait(bar_tab_free(buf), (use - 1u) & 1u);        // (in every segment: the barrier's phases alternate)
         if (!ok) break;
+        if (kOwn && epilogue_merges(p, s_prefix[sg.b + 1] - s_prefix[sg.b], *s_per, before)) continue;
         merge_records<24, 4>(p, sg, s_prefix, C, neg_lse + buf * p.Ralloc, nblk == 1 ? hw * 32 + lane : lane, nblk == 1 ? 64 : 32);
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_tab_full(buf));
@@ -801,6 +830,7 @@ std::atomic<unsigned long long*> g_test_clock_out{nullptr};
 
 struct ScorePlan {
   int R, Ralloc, k_stages, q_bufs, smem_bytes, U, grid;
+  bool own;                // pass 2 with kOwn
   size_t workspace_bytes;
   bool ok;
 };
@@ -838,12 +868,17 @@ ScorePlan plan_score(const sg_shape* s, size_t limit = 0) {
     if (most >= kFewestCtas && most < pl.grid) pl.grid = (int)most;
   }
   pl.workspace_bytes = (size_t)((parts + pl.grid) * record);
+  // The code for the epilogue's own merges costs the hot loop 1 to 3 % (registers), so it is there only where the helper's merge of
+  // the longest part would take longer than all blocks of a CTA.
+  const int64_t per = pl.grid > 0 && tiles > pl.grid ? tiles / pl.grid : 1;
+  const int nrec = (int)((s->max_seqlen / kTileKeys + 1) / per) + 1;
+  pl.own = pl.Ralloc > 128 && helper_trips(pl.Ralloc, nrec) > per * (pl.Ralloc >> 7);
   return pl;
 }
 
-template <int D, int PASS>
+template <int D, int PASS, bool kOwn>
 sg_status launch_pass(const CUtensorMap& q, const CUtensorMap& k, const ScoreParams& p, const ScorePlan& pl, cudaStream_t s) {
-  SG_ENSURE_SMEM((score_kernel<D, PASS>), pl.smem_bytes);
+  SG_ENSURE_SMEM((score_kernel<D, PASS, kOwn>), pl.smem_bytes);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)pl.grid);
   cfg.blockDim = dim3(kThreads);
@@ -854,7 +889,7 @@ sg_status launch_pass(const CUtensorMap& q, const CUtensorMap& k, const ScorePar
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  SG_CUDA_TRY(cudaLaunchKernelEx(&cfg, score_kernel<D, PASS>, q, k, p));
+  SG_CUDA_TRY(cudaLaunchKernelEx(&cfg, score_kernel<D, PASS, kOwn>, q, k, p));
   return SG_OK;
 }
 
@@ -955,9 +990,10 @@ sg_status run_score(const sg_shape* shape, const void* q_win, const void* k_cach
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   p.units = pl.U;
   p.records = static_cast<float2*>(workspace);
-  st = D == 128 ? launch_pass<128, 1>(tmap_q, tmap_k, p, pl, s) : launch_pass<64, 1>(tmap_q, tmap_k, p, pl, s);
+  st = D == 128 ? launch_pass<128, 1, false>(tmap_q, tmap_k, p, pl, s) : launch_pass<64, 1, false>(tmap_q, tmap_k, p, pl, s);
   if (st != SG_OK) return st;
-  return D == 128 ? launch_pass<128, 2>(tmap_q, tmap_k, p, pl, s) : launch_pass<64, 2>(tmap_q, tmap_k, p, pl, s);
+  if (pl.own) return D == 128 ? launch_pass<128, 2, true>(tmap_q, tmap_k, p, pl, s) : launch_pass<64, 2, true>(tmap_q, tmap_k, p, pl, s);
+  return D == 128 ? launch_pass<128, 2, false>(tmap_q, tmap_k, p, pl, s) : launch_pass<64, 2, false>(tmap_q, tmap_k, p, pl, s);
 }
 
 }  // namespace

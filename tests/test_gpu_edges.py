@@ -245,3 +245,22 @@ def test_pack_total_above_the_prefix_array(B, counted):
     want = np.concatenate([kc[0, 12 * b:12 * b + k, 0] for b in range(B)])
     for got in (pk.numpy(), pv.numpy()):
         assert np.array_equal(got[0, :K], want) and np.all(got[0, K:] == 0x5555)
+
+
+@pytest.mark.parametrize("lens,L,W,Hq,Hkv,d", [
+    # 384 rows, three row blocks: as a CTA's second to fifth segment, between segments that the helper merges
+    ((10924, 52, 40, 12611, 44, 69, 65, 22, 5476, 33, 8623, 18, 15, 24, 99), 2, 24, 16, 1, 128),
+    ((20000, 1, 1, 20000, 1, 1, 20000), 1, 64, 16, 1, 64),      # 1024 rows, eight row blocks
+    ((5000, 5000, 60, 5000), 3, 100, 8, 1, 64),            # 800 rows, the last block partial
+    ((700, 20, 3, 900), 1, 128, 16, 4, 64),                # 512 rows, a tile or two per CTA: none
+])
+def test_score_long_parts_behind_short_segments(lens, L, W, Hq, Hkv, d):
+    """Parts over many CTAs whose records the epilogue warps merge themselves, at any place of a CTA's segments."""
+    import gpu_ops
+    rng = np.random.default_rng(18)
+    cu = cu_of(lens)
+    q, k = rand_bf16(rng, (L, len(lens), W, Hq, d)), rand_bf16(rng, (L, int(cu[-1]), Hkv, d))
+    want = oracle.score(q, k, cu).astype(np.float64)
+    for _ in range(3):
+        got = gpu_ops.score(q, k, cu)
+        assert np.all(np.abs(got - want) <= 1e-4 * np.abs(want) + 1e-30)
