@@ -38,13 +38,13 @@ if ROOT not in sys.path:
 METRIC = "prefill select+pack GB/s (sparse-decode tokens/s in decode_tokens_per_s)"
 UNIT = "GB/s"
 
-# dram__bytes_read.sum + dram__bytes_write.sum per launch from ncu --set full captures (bytes; None where no
+# dram__bytes_read.sum + dram__bytes_write.sum per call from ncu --set full captures (bytes; None where no
 # capture exists).  Keyed by workload then kernel.
 NCU_TRAFFIC = {
-    # captured on 8 of the 32 layers: per-launch bytes scaled x4 where a launch
-    # covers all layers; the decode call is per layer.  (pack: its stores were still in L2 when the capture ended.)
-    "c2": {"score": 4 * (142.152e6 + 6.255e6), "select": 4 * 2.125e6, "pack": 4 * (27.097e6 + 0.131e6),
-           "select_pack": (32 / 24) * (86.950e6 + 27.208e6), "decode": 5.146e6},
+    # captured on 8 of the 32 layers (selection + gather on 24): bytes scaled where a call covers all layers; the decode call
+    # is per layer.  score: both launches, each captured with cold caches.  (pack: its stores were still in L2 when the capture ended.)
+    "c2": {"score": 4 * (137.211e6 + 4.092e6 + 137.445e6 + 5.976e6), "select": 4 * 2.123e6, "pack": 4 * (27.089e6 + 0.118e6),
+           "select_pack": (32 / 24) * (86.952e6 + 26.009e6), "decode": 5.155e6},
 }
 
 
