@@ -52,7 +52,7 @@ constexpr uint32_t kKeyNegInf = 0x007fffffu, kKeyPosInf = 0xff800000u;
 // The selection kernels are launched with programmatic stream serialization: when the kernel before them in the
 // stream (normally the scoring kernel) lets its dependents go early, their CTAs are placed while it drains, and
 // the launch latency disappears behind it.  They do not let their own dependents go early: with the gather of 64 ragged rows
-// placed beside its selection (84 SMs free) a call of scoring, selection and packing took 139.0 us, 136.1 without.
+// placed beside its selection (84 SMs free) a call of scoring, selection and packing, replayed from a graph, took 139.0 us, 136.1 without.
 
 template <bool kInSmem>
 __global__ void __launch_bounds__(kSelThreads, 1) select_topk_kernel(const SelParams p) {
@@ -209,8 +209,9 @@ __global__ void __launch_bounds__(kSelThreads, 1) select_topk_kernel(const SelPa
 // through the narrowing (8B shape, 256 rows, cap 20 %: exact top-cap and a trimming kernel behind it took 13.7 + 7.6 us,
 // this 9.0 us when no row reaches its cap).  NaNs do not take part.
 constexpr int kPackUnroll = 4;
-// Interval populations up to kFinishMax are finished by direct ranking.  Rows of 8192 (one CTA each, 256 of them): 64 takes
-// 13.8 us (most rows need another histogram pass), 128 takes 10.1, 256 takes 12.8.  Up to kAtomicGather of them are gathered
+// Interval populations up to kFinishMax are finished by direct ranking.  Rows of 8192 (one CTA each, 256 of them), the selection
+// alone: 64 takes 13.8 us (most rows need another histogram pass), 128 takes 10.1, 256 takes 12.8; with the gather fused in, 43 us
+// in each case.  Up to kAtomicGather of them are gathered
 // with one shared atomic per thread that has any, more of them through a block-wide prefix sum: the atomics of 100 threads
 // took 9 k clocks in a row of 32768, the prefix sum costs rows of 8192 and less 0.1 us when there are few.
 constexpr int kFinishMax = 128;
