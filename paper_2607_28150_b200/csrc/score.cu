@@ -295,10 +295,11 @@ __host__ __device__ __forceinline__ int helper_trips(int Ralloc, int nrec) {
 }
 // A part over many CTAs behind a short segment is not hidden (two layers of one KV head, 1024 query rows, sequences of 30000, 10
 // and 200 keys: 74 records of 1024 rows merged by one warp while a CTA's epilogue stood, 158 us; 82 with this rule, 107
-// before the helpers merged at all): then the epilogue warps merge the records themselves.  `per` = key tiles per CTA.
-__device__ __forceinline__ bool epilogue_merges(const ScoreParams& p, int part_tiles, int per, int blocks_before) {
-  const int nrec = part_tiles / per + 1;
-  return helper_trips(p.Ralloc, nrec) > blocks_before + (p.Ralloc + 32 * kEpiWarps - 1) / (32 * kEpiWarps) * ((nrec + 11) / 12);
+// before the helpers merged at all): then the epilogue warps merge the records themselves.  `per16` = sixteenths of a key tile per
+// CTA.
+__device__ __forceinline__ bool epilogue_merges(const ScoreParams& p, int part_tiles, int per16, int blocks_before) {
+  const int nrec = part_tiles * 16 / per16 + 1;
+  return helper_trips(p.Ralloc, nrec) > blocks_before + 2 + (p.Ralloc + 32 * kEpiWarps - 1) / (32 * kEpiWarps) * ((nrec + 11) / 12);
 }
 
 // kOwn (pass 2): the epilogue warps may merge later segments, too (plan_score says when).
@@ -317,7 +318,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
   uint64_t* bars = reinterpret_cast<uint64_t*>(k_smem + p.k_stages * kKStageBytes);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 38);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  int* const s_per = reinterpret_cast<int*>(bars + 39);              // key tiles per CTA (kOwn)
+  int* const s_per16 = reinterpret_cast<int*>(bars + 39);            // sixteenths of a key tile per CTA (kOwn)
   float* table = reinterpret_cast<float*>(bars + 40);
   // pass 1: [2 buffers][kGroups]{m[Ralloc], l[Ralloc]} running statistics of a segment
   // pass 2: [2 buffers][Ralloc] negated log-sum-exps, [kColSlots][kGroups][128] partial column sums
@@ -391,7 +392,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
       acc += __shfl_sync(0xffffffffu, inc, 31);
     }
     if (lane == 0) s_prefix[0] = 0;
-    if (kOwn && lane == 0) *s_per = max(1, (int)((long long)p.units * acc / gridDim.x));
+    if (kOwn && lane == 0) *s_per16 = max(16, (int)((long long)p.units * acc * 16 / gridDim.x));
   }
   if (p.R < p.Ralloc) {
     // Rows R..Ralloc-1 of the Q operands are never written by TMA: zero them once so that padded MMA
@@ -634,7 +635,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
         __syncwarp();
         if (lane == 0 && ok && sg.u != p.withhold_unit) mbar_arrive(bar_tab_full(buf));
       } else {
-        if (sidx == 0 || (kOwn && epilogue_merges(p, s_prefix[sg.b + 1] - s_prefix[sg.b], *s_per, blocks_before))) {
+        if (sidx == 0 || (kOwn && epilogue_merges(p, s_prefix[sg.b + 1] - s_prefix[sg.b], *s_per16, blocks_before))) {
           // The first segment's log-sum-exps, and those of a part that the helper would be late with, are what the whole
           // CTA waits for: all epilogue threads merge its records.
           if (sidx == 0) pdl_wait();
@@ -760,7 +761,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
         const uint32_t buf = (uint32_t)sidx & 1u, use = (uint32_t)sidx >> 1;
         if (use > 0) ok = wait(bar_tab_free(buf), (use - 1u) & 1u);        // (in every segment: the barrier's phases alternate)
         if (!ok) break;
-        if (kOwn && epilogue_merges(p, s_prefix[sg.b + 1] - s_prefix[sg.b], *s_per, before)) continue;
+        if (kOwn && epilogue_merges(p, s_prefix[sg.b + 1] - s_prefix[sg.b], *s_per16, before)) continue;
         merge_records<24, 4>(p, sg, s_prefix, C, neg_lse + buf * p.Ralloc, nblk == 1 ? hw * 32 + lane : lane, nblk == 1 ? 64 : 32);
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_tab_full(buf));
@@ -868,11 +869,13 @@ ScorePlan plan_score(const sg_shape* s, size_t limit = 0) {
     if (most >= kFewestCtas && most < pl.grid) pl.grid = (int)most;
   }
   pl.workspace_bytes = (size_t)((parts + pl.grid) * record);
-  // The code for the epilogue's own merges costs the hot loop 1 to 3 % (registers), so it is there only where the helper's merge of
-  // the longest part would take longer than all blocks of a CTA.
-  const int64_t per = pl.grid > 0 && tiles > pl.grid ? tiles / pl.grid : 1;
-  const int nrec = (int)((s->max_seqlen / kTileKeys + 1) / per) + 1;
-  pl.own = pl.Ralloc > 128 && helper_trips(pl.Ralloc, nrec) > per * (pl.Ralloc >> 7);
+  // The code for the epilogue's own merges costs the hot loop 1 to 3 % (registers), so it is there only where CTAs have more than a
+  // tile and the helper's merge of the longest part would take clearly longer than all blocks of a CTA.  (Of 330 random shapes of 129
+  // to 1024 rows 14 get 3 to 49 % faster, the others run as before; without the 8 trips more of them gained up to 20 %, but
+  // some thirty with a tile or two per CTA lost 1 to 5 %.)
+  const int64_t per16 = pl.grid > 0 ? tiles * 16 / pl.grid : 0;
+  const int64_t nrec = per16 > 16 ? ((int64_t)s->max_seqlen / kTileKeys + 1) * 16 / per16 + 1 : 0;
+  pl.own = pl.Ralloc > 128 && nrec > 0 && helper_trips(pl.Ralloc, (int)nrec) * 16 > per16 * (pl.Ralloc >> 7) + 8 * 16;
   return pl;
 }
 

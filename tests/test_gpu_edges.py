@@ -248,9 +248,10 @@ def test_pack_total_above_the_prefix_array(B, counted):
 
 
 @pytest.mark.parametrize("lens,L,W,Hq,Hkv,d", [
-    # 384 rows, three row blocks: as a CTA's second to fifth segment, between segments that the helper merges
-    ((10924, 52, 40, 12611, 44, 69, 65, 22, 5476, 33, 8623, 18, 15, 24, 99), 2, 24, 16, 1, 128),
-    ((20000, 1, 1, 20000, 1, 1, 20000), 1, 64, 16, 1, 64),      # 1024 rows, eight row blocks
+    # such a part as a CTA's second, third and fourth segment, between segments that the helper merges: 384 rows, 1024 rows
+    ((12478, 16, 31, 15649, 31, 99, 84, 17425, 94, 32, 10011, 52, 89, 84), 1, 24, 16, 1, 128),
+    ((18982, 60, 13, 5233, 43, 29, 21, 3168, 45, 53, 64), 2, 64, 16, 1, 64),
+    ((20000, 1, 1, 20000, 1, 1, 20000), 1, 64, 16, 1, 64),
     ((5000, 5000, 60, 5000), 3, 100, 8, 1, 64),            # 800 rows, the last block partial
     ((700, 20, 3, 900), 1, 128, 16, 4, 64),                # 512 rows, a tile or two per CTA: none
 ])
