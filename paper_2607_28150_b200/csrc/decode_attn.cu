@@ -128,9 +128,10 @@ __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t v) {
   return r;
 }
 
-// kN: 8-row tiles of the KV head's query rows (1 for G <= 8, 2 up to 16).  kDecWarps warps per CTA, each with a private ring
+// kTwoLane: a counted call with local_skip; a kernel of its own, because a branch on the pointer in front of the first loads cost
+// the plain calls 0.5 to 1 % (a decode step of 32 layers of 820 entries at batch 1 39.8 us, without it 39.5).  kN: 8-row tiles of the KV head's query rows (1 for G <= 8, 2 up to 16).  kDecWarps warps per CTA, each with a private ring
 // of kSlots half slices: three leave room for two 8-warp CTAs per SM (d = 128), six for one.
-template <int D, int kN, int kDecWarps, int kSlots>
+template <int D, int kN, int kDecWarps, int kSlots, bool kTwoLane>
 __global__ void __launch_bounds__(kDecWarps * 32, (kN == 1 && kSlots * D <= 384 ? 16 : 8) / kDecWarps) decode_partial_kernel(const DecParams p) {
   constexpr int kDecThreads = kDecWarps * 32;
   constexpr int kRowBytes = D * 2;
@@ -168,7 +169,7 @@ __global__ void __launch_bounds__(kDecWarps * 32, (kN == 1 && kSlots * D <= 384 
   // Everything it reads is read with plain loads: the compiler may move read-only-cache loads across the wait.  Calls
   // without a skip are those of a decode loop over rows selected and packed long before: one behind another they overlap as
   // plain calls do (one sequence of 820 entries: 1.7 us per call, 4.5 if each waits; 14 of 3277: 17 and 40).
-  if (p.local_skip) pdl_wait();
+  if (kTwoLane) pdl_wait();
   const int b = blockIdx.x / p.csize;                          // grid.x = B * cluster size
   const int c = blockIdx.x - b * p.csize;                      // rank in the cluster
   // A single sequence (the latency-critical case) needs no prefix loads: a dependent round trip to L2 less before the
@@ -179,7 +180,7 @@ __global__ void __launch_bounds__(kDecWarps * 32, (kN == 1 && kSlots * D <= 384 
   const int kbe = p.packed_count ? min(kb, max(0, p.packed_count[(int64_t)b * p.Hkv + g])) : kb;   // ... of which in the list
   const int cl0 = one ? 0 : p.cu_nloc[b];
   const int nl_row = one ? p.NL_tot : p.cu_nloc[b + 1] - cl0;
-  const int lskip = p.local_skip ? min(nl_row, max(0, p.local_skip[(int64_t)b * p.Hkv + g])) : 0;
+  const int lskip = kTwoLane ? min(nl_row, max(0, p.local_skip[(int64_t)b * p.Hkv + g])) : 0;
   const int nl = nl_row - lskip;
   const int c0 = one ? 0 : p.cu[b];
   const int nseq = one ? p.n_tokens : p.cu[b + 1] - c0;
@@ -662,21 +663,27 @@ sg_status decode_launch(const sg_shape* shape, const void* q, const void* packed
   // one launch: sequences with empty lists still get out = 0 and lse = -inf
   cfg.gridDim = dim3((unsigned)grid_x, (unsigned)shape->num_kv_heads);
   cfg.dynamicSmemBytes = (size_t)decode_smem_bytes(D, warps, slots, p.csize > 1);
-#define SG_LAUNCH_DECODE(DD, NN, WW, SS)                                                         \
-  do {                                                                                           \
-    SG_ENSURE_SMEM((decode_partial_kernel<DD, NN, WW, SS>), decode_smem_bytes(DD, WW, SS, true)); \
-    SG_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_partial_kernel<DD, NN, WW, SS>, p));             \
+#define SG_LAUNCH_DECODE(DD, NN, WW, SS, TL)                                                         \
+  do {                                                                                               \
+    SG_ENSURE_SMEM((decode_partial_kernel<DD, NN, WW, SS, TL>), decode_smem_bytes(DD, WW, SS, true)); \
+    SG_CUDA_TRY(cudaLaunchKernelEx(&cfg, decode_partial_kernel<DD, NN, WW, SS, TL>, p));             \
   } while (0)
-#define SG_LAUNCH_DECODE_D(DD)                                            \
-  do {                                                                    \
-    if (G > 8 && warps == 8) SG_LAUNCH_DECODE(DD, 2, 8, 6);               \
-    else if (G > 8) SG_LAUNCH_DECODE(DD, 2, 4, 6);                        \
-    else if (warps == 4) SG_LAUNCH_DECODE(DD, 1, 4, 3);                   \
-    else if (slots == 6) SG_LAUNCH_DECODE(DD, 1, 8, 6);                   \
-    else SG_LAUNCH_DECODE(DD, 1, 8, 3);                                   \
+#define SG_LAUNCH_DECODE_D(DD, TL)                                            \
+  do {                                                                        \
+    if (G > 8 && warps == 8) SG_LAUNCH_DECODE(DD, 2, 8, 6, TL);               \
+    else if (G > 8) SG_LAUNCH_DECODE(DD, 2, 4, 6, TL);                        \
+    else if (warps == 4) SG_LAUNCH_DECODE(DD, 1, 4, 3, TL);                   \
+    else if (slots == 6) SG_LAUNCH_DECODE(DD, 1, 8, 6, TL);                   \
+    else SG_LAUNCH_DECODE(DD, 1, 8, 3, TL);                                   \
   } while (0)
-  if (D == 128) SG_LAUNCH_DECODE_D(128);
-  else SG_LAUNCH_DECODE_D(64);
+  if (local_skip) {
+    if (D == 128) SG_LAUNCH_DECODE_D(128, true);
+    else SG_LAUNCH_DECODE_D(64, true);
+  } else if (D == 128) {
+    SG_LAUNCH_DECODE_D(128, false);
+  } else {
+    SG_LAUNCH_DECODE_D(64, false);
+  }
 #undef SG_LAUNCH_DECODE_D
 #undef SG_LAUNCH_DECODE
   return SG_OK;
