@@ -42,6 +42,10 @@ void sg_testing_score_clock(void* dev_buffer);
 /* Number of CTAs of each of sg_score's launches for this shape on a 148-SM device. */
 int32_t sg_testing_score_grid(const sg_shape* shape);
 
+/* CTAs per (layer, sequence, KV head) of the kernel that scores, selects and packs in one launch, where the prefill sequences take
+ * it for this shape on the current device; else 0. */
+int32_t sg_testing_score_cluster(const sg_shape* shape);
+
 /*
  * sg_testing_decode_overlap -- allowed = 0: the following sg_sparse_decode_attn calls are launched without
  * programmatic stream serialization, i.e. fully ordered behind everything earlier in the stream, so that the

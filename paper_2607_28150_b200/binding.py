@@ -26,7 +26,8 @@ SG_OP_SCORE, SG_OP_SELECT_TOPK, SG_OP_PACK_KV, SG_OP_SPARSE_DECODE_ATTN, SG_OP_S
 EXPORTED = ("sg_workspace_bytes", "sg_score", "sg_select_topk", "sg_pack_kv", "sg_sparse_decode_attn",
             "sg_score_static", "sg_select_pack_kv", "sg_select_threshold", "sg_pack_kv_counted", "sg_sparse_decode_attn_counted", "sg_split_index", "sg_profile_accumulate", "sg_block_importance",
             "sg_transfer_budget", "sg_proactive_mask", "sg_push_blocks", "sg_speculative_delivered", "sg_strerror", "sg_last_cuda_error",
-            "sg_testing_score_fault", "sg_testing_score_clock", "sg_testing_score_grid", "sg_testing_decode_overlap")
+            "sg_testing_score_fault", "sg_testing_score_clock", "sg_testing_score_grid", "sg_testing_score_cluster",
+            "sg_testing_decode_overlap")
 SG_SCORE_STATIC_SCRATCH_BYTES = 8 << 20
 
 if not os.path.exists(LIB_PATH):
@@ -99,6 +100,8 @@ _lib.sg_testing_decode_overlap.restype = None
 _lib.sg_testing_decode_overlap.argtypes = [_i32]
 _lib.sg_testing_score_grid.restype = _i32
 _lib.sg_testing_score_grid.argtypes = [_sp]
+_lib.sg_testing_score_cluster.restype = _i32
+_lib.sg_testing_score_cluster.argtypes = [_sp]
 
 
 def sg_testing_score_fault(withhold_unit: int = -1, wait_limit_ms: int = 0) -> None:
@@ -119,6 +122,10 @@ def sg_testing_decode_overlap(allowed: bool) -> None:
 
 def sg_testing_score_grid(shape: "Shape") -> int:
     return int(_lib.sg_testing_score_grid(ctypes.byref(shape)))
+
+
+def sg_testing_score_cluster(shape: "Shape") -> int:
+    return int(_lib.sg_testing_score_cluster(ctypes.byref(shape)))
 
 
 def make_shape(num_layers: int, num_q_heads: int, num_kv_heads: int, head_dim: int, window: int,

@@ -14,6 +14,9 @@
 
 #include "smartgen.h"
 
+extern "C" sg_status sg_internal_score_select_pack(const sg_shape*, const void*, const void*, const void*, float*, void*, size_t, const int32_t*, int32_t,
+                                                   int32_t*, void*, void*, int32_t*, void*);
+
 namespace {
 
 enum Kind { kBf16, kF32, kI32, kI8 };
@@ -333,7 +336,9 @@ SG_FN(prefill) {
   void *sel = x.ptr(kI32, "sel_idx", total == 0), *pk = x.ptr(kBf16, "packed_k", total == 0), *pv = x.ptr(kBf16, "packed_v", total == 0);
   void *st = x.ptr(kI32, "dev_status", true), *stream = x.stream();
   return call(x, [&]() -> int {
-    int rc = sg_score(s, q, k, (float*)imp, w, wb, (int32_t*)st, stream);
+    int rc = sg_internal_score_select_pack(s, q, k, v, (float*)imp, w, wb, (int32_t*)cu_k, total, (int32_t*)sel, pk, pv, (int32_t*)st, stream);
+    if (rc != SG_ERR_UNSUPPORTED) return rc;           // one kernel did both
+    rc = sg_score(s, q, k, (float*)imp, w, wb, (int32_t*)st, stream);
     if (rc) return rc;
     rc = sg_select_pack_kv(s, (float*)imp, (int32_t*)cu_k, total, k, v, (int32_t*)sel, pk, pv, (int32_t*)st, stream);
     return rc ? rc + 256 : 0;
@@ -352,7 +357,9 @@ SG_FN(prefill_layer) {
   void *sel = x.layer_ptr(kI32, "sel_idx", layer), *pk = x.layer_ptr(kBf16, "packed_k", layer), *pv = x.layer_ptr(kBf16, "packed_v", layer);
   void *st = x.ptr(kI32, "dev_status", true), *stream = x.stream();
   return call(x, [&]() -> int {
-    int rc = sg_score(s, q, k, (float*)imp, w, wb, (int32_t*)st, stream);
+    int rc = sg_internal_score_select_pack(s, q, k, v, (float*)imp, w, wb, (int32_t*)cu_k, total, (int32_t*)sel, pk, pv, (int32_t*)st, stream);
+    if (rc != SG_ERR_UNSUPPORTED) return rc;           // one kernel did both
+    rc = sg_score(s, q, k, (float*)imp, w, wb, (int32_t*)st, stream);
     if (rc) return rc;
     rc = sg_select_pack_kv(s, (float*)imp, (int32_t*)cu_k, total, k, v, (int32_t*)sel, pk, pv, (int32_t*)st, stream);
     return rc ? rc + 256 : 0;

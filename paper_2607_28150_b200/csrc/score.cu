@@ -32,6 +32,8 @@
 
 #include "common.cuh"
 #include "launch.h"
+#include "score_launch.h"
+#include "score_math.cuh"
 #include "tcgen05.cuh"
 
 namespace sg {
@@ -46,7 +48,6 @@ constexpr int kStages = 4;                // 4 x 128 fp32 columns = the whole 51
 constexpr int kColSlots = 4;              // pass 2, several row blocks per tile: partial column sums of four tiles in flight
 constexpr int kMaxKStages = 4;
 constexpr int kSmemLimit = 232448;        // 227 KB opt-in dynamic shared memory per CTA
-constexpr float kLog2e = 1.4426950408889634f;
 
 // Debug build (-DSG_CHECKS): device-side checks of the shared-memory carve-up and of every TMA coordinate (tile inside
 // the tensor or hanging over its end only where the fill value is wanted).  A failed check never traps: it sets the
@@ -85,102 +86,6 @@ struct ScoreParams {
   unsigned long long* clock_out;   // testing only: per CTA {clock64 start, end, globaltimer start, end}, or null
   float scale_log2;
 };
-
-// ---------------------------------------------------------------- exponentials
-// The SFU gives 16 exp2 per clock and SM and is the first unit to fill up: a 128 x 128 block is 1024 clocks of it, while
-// the FMA pipe has 256 clocks of work (scale and sum, two at a time).  So a share of the exponentials is computed on the
-// FMA pipe with packed fp32 instructions.
-__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ float max3(float a, float b, float c) {
-  float r;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
-}
-__device__ __forceinline__ uint64_t pair_of(const uint32_t* v) { return pack2(__uint_as_float(v[0]), __uint_as_float(v[1])); }
-__device__ __forceinline__ uint64_t exp2_sfu2(uint64_t x) {
-  float x0, x1;
-  unpack2(x, x0, x1);
-  return pack2(exp2f(x0), exp2f(x1));
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-// Bounds that let a NaN through (fmaxf and fminf return the bound in its place).
-__device__ __forceinline__ float max_nan(float a, float b) {
-  float r;
-  asm("max.ftz.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ float min_nan(float a, float b) {
-  float r;
-  asm("min.ftz.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-  return r;
-}
-// Two exp2 on the FMA pipe: x = n + f with n an integer and |f| <= 1/2, 2^f by a polynomial of degree 5 (minimax fit of
-// 2^f by iterated weighted least squares, constant term 1; relative error at most 1.7e-7 including the fp32 evaluation),
-// times 2^n put together from its exponent field.  x is clamped to -127, where that field is 0 and so is the factor, and,
-// where x may be large (pass 1, against a stale reference), to 127: a huge finite number, which trips the range test of
-// pass 1 as the SFU's inf does.  A NaN passes the clamps and the polynomial and is a NaN behind the product, as the
-// SFU's is: a non-finite score shows in the sums whatever column it stands in.
-template <bool kAbove>
-__device__ __forceinline__ uint64_t exp2_fma2(uint64_t x) {
-  float x0, x1;
-  unpack2(x, x0, x1);
-  x0 = max_nan(x0, -127.f);
-  x1 = max_nan(x1, -127.f);
-  if (kAbove) { x0 = min_nan(x0, 127.f); x1 = min_nan(x1, 127.f); }
-  x = pack2(x0, x1);
-  const uint64_t t = add2(x, pack2(12582912.f, 12582912.f));                 // 1.5 * 2^23: the low bits of t are round(x)
-  const uint64_t f = fma2(add2(t, pack2(-12582912.f, -12582912.f)), pack2(-1.f, -1.f), x);
-  uint64_t q = fma2(pack2(0.001326472731307149f, 0.001326472731307149f), f, pack2(0.009671512991189957f, 0.009671512991189957f));
-  q = fma2(q, f, pack2(0.05550733581185341f, 0.05550733581185341f));
-  q = fma2(q, f, pack2(0.24022242426872253f, 0.24022242426872253f));
-  q = fma2(q, f, pack2(0.6931470036506653f, 0.6931470036506653f));
-  q = fma2(q, f, pack2(1.f, 1.f));
-  float t0, t1;
-  unpack2(t, t0, t1);
-  return mul2(q, pack2(__int_as_float((__float_as_int(t0) << 23) + 0x3f800000), __int_as_float((__float_as_int(t1) << 23) + 0x3f800000)));
-}
-// Pairs of a 32-column chunk's sixteen whose exponentials run on the FMA pipe, spread evenly.
-constexpr int kFmaPairs1 = 4, kFmaPairs2 = 4;
-__device__ __forceinline__ constexpr bool on_fma(int pair, int share) { return ((pair + 1) * share) / 16 != (pair * share) / 16; }
-// Pass 1: adds exp2(score * scale - m) of a chunk's 32 columns to two pairs of accumulators (nm2 = {-m, -m}).
-__device__ __forceinline__ void chunk_rows(uint32_t (&cur)[32], uint64_t scale2, uint64_t nm2, uint64_t& s0, uint64_t& s1) {
-#pragma unroll
-  for (int i = 0; i < 16; i += 2) {
-    const uint64_t x0 = fma2(pair_of(cur + 2 * i), scale2, nm2), x1 = fma2(pair_of(cur + 2 * i + 2), scale2, nm2);
-    s0 = add2(s0, on_fma(i, kFmaPairs1) ? exp2_fma2<true>(x0) : exp2_sfu2(x0));
-    s1 = add2(s1, on_fma(i + 1, kFmaPairs1) ? exp2_fma2<true>(x1) : exp2_sfu2(x1));
-  }
-}
-// Pass 2: adds exp2(score * scale + nl[column]) of a chunk's 32 columns (nl = negated log-sum-exps).
-__device__ __forceinline__ void chunk_cols(uint32_t (&cur)[32], uint64_t scale2, const float* nl, uint64_t& s0, uint64_t& s1) {
-#pragma unroll
-  for (int i = 0; i < 16; i += 2) {
-    const float4 l4 = *reinterpret_cast<const float4*>(nl + 2 * i);
-    const uint64_t x0 = fma2(pair_of(cur + 2 * i), scale2, pack2(l4.x, l4.y));
-    const uint64_t x1 = fma2(pair_of(cur + 2 * i + 2), scale2, pack2(l4.z, l4.w));
-    s0 = add2(s0, on_fma(i, kFmaPairs2) ? exp2_fma2<false>(x0) : exp2_sfu2(x0));
-    s1 = add2(s1, on_fma(i + 1, kFmaPairs2) ? exp2_fma2<false>(x1) : exp2_sfu2(x1));
-  }
-}
 
 // ---------------------------------------------------------------- schedule
 // CTAs that get tiles (the host sizes the grid by an upper bound of the tile count).
@@ -922,11 +827,19 @@ extern "C" int32_t sg_testing_score_grid(const sg_shape* shape) {
   return pl.ok ? pl.grid : 0;
 }
 
+extern "C" int32_t sg_testing_score_cluster(const sg_shape* shape) {
+  using namespace sg;
+  if (check_shape(shape, true) != SG_OK) return 0;
+  return plan_score(shape).ok ? score_cluster_size(shape, true) : 0;
+}
+
 namespace sg {
 namespace {
 
+// `limit`: as in plan_score, and the two passes whatever the shape.  `pack`: only where one kernel does it all, else SG_ERR_UNSUPPORTED
+// with nothing launched.
 sg_status run_score(const sg_shape* shape, const void* q_win, const void* k_cache, float* importance, void* workspace,
-                    size_t workspace_bytes, size_t limit, int32_t* dev_status, void* stream) {
+                    size_t workspace_bytes, size_t limit, const PackLaunch* pack, int32_t* dev_status, void* stream) {
   sg_status st = check_shape(shape, true);
   if (st != SG_OK) return st;
   if (shape->total_tokens == 0) return SG_OK;
@@ -935,6 +848,9 @@ sg_status run_score(const sg_shape* shape, const void* q_win, const void* k_cach
   const ScorePlan pl = plan_score(shape, limit);
   if (!pl.ok) return SG_ERR_UNSUPPORTED;
   if (!workspace || workspace_bytes < pl.workspace_bytes) return SG_ERR_WORKSPACE;
+  unsigned long long* const clock_out = g_test_clock_out.load(std::memory_order_relaxed);
+  const bool cluster = limit == 0 && !clock_out && score_cluster_size(shape, pack != nullptr) > 0;
+  if (pack && !cluster) return SG_ERR_UNSUPPORTED;
   EncodeTiledFn encode = encode_tiled_fn();
   if (!encode) return cuda_fail((int)cudaErrorUnknown);
 
@@ -987,10 +903,11 @@ sg_status run_score(const sg_shape* shape, const void* q_win, const void* k_cach
   p.withhold_unit = g_test_withhold_unit.load(std::memory_order_relaxed);
   const int limit_ms = g_test_wait_limit_ms.load(std::memory_order_relaxed);
   p.wait_ns = limit_ms > 0 ? (uint32_t)limit_ms * 1000000u : 1000000000u;
-  p.clock_out = g_test_clock_out.load(std::memory_order_relaxed);
+  p.clock_out = clock_out;
   p.scale_log2 = kLog2e / sqrtf((float)D);
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (cluster) return score_cluster_launch(shape, tmap_q, tmap_k, ScoreLaunch{importance, dev_status, p.withhold_unit, p.wait_ns, s}, pack);
   p.units = pl.U;
   p.records = static_cast<float2*>(workspace);
   st = D == 128 ? launch_pass<128, 1, false>(tmap_q, tmap_k, p, pl, s) : launch_pass<64, 1, false>(tmap_q, tmap_k, p, pl, s);
@@ -1004,8 +921,23 @@ sg_status run_score(const sg_shape* shape, const void* q_win, const void* k_cach
 
 extern "C" sg_status sg_score(const sg_shape* shape, const void* q_win, const void* k_cache, float* importance,
                               void* workspace, size_t workspace_bytes, int32_t* dev_status, void* stream) {
-  return sg::run_score(shape, q_win, k_cache, importance, workspace, workspace_bytes, 0, dev_status, stream);
+  return sg::run_score(shape, q_win, k_cache, importance, workspace, workspace_bytes, 0, nullptr, dev_status, stream);
 }
+
+// sg_score, then sg_select_pack_kv, where one kernel does both; SG_ERR_UNSUPPORTED, with nothing launched, for everything else, bad
+// arguments included (the two calls then say what is wrong).  For the sequences of native.cpp.
+extern "C" sg_status sg_internal_score_select_pack(const sg_shape* shape, const void* q_win, const void* k_cache, const void* v_cache,
+                                                   float* importance, void* workspace, size_t workspace_bytes, const int32_t* cu_k,
+                                                   int32_t total_sel, int32_t* sel_idx, void* packed_k, void* packed_v,
+                                                   int32_t* dev_status, void* stream) {
+  using namespace sg;
+  if (total_sel <= 0 || !cu_k || !v_cache || !sel_idx || !packed_k || !packed_v) return SG_ERR_UNSUPPORTED;
+  if (!aligned16(cu_k) || !aligned16(v_cache) || !aligned16(sel_idx) || !aligned16(packed_k) || !aligned16(packed_v)) return SG_ERR_UNSUPPORTED;
+  const PackLaunch pack{cu_k, total_sel, k_cache, v_cache, sel_idx, packed_k, packed_v};
+  const sg_status st = run_score(shape, q_win, k_cache, importance, workspace, workspace_bytes, 0, &pack, dev_status, stream);
+  return st == SG_ERR_CUDA || (st == SG_OK && shape->total_tokens > 0) ? st : SG_ERR_UNSUPPORTED;
+}
+
 
 // ---------------------------------------------------------------------------------------------
 // sg_score_static: sg_score for callers that cannot allocate device memory.
@@ -1039,5 +971,5 @@ extern "C" sg_status sg_score_static(const sg_shape* shape, const void* q_win, c
     if (dev >= 0 && dev < 64) scratch_of_device[dev].store(scratch, std::memory_order_release);
   }
   return run_score(shape, q_win, k_cache, importance, scratch, (size_t)SG_SCORE_STATIC_SCRATCH_BYTES, (size_t)SG_SCORE_STATIC_SCRATCH_BYTES,
-                   dev_status, stream);
+                   nullptr, dev_status, stream);
 }

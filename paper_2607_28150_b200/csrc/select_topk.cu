@@ -9,6 +9,7 @@
 // Both take equal-to-threshold entries from the lowest positions first.  The result is therefore a pure
 // function of the input row: identical on every run and identical to a full sort.
 #include "common.cuh"
+#include "select_key.cuh"
 
 namespace sg {
 namespace {
@@ -39,15 +40,6 @@ struct SelParams {
   int32_t* sel_count;      // [L][B][Hkv]
   float alpha;
 };
-
-// Takes the raw bit pattern: the row is read as uint32 so that no float instruction (and no
-// flush-to-zero of subnormals) ever touches the values.
-__device__ __forceinline__ uint32_t order_key(uint32_t u) {
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-
-__device__ __forceinline__ uint32_t key_to_bits(uint32_t k) { return (k & 0x80000000u) ? (k & 0x7fffffffu) : ~k; }
-constexpr uint32_t kKeyNegInf = 0x007fffffu, kKeyPosInf = 0xff800000u;
 
 // The selection kernels are launched with programmatic stream serialization: when the kernel before them in the
 // stream (normally the scoring kernel) lets its dependents go early, their CTAs are placed while it drains, and
