@@ -532,7 +532,12 @@ constexpr int decode_smem_bytes(int D, int warps, int slots, bool cluster) {
 // A two-lane call names one row of the KV index as its packed and as its indexed list, so avg_tokens is up to twice what it
 // attends.  Planned for the row's length, the chain of split, pack and attention is slower more often than faster
 // (19 sequences of 820 entries 30.2 -> 32.7 us, 1 of 820 11.8 -> 12.3, 64 of 820 87.9 -> 83.4): it stays.
-void decode_plan(const sg_shape* shape, int32_t total_sel, int32_t total_loc, int* csize, int* warps, int* slots) {
+// It does not overlap the next call, so its clusters may fill both CTAs of every SM.  That pays where the longest row is well above the
+// average and its warps have five slices or more: the call lasts as long as that row.  Whole chains of split, pack and attention, 8
+// sequences of 6321 to 32061 tokens, a tenth of them required: 32.8 -> 30.0 us, four tenths 106 -> 90, d = 64 24.8 -> 21.5, 2 heads of 64
+// 14.9 -> 13.3; but 8 of 500 to 4000 tokens 11.8 -> 12.6 and, of equal lengths, 16 of 1638 entries 40.2 -> 41.1, 4 of
+// 1638 18.1 -> 18.5, which the rule leaves as they are.
+void decode_plan(const sg_shape* shape, int32_t total_sel, int32_t total_loc, bool two_lane, int* csize, int* warps, int* slots) {
   const int64_t pairs = (int64_t)shape->batch * shape->num_kv_heads;
   const int64_t avg_tokens = ((int64_t)total_sel + total_loc) / shape->batch;
   const bool packed_only = total_loc == 0;
@@ -547,6 +552,10 @@ void decode_plan(const sg_shape* shape, int32_t total_sel, int32_t total_loc, in
     // short lists: four warps per CTA already give every warp at most ~1.75 slices, and the merge is half as wide
     W = 4 * avg_tokens <= 7 * 4 * kSlice * fit ? 4 : 8;
     while (cs < fit && (int64_t)cs * W * kSlice < avg_tokens) cs *= 2;
+  }
+  if (two_lane && pairs <= kNumSMs && W == 8 && shape->total_tokens > 0) {
+    const int64_t longest = (int64_t)total_sel * shape->max_seqlen / shape->total_tokens, average = total_sel / shape->batch;
+    if (4 * longest >= 5 * average && longest >= 5 * kSlice * W * cs && cs < 8 && pairs * cs <= kNumSMs) cs *= 2;
   }
   *csize = cs;
   *warps = W;
@@ -643,7 +652,7 @@ sg_status decode_launch(const sg_shape* shape, const void* q, const void* packed
   p.NL_tot = total_loc;
   p.n_tokens = shape->total_tokens;
   int warps = 4, slots = 3;
-  decode_plan(shape, total_sel, total_loc, &p.csize, &warps, &slots);
+  decode_plan(shape, total_sel, total_loc, local_skip != nullptr, &p.csize, &warps, &slots);
   p.scale_log2 = (softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)D)) * kLog2e;
   const int64_t grid_x = (int64_t)shape->batch * p.csize;
   if (grid_x > 0x7fffffffLL || shape->num_kv_heads > 65535) return SG_ERR_UNSUPPORTED;

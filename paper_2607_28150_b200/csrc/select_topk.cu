@@ -184,8 +184,8 @@ __global__ void __launch_bounds__(kSelThreads, 1) select_topk_kernel(const SelPa
 
 // ------------------------------------------------------------------------------------------------
 // Register-resident variant for rows of up to 32768 tokens: thread t owns E consecutive positions
-// [t*E, (t+1)*E) and keeps their keys in registers (16-byte loads of its own segment when the row is 16-byte
-// aligned, else coalesced through a padded shared-memory staging buffer).  At most three histogram passes of
+// [t*E, (t+1)*E) and keeps their keys in registers (16-byte loads from the boundary at or before the
+// row's start).  At most three histogram passes of
 // 2048 bins over a shrinking key interval find the k-th largest key exactly; after the first pass only the few
 // keys inside the threshold bin take part.  Because ownership is contiguous, one block-wide prefix sum over
 // per-thread (greater, equal) counts gives every thread the output offset of its first selected position, and
@@ -232,10 +232,12 @@ template <int E, int T, int PD, bool kThr>
 __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
   pdl_wait();
   extern __shared__ __align__(16) uint32_t smem[];
-  uint32_t* hist = smem;                               // [kRegCopies][kRegBins]
-  uint32_t* wsum = hist + kRegCopies * kRegBins;       // [2][T/32]
+  uint32_t* wsum = smem;                               // [2][T/32]
   uint32_t* sh = wsum + 2 * (T / 32);                  // [0] chosen bin, [1] remaining need ... [6], [7] barrier
-  uint32_t* stage = sh + 8;                            // [T][E + 4] keys, or [T * E] values of the row; later lists
+  uint32_t* cand = sh + 8;                             // [kFinishMax + 4] keys that are ranked directly
+  uint32_t* hist = cand + kFinishMax + 4;              // [kRegCopies][kRegBins]
+  uint32_t* stage = hist + kRegCopies * kRegBins;      // E > 16: [T * E] values of the row
+  uint16_t* list = reinterpret_cast<uint16_t*>(E > 16 ? stage : hist);     // [T * E] selected positions (PD > 0), over what has been used
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int row = blockIdx.x;
@@ -311,15 +313,14 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
     return;
   }
   const uint32_t* x = reinterpret_cast<const uint32_t*>(p.importance) + ((int64_t)l * p.Hkv + g) * p.T + c0;
-  // Thread t owns E consecutive values of the row.  Up to 16 of them it reads itself, with 16-byte loads where the row is
-  // 16-byte aligned (the lines of a warp's first load serve its later ones from L1), else coalesced through a padded buffer.
-  // For E = 32 the row comes to shared memory with one bulk copy from the 16-byte boundary at or before it (`off` values
-  // early), the up to three values behind the last boundary with plain loads.  Thread t's values are then the positions
-  // from t*E - off; it reads them 16 bytes at a time, starting at another quad of its segment than its neighbours (no bank
+  // Thread t owns E consecutive values, from the 16-byte boundary at or before the row's start (`off` values early): its positions are
+  // those from t*E - off.  Up to 16 values it reads itself, 16 bytes at a time (the lines of a warp's first load serve its later ones
+  // from L1).  For E = 32 the row comes to shared memory with one bulk copy, the up to three values behind the last boundary with
+  // plain loads; a thread reads its values 16 bytes at a time, starting at another quad of its segment than its neighbours (no bank
   // conflicts), so its registers hold the segment turned by `turn` quads, and bit masks over them are turned back before use.
   // A row of 32768: 5.7 k clocks; by the threads themselves 10.7 k (the row is larger than the L1 that shared memory leaves:
-  // every line comes from L2 several times), coalesced through the padded buffer 8.5 k.  With 16 values or fewer the bulk
-  // copy loses: 3.8 against 2.9 k clocks for a row of 8192, 2.8 against 2.3 k for 1024.
+  // every line comes from L2 several times).  With 16 values or fewer the bulk copy loses: 3.8 against 2.9 k clocks for a row of
+  // 8192, 2.8 against 2.3 k for 1024.
   constexpr bool kBulk = E > 16;
   constexpr uint32_t kAll = E >= 32 ? 0xffffffffu : ((1u << (E & 31)) - 1u);
   constexpr int kQuads = E / 4;
@@ -329,9 +330,10 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
     const int sft = 4 * by;
     return sft == 0 ? m : ((m << sft) | (m >> (E - sft))) & kAll;
   };
-  int off = kBulk ? (int)((reinterpret_cast<uintptr_t>(x) & 15u) >> 2) : 0;
-  const bool bulk = kBulk && N + off <= E * T;         // else the values in front of the row would push its end out of the registers
-  if (!bulk) off = 0;
+  int off = (int)((reinterpret_cast<uintptr_t>(x) & 15u) >> 2);
+  const bool wide = N + off <= E * T;                  // else the values in front of the row would push its end out of the registers
+  const bool bulk = kBulk && wide;
+  if (!wide) off = 0;
   const int span = N + off, whole = bulk ? span & ~3 : 0;                // values from the boundary on; of the bulk copy
   const uint32_t bar = smem_u32(sh + 6);               // 8 bytes, 8-byte aligned
   if (bulk && tid == 0) {
@@ -346,10 +348,8 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
   const int first = tid * E - off;                     // position of the thread's first value (negative: before the row)
   const int nvalid = min(max(N - first, 0), E);
   uint32_t vmask = nvalid >= 32 ? 0xffffffffu : ((1u << nvalid) - 1u);
-  if constexpr (kBulk) {
-    if (first < 0) vmask &= ~((1u << -first) - 1u);    // the boundary's values in front of the row
-    vmask = turned(vmask, (kQuads - turn) % kQuads);   // as the registers hold the segment
-  }
+  if (first < 0) vmask &= ~((1u << -first) - 1u);      // the boundary's values in front of the row
+  vmask = turned(vmask, (kQuads - turn) % kQuads);     // as the registers hold the segment
   uint32_t key[E];
   if constexpr (kBulk) {
     for (int i = whole + tid; i < span; i += T) stage[i] = x[i - off];
@@ -370,18 +370,18 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
       key[4 * q] = order_key(v.x); key[4 * q + 1] = order_key(v.y);
       key[4 * q + 2] = order_key(v.z); key[4 * q + 3] = order_key(v.w);
     }
-  } else if ((reinterpret_cast<uintptr_t>(x) & 15u) == 0) {
+  } else {
     uint4 v[kQuads];
 #pragma unroll
     for (int q = 0; q < kQuads; ++q) {
       const int i = first + 4 * q;
-      if (i + 3 < N) {
+      if (wide && i + 3 < N) {
         v[q] = *reinterpret_cast<const uint4*>(x + i);
       } else {
-        v[q].x = i < N ? x[i] : 0u;
-        v[q].y = i + 1 < N ? x[i + 1] : 0u;
-        v[q].z = i + 2 < N ? x[i + 2] : 0u;
-        v[q].w = 0u;
+        v[q].x = i >= 0 && i < N ? x[i] : 0u;
+        v[q].y = i + 1 >= 0 && i + 1 < N ? x[i + 1] : 0u;
+        v[q].z = i + 2 >= 0 && i + 2 < N ? x[i + 2] : 0u;
+        v[q].w = i + 3 < N ? x[i + 3] : 0u;
       }
     }
 #pragma unroll
@@ -390,20 +390,6 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
       key[4 * q + 2] = order_key(v[q].z); key[4 * q + 3] = order_key(v[q].w);
     }
     __syncthreads();                                   // histogram cleared
-  } else {
-    {
-      uint32_t v[E];                                   // all E loads of the thread are issued before the first store
-#pragma unroll
-      for (int e = 0; e < E; ++e) { const int i = tid + e * T; v[e] = i < N ? x[i] : 0u; }
-#pragma unroll
-      for (int e = 0; e < E; ++e) { const int i = tid + e * T; stage[i + 4 * (i / E)] = i < N ? order_key(v[e]) : 0u; }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int e = 0; e < E; e += 4) {
-      const uint4 v = *reinterpret_cast<const uint4*>(stage + tid * (E + 4) + e);
-      key[e] = v.x; key[e + 1] = v.y; key[e + 2] = v.z; key[e + 3] = v.w;
-    }
   }
 
   // ---- exact k-th largest key by narrowing a key interval [lo, hi] that holds it, 11 bits of the interval per pass.
@@ -490,7 +476,6 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
     if (lo != hi && ncand <= (uint32_t)kFinishMax) {
       // Few keys left in the interval: instead of more block-wide passes, gather them and count for each the keys above it
       // and equal to it; the key whose rank range covers `need` is the threshold.
-      uint32_t* list = stage;
       const uint32_t w = hi - lo;
       uint32_t mine = 0;
 #pragma unroll
@@ -504,17 +489,17 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
       if (mine) {
 #pragma unroll
         for (int e = 0; e < E; ++e)
-          if ((mine >> e) & 1u) list[at++] = key[e];
+          if ((mine >> e) & 1u) cand[at++] = key[e];
       }
       __syncthreads();
       // four lanes per key, a quarter of the list each
       for (int i0 = 0; i0 < (int)ncand; i0 += T / 4) {
         const int i = i0 + (tid >> 2), part = tid & 3;
         if (i0 + (warp << 3) >= (int)ncand) break;     // nothing for this warp
-        const uint32_t k = i < (int)ncand ? list[i] : 0u;
+        const uint32_t k = i < (int)ncand ? cand[i] : 0u;
         uint32_t above = 0, same = 0;
         for (int j = 4 * part; j < (int)ncand; j += 16) {
-          const uint4 o = *reinterpret_cast<const uint4*>(list + j);     // values behind the list's end do not count
+          const uint4 o = *reinterpret_cast<const uint4*>(cand + j);     // values behind the list's end do not count
           const int left = (int)ncand - j;
           above += (o.x > k ? 1u : 0u) + (left > 1 && o.y > k ? 1u : 0u) + (left > 2 && o.z > k ? 1u : 0u) + (left > 3 && o.w > k ? 1u : 0u);
           same += (o.x == k ? 1u : 0u) + (left > 1 && o.y == k ? 1u : 0u) + (left > 2 && o.z == k ? 1u : 0u) + (left > 3 && o.w == k ? 1u : 0u);
@@ -555,7 +540,7 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
     const int e = __ffs(m) - 1;
     m &= m - 1;
     out[slot] = first + e;
-    if constexpr (PD > 0) stage[slot] = (uint32_t)(first + e);
+    if constexpr (PD > 0) list[slot] = (uint16_t)(first + e);
     ++slot;
   }
   if constexpr (kThr) {
@@ -564,12 +549,18 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
   }
   if constexpr (PD > 0) {
     __syncthreads();
-    pack_rows([&](int j) { return (int)stage[j]; });
+    pack_rows([&](int j) { return (int)list[j]; });
   }
 }
 
+// What the selection needs of shared memory is what the gather lacks of L1, which holds the lines that are on their way: 256 rows of
+// 8192 with 57 KB per CTA (rows staged, positions in 32 bits beside the histograms) took 43.6 us, 43.2 with 17 KB; 51 with the whole L1
+// asked for as shared memory.
 template <int E, int T>
-constexpr int select_reg_smem_bytes() { return (kRegCopies * kRegBins + 2 * (T / 32) + 8 + T * (E > 16 ? E : E + 4)) * 4; }
+constexpr int select_reg_smem_bytes(bool lists) {
+  const int hist = kRegCopies * kRegBins * 4, list = lists && E <= 16 ? E * T * 2 : 0;
+  return (2 * (T / 32) + 8 + kFinishMax + 4) * 4 + (hist > list ? hist : list) + (E > 16 ? E * T * 4 : 0);
+}
 
 }  // namespace
 }  // namespace sg
@@ -594,9 +585,9 @@ sg_status select_launch(const sg_shape* shape, SelParams& p, SelectKind kind, vo
 #define SG_LAUNCH_SELECT_REG_PD(E, T, PD, THR)                                                     \
   do {                                                                                          \
     p.capacity = (E) * (T);                                                                     \
-    SG_ENSURE_SMEM((select_topk_reg_kernel<E, T, PD, THR>), (select_reg_smem_bytes<E, T>()));         \
+    SG_ENSURE_SMEM((select_topk_reg_kernel<E, T, PD, THR>), (select_reg_smem_bytes<E, T>(PD > 0)));         \
     cfg.blockDim = dim3(T);                                                                     \
-    cfg.dynamicSmemBytes = select_reg_smem_bytes<E, T>();                                       \
+    cfg.dynamicSmemBytes = select_reg_smem_bytes<E, T>(PD > 0);                                       \
     SG_CUDA_TRY(cudaLaunchKernelEx(&cfg, select_topk_reg_kernel<E, T, PD, THR>, p));                  \
   } while (0)
 #define SG_LAUNCH_SELECT_REG(E, T)                                              \
