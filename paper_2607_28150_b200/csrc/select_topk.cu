@@ -209,7 +209,9 @@ constexpr int kPackUnroll = 4;
 constexpr int kFinishMax = 128;
 constexpr uint32_t kAtomicGather = 64;
 constexpr int64_t kFuseMinRows = kNumSMs;               // fewer rows than SMs cannot fill the machine with their gathers
-constexpr int kRegBins = 2048;
+// Bins of a histogram: four per thread, 2048 at most (eight per thread for 128 and 256 threads: 0.5 to 1 us slower).
+template <int T>
+constexpr int kRegBinBits = T >= 512 ? 11 : T >= 256 ? 10 : 9;
 constexpr int kRegCopies = 2;
 
 // Block-wide exclusive prefix sum of one value per thread (T threads); `wsum` holds T/32 words.  One barrier: every
@@ -231,6 +233,7 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* w
 template <int E, int T, int PD, bool kThr>
 __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
   pdl_wait();
+  constexpr int kBinBits = kRegBinBits<T>, kRegBins = 1 << kBinBits;
   extern __shared__ __align__(16) uint32_t smem[];
   uint32_t* wsum = smem;                               // [2][T/32]
   uint32_t* sh = wsum + 2 * (T / 32);                  // [0] chosen bin, [1] remaining need ... [6], [7] barrier
@@ -434,7 +437,7 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
 #pragma unroll 1
   for (int pass = 0; lo != hi; ++pass) {
     const uint32_t width = hi - lo;
-    const int shift = max(0, 32 - __clz(width) - 11);
+    const int shift = max(0, 32 - __clz(width) - kBinBits);
     const int copies = pass == 0 ? kRegCopies : 1;     // later passes see few candidates: one copy is enough
     uint32_t* my_hist = hist + (warp % copies) * kRegBins;
 #pragma unroll
@@ -558,7 +561,7 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
 // asked for as shared memory.
 template <int E, int T>
 constexpr int select_reg_smem_bytes(bool lists) {
-  const int hist = kRegCopies * kRegBins * 4, list = lists && E <= 16 ? E * T * 2 : 0;
+  const int hist = kRegCopies * (4 << kRegBinBits<T>), list = lists && E <= 16 ? E * T * 2 : 0;
   return (2 * (T / 32) + 8 + kFinishMax + 4) * 4 + (hist > list ? hist : list) + (E > 16 ? E * T * 4 : 0);
 }
 
@@ -597,10 +600,19 @@ sg_status select_launch(const sg_shape* shape, SelParams& p, SelectKind kind, vo
     else if (pd == 64) SG_LAUNCH_SELECT_REG_PD(E, T, 64, false);                \
     else SG_LAUNCH_SELECT_REG_PD(E, T, 0, false);                               \
   } while (0)
+  // Short rows take as many threads as have keys: with 512 for every row a wave held two rows per SM.  Microseconds with 512 threads -> with
+  // 128 (rows of up to 1024) or 256 (2048): the selection alone, 8 rows of 1000 4.3 -> 3.7, 256 of 1024 5.5 -> 4.0, 832 of 640 14.3 -> 5.1,
+  // 1280 of 100 20.9 -> 6.4, 256 of 2000 5.7 -> 4.7; by a threshold, 832 of 640 16.3 -> 10.1, 256 of 2000 7.6 -> 6.3, but 128 of 900 5.1 ->
+  // 6.0.  A gather needs threads for its rows on the way: 832 rows of 640 19.5 -> 9.2, but 256 of 1000, a fifth kept, 13.5 -> 15.9.
+  const int64_t fewest[] = {1, 4 * kNumSMs, kNumSMs};   // rows from which on, by kind
   if (rows < kNumSMs && kind != kPack && shape->max_seqlen <= 8192 && shape->max_seqlen > 4096) {
     // fewer rows than SMs: one CTA per SM anyway, so twice the threads per row (half the keys each) shorten the chains
     if (kind == kThreshold) SG_LAUNCH_SELECT_REG_PD(8, 1024, 0, true);
     else SG_LAUNCH_SELECT_REG_PD(8, 1024, 0, false);
+  } else if (shape->max_seqlen <= 1024 && rows >= fewest[kind]) {
+    SG_LAUNCH_SELECT_REG(8, 128);
+  } else if (shape->max_seqlen <= 2048 && (kind != kPack || rows >= fewest[kind])) {
+    SG_LAUNCH_SELECT_REG(8, 256);
   } else if (shape->max_seqlen <= 4096) {
     SG_LAUNCH_SELECT_REG(8, 512);
   } else if (shape->max_seqlen <= 8192) {

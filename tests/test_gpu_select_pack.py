@@ -47,6 +47,26 @@ def test_fused_route_bit_exact(lens, ks, L, Hkv, d):
     check(*case(3, lens, ks, L, Hkv, d))
 
 
+@pytest.mark.parametrize("lens", [
+    (1024, 5, 1023), (3, 1024), (1, 1021, 1024),            # <= 1024 tokens, rows that start on 16 bytes or 4, 8, 12 behind
+    (1025, 7), (2048, 1, 2047), (3, 2045, 2048),            # <= 2048
+    (2049, 2, 2051), (3, 4096), (1, 4095),                  # <= 4096
+])
+@pytest.mark.parametrize("ties", [False, True])
+def test_row_length_classes_and_alignments(lens, ties):
+    """Selection alone, with the gather, and by a threshold, at the edges of the classes of row lengths; a row of the full length
+    that does not start on 16 bytes has no room for the values in front of it."""
+    from test_gpu_threshold import run
+    L, Hkv = 60, 5
+    assert L * len(lens) * Hkv >= 4 * 148                   # as many rows as the gather's classes ask for
+    ks = tuple(max(1, n // 3) for n in lens)
+    imp, k, v, cu, ck = case(6, lens, ks, L, Hkv, 64, ties)
+    check(imp, k, v, cu, ck)
+    import gpu_ops
+    assert np.array_equal(gpu_ops.select_topk(imp, cu, ck), oracle.select_topk(imp, cu, ck))
+    run(np.minimum(imp, 2.0).astype(np.float32), lens, ks, 1.2 if ties else 1.7)
+
+
 @pytest.mark.parametrize("lens,ks,L,Hkv,d", [
     ((1024,), (128,), 1, 2, 64),                            # few rows: two kernels
     ((2048, 999), (205, 100), 2, 8, 128),
