@@ -207,10 +207,16 @@ __device__ __forceinline__ bool epilogue_merges(const ScoreParams& p, int part_t
   return helper_trips(p.Ralloc, nrec) > blocks_before + 2 + (p.Ralloc + 32 * kEpiWarps - 1) / (32 * kEpiWarps) * ((nrec + 11) / 12);
 }
 
-// kOwn (pass 2): the epilogue warps may merge later segments, too (plan_score says when).
-template <int D, int PASS, bool kOwn>
+// kVariant, pass 1: kTwice, for up to 64 query rows (below); pass 2: kOwn, the epilogue warps may merge later segments, too (plan_score
+// says when).  Kernels of their own: the branches cost the hot loops of the others 0.5 to 3 %.
+template <int D, int PASS, bool kVariant>
 __global__ void __launch_bounds__(kThreads, 1)
 score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k, const ScoreParams p) {
+  constexpr bool kOwn = PASS == 2 && kVariant;
+  // Up to 64 query rows leave half of the lanes of pass 1 with padding.  So the queries stand in rows 64 on once more, and the lanes of
+  // either half take half of the columns: the same MMAs, half of the exponentials.  Scores of 64 rows against heads of 64, in a row: 32 layers
+  // of 8192 tokens 138.8 -> 130.0 us, of 8 x 1500 63.8 -> 55.8, 13 of 8 x 640 52.3 -> 46.3, one of 32768 26.5 -> 24.7.
+  constexpr bool kTwice = PASS == 1 && kVariant;
   constexpr int kSub = D / 64;                        // 64-element (128-byte) sub-tiles along d
   constexpr int kKSubBytes = kTileKeys * 128;         // one sub-tile of a K stage
   constexpr int kKStageBytes = kSub * kKSubBytes;
@@ -302,12 +308,13 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
   if (p.R < p.Ralloc) {
     // Rows R..Ralloc-1 of the Q operands are never written by TMA: zero them once so that padded MMA
     // rows/columns are finite.  (The 128-byte swizzle only permutes 16-byte chunks inside a row's own 128 bytes.)
-    const int words = (p.Ralloc - p.R) * 32;
+    const int span = kTwice ? 64 : p.Ralloc, words = (span - p.R) * 32;
     for (int qb = 0; qb < p.q_bufs; ++qb)
-      for (int dc = 0; dc < kSub; ++dc) {
-        uint32_t* z = reinterpret_cast<uint32_t*>(q_smem + qb * q_buf_bytes + dc * q_sub_bytes + p.R * 128);
-        for (int i = tid; i < words; i += kThreads) z[i] = 0u;
-      }
+      for (int dc = 0; dc < kSub; ++dc)
+        for (int row = p.R; row < p.Ralloc; row += span) {
+          uint32_t* z = reinterpret_cast<uint32_t*>(q_smem + qb * q_buf_bytes + dc * q_sub_bytes + row * 128);
+          for (int i = tid; i < words; i += kThreads) z[i] = 0u;
+        }
     fence_proxy_async();
   }
   tc_fence_before();
@@ -345,10 +352,11 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
         ok = mbar_wait<kBehind>(bar_qempty(qs), (uint32_t)(((nq / p.q_bufs) & 1) ^ 1), abort_flag, p.wait_ns, 100u);
         if (!ok) break;
         ++nq;
-        mbar_arrive_expect_tx(bar_qfull(qs), (uint32_t)(kSub * p.G * p.W * 128));
+        mbar_arrive_expect_tx(bar_qfull(qs), (uint32_t)((kTwice ? 2 : 1) * kSub * p.G * p.W * 128));
 #pragma unroll
         for (int dc = 0; dc < kSub; ++dc)
-          tma_load_4d(smem_u32(q_smem + qs * q_buf_bytes + dc * q_sub_bytes), &tmap_q, bar_qfull(qs), dc * 64, g * p.G, 0, l * p.B + sg.b);
+          for (int at = 0; at <= (kTwice ? 64 : 0); at += 64)
+            tma_load_4d(smem_u32(q_smem + qs * q_buf_bytes + dc * q_sub_bytes + at * 128), &tmap_q, bar_qfull(qs), dc * 64, g * p.G, 0, l * p.B + sg.b);
         const int tiles = sg.tile_end - sg.tile_beg;
         for (int i = 0; i < tiles; ++i) {
           const int tile = tile_at<PASS>(sg, i), ks = nk % p.k_stages;
@@ -462,7 +470,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
         for (int i = 0; i < nblk; ++i) { sm_m[i * 128] = -INFINITY; sm_l[i * 128] = 0.f; }
         const bool all_rows = Weff == p.W;
         for (; n < n_end; n += kGroups) {
-          const uint32_t st = n & (kStages - 1), t_acc = t_lane + st * 128u;
+          const uint32_t st = n & (kStages - 1), col0 = kTwice && quarter >= 2 ? 64u : 0u, t_acc = t_lane + st * 128u + col0;
           SG_PROF_WAIT(w0, ok = wait(bar_afull(st), (n / kStages) & 1u));
           if (!ok) break;
           tc_fence_after();
@@ -488,12 +496,14 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
             uint64_t s0 = 0ull, s1 = 0ull;
             chunk_rows(a, scale2, nm2, s0, s1);
             tmem_ld_wait(b);
-            tmem_ld32_issue(a, t_acc + 64u);
-            chunk_rows(b, scale2, nm2, s0, s1);
-            tmem_ld_wait(a);
-            tmem_ld32_issue(b, t_acc + 96u);
-            chunk_rows(a, scale2, nm2, s0, s1);
-            tmem_ld_wait(b);
+            if (!kTwice) {
+              tmem_ld32_issue(a, t_acc + 64u);
+              chunk_rows(b, scale2, nm2, s0, s1);
+              tmem_ld_wait(a);
+              tmem_ld32_issue(b, t_acc + 96u);
+              chunk_rows(a, scale2, nm2, s0, s1);
+              tmem_ld_wait(b);
+            }
             chunk_rows(b, scale2, nm2, s0, s1);
             float lo, hi;
             unpack2(add2(s0, s1), lo, hi);
@@ -502,12 +512,13 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
             if (!careful) l += s;
           }
           if (careful) {
-            const int r = blk * 128 + row_in_tile;
-            const int cmax = r < p.R && r / p.G < Weff ? first_win + r / p.G - tile * kTileKeys : -1;    // last visible column of this tile
+            const int r = kTwice ? row_in_tile & 63 : blk * 128 + row_in_tile, chunks = kTwice ? 2 : 4;
+            // last visible column of this tile, counted from the first one that the thread takes
+            const int cmax = r < p.R && r / p.G < Weff ? first_win + r / p.G - tile * kTileKeys - (int)col0 : -1;
             float mx = -INFINITY;
             uint32_t cur[32];
 #pragma unroll 1
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < chunks; ++j) {
               tmem_ld32_issue(cur, t_acc + (uint32_t)(j * 32));
               tmem_ld_wait(cur);
 #pragma unroll
@@ -518,7 +529,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
             if (mn != -INFINITY) { l *= exp2f(m - mn); m = mn; }
             const float ref = mn == -INFINITY ? 0.f : mn;
 #pragma unroll 1
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < chunks; ++j) {
               tmem_ld32_issue(cur, t_acc + (uint32_t)(j * 32));
               tmem_ld_wait(cur);
               float s0 = 0.f, s1 = 0.f;
@@ -641,13 +652,17 @@ score_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__
         if (!ok) break;
         const float* sm = stat + (size_t)buf * kGroups * 2 * p.Ralloc;
         float2* rec = p.records + (size_t)(sg.part + (int)blockIdx.x) * p.Ralloc;
-        for (int r = hw * 32 + lane; r < p.Ralloc; r += 64) {
-          float m[kGroups], M = -INFINITY, L = 0.f;
+        for (int r = hw * 32 + lane; r < (kTwice ? 64 : p.Ralloc); r += 64) {
+          float m[2 * kGroups], M = -INFINITY, L = 0.f;
 #pragma unroll
-          for (int w = 0; w < kGroups; ++w) { m[w] = sm[w * 2 * p.Ralloc + r]; M = fmaxf(M, m[w]); }
+          for (int w = 0; w < 2 * kGroups; ++w) {      // (the second half only where the rows stand twice)
+            m[w] = w < kGroups || kTwice ? sm[w % kGroups * 2 * p.Ralloc + r + w / kGroups * 64] : -INFINITY;
+            M = fmaxf(M, m[w]);
+          }
           const float Mu = M == -INFINITY ? 0.f : M;
 #pragma unroll
-          for (int w = 0; w < kGroups; ++w) L += sm[(w * 2 + 1) * p.Ralloc + r] * exp2f(m[w] - Mu);
+          for (int w = 0; w < 2 * kGroups; ++w)
+            if (w < kGroups || kTwice) L += sm[(w % kGroups * 2 + 1) * p.Ralloc + r + w / kGroups * 64] * exp2f(m[w] - Mu);
           rec[r] = make_float2(M, L);
         }
         __syncwarp();
@@ -784,9 +799,9 @@ ScorePlan plan_score(const sg_shape* s, size_t limit = 0) {
   return pl;
 }
 
-template <int D, int PASS, bool kOwn>
+template <int D, int PASS, bool kVariant>
 sg_status launch_pass(const CUtensorMap& q, const CUtensorMap& k, const ScoreParams& p, const ScorePlan& pl, cudaStream_t s) {
-  SG_ENSURE_SMEM((score_kernel<D, PASS, kOwn>), pl.smem_bytes);
+  SG_ENSURE_SMEM((score_kernel<D, PASS, kVariant>), pl.smem_bytes);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)pl.grid);
   cfg.blockDim = dim3(kThreads);
@@ -797,7 +812,7 @@ sg_status launch_pass(const CUtensorMap& q, const CUtensorMap& k, const ScorePar
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  SG_CUDA_TRY(cudaLaunchKernelEx(&cfg, score_kernel<D, PASS, kOwn>, q, k, p));
+  SG_CUDA_TRY(cudaLaunchKernelEx(&cfg, score_kernel<D, PASS, kVariant>, q, k, p));
   return SG_OK;
 }
 
@@ -910,7 +925,8 @@ sg_status run_score(const sg_shape* shape, const void* q_win, const void* k_cach
   if (cluster) return score_cluster_launch(shape, tmap_q, tmap_k, ScoreLaunch{importance, dev_status, p.withhold_unit, p.wait_ns, s}, pack);
   p.units = pl.U;
   p.records = static_cast<float2*>(workspace);
-  st = D == 128 ? launch_pass<128, 1, false>(tmap_q, tmap_k, p, pl, s) : launch_pass<64, 1, false>(tmap_q, tmap_k, p, pl, s);
+  if (p.R <= 64) st = D == 128 ? launch_pass<128, 1, true>(tmap_q, tmap_k, p, pl, s) : launch_pass<64, 1, true>(tmap_q, tmap_k, p, pl, s);
+  else st = D == 128 ? launch_pass<128, 1, false>(tmap_q, tmap_k, p, pl, s) : launch_pass<64, 1, false>(tmap_q, tmap_k, p, pl, s);
   if (st != SG_OK) return st;
   if (pl.own) return D == 128 ? launch_pass<128, 2, true>(tmap_q, tmap_k, p, pl, s) : launch_pass<64, 2, true>(tmap_q, tmap_k, p, pl, s);
   return D == 128 ? launch_pass<128, 2, false>(tmap_q, tmap_k, p, pl, s) : launch_pass<64, 2, false>(tmap_q, tmap_k, p, pl, s);

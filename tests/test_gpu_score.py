@@ -120,3 +120,25 @@ def test_score_late_key_far_above_everything_before_it():
         got = gpu_ops.score(qb, kb, cu)
         assert_close(got, want)
         assert np.all(np.isfinite(got)) and np.abs(got[:, :, where] - W).max() < 1e-2
+
+
+@pytest.mark.parametrize("lens,L,W,Hq,Hkv,d", [
+    ((3000, 129, 5, 1), 3, 16, 8, 2, 64),              # 64 rows: both halves full; prompts shorter than the window
+    ((2000, 700), 2, 15, 8, 2, 128),                   # 60 rows
+    ((1025,), 4, 3, 16, 8, 64),                        # 6 rows
+    ((1000, 64, 300), 2, 1, 4, 4, 128),                # a single row
+    ((1500, 300), 2, 13, 10, 2, 64),                   # 65 rows: the first count that does not stand twice
+])
+def test_score_few_query_rows_in_two_launches(lens, L, W, Hq, Hkv, d):
+    """Up to 64 rows stand twice in pass 1, each half of the lanes with half of the key columns."""
+    import torch
+    import gpu_ops
+    import paper_2607_28150_b200.binding as sg
+    rng = np.random.default_rng(8)
+    cu = cu_of(lens)
+    q, k = rand_bf16(rng, (L, len(lens), W, Hq, d)), rand_bf16(rng, (L, int(cu[-1]), Hkv, d))
+    k[:, 100 % int(cu[-1])] = rand_bf16(rng, (L, Hkv, d), 6.0)         # a key far above its row's first columns
+    imp, st = torch.full((L, Hkv, int(cu[-1])), -7.0, device="cuda"), gpu_ops.status_word()
+    sg.sg_score_static(gpu_ops.shape_of(L, Hq, Hkv, d, W, cu), gpu_ops.dev(q), gpu_ops.dev(k), imp, st)
+    assert gpu_ops.read_status(st) == 0
+    assert_close(imp.cpu().numpy(), oracle.score(q, k, cu))
