@@ -135,7 +135,10 @@ static __device__ __noinline__ bool mbar_wait_cluster(uint32_t bar, volatile int
     }
   }
 }
-template <int D, bool kPack>
+// kTwice: up to 64 query rows stand twice, as in pass 1 of score.cu; else half of the warps, those of two of the four schedulers, would have
+// padding (one layer of 8192 tokens, 8 heads of 64, 21.0 -> 19.3 us, 3000 tokens 13.4 -> 12.8; a kernel of its
+// own, because as a branch it cost 128 rows of 2048 tokens 0.3 us).
+template <int D, bool kPack, bool kTwice>
 __global__ void __launch_bounds__(kThreads, 1)
 score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k, const ClusterParams p) {
   constexpr int kSub = D / 64;
@@ -179,7 +182,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
     for (int s = 0; s < kStages; ++s) { mbar_init(bar_afull(s), 1); mbar_init(bar_aempty(s), kWorkWarps); }
     *abort_flag = 0;
     fence_barrier_init();
-    mbar_arrive_expect_tx(bar_rec, (uint32_t)(p.csize * p.Ralloc * 8));
+    mbar_arrive_expect_tx(bar_rec, (uint32_t)(p.csize * (kTwice ? 64 : p.Ralloc) * 8));
   }
   if (warp == kIssueWarp) {
     tmem_alloc(smem_u32(tmem_slot), 512);
@@ -197,11 +200,12 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
     if (kPack) reinterpret_cast<uint4*>(hist)[tid] = make_uint4(0, 0, 0, 0);
     if (p.R < p.Ralloc) {
       // rows R.. of Q are never written by TMA: zero, so that padded MMA columns are finite
-      const int words = (p.Ralloc - p.R) * 32;
-      for (int dc = 0; dc < kSub; ++dc) {
-        uint32_t* z = reinterpret_cast<uint32_t*>(q_smem + dc * p.Ralloc * 128 + p.R * 128);
-        for (int i = tid; i < words; i += kWork) z[i] = 0u;
-      }
+      const int span = kTwice ? 64 : p.Ralloc, words = (span - p.R) * 32;
+      for (int dc = 0; dc < kSub; ++dc)
+        for (int row = p.R; row < p.Ralloc; row += span) {
+          uint32_t* z = reinterpret_cast<uint32_t*>(q_smem + dc * p.Ralloc * 128 + row * 128);
+          for (int i = tid; i < words; i += kWork) z[i] = 0u;
+        }
       fence_proxy_async();
     }
   }
@@ -231,10 +235,11 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
     used |= 1u << s;
   };
   if (warp == kLoadWarp && lane == 0 && n_my > 0) {
-    mbar_arrive_expect_tx(bar_q, (uint32_t)(kSub * p.G * p.W * 128));
+    mbar_arrive_expect_tx(bar_q, (uint32_t)((kTwice ? 2 : 1) * kSub * p.G * p.W * 128));
 #pragma unroll
     for (int dc = 0; dc < kSub; ++dc)
-      tma_load_4d(smem_u32(q_smem + dc * p.Ralloc * 128), &tmap_q, bar_q, dc * 64, g * p.G, 0, l * p.B + b);
+      for (int at = 0; at <= (kTwice ? 64 : 0); at += 64)
+        tma_load_4d(smem_u32(q_smem + dc * p.Ralloc * 128 + at * 128), &tmap_q, bar_q, dc * 64, g * p.G, 0, l * p.B + b);
     for (int i = 0; i < min(n_my, p.cap); ++i) load(i, 0);
   }
   tc_fence_before();
@@ -330,44 +335,61 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
       const bool hidden = tile >= vis_end || Weff != p.W;
       for (int blk = 0; blk < nblk; ++blk, ++n) {
         const uint32_t st = n & (kStages - 1);
-        const int r = blk * 128 + lane_row, at = part_c * p.Ralloc + r;
         ok = wait(bar_afull(st), (n / kStages) & 1u);
         if (!ok) break;
         tc_fence_after();
-        if (blk * 128 + quarter * 32 >= p.R) { release(st); continue; }
-        uint32_t a[32];
-        tmem_ld32_issue(a, t_lane + st * 128u + part_c * 32u);
-        tmem_ld_wait(a);
-        release(st);
-        if (hidden) {
-          const int cmax = (r < p.R && r / p.G < Weff ? first_win + r / p.G - tile * kTileKeys : -1) - part_c * 32;     // last visible column
+        auto rows_of = [&](auto& a, int r, int col0) {  // row r, columns from col0 on
+          constexpr int kCols = sizeof(a) / 4;
+          if (hidden) {
+            const int cmax = (r < p.R && r / p.G < Weff ? first_win + r / p.G - tile * kTileKeys : -1) - col0;     // last visible column
 #pragma unroll
-          for (int c = 0; c < 32; ++c) a[c] = c <= cmax ? a[c] : 0xff800000u;
+            for (int c = 0; c < kCols; ++c) a[c] = c <= cmax ? a[c] : 0xff800000u;
+          }
+          float x = fmaxf(__uint_as_float(a[0]), __uint_as_float(a[1]));
+#pragma unroll
+          for (int c = 2; c < kCols; c += 2) x = max3(x, __uint_as_float(a[c]), __uint_as_float(a[c + 1]));
+          const int at = part_c * p.Ralloc + blk * 128 + lane_row;
+          const float m = slot_m[at], mn = fmaxf(m, x * p.scale_log2);
+          const float ref = mn == -INFINITY ? 0.f : mn;  // nothing visible yet: all terms are 0 (or NaN)
+          uint64_t s0 = 0ull, s1 = 0ull;
+          chunk_rows(a, scale2, pack2(-ref, -ref), s0, s1);
+          float lo, hi;
+          unpack2(add2(s0, s1), lo, hi);
+          slot_l[at] = slot_l[at] * exp2f(m - ref) + (lo + hi);
+          slot_m[at] = mn;
+        };
+        if constexpr (kTwice) {
+          const int col0 = part_c * 32 + (quarter >> 1) * 16;
+          uint32_t a[16];
+          tmem_ld16_issue(a, t_lane + st * 128u + col0);
+          tmem_ld_wait(a);
+          release(st);
+          if ((quarter & 1) * 32 < p.R) rows_of(a, lane_row & 63, col0);
+        } else {
+          if (blk * 128 + quarter * 32 >= p.R) { release(st); continue; }
+          uint32_t a[32];
+          tmem_ld32_issue(a, t_lane + st * 128u + part_c * 32u);
+          tmem_ld_wait(a);
+          release(st);
+          rows_of(a, blk * 128 + lane_row, part_c * 32);
         }
-        float x = fmaxf(__uint_as_float(a[0]), __uint_as_float(a[1]));
-#pragma unroll
-        for (int c = 2; c < 32; c += 2) x = max3(x, __uint_as_float(a[c]), __uint_as_float(a[c + 1]));
-        const float m = slot_m[at], mn = fmaxf(m, x * p.scale_log2);
-        const float ref = mn == -INFINITY ? 0.f : mn;  // nothing visible yet: all terms are 0 (or NaN)
-        uint64_t s0 = 0ull, s1 = 0ull;
-        chunk_rows(a, scale2, pack2(-ref, -ref), s0, s1);
-        float lo, hi;
-        unpack2(add2(s0, s1), lo, hi);
-        slot_l[at] = slot_l[at] * exp2f(m - ref) + (lo + hi);
-        slot_m[at] = mn;
       }
     }
     ok = work_sync(ok);
     // ---- exchange: every CTA gets every CTA's statistics
     cluster_wait();                                    // all CTAs of the cluster run
     if (ok && u != p.withhold_unit) {
-      for (int r = tid & 127; r < p.Ralloc; r += 128) {
-        float m[4], M = -INFINITY, L = 0.f;
+      for (int r = tid & 127; r < (kTwice ? 64 : p.Ralloc); r += 128) {
+        float m[8], M = -INFINITY, L = 0.f;
 #pragma unroll
-        for (int w = 0; w < 4; ++w) { m[w] = slot_m[w * p.Ralloc + r]; M = fmaxf(M, m[w]); }
+        for (int w = 0; w < 8; ++w) {                  // (the second half only where the rows stand twice)
+          m[w] = w < 4 || kTwice ? slot_m[(w & 3) * p.Ralloc + r + (w >> 2) * 64] : -INFINITY;
+          M = fmaxf(M, m[w]);
+        }
         const float Mu = M == -INFINITY ? 0.f : M;
 #pragma unroll
-        for (int w = 0; w < 4; ++w) L += slot_l[w * p.Ralloc + r] * exp2f(m[w] - Mu);
+        for (int w = 0; w < 8; ++w)
+          if (w < 4 || kTwice) L += slot_l[(w & 3) * p.Ralloc + r + (w >> 2) * 64] * exp2f(m[w] - Mu);
         const uint32_t own_rec = smem_u32(rec + rank * p.Ralloc + r);
         for (int to = tid >> 7; to < p.csize; to += 4) push2(at_rank(own_rec, to), at_rank(bar_rec, to), __float_as_uint(M), __float_as_uint(L));
       }
@@ -710,7 +732,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
 // ---------------------------------------------------------------- host side
 constexpr int kSmemLimit = 232448, kMaxCluster = 16;
 
-template <int D, bool kPack>
+template <int D, bool kPack, bool kTwice>
 cudaError_t prepare_kernel() {
   // once per device: the clusters' size may exceed the portable eight, the shared memory the default
   static std::atomic<int> done[64];
@@ -718,8 +740,8 @@ cudaError_t prepare_kernel() {
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev >= 0 && dev < 64 && done[dev].load(std::memory_order_relaxed)) return cudaSuccess;
-  e = cudaFuncSetAttribute(score_cluster_kernel<D, kPack>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(score_cluster_kernel<D, kPack>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  e = cudaFuncSetAttribute(score_cluster_kernel<D, kPack, kTwice>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(score_cluster_kernel<D, kPack, kTwice>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev].store(1, std::memory_order_relaxed);
   return e;
 }
@@ -731,7 +753,7 @@ int clusters_at_once(int csize) {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
   int n = known[dev][csize].load(std::memory_order_relaxed);
   if (n == 0) {
-    if (prepare_kernel<128, true>() != cudaSuccess) return 0;
+    if (prepare_kernel<128, true, false>() != cudaSuccess) return 0;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
@@ -742,7 +764,7 @@ int clusters_at_once(int csize) {
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int got = 0;
-    if (cudaOccupancyMaxActiveClusters(&got, score_cluster_kernel<128, true>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&got, score_cluster_kernel<128, true, false>, &cfg) != cudaSuccess) {
       (void)cudaGetLastError();
       got = 0;
     }
@@ -778,9 +800,9 @@ ClusterPlan plan_cluster(const sg_shape* s, int Ralloc, bool packs) {
   return pl;
 }
 
-template <int D, bool kPack>
-sg_status launch(const CUtensorMap& q, const CUtensorMap& k, const ClusterParams& p, const ClusterPlan& pl, const sg_shape* shape, cudaStream_t s) {
-  SG_CUDA_TRY((prepare_kernel<D, kPack>()));
+template <int D, bool kPack, bool kTwice>
+sg_status launch_kernel(const CUtensorMap& q, const CUtensorMap& k, const ClusterParams& p, const ClusterPlan& pl, const sg_shape* shape, cudaStream_t s) {
+  SG_CUDA_TRY((prepare_kernel<D, kPack, kTwice>()));
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -793,8 +815,12 @@ sg_status launch(const CUtensorMap& q, const CUtensorMap& k, const ClusterParams
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  SG_CUDA_TRY(cudaLaunchKernelEx(&cfg, score_cluster_kernel<D, kPack>, q, k, p));
+  SG_CUDA_TRY(cudaLaunchKernelEx(&cfg, score_cluster_kernel<D, kPack, kTwice>, q, k, p));
   return SG_OK;
+}
+template <int D, bool kPack>
+sg_status launch(const CUtensorMap& q, const CUtensorMap& k, const ClusterParams& p, const ClusterPlan& pl, const sg_shape* shape, cudaStream_t s) {
+  return p.R <= 64 ? launch_kernel<D, kPack, true>(q, k, p, pl, shape, s) : launch_kernel<D, kPack, false>(q, k, p, pl, shape, s);
 }
 
 }  // namespace

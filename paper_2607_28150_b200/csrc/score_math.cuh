@@ -83,10 +83,11 @@ __device__ __forceinline__ uint64_t exp2_fma2(uint64_t x) {
 // Pairs of a 32-column chunk's sixteen whose exponentials run on the FMA pipe, spread evenly.
 constexpr int kFmaPairs1 = 4, kFmaPairs2 = 4;
 __device__ __forceinline__ constexpr bool on_fma(int pair, int share) { return ((pair + 1) * share) / 16 != (pair * share) / 16; }
-// Pass 1: adds exp2(score * scale - m) of a chunk's columns to two pairs of accumulators (nm2 = {-m, -m}).
-__device__ __forceinline__ void chunk_rows(uint32_t (&cur)[32], uint64_t scale2, uint64_t nm2, uint64_t& s0, uint64_t& s1) {
+// Pass 1: adds exp2(score * scale - m) of a chunk's 32 (or 16) columns to two pairs of accumulators (nm2 = {-m, -m}).
+template <int kCols>
+__device__ __forceinline__ void chunk_rows(uint32_t (&cur)[kCols], uint64_t scale2, uint64_t nm2, uint64_t& s0, uint64_t& s1) {
 #pragma unroll
-  for (int i = 0; i < 16; i += 2) {
+  for (int i = 0; i < kCols / 2; i += 2) {
     const uint64_t x0 = fma2(pair_of(cur + 2 * i), scale2, nm2), x1 = fma2(pair_of(cur + 2 * i + 2), scale2, nm2);
     s0 = add2(s0, on_fma(i, kFmaPairs1) ? exp2_fma2<true>(x0) : exp2_sfu2(x0));
     s1 = add2(s1, on_fma(i + 1, kFmaPairs1) ? exp2_fma2<true>(x1) : exp2_sfu2(x1));
