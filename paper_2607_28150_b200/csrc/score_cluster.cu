@@ -698,6 +698,8 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
         __syncwarp();
         cluster_arrive();
       }
+      // the host's total is larger than cu_k[B]: as sg_pack_kv, entries that no row owns are not written
+      if (rank == 0 && l == 0 && g == 0 && b == p.B - 1 && tid == 0 && ck + kb < p.K_tot) raise(p.dev_status, SG_ERR_INVALID);
       if (kb > 0 && !fits) {
         // longer than max_seqlen promised: as sg_select_pack_kv
         if (rank == 0 && tid == 0) { raise(p.dev_status, SG_ERR_INVALID); raise(p.dev_status, SG_ERR_INDEX); }

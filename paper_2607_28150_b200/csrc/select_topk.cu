@@ -252,6 +252,8 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
   const int N = p.cu[b + 1] - c0;
   const int ck = p.cu_k[b];
   const int kb = p.cu_k[b + 1] - ck;
+  // the host's total is larger than cu_k[B]: as sg_pack_kv, entries that no row owns are not written
+  if (PD > 0 && row == (int)gridDim.x - 1 && tid == 0 && ck + kb < p.K_tot) raise(p.dev_status, SG_ERR_INVALID);
   auto write_count = [&](int n) { if (kThr && tid == 0) p.sel_count[((int64_t)l * p.B + b) * p.Hkv + g] = n; };
   if (kb <= 0) { write_count(0); return; }
   int32_t* out = p.sel_idx + ((int64_t)l * p.Hkv + g) * p.K_tot + ck;

@@ -247,6 +247,47 @@ def test_pack_total_above_the_prefix_array(B, counted):
         assert np.array_equal(got[0, :K], want) and np.all(got[0, K:] == 0x5555)
 
 
+@pytest.mark.parametrize("call", ["prefill", "prefill_layer", "select_pack"])
+@pytest.mark.parametrize("L,lens,Hkv", [
+    (1, (900,), 2), (1, (900, 40, 300), 2),                # one kernel for scoring, selection and packing
+    (8, (400,), 20), (8, (400, 30), 10),                   # 160 rows: selection and packing in one kernel
+    (1, (20000, 9000), 4),                                 # the calls one by one
+])
+def test_selection_total_above_the_prefix_array(call, L, lens, Hkv):
+    """The same through the calls that select and pack: the status bit of sg_pack_kv, and every row of the prefix array right."""
+    import torch
+    import gpu_ops
+    import paper_2607_28150_b200.binding as sg
+    rng = np.random.default_rng(19)
+    W, d, more = 8, 64, 50
+    if call == "prefill_layer":
+        L = 1
+    ks = tuple(max(1, n // 7) for n in lens)
+    cu, ck = cu_of(lens), cu_of(ks)
+    T, Kb = int(cu[-1]), int(ck[-1])
+    K = Kb + more
+    q, k, v = rand_bf16(rng, (L, len(lens), W, Hkv, d)), rand_bf16(rng, (L, T, Hkv, d)), rand_bf16(rng, (L, T, Hkv, d))
+    x = rng.standard_normal((L, Hkv, T)).astype(np.float32)
+    shp, st, d_ck = gpu_ops.shape_of(L, Hkv, Hkv, d, W, cu), gpu_ops.status_word(), gpu_ops.dev(ck)
+    imp, sel = gpu_ops.dev(x), torch.full((L, Hkv, K), -99, dtype=torch.int32, device="cuda")
+    pk, pv = (gpu_ops.Guarded((L, K * Hkv, d), torch.int16, 0x5555) for _ in range(2))
+    ws = sg.alloc_workspace(sg.SG_OP_SCORE, shp)
+    if call == "prefill":
+        sg.prefill(shp, gpu_ops.dev(q), gpu_ops.dev(k), gpu_ops.dev(v), imp, ws, d_ck, K, sel, pk.view, pv.view, st)
+    elif call == "prefill_layer":
+        sg.prefill_layer(shp, 0, gpu_ops.dev(q), gpu_ops.dev(k), gpu_ops.dev(v), imp, ws, d_ck, K, sel, pk.view, pv.view, st)
+    else:
+        sg.sg_select_pack_kv(shp, imp, d_ck, K, gpu_ops.dev(k), gpu_ops.dev(v), sel, pk.view, pv.view, st)
+    got_k, got_v = pk.numpy(), pv.numpy()
+    assert gpu_ops.read_status(st) == 1 << sg.SG_ERR_INVALID
+    sel = sel.cpu().numpy()
+    want = oracle.select_topk(imp.cpu().numpy(), cu, ck)
+    assert np.array_equal(sel[:, :, :Kb], want) and np.all(sel[:, :, Kb:] == -99)
+    want_k, want_v = oracle.pack_kv(k, v, cu, want, ck)
+    for got, rows in ((got_k, want_k), (got_v, want_v)):
+        assert np.array_equal(got[:, :Kb * Hkv], rows) and np.all(got[:, Kb * Hkv:] == 0x5555)
+
+
 @pytest.mark.parametrize("lens,L,W,Hq,Hkv,d", [
     # such a part as a CTA's second, third and fourth segment, between segments that the helper merges: 384 rows, 1024 rows
     ((12478, 16, 31, 15649, 31, 99, 84, 17425, 94, 32, 10011, 52, 89, 84), 1, 24, 16, 1, 128),
