@@ -336,7 +336,8 @@ def sg_push_blocks(shape: Shape, num_blocks: int, layer: int, selected: Optional
 def prefill(shape: Shape, q_win: torch.Tensor, k_cache: torch.Tensor, v_cache: torch.Tensor, importance: torch.Tensor,
             workspace: Optional[torch.Tensor], cu_k: torch.Tensor, total_sel: int, sel_idx: torch.Tensor, packed_k: torch.Tensor,
             packed_v: torch.Tensor, dev_status: Optional[torch.Tensor] = None, stream=None) -> None:
-    """sg_score, then sg_select_pack_kv, marshalled once."""
+    """sg_score, then sg_select_pack_kv, marshalled once; small calls run as one kernel.  With SG_ERR_TIMEOUT in the status word the
+    outputs are not to be used; a part whose wait ran out in that one kernel has -1 and zero rows throughout."""
     rc = _native.prefill(shape, q_win, k_cache, v_cache, importance, workspace, cu_k, total_sel, sel_idx, packed_k, packed_v, dev_status,
                          stream)
     if rc:

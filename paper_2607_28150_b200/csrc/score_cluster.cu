@@ -52,7 +52,7 @@ constexpr int kBins = 2048;
 constexpr int kRankMax = 128;            // keys that are ranked directly
 constexpr int kSweeps = (kMaxOwn * kTileKeys + kWork - 1) / kWork;
 constexpr int kCandAt = (24 + kSweeps * kWorkWarps + 3) & ~3;
-constexpr int kMiscWords = kCandAt + kRankMax + 4;
+constexpr int kFailedAt = kCandAt + kRankMax + 4, kMiscWords = kFailedAt + 4;
 constexpr int kBars = 2 * kMaxCap + 16;
 
 struct ClusterParams {
@@ -95,6 +95,7 @@ __host__ __device__ __forceinline__ Carve carve(int D, int Ralloc, int csize, in
 
 // Relaxed: what the CTAs tell each other is ordered by mbarriers; a releasing arrival took 0.4 us.
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ uint32_t at_rank(uint32_t addr, int rank) {
   uint32_t r;
@@ -135,6 +136,35 @@ static __device__ __noinline__ bool mbar_wait_cluster(uint32_t bar, volatile int
     }
   }
 }
+// Entries from `from` on of a part's kb that name no position: -1 and zero rows, by the workers of all CTAs of the part.
+template <int D>
+__device__ __forceinline__ void clear_entries(int32_t* out, uint16_t* rows_k, uint16_t* rows_v, int from, int kb, int worker, int rank, int csize) {
+  constexpr int kTPR = D / 8, kRowGroups = kWork / kTPR;
+  const int x = worker % kTPR, grp = worker / kTPR;
+  for (int j = from + rank * kRowGroups + grp; j < kb; j += csize * kRowGroups) {
+    if (x == 0) out[j] = -1;
+    *reinterpret_cast<int4*>(rows_k + (int64_t)j * D + x * 8) = make_int4(0, 0, 0, 0);
+    *reinterpret_cast<int4*>(rows_v + (int64_t)j * D + x * 8) = make_int4(0, 0, 0, 0);
+  }
+}
+// A CTA gives up (the workers' first warp): every CTA of the cluster knows it behind the cluster barrier that this warp arrives at.
+__device__ __noinline__ void tell_failed(uint32_t failed, int csize) {
+  const int lane = threadIdx.x & 31;
+  if (lane < csize) asm volatile("st.shared::cluster.u32 [%0], 1;" ::"r"(at_rank(failed, lane)) : "memory");
+  __syncwarp();
+  cluster_arrive_release();
+}
+// All CTAs of a cluster of which one has given up.  It does not know its entries, so none of the part's rows may pass for selected ones.
+// (Out of line, as tell_failed: inside the kernel they cost every call 0.5 us.)
+template <int D, bool kPack>
+__device__ __noinline__ void give_up(const int32_t* cu_k, int32_t* sel_idx, uint16_t* packed_k, uint16_t* packed_v, int K_tot, int Hkv, int csize) {
+  cluster_arrive_release();                            // behind what the other CTAs have packed
+  cluster_wait();
+  if (!kPack || threadIdx.x >= kWork) return;
+  const int l = blockIdx.z, b = blockIdx.y / Hkv, g = blockIdx.y - b * Hkv, ck = cu_k[b], kb = cu_k[b + 1] - ck;
+  const int64_t row0 = (((int64_t)l * K_tot + ck) * Hkv + (int64_t)g * kb) * D;
+  clear_entries<D>(sel_idx + ((int64_t)l * Hkv + g) * K_tot + ck, packed_k + row0, packed_v + row0, 0, kb, threadIdx.x, blockIdx.x, csize);
+}
 // kTwice: up to 64 query rows stand twice, as in pass 1 of score.cu; else half of the warps, those of two of the four schedulers, would have
 // padding (one layer of 8192 tokens, 8 heads of 64, 21.0 -> 19.3 us, 3000 tokens 13.4 -> 12.8; a kernel of its
 // own, because as a branch it cost 128 rows of 2048 tokens 0.3 us).
@@ -170,6 +200,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
   uint32_t* const wsum = misc + 8;                     // [16]
   uint32_t* const wsum2 = misc + 24;                   // [kSweeps][16] selected keys by warp
   uint32_t* const cand = misc + kCandAt;               // [kRankMax + 4]
+  volatile uint32_t* const failed = misc + kFailedAt;  // a CTA of this cluster has given up (it writes the word of every CTA)
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // (an integer division takes a hundred clocks: none where there is one sequence, or where all tiles fit)
@@ -188,6 +219,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
     tmem_alloc(smem_u32(tmem_slot), 512);
     tmem_relinquish();
   }
+  if (warp == kLoadWarp && lane == 1) *failed = 0;
   if (warp == kLoadWarp && lane == 0) {
     tma_prefetch_map(&tmap_q);
     tma_prefetch_map(&tmap_k);
@@ -245,7 +277,10 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  cluster_arrive();                                    // "this CTA runs and its barriers are set up": awaited before the first push
+  // "this CTA runs and its barriers are set up": awaited before the first push.  The arrival of the warp that wrote `failed` releases
+  // it: 0.3 us, which this warp has.
+  if (warp == kLoadWarp) cluster_arrive_release();
+  else cluster_arrive();
   const uint32_t tmem_base = *tmem_slot;
   auto wait = [&](uint32_t bar, uint32_t parity) {
     if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return true;
@@ -266,6 +301,9 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
         if ((used >> s) & 1u) mbar_wait<true>(bar_kfull(s), (odd >> s) & 1u, &never, p.wait_ns, 100u);
       mbar_wait<true>(bar_q, 0u, &never, p.wait_ns, 100u);
     }
+    // the host's total is larger than cu_k[B]: flagged, as by sg_pack_kv, and entries that no row owns are not written (here, because the
+    // workers' chain of steps is what the call takes)
+    if (kPack && lane == 1 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0 && p.cu_k[p.B] < p.K_tot) raise(p.dev_status, SG_ERR_INVALID);
     __syncwarp();
     cluster_wait();
     cluster_arrive();
@@ -323,6 +361,12 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
     int ck = 0, kb = 0;
     if (kPack) { ck = p.cu_k[b]; kb = p.cu_k[b + 1] - ck; }
     const bool selects = kPack && fits && kb > 0 && kb < N;
+    // "this CTA has received everything, and sends nothing more"; or it has given up (`ok` is that of all workers)
+    auto last_arrive = [&] {
+      __syncwarp();
+      if (__builtin_expect(!ok && warp == 0, 0)) tell_failed(smem_u32(const_cast<uint32_t*>(failed)), p.csize);
+      else cluster_arrive();
+    };
     if (selects && tid == 0) mbar_arrive_expect_tx(bar_val, (uint32_t)((ntiles - n_my) * kTileKeys * 4 + ntiles * 8));
 
     // ---- 1. row statistics: a running (maximum, sum of exp2) of the thread's row over its quarter of the columns
@@ -540,14 +584,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
           }
         }
       };
-      auto zero_rows = [&](int from) {                 // entries without a position, over all CTAs of the part
-        for (int j = from + rank * kRowGroups + grp; j < kb; j += p.csize * kRowGroups) {
-          if (x == 0) out[j] = -1;
-          const int64_t dst = (row0 + j) * D + x * 8;
-          *reinterpret_cast<int4*>(p.packed_k + dst) = make_int4(0, 0, 0, 0);
-          *reinterpret_cast<int4*>(p.packed_v + dst) = make_int4(0, 0, 0, 0);
-        }
-      };
+      auto zero_rows = [&](int from) { clear_entries<D>(out, p.packed_k + row0 * D, p.packed_v + row0 * D, from, kb, tid, rank, p.csize); };
       for (int i = 0; i < min(n_my, p.cap) && ok; ++i)  // the tiles' bytes are seen by this thread (the MMAs have used them long ago)
         ok = wait(bar_kfull(i), (uint32_t)(phase2(i) & 1));
       if (selects) {
@@ -556,7 +593,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
         __syncwarp();
         if (ok) ok = wait_cluster(bar_val);
         ok = work_sync(ok);
-        cluster_arrive();                              // this CTA has received everything, and sends nothing more
+        last_arrive();
         if (ok) {
           uint32_t lo = 0xffffffffu, hi = 0u, need = (uint32_t)kb;
           for (int i = lane; i < ntiles; i += 32) { const uint2 v = minmax[i]; lo = min(lo, v.x); hi = max(hi, v.y); }
@@ -695,11 +732,9 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
           pack_own(count, (int)first, [&](int j) { return list[j]; });
         }
       } else {
-        __syncwarp();
-        cluster_arrive();
+        ok = work_sync(ok);
+        last_arrive();
       }
-      // the host's total is larger than cu_k[B]: as sg_pack_kv, entries that no row owns are not written
-      if (rank == 0 && l == 0 && g == 0 && b == p.B - 1 && tid == 0 && ck + kb < p.K_tot) raise(p.dev_status, SG_ERR_INVALID);
       if (kb > 0 && !fits) {
         // longer than max_seqlen promised: as sg_select_pack_kv
         if (rank == 0 && tid == 0) { raise(p.dev_status, SG_ERR_INVALID); raise(p.dev_status, SG_ERR_INDEX); }
@@ -714,14 +749,14 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
         zero_rows(N);
       }
     } else {
-      __syncwarp();
-      cluster_arrive();
+      last_arrive();
     }
   }
   // ---------------------------------------------------------------- teardown
   if (!kPack) pdl_launch_dependents();                 // (the packed rows of a prefill may be inputs that the next kernel reads at once)
   __syncwarp();
   cluster_wait();                                      // nobody sends to this CTA or reads from it any more
+  if (__builtin_expect(*failed, 0)) give_up<D, kPack>(p.cu_k, p.sel_idx, p.packed_k, p.packed_v, p.K_tot, p.Hkv, p.csize);
   tc_fence_before();
   __syncthreads();
   if (warp == kIssueWarp) {

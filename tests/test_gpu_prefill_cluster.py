@@ -173,3 +173,35 @@ def test_expired_wait_ends_cleanly_and_the_next_call_is_correct():
         assert gpu_ops.read_status(st) == ((1 << sg.SG_ERR_TIMEOUT) if fault else 0)
     want = oracle.score(q_h, k_h, cu)
     assert np.all(np.abs(imp.cpu().numpy() - want) <= 1e-4 * np.abs(want) + 1e-30)
+
+
+def test_expired_wait_leaves_no_earlier_rows():
+    """The entries and packed rows of the parts that gave up are -1 and zero, not those of the buffers' previous prompt; the others are right."""
+    import torch
+    import gpu_ops
+    import paper_2607_28150_b200.binding as sg
+    rng = np.random.default_rng(8)
+    lens, budgets, Hkv, d = (2000, 500, 90), (200, 50, 90), 2, 64        # the last one keeps the whole prompt
+    cu, ck = cu_of(lens), cu_of(budgets)
+    T, K = int(cu[-1]), int(ck[-1])
+    q_h, k_h, v_h = rand_bf16(rng, (1, 3, 16, 8, d)), rand_bf16(rng, (1, T, Hkv, d)), rand_bf16(rng, (1, T, Hkv, d))
+    shp, st = gpu_ops.shape_of(1, 8, Hkv, d, 16, cu), gpu_ops.status_word()
+    assert sg.sg_testing_score_cluster(shp) > 0
+    imp = torch.zeros((1, Hkv, T), device="cuda")
+    sel = gpu_ops.Guarded((1, Hkv, K), torch.int32, 3)
+    pk, pv = (gpu_ops.Guarded((1, K * Hkv, d), torch.int16, 77) for _ in range(2))
+    try:
+        sg.sg_testing_score_fault(withhold_unit=1, wait_limit_ms=10)
+        sg.prefill(shp, gpu_ops.dev(q_h), gpu_ops.dev(k_h), gpu_ops.dev(v_h), imp, sg.alloc_workspace(sg.SG_OP_SCORE, shp), gpu_ops.dev(ck), K,
+                   sel.view, pk.view, pv.view, st)
+        torch.cuda.synchronize()
+    finally:
+        sg.sg_testing_score_fault(-1, 0)
+    assert gpu_ops.read_status(st) == 1 << sg.SG_ERR_TIMEOUT
+    want = oracle.select_topk(imp.cpu().numpy(), cu, ck)
+    want_k, want_v = oracle.pack_kv(k_h, v_h, cu, want, ck)
+    want[0, 1] = -1
+    for b, n in enumerate(budgets):
+        lost = slice(int(ck[b]) * Hkv + n, int(ck[b]) * Hkv + 2 * n)      # KV head 1
+        want_k[0, lost], want_v[0, lost] = 0, 0
+    assert np.array_equal(sel.numpy(), want) and np.array_equal(pk.numpy(), want_k) and np.array_equal(pv.numpy(), want_v)
