@@ -20,13 +20,15 @@ extern "C" {
 /*
  * sg_testing_score_fault -- make the scoring kernel's bounded waits observable.
  *   withhold_unit   >= 0: the row statistics that pass 1 gathers for this (layer * H_kv + kv_head) unit are computed
- *                   but never handed to the warps that publish them, whose wait runs out; -1: off.
+ *                   but never handed to the warps that publish them, whose wait runs out (calls that run as one kernel: one
+ *                   CTA of each of the unit's clusters does not send its own to the others); -1: off.
  *   wait_limit_ms   > 0: every bounded wait in the kernels gives up after this many milliseconds instead of about a
  *                   second; 0: the normal limit.  The time of earlier kernels does not count: a wait of the second kernel that
  *                   runs out first waits for the first kernel and then starts its limit once more.
  * A wait that gives up sets the SG_ERR_TIMEOUT bit in the call's device status word; its CTA stops taking work,
  * waits (bounded) for its own outstanding copies and MMAs, frees its tensor memory and returns.  The importance
- * array is then only partly written.  Nothing traps and nothing spins without a limit.
+ * array is then only partly written (and where one kernel also selects and packs, the entries and rows of the parts that
+ * gave up are -1 and zero).  Nothing traps and nothing spins without a limit.
  */
 void sg_testing_score_fault(int32_t withhold_unit, int32_t wait_limit_ms);
 

@@ -68,7 +68,7 @@ struct ClusterParams {
   int64_t T, ls, ts, hs;
   int32_t K_tot, B, Hkv, G, W, R, Ralloc;
   int32_t csize, own, cap;               // CTAs per part; most tiles of a CTA; key tiles that it holds at a time
-  int32_t withhold_unit;                 // testing only: the statistics of this unit are never sent (-1 = none)
+  int32_t withhold_unit;                 // testing only: the first CTA never sends the statistics of this unit (-1 = none)
   uint32_t wait_ns;
   float scale_log2;
 };
@@ -157,8 +157,14 @@ __device__ __noinline__ void tell_failed(uint32_t failed, int csize) {
 // All CTAs of a cluster of which one has given up.  It does not know its entries, so none of the part's rows may pass for selected ones.
 // (Out of line, as tell_failed: inside the kernel they cost every call 0.5 us.)
 template <int D, bool kPack>
-__device__ __noinline__ void give_up(const int32_t* cu_k, int32_t* sel_idx, uint16_t* packed_k, uint16_t* packed_v, int K_tot, int Hkv, int csize) {
-  cluster_arrive_release();                            // behind what the other CTAs have packed
+__device__ __noinline__ void give_up(uint32_t bar_rec, uint32_t bar_val, uint32_t wait_ns, const int32_t* cu_k, int32_t* sel_idx, uint16_t* packed_k,
+                                     uint16_t* packed_v, int K_tot, int Hkv, int csize) {
+  // What the CTAs had sent one another may still be on its way, and nobody may have waited for it: no CTA leaves before it has landed
+  // everywhere.  What was never sent ends the wait at its limit, long behind the landing of what was.
+  const uint64_t t0 = global_timer_ns();
+  while (!(mbar_test_cluster(bar_rec) && (!kPack || mbar_test_cluster(bar_val))) && global_timer_ns() - t0 <= wait_ns) {}
+  __syncwarp();
+  cluster_arrive_release();                            // (behind what the other CTAs have packed, too)
   cluster_wait();
   if (!kPack || threadIdx.x >= kWork) return;
   const int l = blockIdx.z, b = blockIdx.y / Hkv, g = blockIdx.y - b * Hkv, ck = cu_k[b], kb = cu_k[b + 1] - ck;
@@ -277,10 +283,8 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  // "this CTA runs and its barriers are set up": awaited before the first push.  The arrival of the warp that wrote `failed` releases
-  // it: 0.3 us, which this warp has.
-  if (warp == kLoadWarp) cluster_arrive_release();
-  else cluster_arrive();
+  // "this CTA runs and its barriers are set up": awaited before the first push.  (The warp that wrote `failed` arrives below, releasing it.)
+  if (warp != kLoadWarp) cluster_arrive();
   const uint32_t tmem_base = *tmem_slot;
   auto wait = [&](uint32_t bar, uint32_t parity) {
     if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return true;
@@ -293,6 +297,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
 
   if (warp == kLoadWarp) {
     // ------------------------------------------------------------ TMA producer (one thread)
+    cluster_arrive_release();
     if (lane == 0 && n_my > 0) {
       for (int i = p.cap; i < n_my && load_ok; ++i) load(i, i / p.cap);
       for (int i = n_my - p.cap - 1; i >= 0 && load_ok; --i) load(i, phase2(i));
@@ -422,7 +427,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
     ok = work_sync(ok);
     // ---- exchange: every CTA gets every CTA's statistics
     cluster_wait();                                    // all CTAs of the cluster run
-    if (ok && u != p.withhold_unit) {
+    if (ok && (u != p.withhold_unit || rank != 0)) {
       for (int r = tid & 127; r < (kTwice ? 64 : p.Ralloc); r += 128) {
         float m[8], M = -INFINITY, L = 0.f;
 #pragma unroll
@@ -756,7 +761,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
   if (!kPack) pdl_launch_dependents();                 // (the packed rows of a prefill may be inputs that the next kernel reads at once)
   __syncwarp();
   cluster_wait();                                      // nobody sends to this CTA or reads from it any more
-  if (__builtin_expect(*failed, 0)) give_up<D, kPack>(p.cu_k, p.sel_idx, p.packed_k, p.packed_v, p.K_tot, p.Hkv, p.csize);
+  if (__builtin_expect(*failed, 0)) give_up<D, kPack>(bar_rec, bar_val, p.wait_ns, p.cu_k, p.sel_idx, p.packed_k, p.packed_v, p.K_tot, p.Hkv, p.csize);
   tc_fence_before();
   __syncthreads();
   if (warp == kIssueWarp) {

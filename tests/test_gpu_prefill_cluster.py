@@ -205,3 +205,39 @@ def test_expired_wait_leaves_no_earlier_rows():
         lost = slice(int(ck[b]) * Hkv + n, int(ck[b]) * Hkv + 2 * n)      # KV head 1
         want_k[0, lost], want_v[0, lost] = 0, 0
     assert np.array_equal(sel.numpy(), want) and np.array_equal(pk.numpy(), want_k) and np.array_equal(pv.numpy(), want_v)
+
+
+def test_calls_right_behind_one_that_gave_up():
+    """What the CTAs of a part have sent one another has landed when the part ends, also where one of them did not send: calls queued
+    directly behind, whose CTAs take over the shared memory, are right."""
+    import torch
+    import gpu_ops
+    import paper_2607_28150_b200.binding as sg
+    rng = np.random.default_rng(9)
+    cu, ck = cu_of((2000,)), cu_of((200,))
+    q, k = gpu_ops.dev(rand_bf16(rng, (1, 1, 16, 32, 64))), gpu_ops.dev(rand_bf16(rng, (1, 2000, 8, 64)))
+    shp = gpu_ops.shape_of(1, 32, 8, 64, 16, cu)
+    assert sg.sg_testing_score_cluster(shp) > 1
+    ws, d_ck = sg.alloc_workspace(sg.SG_OP_SCORE, shp), gpu_ops.dev(ck)
+
+    def call():
+        out = [torch.zeros((1, 8, 2000), device="cuda"), torch.zeros((1, 8, 200), dtype=torch.int32, device="cuda"),
+               torch.zeros((1, 1600, 64), dtype=torch.int16, device="cuda"), torch.zeros((1, 1600, 64), dtype=torch.int16, device="cuda")]
+        st = gpu_ops.status_word()
+        sg.prefill(shp, q, k, k, out[0], ws, d_ck, 200, out[1], out[2], out[3], st)
+        return out, st
+
+    want, st = call()
+    assert gpu_ops.read_status(st) == 0
+    for unit in (0, 3, 7, 3):
+        try:
+            sg.sg_testing_score_fault(withhold_unit=unit, wait_limit_ms=2)
+            bad, bad_st = call()
+            sg.sg_testing_score_fault(-1, 0)
+            after = [call() for _ in range(3)]
+        finally:
+            sg.sg_testing_score_fault(-1, 0)
+        assert gpu_ops.read_status(bad_st) == 1 << sg.SG_ERR_TIMEOUT
+        assert bool((bad[1][0, unit] == -1).all()) and not bad[2][0, 200 * unit:200 * unit + 200].any()
+        for got, st in after:
+            assert gpu_ops.read_status(st) == 0 and all(torch.equal(x, y) for x, y in zip(got, want))
