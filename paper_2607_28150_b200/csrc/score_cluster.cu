@@ -826,6 +826,7 @@ ClusterPlan plan_cluster(const sg_shape* s, int Ralloc, bool packs) {
   ClusterPlan pl{};
   const int64_t parts = (int64_t)s->num_layers * s->batch * s->num_kv_heads;
   if (parts > kNumSMs) return pl;
+  if (packs && s->batch == 1 && s->max_seqlen < s->total_tokens) return pl;      // broken promise: the selection says so
   const int longest = s->batch == 1 ? s->total_tokens : s->max_seqlen, tiles = longest / kTileKeys + (longest % kTileKeys != 0);
   int cs = kMaxCluster;
   while (cs > 1 && (cs > tiles || parts * cs > kNumSMs || parts > clusters_at_once(cs))) --cs;

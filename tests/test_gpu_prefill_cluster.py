@@ -241,3 +241,33 @@ def test_calls_right_behind_one_that_gave_up():
         assert bool((bad[1][0, unit] == -1).all()) and not bad[2][0, 200 * unit:200 * unit + 200].any()
         for got, st in after:
             assert gpu_ops.read_status(st) == 0 and all(torch.equal(x, y) for x, y in zip(got, want))
+
+
+@pytest.mark.parametrize("max_seqlen", [300, 2999, 3000])
+def test_single_sequence_above_what_max_seqlen_promised(max_seqlen):
+    """As the calls one by one: flagged, no entries, zero rows, where the selection chosen from max_seqlen cannot hold the row."""
+    import torch
+    import gpu_ops
+    import paper_2607_28150_b200.binding as sg
+    rng = np.random.default_rng(10)
+    cu, ck = cu_of((3000,)), cu_of((300,))
+    q, k = gpu_ops.dev(rand_bf16(rng, (1, 1, 16, 8, 64))), gpu_ops.dev(rand_bf16(rng, (1, 3000, 2, 64)))
+    shp, d_ck = gpu_ops.shape_of(1, 8, 2, 64, 16, cu), gpu_ops.dev(ck)
+    shp.max_seqlen = max_seqlen
+    ws = sg.alloc_workspace(sg.SG_OP_SCORE, shp)
+    results = []
+    for together in (True, False):
+        imp, st = torch.zeros((1, 2, 3000), device="cuda"), gpu_ops.status_word()
+        sel = torch.zeros((1, 2, 300), dtype=torch.int32, device="cuda")
+        pk, pv = (torch.ones((1, 600, 64), dtype=torch.int16, device="cuda") for _ in range(2))
+        if together:
+            sg.prefill(shp, q, k, k, imp, ws, d_ck, 300, sel, pk, pv, st)
+        else:
+            sg.sg_score(shp, q, k, imp, ws, st)
+            sg.sg_select_topk(shp, imp, d_ck, 300, sel, None, st)
+            sg.sg_pack_kv(shp, k, k, sel, d_ck, 300, pk, pv, st)
+        results.append((sel, pk, pv, gpu_ops.read_status(st)))
+    for x, y in zip(results[0][:3], results[1][:3]):
+        assert torch.equal(x, y)
+    flagged = (1 << sg.SG_ERR_INVALID) | (1 << sg.SG_ERR_INDEX)
+    assert results[0][3] == results[1][3] == (flagged if max_seqlen == 300 else 0)
