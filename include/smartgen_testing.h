@@ -48,6 +48,9 @@ int32_t sg_testing_score_grid(const sg_shape* shape);
  * it for this shape on the current device; else 0. */
 int32_t sg_testing_score_cluster(const sg_shape* shape);
 
+/* CTAs per (sequence, KV head) of an attention call with these totals; two_lane != 0: a counted call with local_skip. */
+int32_t sg_testing_decode_cluster(const sg_shape* shape, int32_t total_sel, int32_t total_loc, int32_t two_lane);
+
 /*
  * sg_testing_decode_overlap -- allowed = 0: the following sg_sparse_decode_attn calls are launched without
  * programmatic stream serialization, i.e. fully ordered behind everything earlier in the stream, so that the

@@ -27,7 +27,7 @@ EXPORTED = ("sg_workspace_bytes", "sg_score", "sg_select_topk", "sg_pack_kv", "s
             "sg_score_static", "sg_select_pack_kv", "sg_select_threshold", "sg_pack_kv_counted", "sg_sparse_decode_attn_counted", "sg_split_index", "sg_profile_accumulate", "sg_block_importance",
             "sg_transfer_budget", "sg_proactive_mask", "sg_push_blocks", "sg_speculative_delivered", "sg_strerror", "sg_last_cuda_error",
             "sg_testing_score_fault", "sg_testing_score_clock", "sg_testing_score_grid", "sg_testing_score_cluster",
-            "sg_testing_decode_overlap")
+            "sg_testing_decode_cluster", "sg_testing_decode_overlap")
 SG_SCORE_STATIC_SCRATCH_BYTES = 8 << 20
 
 if not os.path.exists(LIB_PATH):
@@ -102,6 +102,8 @@ _lib.sg_testing_score_grid.restype = _i32
 _lib.sg_testing_score_grid.argtypes = [_sp]
 _lib.sg_testing_score_cluster.restype = _i32
 _lib.sg_testing_score_cluster.argtypes = [_sp]
+_lib.sg_testing_decode_cluster.restype = _i32
+_lib.sg_testing_decode_cluster.argtypes = [_sp, _i32, _i32, _i32]
 
 
 def sg_testing_score_fault(withhold_unit: int = -1, wait_limit_ms: int = 0) -> None:
@@ -126,6 +128,10 @@ def sg_testing_score_grid(shape: "Shape") -> int:
 
 def sg_testing_score_cluster(shape: "Shape") -> int:
     return int(_lib.sg_testing_score_cluster(ctypes.byref(shape)))
+
+
+def sg_testing_decode_cluster(shape: "Shape", total_sel: int, total_loc: int, two_lane: bool = False) -> int:
+    return int(_lib.sg_testing_decode_cluster(ctypes.byref(shape), total_sel, total_loc, int(two_lane)))
 
 
 def make_shape(num_layers: int, num_q_heads: int, num_kv_heads: int, head_dim: int, window: int,

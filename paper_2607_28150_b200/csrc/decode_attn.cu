@@ -532,7 +532,8 @@ constexpr int decode_smem_bytes(int D, int warps, int slots, bool cluster) {
 // A two-lane call names one row of the KV index as its packed and as its indexed list, so avg_tokens is up to twice what it
 // attends.  Planned for the row's length, the chain of split, pack and attention is slower more often than faster
 // (19 sequences of 820 entries 30.2 -> 32.7 us, 1 of 820 11.8 -> 12.3, 64 of 820 87.9 -> 83.4): it stays.
-// It does not overlap the next call, so its clusters may fill both CTAs of every SM.  That pays where the longest row is well above the
+// It does not overlap the next call, so its clusters may fill both CTAs of every SM, where two fit (up to eight query rows per KV head; with
+// sixteen the listed chain below took 36.8 -> 40.1 us, a second wave).  That pays where the longest row is well above the
 // average and its warps have five slices or more: the call lasts as long as that row.  Whole chains of split, pack and attention, 8
 // sequences of 6321 to 32061 tokens, a tenth of them required: 32.8 -> 30.0 us, four tenths 106 -> 90, d = 64 24.8 -> 21.5, 2 heads of 64
 // 14.9 -> 13.3; but 8 of 500 to 4000 tokens 11.8 -> 12.6 and, of equal lengths, 16 of 1638 entries 40.2 -> 41.1, 4 of
@@ -553,14 +554,15 @@ void decode_plan(const sg_shape* shape, int32_t total_sel, int32_t total_loc, bo
     W = 4 * avg_tokens <= 7 * 4 * kSlice * fit ? 4 : 8;
     while (cs < fit && (int64_t)cs * W * kSlice < avg_tokens) cs *= 2;
   }
-  if (two_lane && pairs <= kNumSMs && W == 8 && shape->total_tokens > 0) {
+  const bool wide_group = shape->num_q_heads / shape->num_kv_heads > 8;
+  if (two_lane && !wide_group && pairs <= kNumSMs && W == 8 && shape->total_tokens > 0) {
     const int64_t longest = (int64_t)total_sel * shape->max_seqlen / shape->total_tokens, average = total_sel / shape->batch;
     if (4 * longest >= 5 * average && longest >= 5 * kSlice * W * cs && cs < 8 && pairs * cs <= kNumSMs) cs *= 2;
   }
   *csize = cs;
   *warps = W;
   const bool streams = packed_only && W == 8 && avg_tokens >= 6 * kSlice * W * cs && (cs == 1 ? 2 * pairs > kNumSMs : 4 * pairs * cs > 3 * kNumSMs);
-  *slots = shape->num_q_heads / shape->num_kv_heads > 8 || streams ? 6 : 3;
+  *slots = wide_group || streams ? 6 : 3;
 }
 
 size_t decode_workspace_bytes(const sg_shape*, int32_t, int32_t) { return 0; }   // partials stay on chip
@@ -578,6 +580,14 @@ sg_status decode_launch(const sg_shape* shape, const void* q, const void* packed
                         int32_t* dev_status, void* stream);
 }
 }  // namespace sg
+
+extern "C" int32_t sg_testing_decode_cluster(const sg_shape* shape, int32_t total_sel, int32_t total_loc, int32_t two_lane) {
+  using namespace sg;
+  if (check_shape(shape, false) != SG_OK || total_sel < 0 || total_loc < 0) return 0;
+  int csize = 0, warps = 0, slots = 0;
+  decode_plan(shape, total_sel, total_loc, two_lane != 0, &csize, &warps, &slots);
+  return csize;
+}
 
 extern "C" void sg_testing_decode_overlap(int32_t allowed) {
   sg::g_test_decode_overlap.store(allowed, std::memory_order_relaxed);

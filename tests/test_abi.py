@@ -4,6 +4,8 @@ import ctypes
 import os
 import re
 
+import pytest
+
 import paper_2607_28150_b200.binding as sg
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -103,6 +105,24 @@ int main(void) {
                     "-L", libdir, "-lsmartgen", "-Wl,-rpath," + libdir], check=True)
     out = subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout
     assert "c caller ok" in out
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("lens,share,G,Hkv,want", [
+    # (sequence lengths, required share, query heads per KV head, KV heads) -> CTAs per (sequence, KV head)
+    ((32768, 2048, 4096, 9000), 0.1, 4, 8, 8),             # ragged, long rows: twice the CTAs that fit one per SM
+    ((32768, 2048, 4096, 9000), 0.1, 8, 8, 8),
+    ((32768, 2048, 4096, 9000), 0.1, 9, 8, 4),             # one CTA per SM fits: no second wave
+    ((32768, 2048, 4096, 9000), 0.1, 16, 8, 4),
+    ((32768, 2048, 9000, 20000, 8000, 16000, 12000, 30000), 0.1, 4, 8, 4), ((32768, 2048, 9000, 20000, 8000, 16000, 12000, 30000), 0.1, 16, 8, 2),
+    ((16000,) * 4, 0.1, 4, 8, 4),                          # equal lengths
+    ((5000, 300, 64, 77), 0.2, 4, 8, 4),                   # its longest row gives the warps fewer than five slices
+])
+def test_two_lane_clusters_fit_at_once(lens, share, G, Hkv, want, d):
+    T, K = sum(lens), sum(max(1, int(share * n)) for n in lens)
+    s = sg.Shape(1, len(lens), G * Hkv, Hkv, d, 1, T, max(lens), 0x1000, T * Hkv * d, Hkv * d, d)
+    assert sg.sg_testing_decode_cluster(s, K, K, True) == want
+    assert len(lens) * Hkv * want <= (296 if G <= 8 else 148)
 
 
 def test_debug_and_profiling_builds_of_the_scoring_kernel_compile(tmp_path):

@@ -105,6 +105,12 @@ def test_counts_equal_to_the_caps_reproduce_the_plain_calls():
     (tuple(120 + 11 * i for i in range(40)), tuple(10 + i for i in range(40)), 16, 8, 64, 0.2),
     ((2000,), (333,), 32, 2, 128, 1.0),                       # everything remote
     ((2000,), (333,), 32, 2, 128, 0.0),                       # everything local
+    # ragged and long: clusters on both CTAs of an SM, eight per pair ...
+    ((32768, 2048, 4096, 9000), (3277, 205, 410, 900), 32, 8, 128, 0.34),
+    ((32768, 2048, 4096, 9000), (3277, 205, 410, 900), 64, 8, 64, 0.5),
+    ((32768, 2048, 9000, 20000, 8000, 16000, 12000, 30000), (3277, 205, 900, 2000, 800, 1600, 1200, 3000), 16, 8, 64, 0.3),   # four per pair
+    # ... and with sixteen query heads per KV head, where one CTA per SM fits
+    ((32768, 2048, 4096, 9000), (3277, 205, 410, 900), 128, 8, 128, 0.34),
 ])
 def test_two_lane_fetching_on_the_gpu(lens, ks, Hq, Hkv, d, remote_share):
     """Section 4.2 end to end through the C ABI: Algorithm 1 (split + reorder) -> fetch the remote lane into a packed
