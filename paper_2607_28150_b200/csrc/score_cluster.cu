@@ -42,11 +42,7 @@ constexpr int kThreads = 32 * (kIssueWarp + 1);
 constexpr int kTileKeys = 128;
 constexpr int kStages = 4;               // TMEM stages of 128 columns
 constexpr int kMaxCap = 12;              // most key tiles of a CTA in shared memory at a time
-// Most key tiles of a CTA, with selection and packing and without: beyond that the two launches of score.cu, which use all SMs, take
-// less.  Whole calls in a row, 8 KV heads of 128, 128 query rows, one prompt, microseconds with the launches one by one -> in one
-// kernel: 512 tokens 17.6 -> 10.6, 2048 20.0 -> 13.6, 4096 (four tiles) 22.6 -> 17.0, 8192 (seven) 26.2 -> 24.9, 10000 (eight) 30.6 -> 28.1,
-// 12000 (ten) 31.8 -> 32.7; 256 rows, 5000 tokens 35.3 -> 25.4; 2 heads of 64, 64 rows, 1024 tokens 16.7 -> 9.5.  Scores alone: 4096
-// 12.9 -> 11.6, 6500 (six) 14.4 -> 14.9.
+// Most key tiles of a CTA, with selection and packing and without (cluster_pays says when).
 constexpr int kMaxOwn = 8, kMaxOwnScore = 4;
 constexpr int kBins = 2048;
 constexpr int kRankMax = 128;            // keys that are ranked directly
@@ -820,6 +816,27 @@ struct ClusterPlan {
   int csize, own, cap, smem;
   bool ok;
 };
+// Whether one kernel takes less than the launches one by one.  Its time is that of the CTA with the most blocks (key tiles x 128 query
+// rows): 9.5 us and, per tile, 0.65 + 1.4 us per row block.  score.cu deals the tiles of all parts out evenly, so that its time goes with
+// the tiles per SM: with one row block about 18 us with one, 24 with three, 26 with four, 30 with five; with two 22, 33, 37; with four 26
+// with one.  Up to eight tiles of single prompts and of batches of equal lengths that is the one kernel's, but a batch with one long
+// prompt among short ones leaves most of its CTAs idle.  Measured on 400 shapes, calls in a row and on keys not in L2, microseconds one by
+// one -> one kernel; taken, 32 query and 8 KV heads of 128, 128 rows: 512 tokens 16.8 -> 10.2, 2048 19.9 -> 12.6, 4096 (four tiles)
+// 22.6 -> 17.0, 8192 (seven) 25.8 -> 25.0 (keys not in L2 28.8 -> 26.5), 10000 (eight) 30.1 -> 28.3, seven of 100 and one of 1790 (seven)
+// 23.5 -> 23.2, 2040 and 100 in turn, four each (eight) 29.3 -> 25.6; 256 rows: 7500 (six) 35.2 -> 32.8, four of 1270 and of 100 (five)
+// 36.9 -> 27.5; 64 rows, heads of 64, 6000 and 100 (eight) 23.9 -> 20.8.
+// Not taken, 128 rows: seven of 100 and one of 2048 (eight) 23.3 -> 25.0, 3000 and 6000 (eight) 26.0 -> 26.8; 256 rows: seven of 100 and one of
+// 1270 (five) 24.3 -> 27.0, of 2040 28.7 -> 36.5; 512 rows, 2 heads: 20 of 100 and one of 2900 26.6 -> 58.2.
+// Scores alone, taken: 128 rows, 4096 tokens (four) 13.3 -> 11.9; 256 rows, 3000 (three) 0.86 of the time; 512 rows, 8 layers of 2000, 2 heads
+// (three) 0.90.  Not taken: 6500 (six) 14.4 -> 14.9; 256 rows, seven of 100 and one of 1000 (four) 1.18, 512 rows, 20 of 100 and one of 1000 (three) 1.30.
+bool cluster_pays(const sg_shape* s, int own, int Ralloc, bool packs) {
+  const int R = s->num_q_heads / s->num_kv_heads * s->window, blocks = own * (Ralloc / 128);
+  const double parts = (double)s->num_layers * s->batch * s->num_kv_heads;
+  const double even = (s->total_tokens / 64.0 + s->batch) * s->num_layers * s->num_kv_heads / (2 * kNumSMs);     // expected tiles per SM
+  if (!packs) return own <= kMaxOwnScore && (own == 1 || blocks <= 4 || (even >= 1 && blocks <= 4 + 5 * even));
+  if (own == kMaxOwn && !(even >= 4 || (even >= 3 && parts >= 32) || (R <= 64 && (s->head_dim == 64 || even >= 2)))) return false;
+  return own <= kMaxOwn && blocks <= 7 + 1.4 * (Ralloc / 128) * even;
+}
 // The largest cluster with which all parts are resident at once (on B200 15 clusters of 9, 11 of 10, 7 of 16), no larger than the longest
 // sequence has tiles.
 ClusterPlan plan_cluster(const sg_shape* s, int Ralloc, bool packs) {
@@ -833,7 +850,7 @@ ClusterPlan plan_cluster(const sg_shape* s, int Ralloc, bool packs) {
   if (parts > clusters_at_once(cs)) return pl;
   pl.csize = cs;
   pl.own = tiles > cs ? (tiles + cs - 1) / cs : 1;
-  if (pl.own > (packs ? kMaxOwn : kMaxOwnScore)) return pl;
+  if (!cluster_pays(s, pl.own, Ralloc, packs)) return pl;
   pl.cap = pl.own < kMaxCap ? pl.own : kMaxCap;
   while (pl.cap > 0 && carve(s->head_dim, Ralloc, cs, pl.own, pl.cap).total + 1024 > kSmemLimit) --pl.cap;
   if (pl.cap < pl.own && pl.cap < 2) return pl;        // tiles that are loaded twice need a second stage

@@ -13,7 +13,7 @@ from helpers import cu_of, rand_bf16
 pytestmark = pytest.mark.gpu
 
 
-def run(lens, L, W, Hq, Hkv, d, budgets, seed=0, k_h=None, max_seqlen=None, pad_heads=0):
+def run(lens, L, W, Hq, Hkv, d, budgets, seed=0, k_h=None, max_seqlen=None, pad_heads=0, one_kernel=True):
     import torch
     import gpu_ops
     import paper_2607_28150_b200.binding as sg
@@ -28,7 +28,7 @@ def run(lens, L, W, Hq, Hkv, d, budgets, seed=0, k_h=None, max_seqlen=None, pad_
     if max_seqlen is not None:
         shp.max_seqlen = max_seqlen
     cluster = sg.sg_testing_score_cluster(shp)
-    assert cluster > 0
+    assert (cluster > 0) == one_kernel
     q, k, v = (gpu_ops.dev(x) for x in (q_h, *wide))
     st, ws = gpu_ops.status_word(), sg.alloc_workspace(sg.SG_OP_SCORE, shp)
     imp = gpu_ops.Guarded((L, Hkv, T), torch.float32, -7.0)
@@ -66,7 +66,8 @@ def run(lens, L, W, Hq, Hkv, d, budgets, seed=0, k_h=None, max_seqlen=None, pad_
     ((1500, 40), 1, 24, 16, 2, 128, (0, 40)),                   # 192 rows; an empty budget and a whole prompt
     ((700,), 1, 5, 6, 2, 64, (33,)),                            # 15 rows
     ((640, 10), 1, 64, 16, 2, 64, (64, 9)),                     # 512 rows; nine keys of ten
-    ((15000,), 1, 16, 8, 2, 128, (2000,)),                      # sixteen CTAs, eight tiles each, two of them held at a time
+    ((15000,), 1, 16, 16, 4, 128, (2000,)),                     # sixteen CTAs, eight tiles each, two of them held at a time
+    ((14000,), 1, 16, 8, 2, 128, (2000,)),                      # ... seven
     ((100,) * 18, 1, 16, 8, 8, 64, (10,) * 18),                 # 144 parts of one CTA
     ((7000, 3000, 200), 2, 16, 4, 2, 64, (700, 2999, 1)),       # clusters whose CTAs have from none to five tiles
 ])
@@ -75,6 +76,22 @@ def test_prefill_in_one_kernel(lens, L, W, Hq, Hkv, d, budgets):
     assert status == 0
     want = oracle.score(q_h, k_h, cu)
     assert np.all(np.abs(got - want) <= 1e-4 * np.abs(want) + 1e-30)
+
+
+# (query rows, tiles of the longest prompt's CTAs, ...): where the launches one by one are faster, they are taken
+@pytest.mark.parametrize("lens,L,W,Hq,Hkv,d,one_kernel", [
+    ((8192,), 1, 32, 32, 8, 128, True), ((10000,), 1, 32, 32, 8, 128, True), ((8192,), 2, 32, 32, 8, 128, False),
+    ((15000,), 1, 16, 8, 2, 128, False),                        # two parts, eight tiles
+    ((100,) * 7 + (2048,), 1, 32, 32, 8, 128, False), ((100,) * 7 + (1790,), 1, 32, 32, 8, 128, True),
+    ((100,) * 7 + (2048,), 1, 32, 16, 8, 64, True),             # 64 rows, heads of 64
+    ((2040, 100) * 4, 1, 32, 32, 8, 128, True),
+    ((100,) * 7 + (1270,), 1, 64, 32, 8, 128, False), ((100,) * 7 + (900,), 1, 64, 32, 8, 128, True),      # 256 rows
+    ((1270, 100) * 4, 1, 64, 32, 8, 128, True),
+    ((100,) * 20 + (1900,), 1, 64, 16, 2, 64, False),           # 512 rows
+])
+def test_where_one_kernel_pays(lens, L, W, Hq, Hkv, d, one_kernel):
+    """The route, and the same results on either."""
+    assert run(lens, L, W, Hq, Hkv, d, tuple(max(1, n // 9) for n in lens), one_kernel=one_kernel)[-1] == 0
 
 
 def test_prefill_in_one_kernel_from_a_wider_cache():
