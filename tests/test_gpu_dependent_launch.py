@@ -37,10 +37,12 @@ class SlowProducer:
         sg.sg_sparse_decode_attn(self.shape, self.q, None, None, self.cu_k, 0, self.k, self.v, self.idx, self.cu_nloc, self.nloc, self.out)
 
 
+@pytest.mark.parametrize("launches", [1, 2])
 @pytest.mark.parametrize("late", ["keys", "queries"])
-def test_score_waits_for_a_producer_that_lets_it_start_early(late):
+def test_score_waits_for_a_producer_that_lets_it_start_early(late, launches):
     """One sequence and few key tiles leave SMs free for both scoring kernels while the producer of the keys, or of the
-    window queries, is still running: neither may read them before it has ended."""
+    window queries, is still running: neither may read them before it has ended.  sg_score takes one kernel for such a shape,
+    sg_score_static always two."""
     import torch
     import gpu_ops
     import paper_2607_28150_b200.binding as sg
@@ -53,10 +55,17 @@ def test_score_waits_for_a_producer_that_lets_it_start_early(late):
     q = make.out.view(1, 1, W, heads, d) if late == "queries" else gpu_ops.dev(rand_bf16(rng, (1, 1, W, heads, d)))
     shp = gpu_ops.shape_of(1, heads, heads, d, W, cu_of((T,)))
     ws = sg.alloc_workspace(sg.SG_OP_SCORE, shp)
+    assert sg.sg_testing_score_cluster(shp) > 0
+
+    def call(imp, st):
+        if launches == 1:
+            sg.sg_score(shp, q, k, imp, ws, st)
+        else:
+            sg.sg_score_static(shp, q, k, imp, st)
 
     def score():
         imp, st = torch.full((1, heads, T), -1.0, dtype=torch.float32, device="cuda"), gpu_ops.status_word()
-        sg.sg_score(shp, q, k, imp, ws, st)
+        call(imp, st)
         return imp, st
 
     early, _ = score()                                    # on the zeros that the producer will overwrite
@@ -66,10 +75,54 @@ def test_score_waits_for_a_producer_that_lets_it_start_early(late):
         imp, st = torch.full((1, heads, T), -1.0, dtype=torch.float32, device="cuda"), gpu_ops.status_word()
         torch.cuda.synchronize()
         make()
-        sg.sg_score(shp, q, k, imp, ws, st)
+        call(imp, st)
         assert gpu_ops.read_status(st) == 0
         want, _ = score()                                 # again, when everything has been written
         assert torch.equal(imp, want) and not torch.allclose(want, early, rtol=1e-3)
+
+
+@pytest.mark.parametrize("late", ["keys", "values", "queries"])
+def test_prefill_waits_for_a_producer_that_lets_it_start_early(late):
+    """The same for the kernel that also selects and packs."""
+    import torch
+    import gpu_ops
+    import paper_2607_28150_b200.binding as sg
+    rng = np.random.default_rng(24)
+    heads, d, n = 2, 128, 4
+    make = SlowProducer(n, heads, d)
+    T, W = (300, n) if late == "queries" else (n, 2)
+    made = {"keys": make.out.view(1, n, heads, d), "values": make.out.view(1, n, heads, d), "queries": make.out.view(1, 1, n, heads, d)}[late]
+    k, v = (made if late == name else gpu_ops.dev(rand_bf16(rng, (1, T, heads, d))) for name in ("keys", "values"))
+    q = made if late == "queries" else gpu_ops.dev(rand_bf16(rng, (1, 1, W, heads, d)))
+    K = T - 1
+    shp, ck = gpu_ops.shape_of(1, heads, heads, d, W, cu_of((T,))), gpu_ops.dev(cu_of((K,)))
+    ws = sg.alloc_workspace(sg.SG_OP_SCORE, shp)
+    assert sg.sg_testing_score_cluster(shp) > 0
+
+    def prefill():
+        out = [torch.full((1, heads, T), -1.0, device="cuda"), torch.full((1, heads, K), -9, dtype=torch.int32, device="cuda")]
+        out += [torch.full((1, K * heads, d), 5, dtype=torch.int16, device="cuda") for _ in range(2)]
+        st = gpu_ops.status_word()
+        torch.cuda.synchronize()
+        return out, st, lambda: sg.prefill(shp, q, k, v, out[0], ws, ck, K, out[1], out[2], out[3], st)
+
+    def finished():
+        out, st, run = prefill()
+        run()
+        assert gpu_ops.read_status(st) == 0
+        return out
+
+    make.out.zero_()
+    early = finished()                                     # on the zeros that the producer will overwrite
+    for _ in range(3):
+        make.out.zero_()
+        got, st, run = prefill()
+        make()
+        run()
+        assert gpu_ops.read_status(st) == 0
+        want = finished()                                  # again, when everything has been written
+        assert all(torch.equal(x, y) for x, y in zip(got, want))
+        assert not all(torch.equal(x, y) for x, y in zip(want, early))
 
 
 def test_pass_2_of_scoring_waits_as_long_as_pass_1_takes():

@@ -193,27 +193,31 @@ def test_decode_rings_of_short_lists():
     ("query", 4), ("query", 6), ("query", 31), ("query", 127),             # row of the block: exponentials on either pipe
     ("key", 5), ("key", 6), ("key", 262), ("key", 1279), ("key", 1299),    # the same for keys; the last ones are not seen by all rows
 ])
-def test_score_non_finite_input_marks_its_part(value, where, at):
+@pytest.mark.parametrize("W,launches", [(32, 1), (32, 2), (13, 1), (13, 2)])               # 128 query rows; 52, which stand twice
+def test_score_non_finite_input_marks_its_part(value, where, at, W, launches):
     """A NaN or an infinity in one query or key makes every importance of its (layer, KV head, sequence) NaN, wherever it
-    stands, and changes nothing else."""
+    stands, and changes nothing else.  sg_score takes one kernel for such a shape, sg_score_static always two."""
     import torch
     import gpu_ops
     import paper_2607_28150_b200.binding as sg
     rng = np.random.default_rng(14)
-    L, lens, W, Hq, Hkv, d = 2, (700, 1300), 32, 8, 2, 128
+    L, lens, Hq, Hkv, d = 2, (700, 1300), 8, 2, 128
     G, l, b, g = Hq // Hkv, 1, 1, 1
+    at = at % (G * W) if where == "query" else at
     cu = cu_of(lens)
     q = gpu_ops.dev(rand_bf16(rng, (L, 2, W, Hq, d))).view(torch.bfloat16)
     k = gpu_ops.dev(rand_bf16(rng, (L, int(cu[-1]), Hkv, d))).view(torch.bfloat16)
     shp = gpu_ops.shape_of(L, Hq, Hkv, d, W, cu)
     ws, st = sg.alloc_workspace(sg.SG_OP_SCORE, shp), gpu_ops.status_word()
     clean, got = (torch.empty((L, Hkv, int(cu[-1])), dtype=torch.float32, device="cuda") for _ in range(2))
-    sg.sg_score(shp, q, k, clean, ws, st)
+    assert sg.sg_testing_score_cluster(shp) > 0
+    score = (lambda out: sg.sg_score(shp, q, k, out, ws, st)) if launches == 1 else (lambda out: sg.sg_score_static(shp, q, k, out, st))
+    score(clean)
     if where == "query":
         q[l, b, at // G, g * G + at % G, 3] = value
     else:
         k[l, int(cu[b]) + at, g, 3] = value
-    sg.sg_score(shp, q, k, got, ws, st)
+    score(got)
     assert gpu_ops.read_status(st) == 0
     part = torch.zeros_like(got, dtype=torch.bool)
     part[l, g, int(cu[b]):int(cu[b + 1])] = True
