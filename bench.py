@@ -302,7 +302,7 @@ def layerwise_prefill_timing(dev, hp, d_q, d_k, d_v, reps=5):
     one = graph_ms(None)
     two = graph_ms(torch.cuda.Stream(device=dev))
     return {"one_stream_ms": one, "two_stream_ms": two, "layers": hp.L,
-            "note": "4 kernels per layer (scoring 2, selection, packing); compare with score+select+pack of the all-layer calls in stage_ms"}
+            "note": "one stream: one kernel per layer where a layer's parts fit the chip at once, else scoring, selection and packing; two streams: selection and packing beside the next layer's scoring; compare with score+select+pack of the all-layer calls in stage_ms"}
 
 
 def full_first_two_timing(dev, cfg, d_q, d_k, d_v, reps=5):

@@ -68,7 +68,7 @@ def native_stamp() -> str:
 
 def native_is_current() -> bool:
     src = os.path.join(CSRC, "native.cpp")
-    newest = max(os.path.getmtime(p) for p in (src, os.path.join(INCLUDE, "smartgen.h"), os.path.abspath(__file__)))
+    newest = max(os.path.getmtime(p) for p in (src, os.path.join(CSRC, "internal.h"), os.path.join(INCLUDE, "smartgen.h"), os.path.abspath(__file__)))
     if not os.path.exists(NATIVE) or os.path.getmtime(NATIVE) < newest:
         return False
     with open(NATIVE, "rb") as f:

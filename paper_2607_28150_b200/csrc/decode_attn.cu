@@ -535,7 +535,7 @@ constexpr int decode_smem_bytes(int D, int warps, int slots, bool cluster) {
 // It does not overlap the next call, so its clusters may fill both CTAs of every SM, where two fit (up to eight query rows per KV head; with
 // sixteen the listed chain below took 36.8 -> 40.1 us, a second wave).  That pays where the longest row is well above the
 // average and its warps have five slices or more: the call lasts as long as that row.  Whole chains of split, pack and attention, 8
-// sequences of 6321 to 32061 tokens, a tenth of them required: 32.8 -> 30.0 us, four tenths 106 -> 90, d = 64 24.8 -> 21.5, 2 heads of 64
+// sequences of 6321 to 32061 tokens, a tenth of them required: 33.0 -> 30.6 us, four tenths 106 -> 90, d = 64 24.8 -> 21.5, 2 heads of 64
 // 14.9 -> 13.3; but 8 of 500 to 4000 tokens 11.8 -> 12.6 and, of equal lengths, 16 of 1638 entries 40.2 -> 41.1, 4 of
 // 1638 18.1 -> 18.5, which the rule leaves as they are.
 void decode_plan(const sg_shape* shape, int32_t total_sel, int32_t total_loc, bool two_lane, int* csize, int* warps, int* slots) {

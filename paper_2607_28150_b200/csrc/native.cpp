@@ -12,10 +12,7 @@
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
-#include "smartgen.h"
-
-extern "C" sg_status sg_internal_score_select_pack(const sg_shape*, const void*, const void*, const void*, float*, void*, size_t, const int32_t*, int32_t,
-                                                   int32_t*, void*, void*, int32_t*, void*);
+#include "internal.h"
 
 namespace {
 

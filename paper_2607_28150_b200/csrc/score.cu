@@ -31,6 +31,7 @@
 #include <cuda.h>
 
 #include "common.cuh"
+#include "internal.h"
 #include "launch.h"
 #include "score_launch.h"
 #include "score_math.cuh"
@@ -940,8 +941,6 @@ extern "C" sg_status sg_score(const sg_shape* shape, const void* q_win, const vo
   return sg::run_score(shape, q_win, k_cache, importance, workspace, workspace_bytes, 0, nullptr, dev_status, stream);
 }
 
-// sg_score, then sg_select_pack_kv, where one kernel does both; SG_ERR_UNSUPPORTED, with nothing launched, for everything else, bad
-// arguments included (the two calls then say what is wrong).  For the sequences of native.cpp.
 extern "C" sg_status sg_internal_score_select_pack(const sg_shape* shape, const void* q_win, const void* k_cache, const void* v_cache,
                                                    float* importance, void* workspace, size_t workspace_bytes, const int32_t* cu_k,
                                                    int32_t total_sel, int32_t* sel_idx, void* packed_k, void* packed_v,

@@ -22,8 +22,9 @@
 // All sixteen worker warps share every block: a block is 128 x 128 scores in one TMEM stage, warp w takes the lanes of quarter
 // w mod 4 and the columns of quarter w / 4, so that one tile per CTA keeps all schedulers busy.
 //
-// Every wait is bounded, as in score.cu: on expiry the CTA raises SG_ERR_TIMEOUT, waits (bounded) for its own TMA copies and
-// MMAs, frees its TMEM and returns.
+// Every wait on an mbarrier is bounded, as in score.cu: on expiry the CTA raises SG_ERR_TIMEOUT, tells the other CTAs of its cluster, waits
+// (bounded) for its own TMA copies and MMAs and for what is on its way to it, frees its TMEM and returns.  The cluster barriers have no
+// limit of their own: every warp of every CTA arrives at each of them on every path.
 #include <cuda.h>
 
 #include "common.cuh"
@@ -41,7 +42,6 @@ constexpr int kLoadWarp = kWorkWarps, kIssueWarp = kLoadWarp + 1;
 constexpr int kThreads = 32 * (kIssueWarp + 1);
 constexpr int kTileKeys = 128;
 constexpr int kStages = 4;               // TMEM stages of 128 columns
-constexpr int kMaxCap = 12;              // most key tiles of a CTA in shared memory at a time
 // Most key tiles of a CTA, with selection and packing and without (cluster_pays says when).
 constexpr int kMaxOwn = 8, kMaxOwnScore = 4;
 constexpr int kBins = 2048;
@@ -49,7 +49,7 @@ constexpr int kRankMax = 128;            // keys that are ranked directly
 constexpr int kSweeps = (kMaxOwn * kTileKeys + kWork - 1) / kWork;
 constexpr int kCandAt = (24 + kSweeps * kWorkWarps + 3) & ~3;
 constexpr int kFailedAt = kCandAt + kRankMax + 4, kMiscWords = kFailedAt + 4;
-constexpr int kBars = 2 * kMaxCap + 16;
+constexpr int kBars = 2 * kMaxOwn + 16;
 
 struct ClusterParams {
   const int32_t* cu;
@@ -100,10 +100,6 @@ __device__ __forceinline__ uint32_t at_rank(uint32_t addr, int rank) {
 }
 __device__ __forceinline__ void push2(uint32_t addr, uint32_t bar, uint32_t a, uint32_t b) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(addr), "r"(a), "r"(b), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void push4(uint32_t addr, uint32_t bar, uint4 v) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
-               ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar) : "memory");
 }
 // A barrier of the workers that also agrees on whether all of them are well.
 __device__ __forceinline__ bool work_sync(bool ok) {
@@ -195,7 +191,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_co
   auto bar_afull = [&](uint32_t s) { return bar0 + 8u * (8 + s); };
   auto bar_aempty = [&](uint32_t s) { return bar0 + 8u * (12 + s); };
   auto bar_kfull = [&](uint32_t s) { return bar0 + 8u * (16 + s); };
-  auto bar_kempty = [&](uint32_t s) { return bar0 + 8u * (16 + kMaxCap + s); };
+  auto bar_kempty = [&](uint32_t s) { return bar0 + 8u * (16 + kMaxOwn + s); };
   uint32_t* const tmem_slot = misc;
   volatile int* const abort_flag = reinterpret_cast<volatile int*>(misc + 1);
   uint32_t* const sh = misc + 2;                       // [0] chosen bin, [1] remaining need, [2] keys in it, [3] gathered, [4] threshold, [5] need
@@ -851,7 +847,7 @@ ClusterPlan plan_cluster(const sg_shape* s, int Ralloc, bool packs) {
   pl.csize = cs;
   pl.own = tiles > cs ? (tiles + cs - 1) / cs : 1;
   if (!cluster_pays(s, pl.own, Ralloc, packs)) return pl;
-  pl.cap = pl.own < kMaxCap ? pl.own : kMaxCap;
+  pl.cap = pl.own;
   while (pl.cap > 0 && carve(s->head_dim, Ralloc, cs, pl.own, pl.cap).total + 1024 > kSmemLimit) --pl.cap;
   if (pl.cap < pl.own && pl.cap < 2) return pl;        // tiles that are loaded twice need a second stage
   pl.smem = carve(s->head_dim, Ralloc, cs, pl.own, pl.cap).total + 1024;

@@ -187,8 +187,8 @@ __global__ void __launch_bounds__(kSelThreads, 1) select_topk_kernel(const SelPa
 // ------------------------------------------------------------------------------------------------
 // Register-resident variant for rows of up to 32768 tokens: thread t owns E consecutive positions
 // [t*E, (t+1)*E) and keeps their keys in registers (16-byte loads from the boundary at or before the
-// row's start).  At most three histogram passes of
-// 2048 bins over a shrinking key interval find the k-th largest key exactly; after the first pass only the few
+// row's start).  Histogram passes over a shrinking key interval find the k-th largest key exactly, at most three of 2048 bins
+// (512 threads and more; four of 1024 or 512 with 256 or 128); after the first pass only the few
 // keys inside the threshold bin take part.  Because ownership is contiguous, one block-wide prefix sum over
 // per-thread (greater, equal) counts gives every thread the output offset of its first selected position, and
 // it writes its positions in ascending order from two bit masks.
@@ -399,8 +399,8 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
     __syncthreads();                                   // histogram cleared
   }
 
-  // ---- exact k-th largest key by narrowing a key interval [lo, hi] that holds it, 11 bits of the interval per pass.
-  // The digit of a pass is (key - lo) >> shift with shift chosen so that the interval spans at most 2048 bins:
+  // ---- exact k-th largest key by narrowing a key interval [lo, hi] that holds it, kBinBits bits of the interval per pass.
+  // The digit of a pass is (key - lo) >> shift with shift chosen so that the interval spans at most kRegBins bins:
   // unlike the fixed top bits of a float, it spreads whatever range the row really has over all bins, so the
   // threshold bin of the first pass keeps tens of keys, not a quarter of the row, and the later passes touch few.
   if constexpr (kThr) {                                // the keys of -inf .. +inf: everything outside is a NaN
@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(T) select_topk_reg_kernel(const SelParams p) {
       if (((vmask >> e) & 1u) && rel <= width) atomicAdd(&my_hist[rel >> shift], 1u);
     }
     __syncthreads();
-    // suffix search: thread t looks at bins 2047-t*bpt ... (descending) for the bin holding the need-th largest
+    // suffix search: thread t looks at bins kRegBins-1-t*kBpt ... (descending) for the bin holding the need-th largest
     constexpr int kBpt = kRegBins / T;
     uint32_t c[kBpt];
     const int bin0 = kRegBins - 1 - tid * kBpt;        // this thread's highest bin; it owns bin0, bin0-1, ...

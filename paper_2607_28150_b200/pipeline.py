@@ -3,8 +3,9 @@
 `HotPath` owns the device buffers of one batch of prompts -- importance, KV index, packed K/V,
 workspaces, status word -- and issues the library calls in the order of the path:
 
-    prefill side:  sg_score -> sg_select_topk -> sg_pack_kv      (all layers in one call each, or layer by
-                                                                   layer with select+pack on a second stream)
+    prefill side:  sg_score -> sg_select_pack_kv                 (all layers, or layer by layer; calls that fit the chip at once
+                                                                   are one kernel; with a second stream, sg_score there and
+                                                                   sg_select_topk -> sg_pack_kv beside the next layer's)
     decode side :  sg_sparse_decode_attn                          (one call per layer per step)
 
 No arithmetic of the method happens here; every step runs in the library's CUDA kernels.
